@@ -27,6 +27,7 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kVec = 8;                 // elements per lane per step
 constexpr int kChunk = 32 * kVec;       // one warp step = one inverse-CDF chunk (256 elements)
 constexpr int kMaxSplit = 32;
+constexpr int kMaxGamma = 16;           // SPECKV_MAX_GAMMA
 // Measured on b256 (same box, the two builds in turn, five times): 5 CTAs x 3 loads 156.7 us, 4 x 4 161.6 us,
 // 5 x 4 163.6 us, 6 x 3 161.9 us; b256_g8 and b1024_loop the same within 0.1 %.
 constexpr int kSweepLoads = 3;  // 16-byte loads in flight per thread (bf16); fp32 uses half as many vector steps
@@ -806,12 +807,11 @@ struct RowDecide {
     double lse2_q, lse2_p;  // log2-normalisers of draft and target
     int amax;         // greedy rows: argmax of the target row
     bool dbad, tbad;  // non-finite draft row / target row at this position
-    bool badtok, accept, any_dbad;
+    bool badtok, accept;
 };
 
-// The per-position part of the row epilogue: lane i < n_lanes merges the nd partials at pd (draft position
-// i) and the nt partials at pt (target position i) and takes the acceptance test of its position.  One
-// compiled body serves the row epilogue and the prefix epilogue below, so that both reach the same bits.
+// The per-position part of the row epilogue for one warp: lane i < n_lanes merges the nd partials at pd (draft
+// position i) and the nt partials at pt (target position i) and takes the acceptance test of its position.
 template <typename T>
 __device__ __noinline__ void row_decide(const KParams& P, int b, int gam, float Tf, int status, int n_lanes,
                                         const float4* pd, int nd, const float4* pt, int nt, RowDecide& o) {
@@ -862,7 +862,6 @@ __device__ __noinline__ void row_decide(const KParams& P, int b, int gam, float 
     double lse2_q = 0.0, lse2_p = 0.0;
     int amax = -1;
     bool dbad = false, tbad = false, accept = true;  // non-finite draft row / target row at this lane's position
-    bool any_dbad = false;
 
     if (!status) {
         // Partials are merged in fp32 with the same branch-free rules the sweep uses; the draft and
@@ -902,10 +901,9 @@ __device__ __noinline__ void row_decide(const KParams& P, int b, int gam, float 
                 else lse2_p = static_cast<double>(at.x) + log2_split(static_cast<double>(at.y));
             }
         }
-        any_dbad = __any_sync(0xffffffffu, dbad);
     }
 
-    if (status == 0 && !any_dbad && tok_on && !badtok && !tbad) {
+    if (status == 0 && !dbad && tok_on && !badtok && !tbad) {
         if (greedy) {
             accept = (x == amax);
         } else {
@@ -917,58 +915,175 @@ __device__ __noinline__ void row_decide(const KParams& P, int b, int gam, float 
         }
     }
     o.x = x; o.u_res = u_res; o.Hi = Hi; o.ci = ci; o.lse2_q = lse2_q; o.lse2_p = lse2_p; o.amax = amax;
-    o.dbad = dbad; o.tbad = tbad; o.badtok = badtok; o.accept = accept; o.any_dbad = any_dbad;
+    o.dbad = dbad; o.tbad = tbad; o.badtok = badtok; o.accept = accept;
 }
 
-// Prefix epilogue (one warp): run when the partials of a batch row's first positions 0..k are in, while
+// The same for one position by one warp of a CTA that has all its warps at hand (the sliced sweep): lanes 0-15 gather
+// the draft row's partials, lanes 16-31 the target row's, so that up to 32 slices cost one memory round trip and four
+// shuffle steps instead of a chain of them, and one double-precision log2 serves draft row, target row and uniform.
+// Latency-bound: one batch row in 15 slices (fp32, V = 32,000, gamma 4), with a lane per position the prefix and the row
+// epilogue each walked a chain of 11 dependent round trips and the step took 45.1 us; this way 23.0 us.  256 rows of
+// bf16, V = 128,256: 150.5 -> 145.6 us (the chain is also the end of a large step).  The prefix epilogue and the row epilogue call this one compiled body, so that both reach the same bits.
+template <typename T>
+__device__ __noinline__ void decide_position(const KParams& P, int b, int gam, float Tf, int i, const float4* pd,
+                                             const float4* pt, int n, RowDecide& o) {
+    const int lane = threadIdx.x & 31, k = lane & 15;
+    const bool tgt_half = lane >= 16;
+    const bool verify = (P.mode & MODE_VERIFY) != 0;
+    const bool greedy = (Tf == 0.f);
+    const float scale = static_cast<float>(kLog2e / static_cast<double>(greedy ? 1.f : Tf));
+    const bool dr_on = i < gam, tok_on = verify && i < gam;
+
+    // ---- one round trip ----
+    const bool on = tgt_half ? verify : dr_on;
+    const float4* src = tgt_half ? pt : pd;
+    const float4 none = tgt_half && greedy ? make_float4(kFloor, __int_as_float(0x7fffffff), 0.f, 0.f)
+                                           : make_float4(tgt_half ? -3.0e38f : kFloor, 0.f, 0.f, 0.f);
+    float4 a = (on && k < n) ? ldcg4(src + k) : none;
+    const float4 a2 = (on && k + 16 < n) ? ldcg4(src + k + 16) : none;
+    int x = -1;
+    float u_acc = 0.f, u_res = 0.f;
+    float2 tl = make_float2(0.f, 0.f);
+    {
+        const long long at = static_cast<long long>(b) * P.G + i;
+        const long long urow = (static_cast<long long>(b) * (P.G + 1) + i) * 2;
+        if (tok_on) {
+            x = __ldg(P.tok + at);
+            u_acc = __ldg(P.u + urow);
+            if (!greedy) tl = __ldcg(P.tokl + at);  // left by the sweep CTA of the draft position
+        }
+        if (verify) u_res = __ldg(P.u + urow + 1);
+    }
+
+    int amax = -1;
+    bool tbad = false;
+    if (greedy && verify) {  // uniform across the warp; the draft half goes along and is not looked at
+        float4 g = merge_argmax(a, a2);
+#pragma unroll
+        for (int m = 8; m > 0; m >>= 1) g = merge_argmax(g, shfl_xor4(g, m));
+        amax = __shfl_sync(0xffffffffu, __float_as_int(g.y), 16);
+        const float best = __shfl_sync(0xffffffffu, g.x, 16), bad = __shfl_sync(0xffffffffu, g.z, 16);
+        tbad = bad != 0.f || amax == 0x7fffffff || !(best > kFloor);
+    }
+    // draft partial: (m, cnt, Zx, S); target partial (r, Z): both as (reference, cnt, Z, S) with the reference in log2 units
+    // for the target half
+    const float sc = tgt_half ? 1.f : scale;
+    if (tgt_half) {
+        a.z = a.y; a.y = 0.f; a.w = 0.f;
+    }
+    float4 c2 = a2;
+    if (tgt_half) {
+        c2.z = c2.y; c2.y = 0.f; c2.w = 0.f;
+    }
+    float M = fmaxf(a.x, c2.x);
+#pragma unroll
+    for (int m = 8; m > 0; m >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, m));
+    float cnt = 0.f, Z = 0.f, S = 0.f;
+    auto add = [&](const float4& v) {
+        const float dm = v.x - M, f = ex2f(dm * sc), za = v.y + v.z;
+        const bool top = v.x == M;  // below the maximum a count joins the scaled sum
+        cnt += top ? v.y : 0.f;
+        Z += top ? v.z : za * f;
+        S += top ? v.w : fmaf(dm, za, v.w) * f;
+    };
+    add(a);
+    add(c2);
+#pragma unroll
+    for (int m = 8; m > 0; m >>= 1) {
+        cnt += __shfl_xor_sync(0xffffffffu, cnt, m);
+        Z += __shfl_xor_sync(0xffffffffu, Z, m);
+        S += __shfl_xor_sync(0xffffffffu, S, m);
+    }
+    // lane 0: draft normaliser, lane 16: target normaliser, lane 8: accept uniform (lane 8 sees the draft sums)
+    const double arg = lane == 8 ? static_cast<double>(u_acc) : static_cast<double>(cnt) + static_cast<double>(Z);
+    const double l2 = log2_split(arg);
+    const double l2_p = __shfl_sync(0xffffffffu, l2, 16), l2_u = __shfl_sync(0xffffffffu, l2, 8);
+    const float Rp = __shfl_sync(0xffffffffu, M, 16), Zp = __shfl_sync(0xffffffffu, Z, 16);
+    if (lane != 0) return;
+
+    float Hi = 0.f, ci = 0.f;
+    double lse2_q = 0.0, lse2_p = 0.0;
+    bool dbad = false, accept = true;
+    if (dr_on) {
+        const float Zall = cnt + Z;
+        if (!(cnt >= 1.f) || !(Zall < 3e38f) || !(M > kFloor)) {
+            dbad = true;
+        } else {
+            const float lnZ = (cnt == 1.f) ? log1pf(Z) : logf(cnt) + log1pf(Z / cnt);
+            const float rZ = 1.f / Zall;
+            Hi = fmaxf(lnZ - static_cast<float>(kLn2) * scale * S * rZ, 0.f);
+            ci = rZ;
+            lse2_q = static_cast<double>(M) * static_cast<double>(scale) + l2;
+        }
+    }
+    if (verify && !greedy) {
+        if (!(Zp > 0.f) || !(Zp < 3e38f)) tbad = true;
+        else lse2_p = static_cast<double>(Rp) + l2_p;
+    }
+    const bool badtok = tok_on && (x < 0 || x >= P.V);
+    if (tok_on && !dbad && !badtok && !tbad) {
+        if (greedy) {
+            accept = (x == amax);
+        } else {
+            const double sd = static_cast<double>(scale);
+            const double lq = static_cast<double>(tl.x) * sd - lse2_q, lp = static_cast<double>(tl.y) * sd - lse2_p;
+            accept = (l2_u + lq) < lp;  // u * q(x) < p(x); u = 0: log2 is -inf
+        }
+    }
+    o.x = x; o.u_res = u_res; o.Hi = Hi; o.ci = ci; o.lse2_q = lse2_q; o.lse2_p = lse2_p; o.amax = amax;
+    o.dbad = dbad; o.tbad = tbad; o.badtok = badtok; o.accept = accept;
+}
+
+// Prefix epilogue (a whole CTA): run when the partials of a batch row's first positions 0..k are in, while
 // the rest of the row is still being swept.  It takes the acceptance tests of those positions and
 // publishes where the walk stops if it stops there, so that CTAs which have not started yet can leave
 // target rows behind that position unread.  early[b] = stop position + 1, or G + 2 when the walk passes k.
 template <typename T>
-__device__ __noinline__ void prefix_epilogue(const KParams& P, int b, int gam, float Tf) {
-    const int lane = threadIdx.x & 31;
+__device__ __forceinline__ void prefix_epilogue(const KParams& P, int b, int gam, float Tf, RowDecide* pos) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long row0 = static_cast<long long>(b) * P.J;
-    RowDecide d;
-    row_decide<T>(P, b, gam, Tf, 0, P.k_early + 1, P.part + (row0 + P.G + 1 + lane) * P.nsplit, P.nsplit,
-                  P.part + (row0 + lane) * P.nsplit, P.nsplit, d);
-    const bool in = lane <= P.k_early && lane <= gam;
-    const unsigned stop = __ballot_sync(0xffffffffu, in && (d.tbad || d.dbad || (lane < gam && (d.badtok || !d.accept))));
-    if (lane == 0) {
-        const int e = stop ? __ffs(stop) : P.G + 2;
-        asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(P.early + b), "r"(e) : "memory");
+    if (warp <= P.k_early && warp <= gam)
+        decide_position<T>(P, b, gam, Tf, warp, P.part + (row0 + P.G + 1 + warp) * P.nsplit, P.part + (row0 + warp) * P.nsplit,
+                           P.nsplit, pos[warp]);
+    __syncthreads();
+    if (warp == 0) {
+        bool ends = false;
+        if (lane <= P.k_early && lane <= gam) {
+            const RowDecide& d = pos[lane];
+            ends = d.tbad || d.dbad || (lane < gam && (d.badtok || !d.accept));
+        }
+        const unsigned stop = __ballot_sync(0xffffffffu, ends);
+        if (lane == 0) {
+            const int e = stop ? __ffs(stop) : P.G + 2;
+            asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(P.early + b), "r"(e) : "memory");
+        }
     }
+    __syncthreads();  // pos is used again when the same CTA completes the row
 }
 
-// Row epilogue: one warp, run by whoever learns that all partials of batch row b are in.  Lane i
-// merges the nd partials at pd (draft position i) and the nt partials at pt (target position i).
-// gam and Tf are the row's gamma and temperature as the sweep read them.  Everything the row
-// needs from memory that does not depend on other loads is requested first, so the epilogue
-// costs one memory round trip (two when the sweep did not leave the logits at the draft tokens).
+// Status bits a row's gamma and temperature give by themselves.
+__device__ __forceinline__ int row_status0(const KParams& P, int gam, float Tf) {
+    return (gam < 1 || gam > P.G ? 1 : 0) | (!(Tf >= 0.f) || Tf == __int_as_float(0x7f800000) ? 8 : 0);
+}
+
+// Second half of a row epilogue (one warp): the walk over the positions, every output of the row except a drawn token.
+// dec: what lane i has learned about position i; ctl: the controller's parameters, fetched beforehand.
 // Order: what the resample kernel needs (acceptance, stop position, normalisers), the row's
 // completion flag, then the signals and the controller.
-template <typename T>
-__device__ __noinline__ void row_epilogue(const KParams& P, int b, int gam, float Tf, const float4* pd, int nd,
-                                          const float4* pt, int nt) {
+__device__ __noinline__ void row_finish(const KParams& P, int b, int gam, float Tf, const RowDecide& dec, const CtlRegs& ctl) {
     const int lane = threadIdx.x & 31;
     const int G = P.G;
     const bool verify = (P.mode & MODE_VERIFY) != 0;
-
-    int status = 0;
-    if (gam < 1 || gam > G) status |= 1;
-    if (!(Tf >= 0.f) || Tf == __int_as_float(0x7f800000)) status |= 8;
+    int status = row_status0(P, gam, Tf);
     const bool greedy = (Tf == 0.f);
     const float scale = static_cast<float>(kLog2e / static_cast<double>(greedy ? 1.f : Tf));
     const bool tg_on = !status && verify && lane <= gam;
-
-    CtlRegs ctl;
-    if ((P.mode & MODE_MLP) && !status) ctl = ctl_load(P, b, lane);
-    RowDecide dec;
-    row_decide<T>(P, b, gam, Tf, status, 32, pd, nd, pt, nt, dec);
     const int x = dec.x;
     const float u_res = dec.u_res, Hi = dec.Hi, ci = dec.ci;
     const double lse2_q = dec.lse2_q, lse2_p = dec.lse2_p;
     const int amax = dec.amax;
-    const bool tbad = dec.tbad, badtok = dec.badtok, accept = dec.accept, any_dbad = dec.any_dbad;
+    const bool tbad = dec.tbad, badtok = dec.badtok, accept = dec.accept;
+    const bool any_dbad = __any_sync(0xffffffffu, dec.dbad);
 
     // The positions are walked in order; the walk ends at the first one whose target row is non-finite
     // (which flags the row), whose draft token is out of range, or whose token is rejected.  Target rows
@@ -1040,6 +1155,44 @@ __device__ __noinline__ void row_epilogue(const KParams& P, int b, int gam, floa
             if (lane == 0) P.gamma_next[b] = 0;
         }
     }
+}
+
+// Row epilogue: one warp, run by whoever learns that all partials of batch row b are in (ring sweep, sharded step).
+// Lane i merges the nd partials at pd (draft position i) and the nt partials at pt (target position i).
+// gam and Tf are the row's gamma and temperature as the sweep read them.  Everything the row
+// needs from memory that does not depend on other loads is requested first, so the epilogue
+// costs one memory round trip (two when the sweep did not leave the logits at the draft tokens).
+template <typename T>
+__device__ __noinline__ void row_epilogue(const KParams& P, int b, int gam, float Tf, const float4* pd, int nd,
+                                          const float4* pt, int nt) {
+    const int status = row_status0(P, gam, Tf);
+    CtlRegs ctl;
+    if ((P.mode & MODE_MLP) && !status) ctl = ctl_load(P, b, threadIdx.x & 31);
+    RowDecide dec;
+    row_decide<T>(P, b, gam, Tf, status, 32, pd, nd, pt, nt, dec);
+    row_finish(P, b, gam, Tf, dec, ctl);
+}
+
+// Row epilogue of the sliced sweep: a whole CTA, a warp per position.
+template <typename T>
+__device__ __forceinline__ void row_epilogue_cta(const KParams& P, int b, int gam, float Tf, RowDecide* pos) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool verify = (P.mode & MODE_VERIFY) != 0;
+    const long long row0 = static_cast<long long>(b) * P.J;
+    const int n_pos = row_status0(P, gam, Tf) ? 0 : verify ? gam + 1 : gam;
+    // the parameters travel while the positions are decided; warp 0 takes the last turns, so it has the fewest positions
+    CtlRegs ctl;
+    if (warp == 0 && (P.mode & MODE_MLP) && n_pos) ctl = ctl_load(P, b, lane);
+    for (int i = kWarps - 1 - warp; i < n_pos; i += kWarps)
+        decide_position<T>(P, b, gam, Tf, i, P.part + (row0 + (verify ? P.G + 1 + i : i)) * P.nsplit, P.part + (row0 + i) * P.nsplit,
+                           P.nsplit, pos[i]);
+    __syncthreads();
+    if (warp != 0) return;
+    RowDecide dec;
+    dec.x = -1; dec.u_res = 0.f; dec.Hi = dec.ci = 0.f; dec.lse2_q = dec.lse2_p = 0.0; dec.amax = -1;
+    dec.dbad = dec.tbad = dec.badtok = false; dec.accept = true;
+    if (lane < n_pos) dec = pos[lane];
+    row_finish(P, b, gam, Tf, dec, ctl);
 }
 
 // Epilogue of the draft-side sampling sweep (one warp per batch row): lane i merges the partials
@@ -1142,7 +1295,8 @@ __global__ void __launch_bounds__(kThreads, kSweepCtasPerSm) sweep_kernel(const 
         return;
     }
     __shared__ float4 sh_part[kWarps];
-    __shared__ int sh_count;
+    __shared__ RowDecide sh_pos[kMaxGamma + 1];
+    __shared__ int sh_last;
     __shared__ int sh_early;
     __shared__ float sh_m0[kWarps];
     asm volatile("griddepcontrol.launch_dependents;");  // a dependent resample kernel may be scheduled as SMs free up
@@ -1182,7 +1336,6 @@ __global__ void __launch_bounds__(kThreads, kSweepCtasPerSm) sweep_kernel(const 
     int gam = P.gamma ? P.gamma[b] : P.G;
     float Tf = P.temp ? P.temp[b] : P.temp_scalar;
     if (threadIdx.x == 0) {
-        sh_count = 0;
         // one thread reads what is known of the row's stop position, so that the whole CTA takes one decision
         int e = 0;
         if (gen == 2 && !P.read_all)
@@ -1210,8 +1363,7 @@ __global__ void __launch_bounds__(kThreads, kSweepCtasPerSm) sweep_kernel(const 
     const bool skipped = active && gen == 2 && sh_early != 0 && sh_early <= P.k_early + 1;
     if (skipped) {
         // the row epilogue never looks behind the stop position; the partial only has to be finite
-        if (warp != 0) return;
-        if (lane == 0)
+        if (threadIdx.x == 0)
             SPECKV_ST(P.part[pidx], greedy ? make_float4(kFloor, __int_as_float(0x7fffffff), 0.f, 0.f)
                                            : make_float4(kFloor, 0.f, 0.f, 0.f));
     } else if (active) {
@@ -1246,64 +1398,50 @@ __global__ void __launch_bounds__(kThreads, kSweepCtasPerSm) sweep_kernel(const 
             part = sweep_warp<T, ALIGNED, PATH_DRAFT, U, STEP>(row, lo, hi, first, scale, sh_m0);
             path = PATH_DRAFT;
         }
-        // the last warp of the CTA to finish merges the eight warp partials; nobody waits
-        int last = 0;
-        if (lane == 0) {
-            sh_part[warp] = part;
-            __threadfence_block();
-            last = (atomicAdd(&sh_count, 1) == kWarps - 1);
+        if (lane == 0) sh_part[warp] = part;
+        __syncthreads();
+        if (warp == 0) {
+            const float4 none = (path == PATH_ARGMAX) ? make_float4(kFloor, __int_as_float(0x7fffffff), 0.f, 0.f)
+                              : make_float4(path == PATH_TARGET ? -3.0e38f : kFloor, 0.f, 0.f, 0.f);
+            const float4 w = lane < kWarps ? sh_part[lane] : none;
+            const float4 acc = (path == PATH_DRAFT) ? warp_merge<PATH_DRAFT>(w, scale)
+                             : (path == PATH_TARGET) ? warp_merge<PATH_TARGET>(w, scale) : warp_merge<PATH_ARGMAX>(w, scale);
+            if (lane == 0) SPECKV_ST(P.part[pidx], acc);
         }
-        if (!__shfl_sync(0xffffffffu, last, 0)) return;
-        if (lane == 0) {
-            __threadfence_block();
-            const volatile float4* vp = sh_part;
-            float4 acc = make_float4(vp[0].x, vp[0].y, vp[0].z, vp[0].w);
-            for (int w = 1; w < kWarps; ++w) {
-                float4 o = make_float4(vp[w].x, vp[w].y, vp[w].z, vp[w].w);
-                acc = (path == PATH_DRAFT) ? merge_draft(acc, o, scale)
-                    : (path == PATH_TARGET) ? merge_target(acc, o) : merge_argmax(acc, o);
-            }
-            SPECKV_ST(P.part[pidx], acc);
-        }
-        if (P.early && gen == 0) {
-            // first generation: the last of the row's CTAs of positions 0..k_early takes their acceptance tests
-            const int n_pre = (min(P.k_early, gam) + 1 + min(P.k_early + 1, gam)) * P.nsplit;
-            int last_pre = 0;
-            if (lane == 0) {
-                __threadfence();
-                last_pre = (atomicAdd(P.tick_early + b, 1) == n_pre - 1);
-            }
-            if (__shfl_sync(0xffffffffu, last_pre, 0)) {
-                __threadfence();
-                prefix_epilogue<T>(P, b, gam, Tf);
-            }
-        }
-    } else if (row_ok || rem != 0 || warp != 0) {
+    } else if (row_ok || rem != 0) {
         return;  // unused position: nothing to count; a flagged row keeps its first CTA for the epilogue
     }
 
-    // ticket: the last of the row's active CTAs runs the row epilogue; nobody waits
-    const int n_rows = P.sample ? gam : (verify ? 2 * gam + 1 : gam);
-    const int n_tickets = row_ok ? n_rows * P.nsplit : 1;
-    const long long row0 = static_cast<long long>(b) * P.J;
-    int last_row = 0;
-    if (lane == 0) {
+    // tickets: the last of the row's CTAs of positions 0..k_early takes their acceptance tests, the last of all its active
+    // CTAs runs the row epilogue; nobody waits
+    if (threadIdx.x == 0) {
+        const int n_rows = P.sample ? gam : (verify ? 2 * gam + 1 : gam);
+        const int n_tickets = row_ok ? n_rows * P.nsplit : 1;
+        const int n_pre = (min(P.k_early, gam) + 1 + min(P.k_early + 1, gam)) * P.nsplit;
         __threadfence();
-        last_row = (atomicAdd(P.tick1 + b, 1) == n_tickets - 1);
+        int pre = -1;
+        if (P.early && active && gen == 0) pre = atomicAdd(P.tick_early + b, 1);
+        const int all = atomicAdd(P.tick1 + b, 1);
+        const int l = (all == n_tickets - 1 ? 2 : 0) | (pre == n_pre - 1 ? 1 : 0);
+        if (l) __threadfence();
+        sh_last = l;
     }
-    if (!__shfl_sync(0xffffffffu, last_row, 0)) return;
-    __threadfence();
+    __syncthreads();
+    const int last = sh_last;
+    if (last & 1) prefix_epilogue<T>(P, b, gam, Tf, sh_pos);
+    if (!(last & 2)) return;
+    const long long row0 = static_cast<long long>(b) * P.J;
     if (P.sample) {
-        sample_epilogue(P, b, gam, Tf, P.part + (row0 + lane) * P.nsplit, P.nsplit);
+        if (warp == 0) sample_epilogue(P, b, gam, Tf, P.part + (row0 + lane) * P.nsplit, P.nsplit);
         return;
     }
     if (P.export_state) {
-        export_epilogue(P, b, gam, Tf, P.part + (row0 + P.G + 1 + lane) * P.nsplit, P.nsplit,
-                           P.part + (row0 + lane) * P.nsplit, P.nsplit);
+        if (warp == 0)
+            export_epilogue(P, b, gam, Tf, P.part + (row0 + P.G + 1 + lane) * P.nsplit, P.nsplit,
+                            P.part + (row0 + lane) * P.nsplit, P.nsplit);
         return;
     }
-    row_epilogue<T>(P, b, gam, Tf, P.part + (row0 + (verify ? P.G + 1 + lane : lane)) * P.nsplit, P.nsplit,
-                    P.part + (row0 + lane) * P.nsplit, P.nsplit);
+    row_epilogue_cta<T>(P, b, gam, Tf, sh_pos);
 }
 
 // ----------------------------------------------------------------------------------------
