@@ -28,7 +28,6 @@ inline size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 struct Plan {
     int J_full;      // logit rows per batch row with verification: 2*G + 1
-    int nvec;        // kVec-element vectors per logit row
     int nchunk;      // 256-element chunks per logit row
     int R;           // resample CTAs per batch row
     int chunks_per_cta;
@@ -69,22 +68,29 @@ cudaError_t dbg_register(cudaStream_t cs, const speckv_batch* bt, bool target, c
 #endif
 }
 
-// vocabulary slices per logit row for a sweep over J logit rows per batch row
-int choose_nsplit(int B, int J, int V, speckv_dtype dt) {
-    const int nvec = (V + kVec - 1) / kVec;
-    const double row_bytes = static_cast<double>(V) * esize(dt);
-    int ns = static_cast<int>(std::lround(row_bytes / static_cast<double>(kSliceBytes)));
+// Vocabulary slices per logit row for a sweep over J logit rows per batch row, one CTA each, and the granules that one
+// warp takes of a slice: P.nsplit, P.per_warp.  aligned: every row starts on the 16-byte grid.
+void choose_slices(KParams& P, speckv_dtype dt, bool aligned) {
+    const int E = 16 / esize(dt);
+    const int ng = (P.V + E - 1 + (aligned ? 0 : E - 1)) / E;  // granules a row can touch
+    int ns = static_cast<int>(std::lround(16.0 * ng / static_cast<double>(kSliceBytes)));
     if (ns < 1) ns = 1;
     // small batches: enough CTAs to put a few on every SM
-    const long long rows = static_cast<long long>(B) * J;
+    const long long rows = static_cast<long long>(P.B) * P.J;
     const long long want = (1184 + rows - 1) / (rows > 0 ? rows : 1);
     if (want > ns) ns = static_cast<int>(want > kMaxSplit ? kMaxSplit : want);
     if (ns > kMaxSplit) ns = kMaxSplit;
-    // at least one vector per thread in a slice
-    int cap = nvec / kThreads;
-    if (cap < 1) cap = 1;
-    if (ns > cap) ns = cap;
-    return ns;
+    // At least one granule per lane; short ranges are whole rounds of the warp (a round with idle lanes costs as much as a
+    // full one), long ones keep to 128-byte lines.  Rounding down makes more slices: only where they still fit the small-batch
+    // count (500 rows of V = 3,000, bf16, gamma 4: 52 us with one slice per logit row, 68 us with two).
+    int pw = (ng + ns * kWarps - 1) / (ns * kWarps);
+    const int near = (pw + 16) / 32 * 32 < 32 ? 32 : (pw + 16) / 32 * 32;
+    if (pw >= 256) pw = (pw + 7) / 8 * 8;
+    else if (((ng + near * kWarps - 1) / (near * kWarps)) * rows <= 1184 + rows) pw = near;
+    else pw = (pw + 31) / 32 * 32;
+    while ((ng + pw * kWarps - 1) / (pw * kWarps) > kMaxSplit) pw += 32;
+    P.per_warp = pw;
+    P.nsplit = (ng + pw * kWarps - 1) / (pw * kWarps);
 }
 
 constexpr int kEarlyPositions = 2;   // positions whose acceptance tests the sliced sweep takes ahead of the rest of the row
@@ -94,7 +100,6 @@ Plan make_plan(const speckv_batch* bt) {
     Plan p;
     const size_t B = static_cast<size_t>(bt->B);
     p.J_full = 2 * bt->gamma_max + 1;
-    p.nvec = (bt->V + kVec - 1) / kVec;
     p.nchunk = (bt->V + kChunk - 1) / kChunk;
     p.R = (p.nchunk + kRsChunksPerCta - 1) / kRsChunksPerCta;
     if (p.R > 32) p.R = 32;
@@ -275,9 +280,10 @@ speckv_status run(const speckv_batch* bt, int mode, const float* comp, const spe
     KParams P{};
     P.B = bt->B; P.G = bt->gamma_max; P.V = bt->V;
     P.J = verify ? pl.J_full : bt->gamma_max;
-    P.nsplit = choose_nsplit(P.B, P.J, P.V, bt->dtype);
-    P.nvec = pl.nvec;
-    P.per_split = (pl.nvec + P.nsplit - 1) / P.nsplit;
+    const int es = esize(bt->dtype);
+    bool aligned = rows_aligned(bt->draft_logits, bt->draft_stride_b, bt->draft_stride_pos, es);
+    if (verify) aligned = aligned && rows_aligned(bt->target_logits, bt->target_stride_b, bt->target_stride_pos, es);
+    choose_slices(P, bt->dtype, aligned);
     P.nchunk = pl.nchunk; P.R = pl.R; P.chunks_per_cta = pl.chunks_per_cta;
     {
         // small batches: more, shorter shares per row, so that the draw of a handful of rows still spreads
@@ -315,9 +321,6 @@ speckv_status run(const speckv_batch* bt, int mode, const float* comp, const spe
 
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     if (dbg_register(cs, bt, verify, ws, ws_bytes) != cudaSuccess) return SPECKV_ERR_CUDA;
-    const int es = esize(bt->dtype);
-    bool aligned = rows_aligned(bt->draft_logits, bt->draft_stride_b, bt->draft_stride_pos, es);
-    if (verify) aligned = aligned && rows_aligned(bt->target_logits, bt->target_stride_b, bt->target_stride_pos, es);
     const long long row_bytes = static_cast<long long>(P.V) * es;
 
     if (cudaMemsetAsync(P.tick1, 0, (6 * static_cast<size_t>(P.B) + 4) * sizeof(int), cs) != cudaSuccess)
@@ -397,9 +400,8 @@ speckv_status run_sample(const speckv_batch* bt, const float* uniforms, int32_t*
     KParams P{};
     P.B = bt->B; P.G = bt->gamma_max; P.V = bt->V;
     P.J = bt->gamma_max;
-    P.nsplit = choose_nsplit(P.B, P.J, P.V, bt->dtype);
-    P.nvec = (bt->V + kVec - 1) / kVec;
-    P.per_split = (P.nvec + P.nsplit - 1) / P.nsplit;
+    const bool aligned = rows_aligned(bt->draft_logits, bt->draft_stride_b, bt->draft_stride_pos, esize(bt->dtype));
+    choose_slices(P, bt->dtype, aligned);
     P.nchunk = pl.nchunk; P.R = pl.R; P.chunks_per_cta = pl.chunks_per_cta;
     P.mode = MODE_SAMPLE; P.sample = 1; P.rs_reverse = 1;
     P.wait_limit = g_wait_limit.load(std::memory_order_relaxed);
@@ -423,8 +425,6 @@ speckv_status run_sample(const speckv_batch* bt, const float* uniforms, int32_t*
     if (dbg_register(cs, bt, false, ws, ws_bytes) != cudaSuccess) return SPECKV_ERR_CUDA;
     const size_t n_tick = static_cast<size_t>(P.B) * (2 + static_cast<size_t>(P.G));
     if (cudaMemsetAsync(P.tick1, 0, n_tick * sizeof(int), cs) != cudaSuccess) return SPECKV_ERR_CUDA;
-    const int es = esize(bt->dtype);
-    const bool aligned = rows_aligned(bt->draft_logits, bt->draft_stride_b, bt->draft_stride_pos, es);
 constexpr int kSampleCtas = 2368;
     // One pass (speckv_sample.cuh) whenever a row's chunk records fit the searching CTA's shared memory.
     if (P.nchunk <= kRsStage &&
@@ -491,13 +491,12 @@ cudaError_t static_scratch_address(void** out) {
 
 // ---- vocabulary-sharded verification (speckv_shard.cuh) ----
 struct ShardPlan {
-    int nvec, nchunk, R, chunks_per_cta;
+    int nchunk, R, chunks_per_cta;
     size_t off_tick, off_part, off_csum, off_csum2, total;
 };
 ShardPlan make_shard_plan(const speckv_batch* bt) {
     ShardPlan p;
     const size_t B = static_cast<size_t>(bt->B), J = 2 * static_cast<size_t>(bt->gamma_max) + 1;
-    p.nvec = (bt->V + kVec - 1) / kVec;
     p.nchunk = (bt->V + kChunk - 1) / kChunk;
     p.R = (p.nchunk + kRsChunksPerCta - 1) / kRsChunksPerCta;
     if (p.R > 32) p.R = 32;
@@ -523,7 +522,7 @@ speckv_status shard_params(const speckv_batch* bt, void* ws, size_t ws_bytes, KP
     if (!ws || reinterpret_cast<uintptr_t>(ws) % kAlign != 0) return SPECKV_ERR_INVALID_ARG;
     if (ws_bytes < pl.total) return SPECKV_ERR_WORKSPACE;
     P.B = bt->B; P.G = bt->gamma_max; P.V = bt->V; P.J = 2 * bt->gamma_max + 1;
-    P.nvec = pl.nvec; P.nchunk = pl.nchunk; P.R = pl.R; P.chunks_per_cta = pl.chunks_per_cta;
+    P.nchunk = pl.nchunk; P.R = pl.R; P.chunks_per_cta = pl.chunks_per_cta;
     P.mode = MODE_VERIFY; P.bits = bt->entropy_in_bits ? 1 : 0;
     P.d = bt->draft_logits; P.dsb = bt->draft_stride_b; P.dsp = bt->draft_stride_pos;
     P.t = bt->target_logits; P.tsb = bt->target_stride_b; P.tsp = bt->target_stride_pos;
@@ -731,8 +730,8 @@ speckv_status speckv_shard_sweep(const speckv_batch* local, int64_t v_begin, flo
     speckv_status st = shard_params(local, workspace, workspace_bytes, P, pl);
     if (st != SPECKV_OK || local->B == 0) return st;
     if (!shard_state || !shard_tokl || v_begin < 0 || v_begin > (1LL << 30)) return SPECKV_ERR_INVALID_ARG;
-    P.nsplit = choose_nsplit(P.B, P.J, P.V, local->dtype);
-    P.per_split = (P.nvec + P.nsplit - 1) / P.nsplit;
+    const bool al = shard_aligned(local);
+    choose_slices(P, local->dtype, al);
     if (static_cast<long long>(P.B) * P.J * P.nsplit > 0x7fffffffLL) return SPECKV_ERR_UNSUPPORTED;
     P.n_sweep = P.B * P.J * P.nsplit;
     P.v_begin = static_cast<int>(v_begin);
@@ -751,7 +750,6 @@ speckv_status speckv_shard_sweep(const speckv_batch* local, int64_t v_begin, flo
         return SPECKV_ERR_CUDA;
     const unsigned grid = static_cast<unsigned>(P.n_sweep);
     constexpr int Ub = kSweepLoads, Uf = (kSweepLoads + 1) / 2;
-    const bool al = shard_aligned(local);
     // A slice row is short (V / n_shards columns).  One CTA per short row is mostly overhead and the
     // ring sweep pays per logit row as well (segment hand-over to its epilogue warp), so rows of up to
     // 64 KB are swept by one warp each, all of them resident at once; wider slices take the
@@ -760,11 +758,9 @@ speckv_status speckv_shard_sweep(const speckv_batch* local, int64_t v_begin, flo
     if (row_bytes <= kShardWarpRowBytes) {
         const unsigned g2 = static_cast<unsigned>((static_cast<long long>(P.B) * P.J + kWarps - 1) / kWarps);
         if (local->dtype == SPECKV_BF16) {
-            if (al) shard_rows_kernel<__nv_bfloat16, true, Ub><<<g2, kThreads, 0, cs>>>(P);
-            else shard_rows_kernel<__nv_bfloat16, false, Ub><<<g2, kThreads, 0, cs>>>(P);
+            shard_rows_kernel<__nv_bfloat16, Ub><<<g2, kThreads, 0, cs>>>(P);
         } else {
-            if (al) shard_rows_kernel<float, true, Uf><<<g2, kThreads, 0, cs>>>(P);
-            else shard_rows_kernel<float, false, Uf><<<g2, kThreads, 0, cs>>>(P);
+            shard_rows_kernel<float, Uf><<<g2, kThreads, 0, cs>>>(P);
         }
         return cudaGetLastError() == cudaSuccess ? SPECKV_OK : SPECKV_ERR_CUDA;
     }

@@ -190,20 +190,6 @@ __device__ __forceinline__ void unit_elems(int gran0, int unit, int lane, int& e
     }
 }
 
-// argmax step whose two halves of kVec/2 elements start at element ea and eb
-template <typename T>
-__device__ __forceinline__ void argmax_step_split(ArgmaxState& as, const Raw<T>& raw, int ea, int eb) {
-    if (!raw_exceeds<false>(raw, as.best)) return;
-    float x[kVec];
-    unpack<T>(raw, x);
-#pragma unroll
-    for (int j = 0; j < kVec; ++j) {
-        const int idx = (j < kVec / 2) ? ea + j : eb + j - kVec / 2;
-        as.bad |= (x[j] != x[j]) || (x[j] == __int_as_float(0x7f800000));
-        if (x[j] > as.best || (x[j] == as.best && idx < as.idx)) { as.best = x[j]; as.idx = idx; }
-    }
-}
-
 // ---- per-warp sweep state -------------------------------------------------------------------
 // The running maximum M is the same in all 32 lanes of a warp, so a stage is checked once (one
 // warp-wide maximum over everything the warp holds of the stage) instead of once per vector, no
@@ -345,7 +331,7 @@ __device__ __forceinline__ void pipe_fold_rare(const uint4* stage, int n_gran, i
         if (path == PATH_ARGMAX) {
             int ea, eb;
             unit_elems<T>(gran0, unit, lane, ea, eb);
-            argmax_step_split<T>(st.as, raw, ea, eb);
+            st.as.template step<T>(raw, ea, eb);
             continue;
         }
         const float um = raw_max(raw);

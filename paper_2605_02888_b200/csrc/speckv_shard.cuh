@@ -19,7 +19,7 @@ namespace speckv {
 // Phase 1 for short slice rows: one warp per (batch row, logit row), every warp on its own row with
 // U loads of 16 bytes in flight per lane; the warp's merged state is the shard's state of that row.
 // No partials, no tickets.  (Wider slices use sweep_kernel with export_state set.)
-template <typename T, bool ALIGNED, int U>
+template <typename T, int U>
 __global__ void __launch_bounds__(kThreads, kSweepCtasPerSm) shard_rows_kernel(const __grid_constant__ KParams P) {
     const int lane = threadIdx.x & 31;
     const long long w = static_cast<long long>(blockIdx.x) * kWarps + (threadIdx.x >> 5);
@@ -38,11 +38,11 @@ __global__ void __launch_bounds__(kThreads, kSweepCtasPerSm) shard_rows_kernel(c
         if (is_target) {
             const T* row = static_cast<const T*>(P.t) + static_cast<long long>(b) * P.tsb + static_cast<long long>(pos) * P.tsp;
             if (greedy) {
-                st = sweep_warp<T, ALIGNED, PATH_ARGMAX, U, 32, false>(row, 0, P.V, lane, scale, nullptr);
+                st = sweep_warp<T, PATH_ARGMAX, U, false>(make_row(row, P.V), 0, 0x7fffffff, scale, nullptr);
                 const int idx = __float_as_int(st.y);
                 if (idx != 0x7fffffff) st.y = __int_as_float(idx + P.v_begin);
             } else {
-                st = sweep_warp<T, ALIGNED, PATH_TARGET, U, 32, false>(row, 0, P.V, lane, scale, nullptr);
+                st = sweep_warp<T, PATH_TARGET, U, false>(make_row(row, P.V), 0, 0x7fffffff, scale, nullptr);
             }
         } else {
             const T* row = static_cast<const T*>(P.d) + static_cast<long long>(b) * P.dsb + static_cast<long long>(pos) * P.dsp;
@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(kThreads, kSweepCtasPerSm) shard_rows_kernel(c
                     SPECKV_ST(P.tokl[static_cast<long long>(b) * P.G + pos], make_float2(elem_to_float(row, x), elem_to_float(trow, x)));
                 }
             }
-            st = sweep_warp<T, ALIGNED, PATH_DRAFT, U, 32, false>(row, 0, P.V, lane, scale, nullptr);
+            st = sweep_warp<T, PATH_DRAFT, U, false>(make_row(row, P.V), 0, 0x7fffffff, scale, nullptr);
         }
     }
     if (lane == 0) P.state[static_cast<long long>(b) * P.J + j] = st;

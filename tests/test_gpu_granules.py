@@ -1,0 +1,52 @@
+"""Rows that start and end off the 16-byte grid: the sweep loads whole 16-byte granules and takes only a row's incomplete
+first and last one element by element.  Vocabularies below one granule, of one granule, of whole and partial rounds of a
+warp and of a CTA, rows cut into several slices whose last one is empty for some alignments, both types; the maximum, a
+NaN and -inf placed in the edge elements.  Against the oracle under the rules of tests/parity.py."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2605_02888_b200 as speckv
+from paper_2605_02888_b200 import synth
+
+from parity import compare_step, gpu_batch, mlp_pair, oracle_batch
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+def _check(s, w):
+    gm, om = mlp_pair(synth.make_mlp(w, DEV))
+    out = speckv.speckv_step(gpu_batch(s), s["comp"], gm)
+    torch.cuda.synchronize()
+    compare_step(out, oracle.step(oracle_batch(s), s["comp"].cpu().numpy(), om))
+    return out
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("V", [1, 3, 7, 9, 15, 17, 255, 257, 1023, 2047, 2049, 16385, 33333])
+def test_rows_off_the_grid(dtype, V):
+    w = synth.Workload("g", B=7, gamma_max=3, V=V, dtype=dtype, gamma_mode="ragged", temperature_mode="mixed",
+                       sigma_d=(0.3, 0.6), seed=V)
+    _check(synth.make_step(w, 0, DEV), w)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("where", ["first", "last"])
+def test_edge_elements_count(dtype, where):
+    w = synth.Workload("g", B=6, gamma_max=2, V=5003, dtype=dtype, gamma_mode="fixed", gamma_fixed=2, temperature_mode="mixed",
+                       sigma_d=(0.5,), seed=11)
+    s = synth.make_step(w, 0, DEV)
+    k = 0 if where == "first" else w.V - 1
+    s["draft"][1:4, :, k] = 40.0     # the maximum sits in the row's edge granule
+    s["target"][2:5, :, k] = 40.0
+    s["draft_tokens"][1:4] = k
+    s["target"][5, 0, k] = float("-inf")
+    s["draft"][5, :, k] = float("-inf")
+    _check(s, w)
+    s["draft"][0, 1, k] = float("nan")
+    s["target"][3, 0, k] = float("inf")
+    out = _check(s, w)
+    st = out["row_status"].cpu().numpy()
+    assert np.array_equal(st, np.array([4, 0, 0, 4, 0, 0]))
