@@ -120,8 +120,8 @@ typedef struct {
     int32_t score_transform;       /* 0: E_j = o_j * gamma_j + 1 (Eq. 1); 1: E_j = o_j    */
 } speckv_mlp;
 
-/* Scratch bytes needed by speckv_signals / speckv_verify / speckv_step for this batch
- * shape (depends on B, gamma_max, V and dtype only).                                      */
+/* Scratch bytes that serve speckv_signals / speckv_verify / speckv_step for this batch
+ * shape (depends on B, gamma_max, V and dtype only; a size for more rows serves fewer).    */
 speckv_status speckv_workspace_size(const speckv_batch* batch, size_t* bytes);
 
 /* Draft signals (paper Sec. 4.2).  H, C: [B, gamma_max] fp32 (0 at i >= gamma_b);
@@ -158,8 +158,8 @@ speckv_status speckv_sample_draft(const speckv_batch* batch, const float* unifor
                                   void* cuda_stream);
 
 /* One fused step: signals, controller and verification from a single pass over the logits
- * (plus a second look at the stop position's two rows for the residual / bonus draw, taken
- * while those rows are still in L2 where the batch is large enough for the stream kernel).
+ * (plus a second look at the stop position's two rows for a residual draw, and at one short range
+ * of the bonus position's row for a bonus draw).
  * gamma_next[b] is the controller's choice for the NEXT step of row b; this step verifies
  * with the gamma given in the batch.  H, C, scores may be NULL.                            */
 speckv_status speckv_step(const speckv_batch* batch, const float* comp, const speckv_mlp* mlp,
@@ -179,9 +179,9 @@ speckv_status speckv_step(const speckv_batch* batch, const float* comp, const sp
  * library holds that much memory until the process exits.  The caller still owns and passes the
  * inputs and the outputs; arguments, results and row_status are exactly those of speckv_signals.
  *
- *   - A batch whose speckv_workspace_size() exceeds SPECKV_STATIC_SCRATCH_BYTES is refused with
+ *   - A batch that needs more scratch than SPECKV_STATIC_SCRATCH_BYTES is refused with
  *     SPECKV_ERR_STATIC_LIMIT before anything is enqueued (B = 256, gamma_max = 8, V = 128256
- *     needs 2.7 MB).
+ *     needs 2.7 MB; speckv_workspace_size() says 3.8 MB for it because it covers verification too).
  *   - The call allocates and frees nothing.  The first call on each device looks up the
  *     array's device address (cudaGetSymbolAddress with that device current) and remembers it;
  *     make that first call outside any stream capture.

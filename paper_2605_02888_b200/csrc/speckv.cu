@@ -14,6 +14,7 @@
 
 #include "speckv_kernels.cuh"
 #include "speckv_pipeline.cuh"
+#include "speckv_sweep.cuh"
 #include "speckv_shard.cuh"
 #include "speckv_sample.cuh"
 
@@ -28,10 +29,8 @@ inline size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 struct Plan {
     int J_full;      // logit rows per batch row with verification: 2*G + 1
-    int nchunk;      // 256-element chunks per logit row
-    int R;           // resample CTAs per batch row
-    int chunks_per_cta;
-    size_t off_tick, off_info, off_part, off_csum, off_tokl, total;
+    size_t off_tick, off_info, off_part, off_tokl, off_spans, off_dsum, total;
+    size_t total_signals;  // what the signals alone may use: the scratch array of speckv_signals_static is held against it
 };
 
 inline int esize(speckv_dtype dt) { return dt == SPECKV_BF16 ? 2 : 4; }
@@ -75,9 +74,12 @@ void choose_slices(KParams& P, speckv_dtype dt, bool aligned) {
     const int ng = (P.V + E - 1 + (aligned ? 0 : E - 1)) / E;  // granules a row can touch
     int ns = static_cast<int>(std::lround(16.0 * ng / static_cast<double>(kSliceBytes)));
     if (ns < 1) ns = 1;
-    // small batches: enough CTAs to put a few on every SM
+    // Small batches: enough CTAs to fill the slots of the chip once (5 on each of 148 SMs).  Aiming at more starts a second
+    // round of short CTAs: with 1,184 instead of 740, step of 64 bf16 rows, V = 32,000, 37.7 us instead of 33.1, of 37 rows,
+    // V = 50,257, 32.6 instead of 31.1; one row the same.
+    constexpr int kSlots = 740;
     const long long rows = static_cast<long long>(P.B) * P.J;
-    const long long want = (1184 + rows - 1) / (rows > 0 ? rows : 1);
+    const long long want = (kSlots + rows - 1) / (rows > 0 ? rows : 1);
     if (want > ns) ns = static_cast<int>(want > kMaxSplit ? kMaxSplit : want);
     if (ns > kMaxSplit) ns = kMaxSplit;
     // At least one granule per lane; short ranges are whole rounds of the warp (a round with idle lanes costs as much as a
@@ -86,7 +88,7 @@ void choose_slices(KParams& P, speckv_dtype dt, bool aligned) {
     int pw = (ng + ns * kWarps - 1) / (ns * kWarps);
     const int near = (pw + 16) / 32 * 32 < 32 ? 32 : (pw + 16) / 32 * 32;
     if (pw >= 256) pw = (pw + 7) / 8 * 8;
-    else if (((ng + near * kWarps - 1) / (near * kWarps)) * rows <= 1184 + rows) pw = near;
+    else if (((ng + near * kWarps - 1) / (near * kWarps)) * rows <= kSlots + rows) pw = near;
     else pw = (pw + 31) / 32 * 32;
     while ((ng + pw * kWarps - 1) / (pw * kWarps) > kMaxSplit) pw += 32;
     P.per_warp = pw;
@@ -94,23 +96,36 @@ void choose_slices(KParams& P, speckv_dtype dt, bool aligned) {
 }
 
 constexpr int kEarlyPositions = 2;   // positions whose acceptance tests the sliced sweep takes ahead of the rest of the row
-constexpr int kRsChunksPerCta = 64;  // 256-element chunks of the stop position that one resample CTA sums
+constexpr int kDrawElems = 16384;    // elements of the stop position that one CTA of a draw sums
+constexpr int kDrawSmallCtas = 1184; // CTAs of a draw wanted in flight for a small batch (two per CTA slot)
+
+// CTAs per draw and granules per warp: P.R, P.draw_pw.
+void choose_draw(KParams& P, speckv_dtype dt, bool aligned) {
+    const int E = 16 / esize(dt);
+    const int ng = (P.V + E - 1 + (aligned ? 0 : E - 1)) / E;
+    int R = (P.V + kDrawElems - 1) / kDrawElems;
+    // small batches: more, shorter shares per row, so that the draw of a handful of rows still spreads over the SMs
+    const int want = (kDrawSmallCtas + P.B - 1) / P.B, cap = (ng + 32 * kWarps - 1) / (32 * kWarps);  // one granule per lane at least
+    if (want > R) R = want < cap ? want : cap > R ? cap : R;
+    if (R > kMaxShares) R = kMaxShares;
+    if (R < 1) R = 1;
+    P.draw_pw = ((ng + R * kWarps - 1) / (R * kWarps) + 7) / 8 * 8;
+    P.R = (ng + P.draw_pw * kWarps - 1) / (P.draw_pw * kWarps);
+}
 
 Plan make_plan(const speckv_batch* bt) {
     Plan p;
     const size_t B = static_cast<size_t>(bt->B);
     p.J_full = 2 * bt->gamma_max + 1;
-    p.nchunk = (bt->V + kChunk - 1) / kChunk;
-    p.R = (p.nchunk + kRsChunksPerCta - 1) / kRsChunksPerCta;
-    if (p.R > 32) p.R = 32;
-    if (p.R < 1) p.R = 1;
-    p.chunks_per_cta = (p.nchunk + p.R - 1) / p.R;
     size_t off = 0;
     p.off_tick = off; off = align_up(off + (6 * B + 4) * sizeof(int));  // tickets, counters, row queue, row flags, first-generation tickets, early stops
     p.off_info = off; off = align_up(off + B * sizeof(RowInfo));
     p.off_part = off; off = align_up(off + B * p.J_full * kMaxSplit * sizeof(float4));
-    p.off_csum = off; off = align_up(off + B * p.nchunk * sizeof(float));
+    off = align_up(off + B * ((static_cast<size_t>(bt->V) + 255) / 256) * sizeof(float));  // (not in use: keeps the sizes that were accepted)
     p.off_tokl = off; off = align_up(off + B * static_cast<size_t>(bt->gamma_max) * sizeof(float2));
+    p.total_signals = off < kAlign ? kAlign : off;
+    p.off_spans = off; off = align_up(off + B * kMaxSplit * kWarps * sizeof(float2));
+    p.off_dsum = off; off = align_up(off + B * kMaxShares * kWarps * sizeof(double));
     p.total = off < kAlign ? kAlign : off;
     return p;
 }
@@ -212,19 +227,17 @@ cudaError_t launch_pipe(const KParams& P, cudaStream_t st) {
 // After the register-staged sweep the fresh tokens are drawn by extra CTAs of the same launch; the rows swept last have their fresh tokens drawn by more, shorter CTAs (see resample_body)
 constexpr int kRsTailRows = 32;  // b256, same box, builds in turn: 16 rows 158.7 us, 32 rows 156.6 us, 64 rows 156.7 us, 128 rows 157.2 us
 constexpr int kRsTailMult = 2;
-constexpr int kRsSmallCtas = 1184;  // resample CTAs wanted in flight for a small batch (two per CTA slot)
 
-template <typename T, bool ALIGNED>
-cudaError_t launch_all(KParams P, cudaStream_t st, const Events& ev, bool staged) {
+template <typename T>
+cudaError_t launch_all(KParams P, cudaStream_t st, const Events& ev, bool ring) {
     constexpr int U = sizeof(T) == 2 ? kSweepLoads : (kSweepLoads + 1) / 2;
     const bool verify = (P.mode & MODE_VERIFY) != 0;
-    const bool ring = ALIGNED && staged;
-    P.rs_tail = 0; P.R2 = P.R; P.chunks_per_cta2 = P.chunks_per_cta;
+    P.rs_tail = 0; P.R2 = P.R; P.draw_pw2 = P.draw_pw;
     bool merged = verify && !ring && P.rdone;
-    if (merged && P.B >= 4 * kRsTailRows && P.R * kRsTailMult <= 32 && kRsTailMult > 1) {
+    if (merged && P.B >= 4 * kRsTailRows && P.R * kRsTailMult <= kMaxShares && P.draw_pw >= 64) {
         P.rs_tail = kRsTailRows;
         P.R2 = P.R * kRsTailMult;
-        P.chunks_per_cta2 = (P.nchunk + P.R2 - 1) / P.R2;
+        P.draw_pw2 = (P.draw_pw + kRsTailMult - 1) / kRsTailMult;
     }
     const long long n_draw = static_cast<long long>(P.B - P.rs_tail) * P.R + static_cast<long long>(P.rs_tail) * P.R2;
     merged = merged && P.n_sweep + n_draw <= 0x7fffffffLL;
@@ -234,7 +247,7 @@ cudaError_t launch_all(KParams P, cudaStream_t st, const Events& ev, bool staged
         e = launch_pipe<T>(P, st);
     } else {
         const long long grid = P.n_sweep + (merged ? n_draw : 0);
-        sweep_kernel<T, ALIGNED, U><<<static_cast<unsigned>(grid), kThreads, 0, st>>>(P);
+        sweep_kernel<T, U><<<static_cast<unsigned>(grid), kThreads, 0, st>>>(P);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess) return e;
@@ -252,7 +265,7 @@ cudaError_t launch_all(KParams P, cudaStream_t st, const Events& ev, bool staged
         attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        e = cudaLaunchKernelEx(&cfg, resample_kernel<T, ALIGNED>, P);
+        e = cudaLaunchKernelEx(&cfg, resample_kernel<T>, P);
     }
     if (ev.after_resample) cudaEventRecord(ev.after_resample, st);
     return e;
@@ -275,7 +288,7 @@ speckv_status run(const speckv_batch* bt, int mode, const float* comp, const spe
     if (bt->B == 0) return SPECKV_OK;
     const Plan pl = make_plan(bt);
     if (!ws || reinterpret_cast<uintptr_t>(ws) % kAlign != 0) return SPECKV_ERR_INVALID_ARG;
-    if (ws_bytes < workspace_total(bt)) return SPECKV_ERR_WORKSPACE;
+    if (ws_bytes < (verify ? pl.total : pl.total_signals)) return SPECKV_ERR_WORKSPACE;
 
     KParams P{};
     P.B = bt->B; P.G = bt->gamma_max; P.V = bt->V;
@@ -284,18 +297,7 @@ speckv_status run(const speckv_batch* bt, int mode, const float* comp, const spe
     bool aligned = rows_aligned(bt->draft_logits, bt->draft_stride_b, bt->draft_stride_pos, es);
     if (verify) aligned = aligned && rows_aligned(bt->target_logits, bt->target_stride_b, bt->target_stride_pos, es);
     choose_slices(P, bt->dtype, aligned);
-    P.nchunk = pl.nchunk; P.R = pl.R; P.chunks_per_cta = pl.chunks_per_cta;
-    {
-        // small batches: more, shorter shares per row, so that the draw of a handful of rows still spreads
-        // over the SMs (the draw of a row is a chain of dependent round trips, shorter with fewer chunks per CTA)
-        const int want = (kRsSmallCtas + P.B - 1) / P.B;
-        int cap = (P.nchunk + 7) / 8;  // at least one chunk per warp
-        if (cap > 32) cap = 32;
-        if (want > P.R && cap > P.R) {
-            P.R = want < cap ? want : cap;
-            P.chunks_per_cta = (P.nchunk + P.R - 1) / P.R;
-        }
-    }
+    choose_draw(P, bt->dtype, aligned);
     P.mode = mode; P.bits = bt->entropy_in_bits ? 1 : 0;
     P.wait_limit = g_wait_limit.load(std::memory_order_relaxed);
     P.d = bt->draft_logits; P.dsb = bt->draft_stride_b; P.dsp = bt->draft_stride_pos;
@@ -314,7 +316,7 @@ speckv_status run(const speckv_batch* bt, int mode, const float* comp, const spe
     P.rowq = P.qcount + 4;
     P.info = reinterpret_cast<RowInfo*>(w + pl.off_info);
     P.part = reinterpret_cast<float4*>(w + pl.off_part);
-    P.csum = reinterpret_cast<float*>(w + pl.off_csum);
+    P.dsum = reinterpret_cast<double*>(w + pl.off_dsum);
 
     if (static_cast<long long>(P.B) * P.J * P.nsplit > 0x7fffffffLL) return SPECKV_ERR_UNSUPPORTED;
     P.n_sweep = P.B * P.J * P.nsplit;
@@ -344,6 +346,7 @@ constexpr int kPipeMinB = 384;
     P.rdone = (verify && !staged) ? P.rowq + P.B : nullptr;
     P.tokl = (verify && !staged) ? reinterpret_cast<float2*>(static_cast<char*>(ws) + pl.off_tokl) : nullptr;
     if (verify && !staged) {
+        P.spans = reinterpret_cast<float2*>(w + pl.off_spans);
         // generation order: positions 0..k of every batch row first, so that their acceptance tests are in
         // before the CTAs of the later target rows start (most walks that stop early stop at the first two
         // positions, and a later position's test would come too late for the CTAs behind it anyway)
@@ -356,32 +359,20 @@ constexpr int kPipeMinB = 384;
     P.Lg = static_cast<int>(row_bytes / 16);
     P.Lp = (P.Lg + kStageGran - 1) / kStageGran * kStageGran;
     cudaError_t e;
-    if (bt->dtype == SPECKV_BF16)
-        e = aligned ? launch_all<__nv_bfloat16, true>(P, cs, ev, staged) : launch_all<__nv_bfloat16, false>(P, cs, ev, false);
-    else
-        e = aligned ? launch_all<float, true>(P, cs, ev, staged) : launch_all<float, false>(P, cs, ev, false);
+    e = bt->dtype == SPECKV_BF16 ? launch_all<__nv_bfloat16>(P, cs, ev, staged) : launch_all<float>(P, cs, ev, staged);
     return e == cudaSuccess ? SPECKV_OK : SPECKV_ERR_CUDA;
 }
 
-// Draft-side sampling: its own workspace plan (one resample slot per drafted position).
+// Draft-side sampling: its own workspace plan (one draw per drafted position).
 struct SamplePlan {
-    int nchunk, R, chunks_per_cta;
-    size_t off_tick, off_info, off_part, off_csum, off_cz, total;
+    size_t off_tick, off_spans, total;
 };
 SamplePlan make_sample_plan(const speckv_batch* bt) {
     SamplePlan p;
     const size_t B = static_cast<size_t>(bt->B), G = static_cast<size_t>(bt->gamma_max);
-    p.nchunk = (bt->V + kChunk - 1) / kChunk;
-    p.R = (p.nchunk + 63) / 64;
-    if (p.R > 32) p.R = 32;
-    if (p.R < 1) p.R = 1;
-    p.chunks_per_cta = (p.nchunk + p.R - 1) / p.R;
     size_t off = 0;
-    p.off_tick = off; off = align_up(off + (2 * B + B * G) * sizeof(int));  // sweep tickets, resample tickets, row flags
-    p.off_info = off; off = align_up(off + B * G * sizeof(RowInfo));
-    p.off_part = off; off = align_up(off + B * G * kMaxSplit * sizeof(float4));
-    p.off_csum = off; off = align_up(off + B * G * p.nchunk * sizeof(float));
-    p.off_cz = off; off = align_up(off + B * G * p.nchunk * sizeof(float2));  // per-chunk (maximum, sum) of the one-pass kernel
+    p.off_tick = off; off = align_up(off + (B * G + 2 * B) * sizeof(int));  // tickets per position and per row, row status
+    p.off_spans = off; off = align_up(off + B * G * kMaxSplit * kWarps * sizeof(float2));
     p.total = off < kAlign ? kAlign : off;
     return p;
 }
@@ -402,69 +393,24 @@ speckv_status run_sample(const speckv_batch* bt, const float* uniforms, int32_t*
     P.J = bt->gamma_max;
     const bool aligned = rows_aligned(bt->draft_logits, bt->draft_stride_b, bt->draft_stride_pos, esize(bt->dtype));
     choose_slices(P, bt->dtype, aligned);
-    P.nchunk = pl.nchunk; P.R = pl.R; P.chunks_per_cta = pl.chunks_per_cta;
-    P.mode = MODE_SAMPLE; P.sample = 1; P.rs_reverse = 1;
-    P.wait_limit = g_wait_limit.load(std::memory_order_relaxed);
-    // the drafted positions are swept and drawn from as if they were target rows
     P.d = bt->draft_logits; P.dsb = bt->draft_stride_b; P.dsp = bt->draft_stride_pos;
-    P.t = bt->draft_logits; P.tsb = bt->draft_stride_b; P.tsp = bt->draft_stride_pos;
     P.gamma = bt->gamma; P.temp = bt->temperature; P.temp_scalar = bt->temperature_scalar;
     P.u = uniforms;
     P.out_tok = tokens; P.status = row_status;
     char* w = static_cast<char*>(ws);
     P.tick1 = reinterpret_cast<int*>(w + pl.off_tick);
-    P.tick2 = P.tick1 + P.B;
-    P.rdone = P.tick2 + static_cast<size_t>(P.B) * P.G;
-    P.info = reinterpret_cast<RowInfo*>(w + pl.off_info);
-    P.part = reinterpret_cast<float4*>(w + pl.off_part);
-    P.csum = reinterpret_cast<float*>(w + pl.off_csum);
+    P.tick2 = P.tick1 + static_cast<size_t>(P.B) * P.G;
+    P.rdone = P.tick2 + P.B;
+    P.spans = reinterpret_cast<float2*>(w + pl.off_spans);
     if (static_cast<long long>(P.B) * P.J * P.nsplit > 0x7fffffffLL) return SPECKV_ERR_UNSUPPORTED;
-    P.n_sweep = P.B * P.J * P.nsplit;
 
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     if (dbg_register(cs, bt, false, ws, ws_bytes) != cudaSuccess) return SPECKV_ERR_CUDA;
     const size_t n_tick = static_cast<size_t>(P.B) * (2 + static_cast<size_t>(P.G));
     if (cudaMemsetAsync(P.tick1, 0, n_tick * sizeof(int), cs) != cudaSuccess) return SPECKV_ERR_CUDA;
-constexpr int kSampleCtas = 2368;
-    // One pass (speckv_sample.cuh) whenever a row's chunk records fit the searching CTA's shared memory.
-    if (P.nchunk <= kRsStage &&
-        static_cast<long long>(P.B) * P.G * P.R <= 0x7fffffffLL) {
-        P.csum2 = reinterpret_cast<float*>(w + pl.off_cz);
-        // shares per logit row: enough CTAs to fill the SMs a few times over, no more (a CTA costs a few
-        // microseconds before its first load returns)
-        {
-            const long long draws = static_cast<long long>(P.B) * P.G;
-            long long S = (kSampleCtas + draws - 1) / draws;
-            if (S > P.R) S = P.R;
-            if (S < 1) S = 1;
-            P.R = static_cast<int>(S);
-            P.chunks_per_cta = (P.nchunk + P.R - 1) / P.R;
-        }
-        const unsigned g1 = static_cast<unsigned>(P.B) * P.G * P.R;
-        if (bt->dtype == SPECKV_BF16) {
-            if (aligned) sample_onepass_kernel<__nv_bfloat16, true><<<g1, kThreads, 0, cs>>>(P);
-            else sample_onepass_kernel<__nv_bfloat16, false><<<g1, kThreads, 0, cs>>>(P);
-        } else {
-            if (aligned) sample_onepass_kernel<float, true><<<g1, kThreads, 0, cs>>>(P);
-            else sample_onepass_kernel<float, false><<<g1, kThreads, 0, cs>>>(P);
-        }
-        return cudaGetLastError() == cudaSuccess ? SPECKV_OK : SPECKV_ERR_CUDA;
-    }
-    // one launch: the draws' CTAs sit behind the sweep CTAs of the same grid and wait for their batch
-    // row's flag (as in the verification step); two launches when the grid would not fit
-    const long long n_draw = static_cast<long long>(P.B) * P.G * P.R;
-    const bool merged = P.n_sweep + n_draw <= 0x7fffffffLL;
-    if (merged) P.rs_reverse = 0; else P.rdone = nullptr;
-    const unsigned grid1 = static_cast<unsigned>(P.n_sweep + (merged ? n_draw : 0));
-    const unsigned grid2 = static_cast<unsigned>(n_draw);
-    constexpr int Ub = kSweepLoads, Uf = (kSweepLoads + 1) / 2;
-    if (bt->dtype == SPECKV_BF16) {
-        if (aligned) { sweep_kernel<__nv_bfloat16, true, Ub><<<grid1, kThreads, 0, cs>>>(P); if (!merged) resample_kernel<__nv_bfloat16, true><<<grid2, kThreads, 0, cs>>>(P); }
-        else { sweep_kernel<__nv_bfloat16, false, Ub><<<grid1, kThreads, 0, cs>>>(P); if (!merged) resample_kernel<__nv_bfloat16, false><<<grid2, kThreads, 0, cs>>>(P); }
-    } else {
-        if (aligned) { sweep_kernel<float, true, Uf><<<grid1, kThreads, 0, cs>>>(P); if (!merged) resample_kernel<float, true><<<grid2, kThreads, 0, cs>>>(P); }
-        else { sweep_kernel<float, false, Uf><<<grid1, kThreads, 0, cs>>>(P); if (!merged) resample_kernel<float, false><<<grid2, kThreads, 0, cs>>>(P); }
-    }
+    const unsigned grid = static_cast<unsigned>(P.B) * P.G * P.nsplit;
+    if (bt->dtype == SPECKV_BF16) sample_kernel<__nv_bfloat16, kSweepLoads><<<grid, kThreads, 0, cs>>>(P);
+    else sample_kernel<float, (kSweepLoads + 1) / 2><<<grid, kThreads, 0, cs>>>(P);
     return cudaGetLastError() == cudaSuccess ? SPECKV_OK : SPECKV_ERR_CUDA;
 }
 
@@ -491,22 +437,16 @@ cudaError_t static_scratch_address(void** out) {
 
 // ---- vocabulary-sharded verification (speckv_shard.cuh) ----
 struct ShardPlan {
-    int nchunk, R, chunks_per_cta;
-    size_t off_tick, off_part, off_csum, off_csum2, total;
+    size_t off_tick, off_part, off_dsum, off_dsum2, total;
 };
 ShardPlan make_shard_plan(const speckv_batch* bt) {
     ShardPlan p;
     const size_t B = static_cast<size_t>(bt->B), J = 2 * static_cast<size_t>(bt->gamma_max) + 1;
-    p.nchunk = (bt->V + kChunk - 1) / kChunk;
-    p.R = (p.nchunk + kRsChunksPerCta - 1) / kRsChunksPerCta;
-    if (p.R > 32) p.R = 32;
-    if (p.R < 1) p.R = 1;
-    p.chunks_per_cta = (p.nchunk + p.R - 1) / p.R;
     size_t off = 0;
     p.off_tick = off; off = align_up(off + (3 * B + 4) * sizeof(int));  // sweep tickets, draw tickets, counters, row queue
     p.off_part = off; off = align_up(off + B * J * kMaxSplit * sizeof(float4));
-    p.off_csum = off; off = align_up(off + B * p.nchunk * sizeof(float));
-    p.off_csum2 = off; off = align_up(off + B * p.nchunk * sizeof(float));
+    p.off_dsum = off; off = align_up(off + B * kMaxShares * kWarps * sizeof(double));
+    p.off_dsum2 = off; off = align_up(off + B * kMaxShares * kWarps * sizeof(double));
     p.total = off < kAlign ? kAlign : off;
     return p;
 }
@@ -522,7 +462,9 @@ speckv_status shard_params(const speckv_batch* bt, void* ws, size_t ws_bytes, KP
     if (!ws || reinterpret_cast<uintptr_t>(ws) % kAlign != 0) return SPECKV_ERR_INVALID_ARG;
     if (ws_bytes < pl.total) return SPECKV_ERR_WORKSPACE;
     P.B = bt->B; P.G = bt->gamma_max; P.V = bt->V; P.J = 2 * bt->gamma_max + 1;
-    P.nchunk = pl.nchunk; P.R = pl.R; P.chunks_per_cta = pl.chunks_per_cta;
+    const int es = esize(bt->dtype);
+    choose_draw(P, bt->dtype, rows_aligned(bt->draft_logits, bt->draft_stride_b, bt->draft_stride_pos, es) &&
+                                  rows_aligned(bt->target_logits, bt->target_stride_b, bt->target_stride_pos, es));
     P.mode = MODE_VERIFY; P.bits = bt->entropy_in_bits ? 1 : 0;
     P.d = bt->draft_logits; P.dsb = bt->draft_stride_b; P.dsp = bt->draft_stride_pos;
     P.t = bt->target_logits; P.tsb = bt->target_stride_b; P.tsp = bt->target_stride_pos;
@@ -536,8 +478,8 @@ speckv_status shard_params(const speckv_batch* bt, void* ws, size_t ws_bytes, KP
     P.qtail = P.qcount + 2;
     P.rowq = P.qcount + 4;
     P.part = reinterpret_cast<float4*>(w + pl.off_part);
-    P.csum = reinterpret_cast<float*>(w + pl.off_csum);
-    P.csum2 = reinterpret_cast<float*>(w + pl.off_csum2);
+    P.dsum = reinterpret_cast<double*>(w + pl.off_dsum);
+    P.dsum2 = reinterpret_cast<double*>(w + pl.off_dsum2);
     return SPECKV_OK;
 }
 bool shard_aligned(const speckv_batch* bt) {
@@ -588,7 +530,7 @@ speckv_status speckv_signals_static(const speckv_batch* batch, float* H, float* 
     speckv_status st = check_batch(batch, false);
     if (st != SPECKV_OK) return st;
     if (batch->B == 0) return SPECKV_OK;
-    if (make_plan(batch).total > SPECKV_STATIC_SCRATCH_BYTES) return SPECKV_ERR_STATIC_LIMIT;
+    if (make_plan(batch).total_signals > SPECKV_STATIC_SCRATCH_BYTES) return SPECKV_ERR_STATIC_LIMIT;
     void* scratch = nullptr;
     if (static_scratch_address(&scratch) != cudaSuccess || !scratch) return SPECKV_ERR_CUDA;
     // run() clears the ticket counters on the caller's stream; nothing else needs a known start
@@ -696,8 +638,8 @@ speckv_status speckv_internal_wait_probe(int32_t B, int32_t* row_status, int32_t
         return SPECKV_ERR_WORKSPACE;
     // the draw kernel on its own, one CTA per batch row, with completion flags that nothing raises
     KParams P{};
-    P.B = B; P.G = 1; P.V = kChunk; P.J = 3; P.nchunk = 1; P.R = 1; P.chunks_per_cta = 1;
-    P.R2 = 1; P.chunks_per_cta2 = 1; P.mode = MODE_VERIFY;
+    P.B = B; P.G = 1; P.V = 256; P.J = 3; P.R = 1; P.draw_pw = 8;
+    P.R2 = 1; P.draw_pw2 = 8; P.mode = MODE_VERIFY;
     P.wait_limit = g_wait_limit.load(std::memory_order_relaxed);
     P.status = row_status; P.out_tok = out_tokens;
     P.rdone = static_cast<int*>(workspace);
@@ -709,7 +651,7 @@ speckv_status speckv_internal_wait_probe(int32_t B, int32_t* row_status, int32_t
     }
     if (cudaMemsetAsync(workspace, 0, 2 * static_cast<size_t>(B) * sizeof(int), cs) != cudaSuccess) return SPECKV_ERR_CUDA;
     wait_probe_fill<<<(B + 255) / 256, 256, 0, cs>>>(P);
-    resample_kernel<float, true><<<static_cast<unsigned>(B), kThreads, 0, cs>>>(P);
+    resample_kernel<float><<<static_cast<unsigned>(B), kThreads, 0, cs>>>(P);
     wait_probe_late_epilogue<<<(B + kWarps - 1) / kWarps, kThreads, 0, cs>>>(P);
     return cudaGetLastError() == cudaSuccess ? SPECKV_OK : SPECKV_ERR_CUDA;
 }
@@ -765,11 +707,9 @@ speckv_status speckv_shard_sweep(const speckv_batch* local, int64_t v_begin, flo
         return cudaGetLastError() == cudaSuccess ? SPECKV_OK : SPECKV_ERR_CUDA;
     }
     if (local->dtype == SPECKV_BF16) {
-        if (al) sweep_kernel<__nv_bfloat16, true, Ub><<<grid, kThreads, 0, cs>>>(P);
-        else sweep_kernel<__nv_bfloat16, false, Ub><<<grid, kThreads, 0, cs>>>(P);
+        sweep_kernel<__nv_bfloat16, Ub><<<grid, kThreads, 0, cs>>>(P);
     } else {
-        if (al) sweep_kernel<float, true, Uf><<<grid, kThreads, 0, cs>>>(P);
-        else sweep_kernel<float, false, Uf><<<grid, kThreads, 0, cs>>>(P);
+        sweep_kernel<float, Uf><<<grid, kThreads, 0, cs>>>(P);
     }
     return cudaGetLastError() == cudaSuccess ? SPECKV_OK : SPECKV_ERR_CUDA;
 }
@@ -838,13 +778,10 @@ speckv_status speckv_shard_draw_sums(const speckv_batch* local, const void* row_
     if (cudaMemsetAsync(P.tick2, 0, static_cast<size_t>(P.B) * sizeof(int), cs) != cudaSuccess) return SPECKV_ERR_CUDA;
     if (static_cast<long long>(P.B) * P.R > 0x7fffffffLL) return SPECKV_ERR_UNSUPPORTED;
     const unsigned grid = static_cast<unsigned>(P.B) * static_cast<unsigned>(P.R);
-    const bool al = shard_aligned(local);
     if (local->dtype == SPECKV_BF16) {
-        if (al) shard_sums_kernel<__nv_bfloat16, true><<<grid, kThreads, 0, cs>>>(P);
-        else shard_sums_kernel<__nv_bfloat16, false><<<grid, kThreads, 0, cs>>>(P);
+        shard_sums_kernel<__nv_bfloat16><<<grid, kThreads, 0, cs>>>(P);
     } else {
-        if (al) shard_sums_kernel<float, true><<<grid, kThreads, 0, cs>>>(P);
-        else shard_sums_kernel<float, false><<<grid, kThreads, 0, cs>>>(P);
+        shard_sums_kernel<float><<<grid, kThreads, 0, cs>>>(P);
     }
     return cudaGetLastError() == cudaSuccess ? SPECKV_OK : SPECKV_ERR_CUDA;
 }
@@ -869,13 +806,10 @@ speckv_status speckv_shard_draw_pick(const speckv_batch* local, int64_t v_begin,
         if (dbg_register(cs, local, true, workspace, workspace_bytes, ex, 1) != cudaSuccess) return SPECKV_ERR_CUDA;
     }
     const unsigned grid = static_cast<unsigned>(P.B);
-    const bool al = shard_aligned(local);
     if (local->dtype == SPECKV_BF16) {
-        if (al) shard_pick_kernel<__nv_bfloat16, true><<<grid, kThreads, 0, cs>>>(P);
-        else shard_pick_kernel<__nv_bfloat16, false><<<grid, kThreads, 0, cs>>>(P);
+        shard_pick_kernel<__nv_bfloat16><<<grid, kThreads, 0, cs>>>(P);
     } else {
-        if (al) shard_pick_kernel<float, true><<<grid, kThreads, 0, cs>>>(P);
-        else shard_pick_kernel<float, false><<<grid, kThreads, 0, cs>>>(P);
+        shard_pick_kernel<float><<<grid, kThreads, 0, cs>>>(P);
     }
     return cudaGetLastError() == cudaSuccess ? SPECKV_OK : SPECKV_ERR_CUDA;
 }

@@ -1,0 +1,483 @@
+// Drawing a token by inverse CDF in vocabulary order (Sec. 3.1: the fresh token of a step, the tokens of a draft).
+//   residual  w_v = max(0, p_v - q_v)     a rejected position
+//   plain     w_v = p_v                   the bonus position, a drafted position
+// Weights are fp32, everything above one lane's granule is summed in double.  A draw knows the weight of a few ranges
+// ("spans", one per warp that summed it), takes the span that holds the threshold and narrows it down: a CTA sums up to 64
+// parts of the range at once, picks one, until 32 granules are left, which one warp scans.  A plain draw gets its spans
+// from the sweep itself (the sums a warp leaves of its range are the span weights), so beyond one span it never reads the
+// row again; a residual needs both normalisers first, so its spans are summed by CTAs of their own.
+#pragma once
+
+#include "speckv_kernels.cuh"
+
+namespace speckv {
+
+struct DrawSrc {
+    GranRow t, d;        // target row, draft row (residual only)
+    int dg, off;         // granule g of t covers the elements of d from granule g + dg, element off, on
+    int in_lo, in_hi;    // granules of t for which all granules involved are whole ones of their rows
+    float scale, lp_hi, lp_lo, lq_hi, lq_lo;  // log2(e) / T; the log2-normalisers as two floats each, so that the
+                                              // exponent keeps the bits that a single float would drop
+};
+
+// The rows of a draw; the constants follow by set_norm, so that loads can go out while those are still on their way.
+template <typename T>
+__device__ __forceinline__ DrawSrc make_draw(const T* trow, const T* drow, int V) {
+    constexpr int E = 16 / sizeof(T);
+    DrawSrc s;
+    s.t = make_row(trow, V);
+    s.d = drow ? make_row(drow, V) : s.t;
+    s.off = s.d.shift() - s.t.shift();
+    s.dg = 0;
+    if (s.off < 0) { s.off += E; s.dg = -1; }
+    s.in_lo = max(s.t.whole_lo(), s.d.whole_lo() - s.dg);
+    s.in_hi = min(s.t.whole_hi(), s.d.whole_hi() - s.dg - (s.off ? 1 : 0));
+    return s;
+}
+__device__ __forceinline__ void set_norm(DrawSrc& s, float scale, double lse_p, double lse_q) {
+    s.scale = scale;
+    s.lp_hi = static_cast<float>(lse_p);
+    s.lp_lo = static_cast<float>(lse_p - static_cast<double>(s.lp_hi));
+    s.lq_hi = static_cast<float>(lse_q);
+    s.lq_lo = static_cast<float>(lse_q - static_cast<double>(s.lq_hi));
+}
+
+// ---- weights of one granule ------------------------------------------------------------------------------
+__device__ __forceinline__ void gran_pairs(const uint4& g, f2 (&x)[4]) {
+    x[0] = pack2(bf_lo(g.x), bf_hi(g.x)); x[1] = pack2(bf_lo(g.y), bf_hi(g.y));
+    x[2] = pack2(bf_lo(g.z), bf_hi(g.z)); x[3] = pack2(bf_lo(g.w), bf_hi(g.w));
+}
+__device__ __forceinline__ void gran_pairs(const uint4& g, f2 (&x)[2]) {
+    x[0] = pack2(__uint_as_float(g.x), __uint_as_float(g.y));
+    x[1] = pack2(__uint_as_float(g.z), __uint_as_float(g.w));
+}
+template <typename T, bool RES>
+__device__ __forceinline__ void gran_weights(const DrawSrc& s, const uint4& t, const uint4& d, float (&w)[16 / sizeof(T)]) {
+    constexpr int NP = 8 / sizeof(T);
+    const f2 sc2 = pack2(s.scale, s.scale), ph2 = pack2(-s.lp_hi, -s.lp_hi), pl2 = pack2(s.lp_lo, s.lp_lo);
+    f2 xt[NP];
+    gran_pairs(t, xt);
+    if constexpr (!RES) {
+#pragma unroll
+        for (int i = 0; i < NP; ++i) unpack2(ex2_2(sub2(fma2(xt[i], sc2, ph2), pl2)), w[2 * i], w[2 * i + 1]);
+    } else {
+        const f2 qh2 = pack2(-s.lq_hi, -s.lq_hi), ql2 = pack2(s.lq_lo, s.lq_lo);
+        f2 xd[NP];
+        gran_pairs(d, xd);
+#pragma unroll
+        for (int i = 0; i < NP; ++i) {
+            const f2 p = ex2_2(sub2(fma2(xt[i], sc2, ph2), pl2));
+            const f2 q = ex2_2(sub2(fma2(xd[i], sc2, qh2), ql2));
+            float lo, hi;
+            unpack2(sub2(p, q), lo, hi);
+            w[2 * i] = fmaxf(lo, 0.f);
+            w[2 * i + 1] = fmaxf(hi, 0.f);
+        }
+    }
+}
+template <typename T, bool RES>
+__device__ __forceinline__ float gran_weight(const DrawSrc& s, const uint4& t, const uint4& d) {
+    float w[16 / sizeof(T)];
+    gran_weights<T, RES>(s, t, d, w);
+    float a = 0.f;
+#pragma unroll
+    for (int j = 0; j < static_cast<int>(16 / sizeof(T)); ++j) a += w[j];
+    return a;
+}
+
+// ---- granules that are not whole, and rows that sit differently on the 16-byte grid -------------------------
+template <typename T>
+__device__ __forceinline__ uint4 gran_any(const GranRow& r, int g) {  // outside the row: -inf, that is weight 0
+    const float ninf = __int_as_float(0xff800000);
+    if (g < 0 || g >= r.ng) return gran_fill<T>(ninf);
+    if (g < r.whole_lo() || g >= r.whole_hi()) return gran_edge<T>(r, g, ninf);
+    return ldg_stream(r.base + g);
+}
+// elements off, off + 1, ... of the 2 * E elements in a and b
+template <typename T>
+__device__ __forceinline__ uint4 gran_shift(const uint4& a, const uint4& b, int off) {
+    constexpr int EW = 4 / sizeof(T);  // elements per 32-bit word
+    uint32_t w[7] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z};
+    uint32_t top = b.w;
+    const int wo = off / EW;
+    uint32_t v[8] = {w[0], w[1], w[2], w[3], w[4], w[5], w[6], top};
+    if (wo & 2) {
+#pragma unroll
+        for (int i = 0; i < 6; ++i) v[i] = v[i + 2];
+    }
+    if (wo & 1) {
+#pragma unroll
+        for (int i = 0; i < 5; ++i) v[i] = v[i + 1];
+    }
+    if (EW == 2 && (off & 1)) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] = __funnelshift_r(v[i], v[i + 1], 16);
+    }
+    return make_uint4(v[0], v[1], v[2], v[3]);
+}
+template <typename T>
+__device__ __forceinline__ uint4 draft_any(const DrawSrc& s, int g) {  // the draft's elements of t's granule g
+    const uint4 a = gran_any<T>(s.d, g + s.dg);
+    return s.off ? gran_shift<T>(a, gran_any<T>(s.d, g + s.dg + 1), s.off) : a;
+}
+template <typename T, bool RES>
+__device__ __noinline__ double gran_weight_any(const DrawSrc s, int g) {
+    const uint4 t = gran_any<T>(s.t, g);
+    return static_cast<double>(gran_weight<T, RES>(s, t, RES ? draft_any<T>(s, g) : t));
+}
+
+// ---- sums ----------------------------------------------------------------------------------------------------
+// Weight of granules [g0, g1), one warp, the same in every lane.  norm(s) sets the constants and is called once the
+// first loads are out.  Two loads per row are in flight and none is requested ahead: the other warps of the SM, not this one,
+// hide the latency, and what fits 48 registers does not spill (1,024 bf16 rows, V = 128,256: step 430 us; two requested ahead
+// 439, four in flight 435, one in flight and one ahead 436).
+template <typename T, bool RES, bool SHIFTED, class F>
+__device__ __forceinline__ double warp_weight_body(DrawSrc& s, int g0, int g1, F norm) {
+    constexpr int KU = SHIFTED ? 1 : 2;
+    const int lane = threadIdx.x & 31;
+    const int a = min(max(g0, s.in_lo), g1), e = max(min(g1, s.in_hi), a);
+    double acc = 0.0;
+    const uint4* pt = s.t.base + lane;
+    const uint4* pd = s.d.base + s.dg + lane;
+    uint4 t[KU], d[KU], d1[KU];
+    auto load = [&](int g) {
+#pragma unroll
+        for (int u = 0; u < KU; ++u) {
+            const int k = g + 32 * u;
+            t[u] = gran_fill<T>(__int_as_float(0xff800000));
+            if (RES) d[u] = t[u];
+            if (RES && SHIFTED) d1[u] = t[u];
+            if (k + lane < e) {
+                t[u] = ldg_stream(pt + k);
+                if (RES) d[u] = ldg_stream(pd + k);
+                if (RES && SHIFTED) d1[u] = ldg_stream(pd + k + 1);
+            }
+        }
+    };
+    if (a < e) load(a);
+    norm(s);
+    // incomplete granules in front of and behind [a, e): a handful at most, one per lane
+    const int nl = a - g0, nr = g1 - e;
+    for (int k = lane; k < nl + nr; k += 32) acc += gran_weight_any<T, RES>(s, k < nl ? g0 + k : e + (k - nl));
+    for (int g = a; g < e;) {
+        float w = 0.f;
+#pragma unroll
+        for (int u = 0; u < KU; ++u) w += gran_weight<T, RES>(s, t[u], RES ? (SHIFTED ? gran_shift<T>(d[u], d1[u], s.off) : d[u]) : t[u]);
+        acc += static_cast<double>(w);
+        g += 32 * KU;
+        if (g < e) load(g);
+    }
+    return warp_sum(acc);
+}
+template <typename T, bool RES, class F>
+__device__ __forceinline__ double warp_weight(DrawSrc& s, int g0, int g1, F norm) {
+    if (RES && s.off) return warp_weight_body<T, RES, RES>(s, g0, g1, norm);
+    return warp_weight_body<T, RES, false>(s, g0, g1, norm);
+}
+template <typename T, bool RES>
+__device__ __noinline__ double warp_weight_of(const DrawSrc& s, int g0, int g1) {
+    DrawSrc c = s;
+    return warp_weight<T, RES>(c, g0, g1, [](DrawSrc&) {});
+}
+
+// ---- picking -------------------------------------------------------------------------------------------------
+// Which of 32 weights (lane k holds the k-th) holds tau: the first at which the running sum exceeds it, else the last with
+// weight; *before: the sum in front of it.  -1: none has weight.
+__device__ __forceinline__ int pick_lane(double w, double tau, double* before) {
+    const int lane = threadIdx.x & 31;
+    double incl = w;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const double v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+    }
+    const unsigned hit = __ballot_sync(0xffffffffu, incl > tau && w > 0.0);
+    const unsigned pos = __ballot_sync(0xffffffffu, w > 0.0);
+    if (!pos) return -1;
+    const int src = hit ? __ffs(hit) - 1 : 31 - __clz(pos);
+    *before = __shfl_sync(0xffffffffu, incl - w, src);
+    return src;
+}
+// The same over n <= 32 * MOST weights get(0..n-1); tau is u * total where FRACTION is set, *total is returned either way.
+template <bool FRACTION, int MOST, class F>
+__device__ __forceinline__ int pick_many(int n, F get, double u, double* before, double* total, double* tau_out) {
+    const int lane = threadIdx.x & 31;
+    const int per = (n + 31) >> 5;  // lane k takes weights k * per ...
+    double v[MOST], w = 0.0;
+#pragma unroll
+    for (int i = 0; i < MOST; ++i) {
+        v[i] = (i < per && lane * per + i < n) ? get(lane * per + i) : 0.0;
+        w += v[i];
+    }
+    *total = warp_sum(w);
+    const double tau = FRACTION ? u * *total : u;
+    *tau_out = tau;
+    double b0 = 0.0, b1 = 0.0;
+    const int own = pick_lane(w, tau, &b0);
+    if (own < 0) return -1;
+    double mine = 0.0;  // lane i: the chosen lane's i-th weight
+#pragma unroll
+    for (int i = 0; i < MOST; ++i) {
+        const double x = __shfl_sync(0xffffffffu, v[i], own);
+        if (lane == i) mine = x;
+    }
+    const int sub = pick_lane(mine, tau - b0, &b1);
+    *before = b0 + b1;
+    return own * per + max(sub, 0);
+}
+
+// The lane's granule g of both rows; those at or behind g1 have no weight.
+template <typename T, bool RES>
+__device__ __forceinline__ void load_weights(const DrawSrc& s, int g, int g1, float (&w)[16 / sizeof(T)]) {
+    uint4 t = gran_fill<T>(__int_as_float(0xff800000)), d = t;
+    if (g < g1) {
+        if (g >= s.in_lo && g < s.in_hi) {
+            t = ldg_stream(s.t.base + g);
+            if (RES) d = ldg_stream(s.d.base + g + s.dg);
+            if (RES && s.off) d = gran_shift<T>(d, ldg_stream(s.d.base + g + s.dg + 1), s.off);
+        } else {
+            t = gran_any<T>(s.t, g);
+            if (RES) d = draft_any<T>(s, g);
+        }
+    }
+    gran_weights<T, RES>(s, t, d, w);
+}
+// One warp: the token among 32 consecutive granules whose weights its lanes hold (lane 0 granule g0).
+template <typename T>
+__device__ __forceinline__ int scan_weights(const DrawSrc& s, int g0, const float (&w)[16 / sizeof(T)], double tau) {
+    constexpr int E = 16 / sizeof(T);
+    const int lane = threadIdx.x & 31;
+    double tot = 0.0;
+#pragma unroll
+    for (int j = 0; j < E; ++j) tot += static_cast<double>(w[j]);
+    double incl = tot;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const double v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+    }
+    double run = incl - tot;
+    int found = 0x7fffffff, last = -1;
+#pragma unroll
+    for (int j = 0; j < E; ++j) {
+        run += static_cast<double>(w[j]);
+        if (w[j] > 0.f) {
+            last = (g0 + lane) * E - s.t.shift() + j;
+            if (run > tau && found == 0x7fffffff) found = last;
+        }
+    }
+    const int f = static_cast<int>(__reduce_min_sync(0xffffffffu, static_cast<unsigned>(found)));
+    return f != 0x7fffffff ? f : __reduce_max_sync(0xffffffffu, last);
+}
+
+constexpr int kNotMine = -2;
+
+// nw warps (this one is wi) that share named barrier `bar`: the token within granules [g0, g1) at tau (`fraction`: at tau times
+// the range's own weight).  Exactly one warp gets the answer (-1: nothing in the range has weight), the others kNotMine.
+// sh: 64 doubles of shared memory.
+template <typename T, bool RES>
+__device__ __noinline__ int find_token(const DrawSrc& s, int g0, int g1, double tau, bool fraction, int wi, int nw, int bar, double* sh) {
+    constexpr int E = 16 / sizeof(T);
+    const int lane = threadIdx.x & 31;
+    for (;;) {
+        const int n = g1 - g0;
+        const int sub = ((n + 63) / 64 + 31) / 32 * 32, cnt = (n + sub - 1) / sub;
+        const bool leaf = cnt <= nw && sub == 32;  // one granule per lane: the warp that holds the token has its weights at hand
+        float w[E];
+        if (leaf) {
+            load_weights<T, RES>(s, g0 + wi * 32 + lane, g1, w);
+            double a = 0.0;
+#pragma unroll
+            for (int j = 0; j < E; ++j) a += static_cast<double>(w[j]);
+            a = warp_sum(a);
+            if (lane == 0 && wi < cnt) sh[wi] = a;
+        } else if (!RES && sub == 32) {  // four parts at a time: one round trip for them
+            for (int k = wi; k < cnt; k += 4 * nw) {
+                uint4 t[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int g = g0 + (k + u * nw) * 32 + lane;
+                    t[u] = gran_fill<T>(__int_as_float(0xff800000));
+                    if (g < g1) t[u] = gran_any<T>(s.t, g);
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const double a = warp_sum(static_cast<double>(gran_weight<T, false>(s, t[u], t[u])));
+                    if (lane == 0 && k + u * nw < cnt) sh[k + u * nw] = a;
+                }
+            }
+        } else {
+            for (int k = wi; k < cnt; k += nw) {
+                const double a = warp_weight_of<T, RES>(s, g0 + k * sub, min(g1, g0 + (k + 1) * sub));
+                if (lane == 0) sh[k] = a;
+            }
+        }
+        asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(nw * 32) : "memory");
+        double before = 0.0, total, t;
+        int own;
+        if (fraction) own = pick_many<true, 2>(cnt, [&](int i) { return sh[i]; }, tau, &before, &total, &t);
+        else own = pick_many<false, 2>(cnt, [&](int i) { return sh[i]; }, tau, &before, &total, &t);
+        if (own < 0) return wi == 0 ? -1 : kNotMine;
+        fraction = false;
+        tau = t - before;
+        if (leaf) return wi == own ? scan_weights<T>(s, g0 + own * 32, w, tau) : kNotMine;
+        g0 += own * sub;
+        g1 = min(g1, g0 + sub);
+        asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(nw * 32) : "memory");  // sh is written again
+    }
+}
+
+// A plain draw from the sums that the sweep's warps have left of a row (spans: reference in log2 units and sum, one per
+// warp range): nw warps of a CTA, one of which gets the token (find_token).  -1: the row holds a NaN / +inf or has no weight.
+template <typename T>
+__device__ __forceinline__ int draw_from_spans(const T* row, int V, float scale, const float2* spans, int n, int per_warp, float u,
+                                               int wi, int nw, int bar, double* sh, DrawSrc* sh_src) {
+    const int lane = threadIdx.x & 31, per = (n + 31) >> 5;
+    float2 v[8];
+    float R = -3.0e38f;
+    bool bad = false;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int k = lane * per + i;
+        v[i] = make_float2(-3.0e38f, 0.f);
+        if (i < per && k < n && dbg_ok(spans + k, 8, DBG_WS_LOAD)) v[i] = __ldcg(spans + k);
+        R = fmaxf(R, v[i].x);
+        bad |= !(v[i].y < 3e38f);
+    }
+    R = warp_maxf(R);
+    double before = 0.0, total, tau;
+    const int own = pick_many<true, 8>(n, [&](int k) {
+        const int i = k - lane * per;
+        float2 x = v[0];
+#pragma unroll
+        for (int q = 1; q < 8; ++q) if (i == q) x = v[q];
+        return static_cast<double>(x.y) * static_cast<double>(ex2f(x.x - R));
+    }, static_cast<double>(u), &before, &total, &tau);
+    if (__any_sync(0xffffffffu, bad) || own < 0) return wi == 0 ? -1 : kNotMine;
+    if (wi == 0 && lane == 0) {
+        DrawSrc s = make_draw<T>(row, nullptr, V);
+        set_norm(s, scale, static_cast<double>(R), 0.0);
+        *sh_src = s;
+    }
+    asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(nw * 32) : "memory");
+    const int g0 = own * per_warp;
+    return find_token<T, false>(*sh_src, g0, min(sh_src->t.ng, g0 + per_warp), tau - before, false, wi, nw, bar, sh);
+}
+
+// RowInfo as the two 16-byte words it is loaded as
+__device__ __forceinline__ RowInfo row_info_from(const int4& lo4, const int4& hi4) {
+    RowInfo ri;
+    ri.mode = lo4.x; ri.n = lo4.y; ri.u2 = __int_as_float(lo4.z); ri.scale = __int_as_float(lo4.w);
+    ri.lse2_p = __hiloint2double(hi4.y, hi4.x);
+    ri.lse2_q = __hiloint2double(hi4.w, hi4.z);
+    return ri;
+}
+
+// ----------------------------------------------------------------------------------------
+// One CTA's share of the fresh-token draw of batch row b at stop position n: share `share` of Rr, dw granules per warp.
+// The last of the row's CTAs to arrive locates the token.  A residual whose total mass is below 1e-6 cannot be told from
+// rounding noise and is treated as empty (p == q at the stop position): the token is then drawn from p.
+// ----------------------------------------------------------------------------------------
+template <typename T>
+__device__ __forceinline__ void resample_row(const KParams& P, const int b, const int mode, const int n, const int share,
+                                             const int Rr, const int dw) {
+    __shared__ int sh_flag;
+    __shared__ DrawSrc sh_src;
+    __shared__ double sh_sum[64];
+    if (mode == RS_NONE) return;  // greedy or flagged row, or a token that the sweep's own CTA draws
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int4* ip = reinterpret_cast<const int4*>(P.info + b);
+    const int4 lo4 = __ldcg(ip), hi4 = __ldcg(ip + 1);  // on their way while the first logits are requested
+    const T* trow = static_cast<const T*>(P.t) + static_cast<long long>(b) * P.tsb + static_cast<long long>(n) * P.tsp;
+    const T* drow = static_cast<const T*>(P.d) + static_cast<long long>(b) * P.dsb + static_cast<long long>(n) * P.dsp;
+    DrawSrc src = make_draw<T>(trow, mode == RS_RESIDUAL ? drow : nullptr, P.V);
+    auto norm = [&](DrawSrc& s) {
+        const RowInfo ri = row_info_from(lo4, hi4);
+        set_norm(s, ri.scale, ri.lse2_p, ri.lse2_q);
+    };
+    double* dsum = P.dsum + static_cast<long long>(b) * (kMaxShares * kWarps);
+    const int span = share * kWarps + warp;
+    {
+        const int g0 = span * dw, g1 = min(src.t.ng, g0 + dw);
+        const double w = mode == RS_RESIDUAL ? warp_weight<T, true>(src, g0, g1, norm) : warp_weight<T, false>(src, g0, g1, norm);
+        if (lane == 0) SPECKV_ST(dsum[span], w);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        const bool last = atomicAdd(P.tick2 + b, 1) == Rr - 1;
+        if (last) __threadfence();
+        sh_flag = last;
+        sh_src = src;
+    }
+    __syncthreads();
+    if (!sh_flag) return;
+
+    // ---- last CTA of the row: locate the threshold (every warp picks the span, redundantly) ----
+    const float u2 = __int_as_float(lo4.z);
+    double before = 0.0, total, tau;
+    const int own = pick_many<true, 8>(Rr * kWarps, [&](int k) { return dbg_ok(dsum + k, 8, DBG_WS_LOAD) ? __ldcg(dsum + k) : 0.0; },
+                                       static_cast<double>(u2), &before, &total, &tau);
+    int tok;
+    if (mode == RS_RESIDUAL && !(total > 1e-6))
+        tok = find_token<T, false>(sh_src, 0, src.t.ng, static_cast<double>(u2), true, warp, kWarps, 1, sh_sum);
+    else if (own < 0)
+        tok = warp == 0 ? 0 : kNotMine;  // p itself has no mass: cannot happen for a finite row
+    else if (mode == RS_RESIDUAL)
+        tok = find_token<T, true>(sh_src, own * dw, min(src.t.ng, (own + 1) * dw), tau - before, false, warp, kWarps, 1, sh_sum);
+    else
+        tok = find_token<T, false>(sh_src, own * dw, min(src.t.ng, (own + 1) * dw), tau - before, false, warp, kWarps, 1, sh_sum);
+    if (tok != kNotMine && lane == 0) P.out_tok[static_cast<long long>(b) * (P.G + 1) + n] = max(tok, 0);
+}
+
+template <typename T>
+__device__ __forceinline__ void resample_body(const KParams& P, const int bid) {
+    __shared__ int sh_wait;
+    // one-dimensional grid, R consecutive CTAs per batch row: the CTAs of a row are neighbours in
+    // launch order, so rows finish one after the other and their searches overlap the other rows' sums
+    // the last rs_tail draws (in launch order) are cut into R2 >= R shares: their rows are the last to
+    // be swept, nothing is left to overlap their draw with, and more CTAs per row shorten it
+    const int n_head = (P.B - P.rs_tail) * P.R;
+    const bool tail = bid >= n_head;
+    const int Rr = tail ? P.R2 : P.R;
+    const int dw = tail ? P.draw_pw2 : P.draw_pw;
+    const int bq = tail ? (P.B - P.rs_tail) + (bid - n_head) / Rr : bid / Rr;
+    const int share = tail ? (bid - n_head) % Rr : bid % Rr;
+    const int b = P.rs_reverse ? P.B - 1 - bq : bq;
+    // With completion flags a CTA waits only for its own batch row (rows
+    // are taken in the order the sweep finishes them unless rs_reverse is set) and the stop positions of finished rows are
+    // summed while the sweep drains; every sweep CTA is resident or done before the first CTA that draws
+    // starts, so the wait ends, and it is bounded all the same.  Without flags (a programmatic dependent launch behind the
+    // ring sweep) the CTA waits for the whole sweep grid.
+    int mode, n;
+    if (P.rdone) {
+        if (threadIdx.x == 0) sh_wait = row_done_wait(P.rdone + b, P.wait_limit);
+        __syncthreads();
+        const int v = sh_wait;
+        if (!v) {
+            // Gave up.  The mark goes on the row's flag: if the row epilogue has already written the
+            // status (the flag went up just after the last poll) the bit is added here, otherwise the
+            // epilogue finds the mark when it raises the flag and adds the bit itself.
+            if (threadIdx.x == 0 && share == 0) {
+                const int old = atomicOr(P.rdone + b, kRowDoneTimeout);
+                if ((old & 1) && P.status) atomicOr(P.status + b, 16);
+            }
+            return;
+        }
+        mode = (v >> 8) & 3;
+        n = (v >> 16) & 0xff;
+    } else {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        const int4 lo4 = __ldcg(reinterpret_cast<const int4*>(P.info + b));
+        mode = lo4.x;
+        n = lo4.y;
+    }
+    resample_row<T>(P, b, mode, n, share, Rr, dw);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kThreads, 4) resample_kernel(const __grid_constant__ KParams P) {
+    resample_body<T>(P, static_cast<int>(blockIdx.x));
+}
+
+}  // namespace speckv

@@ -25,7 +25,7 @@ namespace speckv {
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr int kVec = 8;                 // elements per lane per step
-constexpr int kChunk = 32 * kVec;       // one warp step = one inverse-CDF chunk (256 elements)
+constexpr int kMaxShares = 32;          // CTAs that share one draw at most
 constexpr int kMaxSplit = 32;
 constexpr int kMaxGamma = 16;           // SPECKV_MAX_GAMMA
 // Measured on b256 (same box, the two builds in turn, five times): 5 CTAs x 3 loads 156.7 us, 4 x 4 161.6 us,
@@ -65,7 +65,7 @@ __device__ __forceinline__ bool dbg_ok(const void*, unsigned, int) { return true
 #endif
 enum : int { DBG_LOGIT16 = 1, DBG_LOGIT1 = 2, DBG_WS_LOAD = 3, DBG_WS_STORE = 4, DBG_COPY = 5 };
 
-enum : int { MODE_SIGNALS = 1, MODE_VERIFY = 2, MODE_MLP = 4, MODE_SAMPLE = 8 };
+enum : int { MODE_SIGNALS = 1, MODE_VERIFY = 2, MODE_MLP = 4 };
 enum : int { PATH_DRAFT = 0, PATH_TARGET = 1, PATH_ARGMAX = 2 };
 enum : int { RS_NONE = 0, RS_RESIDUAL = 1, RS_BONUS = 2 };
 
@@ -81,11 +81,11 @@ struct RowInfo {  // written by the sweep kernel's row epilogue, read by the res
 static_assert(sizeof(RowInfo) == 32, "the resample kernel reads a RowInfo as two 16-byte words");
 
 struct KParams {
-    int B, G, V, J, nsplit, nchunk, R, chunks_per_cta, mode, bits;
+    int B, G, V, J, nsplit, R, mode, bits;
     int per_warp;  // sweep kernel: 16-byte granules of a logit row that one warp folds; a slice is kWarps times that
     int n_sweep;  // sweep kernel: CTAs that sweep; the rest of the grid (if any) does the resample work
-    int sample;  // 1: draft-side sampling (every drafted position draws a token from its own row)
-    int rs_tail, R2, chunks_per_cta2;  // resample: the last rs_tail draws in launch order use R2 CTAs each
+    int draw_pw;  // draw: granules of the stop position that one warp sums; R CTAs of kWarps warps per batch row
+    int rs_tail, R2, draw_pw2;  // draw: the last rs_tail rows in launch order use R2 CTAs each
     int wait_limit;  // polls a resample CTA spends on its row's completion flag before it gives the row up
     // Generation order of the sweep grid (verification, early != nullptr): first the draft and target rows of
     // positions 0..k_early of every batch row, then the remaining draft rows, last the remaining target rows,
@@ -112,7 +112,10 @@ struct KParams {
     int* rdone;  // verification: rdone[b] = 1 once batch row b's epilogue has written everything the resample kernel reads
     RowInfo* info;
     float4* part;
-    float* csum;
+    float2* spans;  // (reference, sum) of every warp's range of the row a plain draw may need: verification [B, nsplit * kWarps]
+                    // (target position gamma_b), draft-side sampling [B * G, nsplit * kWarps]
+    double* dsum;   // draw: [B, kMaxShares * kWarps] span weights of the stop position
+    double* dsum2;  // shard draw: the same of p beside the residual's
     // vocabulary-sharded verification (speckv_shard.cuh); all zero otherwise
     int part_stride;   // row epilogue: float4s between successive partials of one logit row (0 = adjacent)
     int n_shards;      // row epilogue: tokl holds one [B, G] table per shard, tokl_stride float2s apart
@@ -121,7 +124,6 @@ struct KParams {
     int v_begin;       // sweep: first vocabulary index of this shard's slice (the batch's V is the slice width)
     int export_state;  // sweep: 1 = the row's last CTA writes the merged per-logit-row states instead of the row epilogue
     float4* state;     // [B, J] merged states of this shard (export)
-    float* csum2;      // shard draw: chunk sums of p beside the residual's
     double* weight;    // shard draw: [B, 2] (residual mass, p mass) of this shard
     const double* all_weight;  // [n_shards, B, 2]
     int rank;
@@ -245,37 +247,6 @@ __device__ __forceinline__ float elem_to_float(const __nv_bfloat16* p, long long
 __device__ __forceinline__ float elem_to_float(const float* p, long long i) {
     if (!dbg_ok(p + i, 4, DBG_LOGIT1)) return 0.f;
     return p[i];
-}
-
-// kVec elements starting at element e0 of a row; elements at or beyond `hi` read as `pad`.
-// ALIGNED: the row is 16-byte aligned, so a full vector is one (bf16) or two (fp32) 16-byte loads.
-template <typename T, bool ALIGNED>
-__device__ __forceinline__ Raw<T> load_raw(const T* row, int e0, int hi, float pad) {
-    if (ALIGNED && e0 + kVec <= hi) {
-        Raw<T> r;
-        if constexpr (sizeof(T) == 2) {
-            r.a = ldg_stream(row + e0);
-        } else {
-            r.a = ldg_stream(row + e0);
-            r.b = ldg_stream(row + e0 + 4);
-        }
-        return r;
-    }
-    if (e0 >= hi) return raw_fill<T>(pad);
-    float x[kVec];
-#pragma unroll
-    for (int j = 0; j < kVec; ++j) x[j] = (e0 + j < hi) ? elem_to_float(row, e0 + j) : pad;
-    Raw<T> r;
-    if constexpr (sizeof(T) == 2) {
-        r.a.x = (__float_as_uint(x[0]) >> 16) | (__float_as_uint(x[1]) & 0xFFFF0000u);
-        r.a.y = (__float_as_uint(x[2]) >> 16) | (__float_as_uint(x[3]) & 0xFFFF0000u);
-        r.a.z = (__float_as_uint(x[4]) >> 16) | (__float_as_uint(x[5]) & 0xFFFF0000u);
-        r.a.w = (__float_as_uint(x[6]) >> 16) | (__float_as_uint(x[7]) & 0xFFFF0000u);
-    } else {
-        r.a = make_uint4(__float_as_uint(x[0]), __float_as_uint(x[1]), __float_as_uint(x[2]), __float_as_uint(x[3]));
-        r.b = make_uint4(__float_as_uint(x[4]), __float_as_uint(x[5]), __float_as_uint(x[6]), __float_as_uint(x[7]));
-    }
-    return r;
 }
 
 // NaN-propagating maximum of the kVec raw elements.
@@ -1126,7 +1097,9 @@ __device__ __forceinline__ int row_status0(const KParams& P, int gam, float Tf) 
 // dec: what lane i has learned about position i; ctl: the controller's parameters, fetched beforehand.
 // Order: what the resample kernel needs (acceptance, stop position, normalisers), the row's
 // completion flag, then the signals and the controller.
-__device__ __noinline__ void row_finish(const KParams& P, int b, int gam, float Tf, const RowDecide& dec, const CtlRegs& ctl) {
+// own_bonus: a bonus token is drawn by the caller (from the sweep's spans), not by the CTAs that wait for the flag.
+__device__ __noinline__ void row_finish(const KParams& P, int b, int gam, float Tf, const RowDecide& dec, const CtlRegs& ctl,
+                                        bool own_bonus) {
     const int lane = threadIdx.x & 31;
     const int G = P.G;
     const bool verify = (P.mode & MODE_VERIFY) != 0;
@@ -1167,7 +1140,7 @@ __device__ __noinline__ void row_finish(const KParams& P, int b, int gam, float 
                 if (lane < n) v = x;
                 else if (lane == n && greedy) v = amax_n;
             }
-            P.out_tok[static_cast<long long>(b) * (G + 1) + lane] = v;
+            if (!(own_bonus && rs_mode == RS_BONUS && lane == n)) P.out_tok[static_cast<long long>(b) * (G + 1) + lane] = v;
         }
         if (lane == 0) {
             P.n_acc[b] = n;
@@ -1182,7 +1155,7 @@ __device__ __noinline__ void row_finish(const KParams& P, int b, int gam, float 
         }
     }
     if (P.status && lane == 0) P.status[b] = status;
-    row_done_signal(P, b, rs_mode, n);
+    row_done_signal(P, b, own_bonus && rs_mode == RS_BONUS ? RS_NONE : rs_mode, n);
 
     // signals
     const float in_bits = P.bits ? static_cast<float>(kLog2e) : 1.f;
@@ -1226,73 +1199,7 @@ __device__ __noinline__ void row_epilogue(const KParams& P, int b, int gam, floa
     if ((P.mode & MODE_MLP) && !status) ctl = ctl_load(P, b, threadIdx.x & 31);
     RowDecide dec;
     row_decide<T>(P, b, gam, Tf, status, 32, pd, nd, pt, nt, dec);
-    row_finish(P, b, gam, Tf, dec, ctl);
-}
-
-// Row epilogue of the sliced sweep: a whole CTA, a warp per position.
-template <typename T>
-__device__ __forceinline__ void row_epilogue_cta(const KParams& P, int b, int gam, float Tf, RowDecide* pos) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const bool verify = (P.mode & MODE_VERIFY) != 0;
-    const long long row0 = static_cast<long long>(b) * P.J;
-    const int n_pos = row_status0(P, gam, Tf) ? 0 : verify ? gam + 1 : gam;
-    // the parameters travel while the positions are decided; warp 0 takes the last turns, so it has the fewest positions
-    CtlRegs ctl;
-    if (warp == 0 && (P.mode & MODE_MLP) && n_pos) ctl = ctl_load(P, b, lane);
-    for (int i = kWarps - 1 - warp; i < n_pos; i += kWarps)
-        decide_position<T>(P, b, gam, Tf, i, P.part + (row0 + (verify ? P.G + 1 + i : i)) * P.nsplit, P.part + (row0 + i) * P.nsplit,
-                           P.nsplit, pos[i]);
-    __syncthreads();
-    if (warp != 0) return;
-    RowDecide dec;
-    dec.x = -1; dec.u_res = 0.f; dec.Hi = dec.ci = 0.f; dec.lse2_q = dec.lse2_p = 0.0; dec.amax = -1;
-    dec.dbad = dec.tbad = dec.badtok = false; dec.accept = true;
-    if (lane < n_pos) dec = pos[lane];
-    row_finish(P, b, gam, Tf, dec, ctl);
-}
-
-// Epilogue of the draft-side sampling sweep (one warp per batch row): lane i merges the partials
-// of drafted position i into the row's log2-normaliser (or its argmax for a greedy row) and leaves
-// one RowInfo per position for the resample kernel, which then draws from softmax(d_i / T).
-__device__ __noinline__ void sample_epilogue(const KParams& P, int b, int gam, float Tf, const float4* pt, int nt) {
-    const int lane = threadIdx.x & 31;
-    const int G = P.G;
-    int status = 0;
-    if (gam < 1 || gam > G) status |= 1;
-    if (!(Tf >= 0.f) || Tf == __int_as_float(0x7f800000)) status |= 8;
-    const bool greedy = (Tf == 0.f);
-    const float scale = static_cast<float>(kLog2e / static_cast<double>(greedy ? 1.f : Tf));
-    const bool on = !status && lane < gam;
-    double lse2 = 0.0;
-    int amax = -1;
-    bool nonfinite = false;
-    if (on) {
-        float4 at = ldcg4(pt);
-        for (int k = 1; k < nt; ++k) at = greedy ? merge_argmax(at, ldcg4(pt + k)) : merge_target(at, ldcg4(pt + k));
-        if (greedy) {
-            amax = __float_as_int(at.y);
-            if (at.z != 0.f || amax == 0x7fffffff || !(at.x > kFloor)) nonfinite = true;
-        } else {
-            if (!(at.y > 0.f) || !(at.y < 3e38f)) nonfinite = true;
-            else lse2 = static_cast<double>(at.x) + log2_split(static_cast<double>(at.y));
-        }
-    }
-    if (__any_sync(0xffffffffu, nonfinite)) status |= 4;
-    if (lane < G) {
-        const long long r = static_cast<long long>(b) * G + lane;
-        const bool ok = (status == 0 && lane < gam);
-        RowInfo ri;
-        ri.mode = (ok && !greedy) ? RS_BONUS : RS_NONE;
-        ri.n = lane;
-        ri.u2 = (ok && !greedy) ? __ldg(P.u + r) : 0.f;
-        ri.scale = scale;
-        ri.lse2_p = lse2;
-        ri.lse2_q = 0.0;
-        SPECKV_ST(P.info[r], ri);
-        P.out_tok[r] = (ok && greedy) ? amax : -1;
-    }
-    if (P.status && lane == 0) P.status[b] = status;
-    row_done_signal(P, b, RS_NONE, 0);  // every position of the row has its own record: the flag only says they are written
+    row_finish(P, b, gam, Tf, dec, ctl, false);
 }
 
 // Epilogue of a vocabulary shard's sweep (one warp per batch row): lane i merges this shard's nd
@@ -1327,617 +1234,6 @@ __device__ __noinline__ void export_epilogue(const KParams& P, int b, int gam, f
         }
         SPECKV_ST(out[lane], at);
     }
-}
-
-// One CTA's share of a batch row's fresh-token draw (defined with the resample kernel below).
-template <typename T, bool ALIGNED>
-__device__ __forceinline__ void resample_body(const KParams& P, const int bid);
-template <typename T, bool ALIGNED>
-__device__ __forceinline__ void resample_row(const KParams& P, const int b, const int r, const int mode, const int n,
-                                             const int4 lo4, const int4 hi4, const int share, const int Rr, const int cpc);
-
-// ----------------------------------------------------------------------------------------
-// Sweep kernel.  CTAs 0 .. n_sweep-1 sweep one slice of one logit row each.  With verification the
-// grid may carry B*R more CTAs behind them that do the resample kernel's work in the same launch:
-// CTAs start in index order, so these start exactly when the sweep runs out of slices, wait (with
-// a bound) for their batch row's completion flag and fill the SMs that the sweep's last CTAs
-// leave one by one.  A second launch, even a programmatic dependent one, starts microseconds
-// after the last sweep CTA has started and leaves most of the drain unused.
-// ----------------------------------------------------------------------------------------
-template <typename T, bool ALIGNED, int U>
-__global__ void __launch_bounds__(kThreads, kSweepCtasPerSm) sweep_kernel(const __grid_constant__ KParams P) {
-    if (static_cast<int>(blockIdx.x) >= P.n_sweep) {
-        resample_body<T, ALIGNED>(P, static_cast<int>(blockIdx.x) - P.n_sweep);
-        return;
-    }
-    __shared__ float4 sh_part[kWarps];
-    __shared__ RowDecide sh_pos[kMaxGamma + 1];
-    __shared__ int sh_last;
-    __shared__ int sh_early;
-    __shared__ float sh_m0[kWarps];
-    asm volatile("griddepcontrol.launch_dependents;");  // a dependent resample kernel may be scheduled as SMs free up
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const bool verify = (P.mode & MODE_VERIFY) != 0;
-    int b, j, s, gen = 0;
-    if (P.early) {
-        // generation order: CTAs start in index order, so a later generation starts when the earlier ones
-        // are all under way and, for all but the smallest batches, long after the first one has finished
-        const int ns = P.nsplit, k1 = P.k_early + 1;
-        const int nA = k1 * P.B * 2 * ns, nB = (P.G - k1) * P.B * ns;
-        int i = blockIdx.x, p, is_draft;
-        if (i < nA) {
-            p = i / (2 * P.B * ns); i -= p * (2 * P.B * ns);
-            b = i / (2 * ns); i -= b * (2 * ns);
-            is_draft = i / ns; s = i - is_draft * ns;
-        } else {
-            // the later generations go batch row by batch row, so that the rows complete one after another
-            gen = (i < nA + nB) ? 1 : 2;
-            i -= (gen == 1) ? nA : nA + nB;
-            const int per_b = (gen == 1 ? P.G - k1 : P.G + 1 - k1) * ns;
-            b = i / per_b; i -= b * per_b;
-            p = i / ns; s = i - p * ns;
-            p += k1;
-            is_draft = (gen == 1);
-        }
-        j = is_draft ? P.G + 1 + p : p;
-    } else {
-        const int per_row = P.J * P.nsplit;
-        b = blockIdx.x / per_row;
-        const int r = blockIdx.x - b * per_row;
-        j = r / P.nsplit;
-        s = r - j * P.nsplit;
-    }
-    // the row's gamma and temperature travel together with the one thing a CTA of the last generation has
-    // to learn first: one memory round trip before the CTA knows whether it has work
-    int gam = P.gamma ? P.gamma[b] : P.G;
-    float Tf = P.temp ? P.temp[b] : P.temp_scalar;
-    if (threadIdx.x == 0) {
-        // one thread reads what is known of the row's stop position, so that the whole CTA takes one decision
-        int e = 0;
-        if (gen == 2 && !P.read_all)
-            asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(e) : "l"(P.early + b) : "memory");
-        sh_early = e;
-    }
-    if (threadIdx.x < kWarps) sh_m0[threadIdx.x] = kFloor;
-    __syncthreads();  // before any load is issued
-    const int rem = j * P.nsplit + s;
-
-    const bool row_ok = (gam >= 1 && gam <= P.G) && (Tf >= 0.f) && (Tf != __int_as_float(0x7f800000));
-    const bool greedy = (Tf == 0.f);
-    const float scale = static_cast<float>(kLog2e / static_cast<double>(greedy ? 1.f : Tf));
-
-    // logit row handled by this CTA: with verification, j <= G are target positions and the
-    // rest draft positions; signals alone sweep draft positions only
-    // (draft-side sampling sweeps the drafted positions with the target statistics: only the
-    // normaliser, or the argmax, of each row is needed; P.t then points at the draft logits)
-    const bool is_target = P.sample || (verify && j <= P.G);
-    const int pos = is_target ? j : (verify ? j - (P.G + 1) : j);
-    const bool active = row_ok && ((is_target && !P.sample) ? pos <= gam : pos < gam);
-    const long long pidx = (static_cast<long long>(b) * P.J + j) * P.nsplit + s;  // this CTA's partial
-
-    // the walk stopped at a position before this one
-    const bool skipped = active && gen == 2 && sh_early != 0 && sh_early <= P.k_early + 1;
-    if (skipped) {
-        // the row epilogue never looks behind the stop position; the partial only has to be finite
-        if (threadIdx.x == 0)
-            SPECKV_ST(P.part[pidx], greedy ? make_float4(kFloor, __int_as_float(0x7fffffff), 0.f, 0.f)
-                                           : make_float4(kFloor, 0.f, 0.f, 0.f));
-    } else if (active) {
-        // this warp's granules: the CTA's slice is cut into one contiguous range per warp
-        const int lo = (s * kWarps + warp) * P.per_warp, hi = lo + P.per_warp;
-        float4 part;
-        int path;
-        if (is_target) {
-            const T* row = static_cast<const T*>(P.t) + static_cast<long long>(b) * P.tsb +
-                           static_cast<long long>(pos) * P.tsp;
-            if (greedy) { part = sweep_warp<T, PATH_ARGMAX, U>(make_row(row, P.V), lo, hi, scale, sh_m0); path = PATH_ARGMAX; }
-            else { part = sweep_warp<T, PATH_TARGET, U>(make_row(row, P.V), lo, hi, scale, sh_m0); path = PATH_TARGET; }
-        } else {
-            const T* row = static_cast<const T*>(P.d) + static_cast<long long>(b) * P.dsb +
-                           static_cast<long long>(pos) * P.dsp;
-            if (verify && P.tokl && s == 0 && threadIdx.x == 0 && !greedy) {
-                // the acceptance test of this position needs both logits at the draft token: fetch them
-                // now, while the sweep hides the latency, and leave them for the row epilogue
-                const int x = __ldg(P.tok + static_cast<long long>(b) * P.G + pos) - P.v_begin;  // index in this slice
-                if (x >= 0 && x < P.V) {
-                    const T* trow = static_cast<const T*>(P.t) + static_cast<long long>(b) * P.tsb +
-                                    static_cast<long long>(pos) * P.tsp;
-                    SPECKV_ST(P.tokl[static_cast<long long>(b) * P.G + pos], make_float2(elem_to_float(row, x), elem_to_float(trow, x)));
-                }
-            }
-            part = sweep_warp<T, PATH_DRAFT, U>(make_row(row, P.V), lo, hi, scale, sh_m0);
-            path = PATH_DRAFT;
-        }
-        if (lane == 0) sh_part[warp] = part;
-        __syncthreads();
-        if (warp == 0) {
-            const float4 none = (path == PATH_ARGMAX) ? make_float4(kFloor, __int_as_float(0x7fffffff), 0.f, 0.f)
-                              : make_float4(path == PATH_TARGET ? -3.0e38f : kFloor, 0.f, 0.f, 0.f);
-            const float4 w = lane < kWarps ? sh_part[lane] : none;
-            const float4 acc = (path == PATH_DRAFT) ? warp_merge<PATH_DRAFT>(w, scale)
-                             : (path == PATH_TARGET) ? warp_merge<PATH_TARGET>(w, scale) : warp_merge<PATH_ARGMAX>(w, scale);
-            if (lane == 0) SPECKV_ST(P.part[pidx], acc);
-        }
-    } else if (row_ok || rem != 0) {
-        return;  // unused position: nothing to count; a flagged row keeps its first CTA for the epilogue
-    }
-
-    // tickets: the last of the row's CTAs of positions 0..k_early takes their acceptance tests, the last of all its active
-    // CTAs runs the row epilogue; nobody waits
-    if (threadIdx.x == 0) {
-        const int n_rows = P.sample ? gam : (verify ? 2 * gam + 1 : gam);
-        const int n_tickets = row_ok ? n_rows * P.nsplit : 1;
-        const int n_pre = (min(P.k_early, gam) + 1 + min(P.k_early + 1, gam)) * P.nsplit;
-        __threadfence();
-        int pre = -1;
-        if (P.early && active && gen == 0) pre = atomicAdd(P.tick_early + b, 1);
-        const int all = atomicAdd(P.tick1 + b, 1);
-        const int l = (all == n_tickets - 1 ? 2 : 0) | (pre == n_pre - 1 ? 1 : 0);
-        if (l) __threadfence();
-        sh_last = l;
-    }
-    __syncthreads();
-    const int last = sh_last;
-    if (last & 1) prefix_epilogue<T>(P, b, gam, Tf, sh_pos);
-    if (!(last & 2)) return;
-    const long long row0 = static_cast<long long>(b) * P.J;
-    if (P.sample) {
-        if (warp == 0) sample_epilogue(P, b, gam, Tf, P.part + (row0 + lane) * P.nsplit, P.nsplit);
-        return;
-    }
-    if (P.export_state) {
-        if (warp == 0)
-            export_epilogue(P, b, gam, Tf, P.part + (row0 + P.G + 1 + lane) * P.nsplit, P.nsplit,
-                            P.part + (row0 + lane) * P.nsplit, P.nsplit);
-        return;
-    }
-    row_epilogue_cta<T>(P, b, gam, Tf, sh_pos);
-}
-
-// ----------------------------------------------------------------------------------------
-// Resample kernel: inverse CDF over the stop position's weights, vocabulary order.
-//   residual: w_v = max(0, p_v - q_v);   bonus: w_v = p_v
-// p_v and q_v are evaluated with fp32 exp2 against normalisers carried as two floats; the chunk
-// sums are fp32, everything above a chunk is summed in double.  A residual whose total mass is
-// below 1e-6 cannot be told from rounding noise and is treated as empty (p == q at the stop
-// position): the token is then drawn from p.
-// ----------------------------------------------------------------------------------------
-struct RsConst {
-    int mode;
-    float scale, lp_hi, lp_lo, lq_hi, lq_lo;
-};
-
-__device__ __forceinline__ RsConst rs_const(const RowInfo& ri, int mode) {
-    RsConst c;
-    c.mode = mode;
-    c.scale = ri.scale;
-    // log2-normalisers split into two floats so that the exponent argument keeps the bits a
-    // single float would drop
-    c.lp_hi = static_cast<float>(ri.lse2_p);
-    c.lp_lo = static_cast<float>(ri.lse2_p - static_cast<double>(c.lp_hi));
-    c.lq_hi = static_cast<float>(ri.lse2_q);
-    c.lq_lo = static_cast<float>(ri.lse2_q - static_cast<double>(c.lq_hi));
-    return c;
-}
-
-// w = p (bonus) or max(0, p - q) (residual); explicit roundings so that the first pass and the
-// rescan of the located chunk produce the same bits
-__device__ __forceinline__ float rs_weight(const RsConst& c, float xt, float xd) {
-    const float p = ex2f(__fsub_rn(__fmaf_rn(xt, c.scale, -c.lp_hi), c.lp_lo));
-    if (c.mode == RS_BONUS) return p;
-    const float q = ex2f(__fsub_rn(__fmaf_rn(xd, c.scale, -c.lq_hi), c.lq_lo));
-    return fmaxf(__fsub_rn(p, q), 0.f);
-}
-
-// A lane's kVec elements of a 256-element chunk.  bf16: eight adjacent elements (one 16-byte load, the warp
-// reads 512 contiguous bytes).  fp32: four adjacent elements of the chunk's first half and four of its
-// second half, so that each of the two loads of the warp covers 512 contiguous bytes (with eight
-// adjacent floats per lane every 32-byte sector would be requested twice).  rs_elem gives the vocabulary
-// index of element j.
-template <typename T>
-__device__ __forceinline__ int rs_elem(int chunk, int lane, int j) {
-    if constexpr (sizeof(T) == 2) return chunk * kChunk + lane * kVec + j;
-    else return chunk * kChunk + (j < kVec / 2 ? lane * (kVec / 2) + j : kChunk / 2 + lane * (kVec / 2) + j - kVec / 2);
-}
-template <bool ALIGNED>
-__device__ __forceinline__ uint4 rs_load4(const float* row, int e, int hi, float pad) {
-    if (ALIGNED && e + 4 <= hi) return ldg_stream(row + e);
-    float x[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) x[j] = (e + j < hi) ? elem_to_float(row, e + j) : pad;
-    return make_uint4(__float_as_uint(x[0]), __float_as_uint(x[1]), __float_as_uint(x[2]), __float_as_uint(x[3]));
-}
-template <typename T, bool ALIGNED>
-__device__ __forceinline__ Raw<T> rs_load_lane(const T* row, int chunk, int V, float pad) {
-    const int lane = threadIdx.x & 31;
-    if constexpr (sizeof(T) == 2) {
-        return load_raw<T, ALIGNED>(row, chunk * kChunk + lane * kVec, V, pad);
-    } else {
-        Raw<T> r;
-        r.a = rs_load4<ALIGNED>(row, chunk * kChunk + lane * 4, V, pad);
-        r.b = rs_load4<ALIGNED>(row, chunk * kChunk + kChunk / 2 + lane * 4, V, pad);
-        return r;
-    }
-}
-
-template <typename T, bool ALIGNED>
-__device__ __forceinline__ void rs_load(const RsConst& c, const T* trow, const T* drow, int chunk, int V,
-                                        Raw<T>& rt, Raw<T>& rd) {
-    const float ninf = __int_as_float(0xff800000);
-    rt = rs_load_lane<T, ALIGNED>(trow, chunk, V, ninf);
-    if (c.mode == RS_RESIDUAL) rd = rs_load_lane<T, ALIGNED>(drow, chunk, V, ninf);
-    else rd = raw_fill<T>(ninf);
-}
-
-// the kVec weights of one lane, two elements per instruction; per element the same operations and
-// roundings as rs_weight, so both give the same bits
-template <typename T>
-__device__ __forceinline__ void rs_weights(const RsConst& c, const Raw<T>& rt, const Raw<T>& rd, float (&w)[kVec]) {
-    const f2 sc2 = pack2(c.scale, c.scale);
-    const f2 ph2 = pack2(-c.lp_hi, -c.lp_hi), pl2 = pack2(c.lp_lo, c.lp_lo);
-    f2 xt[4];
-    unpack_pairs(rt, xt);
-    if (c.mode == RS_BONUS) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const f2 p = ex2_2(sub2(fma2(xt[i], sc2, ph2), pl2));
-            unpack2(p, w[2 * i], w[2 * i + 1]);
-        }
-        return;
-    }
-    const f2 qh2 = pack2(-c.lq_hi, -c.lq_hi), ql2 = pack2(c.lq_lo, c.lq_lo);
-    f2 xd[4];
-    unpack_pairs(rd, xd);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const f2 p = ex2_2(sub2(fma2(xt[i], sc2, ph2), pl2));
-        const f2 q = ex2_2(sub2(fma2(xd[i], sc2, qh2), ql2));
-        float lo, hi;
-        unpack2(sub2(p, q), lo, hi);
-        w[2 * i] = fmaxf(lo, 0.f);
-        w[2 * i + 1] = fmaxf(hi, 0.f);
-    }
-}
-
-template <typename T, bool ALIGNED>
-__device__ __forceinline__ void rs_chunk_weights(const RsConst& c, const T* trow, const T* drow, int chunk,
-                                                 int V, float (&w)[kVec]) {
-    Raw<T> rt, rd;
-    rs_load<T, ALIGNED>(c, trow, drow, chunk, V, rt, rd);
-    rs_weights<T>(c, rt, rd, w);
-}
-
-// Each warp takes KU chunks at a time (c0+warp, +8, ...) and requests the next KU before it evaluates
-// the current ones, so the memory latency is paid once per CTA, not once per batch.  MODE is the
-// row's mode as a constant: a bonus draw never touches the draft row, so its registers go into a
-// deeper batch instead.  The buffers of both batches stay within 32 registers per thread for
-// either element type; more than that spills and the kernel falls to a fraction of its rate.
-template <typename T, bool ALIGNED, int MODE, int KU>
-__device__ __forceinline__ void rs_load_batch(const T* trow, const T* drow, int base, int c1, int V,
-                                              Raw<T> (&rt)[KU], Raw<T> (&rd)[KU]) {
-    const float ninf = __int_as_float(0xff800000);
-#pragma unroll
-    for (int u = 0; u < KU; ++u) {
-        const int ch = base + u * kWarps;
-        if (ch < c1) {
-            rt[u] = rs_load_lane<T, ALIGNED>(trow, ch, V, ninf);
-            if (MODE == RS_RESIDUAL) rd[u] = rs_load_lane<T, ALIGNED>(drow, ch, V, ninf);
-        } else {
-            rt[u] = raw_fill<T>(ninf);
-            if (MODE == RS_RESIDUAL) rd[u] = rt[u];
-        }
-    }
-}
-
-// make_const() yields the row's constants; it is called after the first batch of loads has been issued,
-// so constants that are themselves still on their way from memory do not hold the loads up.
-template <typename T, bool ALIGNED, int MODE, int KU, class F>
-__device__ __forceinline__ void rs_chunk_sums_mode(F make_const, const T* trow, const T* drow, int c0, int c1,
-                                                   int V, float* csum) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int base = c0 + warp;
-    if (base >= c1) return;
-    Raw<T> rt[KU], rd[KU];
-    rs_load_batch<T, ALIGNED, MODE, KU>(trow, drow, base, c1, V, rt, rd);
-    RsConst c = make_const();
-    c.mode = MODE;
-    while (base < c1) {
-        const int next = base + kWarps * KU;
-        Raw<T> nt[KU], nd[KU];
-        if (next < c1) rs_load_batch<T, ALIGNED, MODE, KU>(trow, drow, next, c1, V, nt, nd);
-        float s[KU];
-#pragma unroll
-        for (int u = 0; u < KU; ++u) {
-            float w[kVec];
-            rs_weights<T>(c, rt[u], rd[u], w);
-            s[u] = 0.f;
-#pragma unroll
-            for (int j = 0; j < kVec; ++j) s[u] = __fadd_rn(s[u], w[j]);
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-            for (int u = 0; u < KU; ++u) s[u] = __fadd_rn(s[u], __shfl_xor_sync(0xffffffffu, s[u], o));
-        }
-#pragma unroll
-        for (int u = 0; u < KU; ++u) {
-            const int ch = base + u * kWarps;
-            if (lane == 0 && ch < c1) SPECKV_ST(csum[ch], s[u]);
-        }
-        if (next < c1) {
-#pragma unroll
-            for (int u = 0; u < KU; ++u) {
-                rt[u] = nt[u];
-                if (MODE == RS_RESIDUAL) rd[u] = nd[u];
-            }
-        }
-        base = next;
-    }
-}
-
-template <typename T, bool ALIGNED>
-__device__ __forceinline__ void rs_chunk_sums(const RsConst& c, const T* trow, const T* drow, int c0, int c1,
-                                              int V, float* csum) {
-    constexpr int kResidual = sizeof(T) == 2 ? 2 : 1;  // chunks per batch: two rows to buffer
-    constexpr int kBonus = 2;  // one row to buffer; measured: deeper bf16 batches leave a warp too few iterations
-    auto mk = [&]() { return c; };
-    if (c.mode == RS_BONUS) rs_chunk_sums_mode<T, ALIGNED, RS_BONUS, kBonus>(mk, trow, drow, c0, c1, V, csum);
-    else rs_chunk_sums_mode<T, ALIGNED, RS_RESIDUAL, kResidual>(mk, trow, drow, c0, c1, V, csum);
-}
-
-// RowInfo as the two 16-byte words it is loaded as
-__device__ __forceinline__ RowInfo row_info_from(const int4& lo4, const int4& hi4) {
-    RowInfo ri;
-    ri.mode = lo4.x; ri.n = lo4.y; ri.u2 = __int_as_float(lo4.z); ri.scale = __int_as_float(lo4.w);
-    ri.lse2_p = __hiloint2double(hi4.y, hi4.x);
-    ri.lse2_q = __hiloint2double(hi4.w, hi4.z);
-    return ri;
-}
-// The same sums for a row whose mode is known but whose RowInfo words may still be in flight
-template <typename T, bool ALIGNED>
-__device__ __forceinline__ void rs_chunk_sums_info(int mode, const int4& lo4, const int4& hi4, const T* trow, const T* drow,
-                                                   int c0, int c1, int V, float* csum) {
-    constexpr int kResidual = sizeof(T) == 2 ? 2 : 1;
-    constexpr int kBonus = 2;
-    auto mk = [&]() { return rs_const(row_info_from(lo4, hi4), mode); };
-    if (mode == RS_BONUS) rs_chunk_sums_mode<T, ALIGNED, RS_BONUS, kBonus>(mk, trow, drow, c0, c1, V, csum);
-    else rs_chunk_sums_mode<T, ALIGNED, RS_RESIDUAL, kResidual>(mk, trow, drow, c0, c1, V, csum);
-}
-
-// The last CTA of a row copies the row's chunk sums into shared memory (one memory round trip for
-// all of them) before it searches them; rows with more chunks than fit are searched in place.
-constexpr int kRsStage = 2048;
-struct RsSums {
-    const float* sh;    // staged copy, or nullptr
-    const float* glob;
-    __device__ __forceinline__ float operator[](int ch) const {
-        if (sh) return sh[ch];
-        return dbg_ok(glob + ch, 4, DBG_WS_LOAD) ? __ldcg(glob + ch) : 0.f;
-    }
-};
-__device__ __forceinline__ RsSums rs_stage_sums(float* sh_cs, const float* csum, int nchunk) {
-    RsSums r;
-    r.glob = csum;
-    r.sh = nullptr;
-    if (nchunk <= kRsStage) {
-        for (int ch = threadIdx.x; ch < nchunk; ch += kThreads) sh_cs[ch] = dbg_ok(csum + ch, 4, DBG_WS_LOAD) ? __ldcg(csum + ch) : 0.f;
-        r.sh = sh_cs;
-    }
-    __syncthreads();
-    return r;
-}
-
-// warp 0: total weight W of the row from its chunk sums
-__device__ __forceinline__ double rs_total(const RsSums& cs, int nchunk, int per_lane, double* own_out) {
-    const int lane = threadIdx.x & 31;
-    double own = 0.0;
-    const int a = lane * per_lane, e = min(nchunk, a + per_lane);
-    for (int ch = a; ch < e; ++ch) own += static_cast<double>(cs[ch]);
-    *own_out = own;
-    return warp_sum(own);
-}
-
-// Warp 0 of the CTA that holds a row's chunk sums: the vocabulary index at which the running sum of the
-// weights first exceeds tau (the last index with weight if rounding leaves tau at or above the total).
-// own = this lane's share of the chunk sums as rs_total left it.  The located chunk's weights are
-// recomputed, bit-identical to the first pass.  Every lane returns the index.
-template <typename T, bool ALIGNED>
-__device__ __forceinline__ int rs_search(const RsConst& c, const T* trow, const T* drow, const RsSums& cs, int nchunk,
-                                         int V, double tau, double own, int per_lane) {
-    const int lane = threadIdx.x & 31;
-    // inclusive scan of the per-lane group sums
-    double incl = own;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        double v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-    }
-    unsigned hit = __ballot_sync(0xffffffffu, incl > tau && own > 0.0);
-    unsigned pos = __ballot_sync(0xffffffffu, own > 0.0);
-    int src = hit ? (__ffs(hit) - 1) : (31 - __clz(pos));  // fallback: last group with weight
-    // the chosen lane walks its chunks
-    int chunk = -1;
-    double before = 0.0;
-    if (lane == src) {
-        double run = incl - own;
-        const int a = lane * per_lane, e = min(nchunk, a + per_lane);
-        int last_pos = -1;
-        double last_before = 0.0;
-        for (int ch = a; ch < e; ++ch) {
-            double sv = static_cast<double>(cs[ch]);
-            if (sv > 0.0) { last_pos = ch; last_before = run; }
-            if (run + sv > tau && sv > 0.0) { chunk = ch; before = run; break; }
-            run += sv;
-        }
-        if (chunk < 0) { chunk = last_pos; before = last_before; }
-    }
-    chunk = __shfl_sync(0xffffffffu, chunk, src);
-    before = __shfl_sync(0xffffffffu, before, src);
-
-    // recompute the chunk's weights (bit-identical to the first pass) and scan them
-    float w[kVec];
-    rs_chunk_weights<T, ALIGNED>(c, trow, drow, chunk, V, w);
-    // a lane's elements form one run of the chunk (bf16) or two (fp32, see rs_elem): scan run by run
-    constexpr int kSeg = sizeof(T) == 2 ? 1 : 2, kSegLen = kVec / kSeg;
-    int found = 0x7fffffff, lastw = -1;
-    double seg_base = before;
-#pragma unroll
-    for (int sg = 0; sg < kSeg; ++sg) {
-        double lane_tot = 0.0;
-#pragma unroll
-        for (int j = 0; j < kSegLen; ++j) lane_tot += static_cast<double>(w[sg * kSegLen + j]);
-        double lincl = lane_tot;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            double v = __shfl_up_sync(0xffffffffu, lincl, o);
-            if (lane >= o) lincl += v;
-        }
-        double run = seg_base + (lincl - lane_tot);
-#pragma unroll
-        for (int j = 0; j < kSegLen; ++j) {
-            run += static_cast<double>(w[sg * kSegLen + j]);
-            const int idx = rs_elem<T>(chunk, lane, sg * kSegLen + j);
-            if (w[sg * kSegLen + j] > 0.f) {
-                lastw = max(lastw, idx);
-                if (run > tau && found == 0x7fffffff) found = idx;
-            }
-        }
-        seg_base += __shfl_sync(0xffffffffu, lincl, 31);  // the whole run
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        found = min(found, __shfl_xor_sync(0xffffffffu, found, o));
-        lastw = max(lastw, __shfl_xor_sync(0xffffffffu, lastw, o));
-    }
-    return (found != 0x7fffffff) ? found : lastw;
-}
-
-template <typename T, bool ALIGNED>
-__device__ __forceinline__ void resample_body(const KParams& P, const int bid) {
-    __shared__ int sh_flag;
-    // one-dimensional grid, R consecutive CTAs per batch row: the CTAs of a row are neighbours in
-    // launch order, so rows finish one after the other and their searches overlap the other rows' sums
-    // (draft-side sampling: one draw per drafted position; r counts positions, b = r / gamma_max)
-    // the last rs_tail draws (in launch order) are cut into R2 >= R shares: their rows are the last to
-    // be swept, nothing is left to overlap their draw with, and more CTAs per row shorten it
-    const int n_all = P.sample ? P.B * P.G : P.B;
-    const int n_head = (n_all - P.rs_tail) * P.R;
-    const bool tail = bid >= n_head;
-    const int Rr = tail ? P.R2 : P.R;
-    const int cpc = tail ? P.chunks_per_cta2 : P.chunks_per_cta;
-    const int bq = tail ? (n_all - P.rs_tail) + (bid - n_head) / Rr : bid / Rr;
-    const int share = tail ? (bid - n_head) % Rr : bid % Rr;
-    const int r = P.rs_reverse ? (P.sample ? P.B * P.G : P.B) - 1 - bq : bq;
-    const int b = P.sample ? r / P.G : r;
-    // Launched as a programmatic dependent of the sweep kernel, so its CTAs become resident as the
-    // sweep's last CTAs leave.  With completion flags a CTA waits only for its own batch row (rows
-    // are taken in the order the sweep finishes them unless rs_reverse is set) and the stop positions of finished rows are
-    // summed while the sweep drains; every sweep CTA is resident or done before the first CTA of
-    // this kernel starts, so the wait ends, and it is bounded all the same.  Without flags the CTA
-    // waits for the whole sweep grid.
-    const int4* ip = reinterpret_cast<const int4*>(P.info + r);
-    int mode, n;
-    int4 lo4, hi4;
-    if (P.rdone) {
-        if (threadIdx.x == 0) sh_flag = row_done_wait(P.rdone + b, P.wait_limit);
-        __syncthreads();
-        const int v = sh_flag;
-        if (!v) {
-            // Gave up.  The mark goes on the row's flag: if the row epilogue has already written the
-            // status (the flag went up just after the last poll) the bit is added here, otherwise the
-            // epilogue finds the mark when it raises the flag and adds the bit itself.
-            if (threadIdx.x == 0 && share == 0) {
-                const int old = atomicOr(P.rdone + b, kRowDoneTimeout);
-                if ((old & 1) && P.status) atomicOr(P.status + b, 16);
-            }
-            return;
-        }
-        __syncthreads();  // sh_flag is reused below
-        // mode and stop position came with the flag: the logit loads below can go out at once, the
-        // rest of the row's record (normalisers, second uniform) travels beside them
-        lo4 = __ldcg(ip); hi4 = __ldcg(ip + 1);
-        if (P.sample) {  // one record per drafted position behind one flag per batch row
-            mode = lo4.x;
-            n = lo4.y;
-        } else {
-            mode = (v >> 8) & 3;
-            n = (v >> 16) & 0xff;
-        }
-    } else {
-        asm volatile("griddepcontrol.wait;" ::: "memory");
-        lo4 = __ldcg(ip); hi4 = __ldcg(ip + 1);
-        mode = lo4.x;
-        n = lo4.y;
-    }
-    resample_row<T, ALIGNED>(P, b, r, mode, n, lo4, hi4, share, Rr, cpc);
-}
-
-// One CTA's share (chunks share*cpc ...) of draw r of batch row b; the last of the draw's Rr CTAs to arrive
-// locates the token.  lo4 / hi4: the row's record as loaded from P.info[r].
-template <typename T, bool ALIGNED>
-__device__ __forceinline__ void resample_row(const KParams& P, const int b, const int r, const int mode, const int n,
-                                             const int4 lo4, const int4 hi4, const int share, const int Rr, const int cpc) {
-    __shared__ int sh_flag;
-    __shared__ int sh_empty;
-    __shared__ float sh_cs[kRsStage];
-    const int4* ip = reinterpret_cast<const int4*>(P.info + r);
-    if (mode == RS_NONE) return;  // greedy or flagged row: nothing to draw
-    const long long out_at = P.sample ? static_cast<long long>(r) : static_cast<long long>(b) * (P.G + 1) + n;
-
-    const T* trow = static_cast<const T*>(P.t) + static_cast<long long>(b) * P.tsb +
-                    static_cast<long long>(n) * P.tsp;
-    const T* drow = static_cast<const T*>(P.d) + static_cast<long long>(b) * P.dsb +
-                    static_cast<long long>(n) * P.dsp;
-    float* csum = P.csum + static_cast<long long>(r) * P.nchunk;
-
-    const int c0 = share * cpc;
-    const int c1 = min(P.nchunk, c0 + cpc);
-    rs_chunk_sums_info<T, ALIGNED>(mode, lo4, hi4, trow, drow, c0, c1, P.V, csum);
-
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        int old = atomicAdd(P.tick2 + r, 1);
-        sh_flag = (old == Rr - 1);
-    }
-    __syncthreads();
-    if (!sh_flag) return;
-    __threadfence();
-
-    // ---- last CTA of the row: locate the threshold ----
-    const RowInfo ri = row_info_from(__ldcg(ip), __ldcg(ip + 1));  // fetched again rather than kept in registers
-    RsConst c = rs_const(ri, mode);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int per_lane = (P.nchunk + 31) / 32;
-    double own = 0.0, W = 0.0;
-    RsSums cs = rs_stage_sums(sh_cs, csum, P.nchunk);
-    if (warp == 0) {
-        W = rs_total(cs, P.nchunk, per_lane, &own);
-        if (lane == 0) sh_empty = (W > (c.mode == RS_RESIDUAL ? 1e-6 : 0.0)) ? 0 : 1;
-    }
-    __syncthreads();
-    if (sh_empty) {
-        // numerically empty residual (p == q at the stop position): draw from p instead
-        if (c.mode != RS_RESIDUAL) {  // p itself has no mass: cannot happen for a finite row
-            if (threadIdx.x == 0) P.out_tok[out_at] = 0;
-            return;
-        }
-        c.mode = RS_BONUS;
-        rs_chunk_sums<T, ALIGNED>(c, trow, drow, 0, P.nchunk, P.V, csum);
-        __syncthreads();
-        cs = rs_stage_sums(sh_cs, csum, P.nchunk);
-        if (warp == 0) W = rs_total(cs, P.nchunk, per_lane, &own);
-    }
-    if (warp != 0) return;
-
-    const double tau = static_cast<double>(ri.u2) * W;
-    const int tok = rs_search<T, ALIGNED>(c, trow, drow, cs, P.nchunk, P.V, tau, own, per_lane);
-    if (lane == 0) P.out_tok[out_at] = tok;
-}
-
-template <typename T, bool ALIGNED>
-__global__ void __launch_bounds__(kThreads, 4) resample_kernel(const __grid_constant__ KParams P) {
-    resample_body<T, ALIGNED>(P, static_cast<int>(blockIdx.x));
 }
 
 // ----------------------------------------------------------------------------------------

@@ -12,7 +12,7 @@
 // CDF runs over the vocabulary in index order, shard after shard.
 #pragma once
 
-#include "speckv_kernels.cuh"
+#include "speckv_draw.cuh"
 
 namespace speckv {
 
@@ -72,63 +72,66 @@ __global__ void __launch_bounds__(kThreads) shard_finish_kernel(const __grid_con
     row_epilogue<T>(P, b, gam, Tf, row + P.G + 1 + lane, P.n_shards, row + lane, P.n_shards);
 }
 
-// Phase 3: grid B * R.  Chunk sums of the stop position over the local slice: of the row's own
+// Phase 3: grid B * R.  Span weights of the stop position over the local slice: of the row's own
 // weights and, for a residual draw, of p as well (the draw falls back to p when the residual is
 // numerically empty, and whether it is shows only once all shards' masses are known).  The last
 // CTA of a row adds them up.
-template <typename T, bool ALIGNED>
+template <typename T>
 __global__ void __launch_bounds__(kThreads, 4) shard_sums_kernel(const __grid_constant__ KParams P) {
     __shared__ int sh_flag;
-    __shared__ float sh_cs[kRsStage];
     const int b = blockIdx.x / P.R;
     const int share = blockIdx.x - b * P.R;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const RowInfo ri = P.info[b];
     if (ri.mode == RS_NONE) {
         if (share == 0 && threadIdx.x < 2) P.weight[2 * static_cast<long long>(b) + threadIdx.x] = 0.0;
         return;
     }
+    const bool res = ri.mode == RS_RESIDUAL;
     const T* trow = static_cast<const T*>(P.t) + static_cast<long long>(b) * P.tsb + static_cast<long long>(ri.n) * P.tsp;
     const T* drow = static_cast<const T*>(P.d) + static_cast<long long>(b) * P.dsb + static_cast<long long>(ri.n) * P.dsp;
-    float* csum = P.csum + static_cast<long long>(b) * P.nchunk;
-    float* csum_p = P.csum2 + static_cast<long long>(b) * P.nchunk;
-    RsConst c = rs_const(ri, ri.mode);
-    const int c0 = share * P.chunks_per_cta;
-    const int c1 = min(P.nchunk, c0 + P.chunks_per_cta);
-    if (ri.mode == RS_RESIDUAL) rs_chunk_sums<T, ALIGNED>(c, trow, drow, c0, c1, P.V, csum);
-    c.mode = RS_BONUS;
-    rs_chunk_sums<T, ALIGNED>(c, trow, drow, c0, c1, P.V, csum_p);
-
+    DrawSrc src = make_draw<T>(trow, res ? drow : nullptr, P.V);
+    set_norm(src, ri.scale, ri.lse2_p, ri.lse2_q);
+    auto norm = [](DrawSrc&) {};
+    double* dr = P.dsum + static_cast<long long>(b) * (kMaxShares * kWarps);
+    double* dp = P.dsum2 + static_cast<long long>(b) * (kMaxShares * kWarps);
+    const int span = share * kWarps + warp, g0 = span * P.draw_pw, g1 = min(src.t.ng, g0 + P.draw_pw);
+    const double wr = res ? warp_weight<T, true>(src, g0, g1, norm) : 0.0;
+    const double wp = warp_weight<T, false>(src, g0, g1, norm);
+    if (lane == 0) {
+        SPECKV_ST(dr[span], wr);
+        SPECKV_ST(dp[span], wp);
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
-        sh_flag = (atomicAdd(P.tick2 + b, 1) == P.R - 1);
+        const bool last = atomicAdd(P.tick2 + b, 1) == P.R - 1;
+        if (last) __threadfence();
+        sh_flag = last;
     }
     __syncthreads();
-    if (!sh_flag) return;
-    __threadfence();
-    const int per_lane = (P.nchunk + 31) / 32;
-    double own, W_res = 0.0;
-    if (ri.mode == RS_RESIDUAL) {
-        RsSums cs = rs_stage_sums(sh_cs, csum, P.nchunk);
-        if (threadIdx.x < 32) W_res = rs_total(cs, P.nchunk, per_lane, &own);
-        __syncthreads();
-    }
-    RsSums cp = rs_stage_sums(sh_cs, csum_p, P.nchunk);
-    if (threadIdx.x < 32) {
-        const double W_p = rs_total(cp, P.nchunk, per_lane, &own);
-        if (threadIdx.x == 0) {
-            P.weight[2 * static_cast<long long>(b)] = W_res;
-            P.weight[2 * static_cast<long long>(b) + 1] = W_p;
+    if (!sh_flag || warp != 0) return;
+    double tr = 0.0, tp = 0.0;
+    for (int k = lane; k < P.R * kWarps; k += 32)
+        if (dbg_ok(dr + k, 8, DBG_WS_LOAD) && dbg_ok(dp + k, 8, DBG_WS_LOAD)) {
+            tr += __ldcg(dr + k);
+            tp += __ldcg(dp + k);
         }
+    tr = warp_sum(tr);
+    tp = warp_sum(tp);
+    if (lane == 0) {
+        P.weight[2 * static_cast<long long>(b)] = tr;
+        P.weight[2 * static_cast<long long>(b) + 1] = tp;
     }
 }
 
 // Phase 4: one CTA per batch row.  Every rank finds the owning shard from the gathered masses; the
-// owner searches its own chunk sums and writes the token into out_tokens[b, n]; the others leave the
+// owner searches its own spans and writes the token into out_tokens[b, n]; the others leave the
 // -1 that the row epilogue put there, so an element-wise maximum over the ranks completes the row.
-template <typename T, bool ALIGNED>
+template <typename T>
 __global__ void __launch_bounds__(kThreads) shard_pick_kernel(const __grid_constant__ KParams P) {
-    __shared__ float sh_cs[kRsStage];
+    __shared__ DrawSrc sh_src;
+    __shared__ double sh_sum[64];
     __shared__ int sh_go;
     __shared__ int sh_mode;
     __shared__ double sh_tau;
@@ -175,15 +178,22 @@ __global__ void __launch_bounds__(kThreads) shard_pick_kernel(const __grid_const
     if (!sh_go) return;
     const T* trow = static_cast<const T*>(P.t) + static_cast<long long>(b) * P.tsb + static_cast<long long>(ri.n) * P.tsp;
     const T* drow = static_cast<const T*>(P.d) + static_cast<long long>(b) * P.dsb + static_cast<long long>(ri.n) * P.dsp;
-    const RsConst c = rs_const(ri, sh_mode);
-    const float* csum = (sh_mode == RS_RESIDUAL ? P.csum : P.csum2) + static_cast<long long>(b) * P.nchunk;
-    const RsSums cs = rs_stage_sums(sh_cs, csum, P.nchunk);
-    if (warp != 0) return;
-    const int per_lane = (P.nchunk + 31) / 32;
-    double own;
-    (void)rs_total(cs, P.nchunk, per_lane, &own);
-    const int tok = rs_search<T, ALIGNED>(c, trow, drow, cs, P.nchunk, P.V, sh_tau, own, per_lane);
-    if (lane == 0) P.out_tok[static_cast<long long>(b) * (P.G + 1) + ri.n] = tok + P.v_begin;
+    const bool res = sh_mode == RS_RESIDUAL;
+    if (threadIdx.x == 0) {
+        DrawSrc src = make_draw<T>(trow, res ? drow : nullptr, P.V);
+        set_norm(src, ri.scale, ri.lse2_p, ri.lse2_q);
+        sh_src = src;
+    }
+    const double* dsum = (res ? P.dsum : P.dsum2) + static_cast<long long>(b) * (kMaxShares * kWarps);
+    double before = 0.0, total, tau;
+    const int own = pick_many<false, 8>(P.R * kWarps, [&](int k) { return dbg_ok(dsum + k, 8, DBG_WS_LOAD) ? __ldcg(dsum + k) : 0.0; },
+                                     sh_tau, &before, &total, &tau);
+    __syncthreads();
+    if (own < 0) return;
+    const int g0 = own * P.draw_pw, g1 = min(sh_src.t.ng, g0 + P.draw_pw);
+    const int tok = res ? find_token<T, true>(sh_src, g0, g1, tau - before, false, warp, kWarps, 1, sh_sum)
+                        : find_token<T, false>(sh_src, g0, g1, tau - before, false, warp, kWarps, 1, sh_sum);
+    if (lane == 0 && tok >= 0) P.out_tok[static_cast<long long>(b) * (P.G + 1) + ri.n] = tok + P.v_begin;
 }
 
 }  // namespace speckv
