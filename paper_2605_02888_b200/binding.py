@@ -1,4 +1,4 @@
-"""Thin ctypes binding of libspeckv (argument marshalling only).
+"""Thin binding of libspeckv (argument marshalling only; natively in csrc/speckv_torch.cpp where a call is an ordinary one).
 
 Every step of the path runs in the CUDA kernels behind the C ABI of ``include/speckv.h``;
 this module only turns torch tensors into pointers, allocates outputs and scratch through
@@ -112,6 +112,43 @@ def load_library(path: Optional[str] = None) -> C.CDLL:
     if path is None:
         _lib = L
     return L
+
+
+# Addresses of the entry points of the library in use, for the native marshalling: (library, {name: address}).
+_addresses = (None, {})
+_native = None      # the module of csrc/speckv_torch.cpp; False where it is not to be had
+
+
+def _load_native():
+    """The native marshalling module, built if need be.  Where it cannot be had (no compiler, another torch) the same
+    checks run in Python."""
+    global _native
+    import importlib.machinery
+    import importlib.util
+    try:
+        path = _build.build_torch()
+        loader = importlib.machinery.ExtensionFileLoader("_speckv_torch", path)
+        mod = importlib.util.module_from_spec(importlib.util.spec_from_loader("_speckv_torch", loader))
+        loader.exec_module(mod)
+        _native = mod
+    except Exception as e:
+        import warnings
+        warnings.warn(f"native argument marshalling not available, using the slower Python path: {e}")
+        _native = False
+    return _native
+
+
+def _entry(L: C.CDLL):
+    """(native module or False, addresses of the library's functions)"""
+    global _addresses
+    lib, addr = _addresses
+    if lib is not L:
+        addr = {n: C.cast(getattr(L, n), C.c_void_p).value
+                for n in ("speckv_workspace_size", "speckv_signals", "speckv_select_gamma", "speckv_verify", "speckv_step",
+                          "speckv_sample_workspace_size", "speckv_sample_draft", "speckv_shard_sweep", "speckv_shard_finish",
+                          "speckv_shard_draw_sums", "speckv_shard_draw_pick")}
+        _addresses = (L, addr)
+    return (_native if _native is not None else _load_native()), addr
 
 
 def status_string(code: int) -> str:
@@ -296,8 +333,8 @@ class StepOutputs:
                            workspace=_workspace(batch, None))
 
     def as_dict(self):
-        return {k: getattr(self, k) for k in ("H", "C", "feat", "scores", "gamma_next", "n_accepted",
-                                              "out_tokens", "row_status")}
+        return dict(H=self.H, C=self.C, feat=self.feat, scores=self.scores, gamma_next=self.gamma_next,
+                    n_accepted=self.n_accepted, out_tokens=self.out_tokens, row_status=self.row_status)
 
     def pointers(self, batch: "Batch", n_out: int) -> dict:
         """Device pointers of the buffers, each checked against the batch it is about to be used with."""
@@ -323,12 +360,15 @@ class StepOutputs:
 def speckv_signals(batch: Batch, out: Optional[StepOutputs] = None):
     """Draft signals (paper Sec. 4.2): H, C [B, gamma_max]; feat [B, 4]; row_status [B]."""
     L = load_library()
-    c = batch._c()
     o = out or StepOutputs.allocate(batch)
-    q = o.pointers(batch, 0)
-    with torch.cuda.device(batch.draft_logits.device):
-        rc = L.speckv_signals(C.byref(c), q["H"], q["C"], q["feat"], q["row_status"],
-                              q["workspace"], o.workspace.numel(), _stream(batch.draft_logits.device))
+    nat, addr = _entry(L)
+    rc = nat.signals(addr["speckv_signals"], addr["speckv_workspace_size"], batch, o) if nat else None
+    if rc is None:
+        c = batch._c()
+        q = o.pointers(batch, 0)
+        with torch.cuda.device(batch.draft_logits.device):
+            rc = L.speckv_signals(C.byref(c), q["H"], q["C"], q["feat"], q["row_status"],
+                                  q["workspace"], o.workspace.numel(), _stream(batch.draft_logits.device))
     if rc != OK:
         raise SpeckvError(rc, "speckv_signals")
     return dict(H=o.H, C=o.C, feat=o.feat, row_status=o.row_status)
@@ -359,6 +399,14 @@ def speckv_sample_draft(batch: Batch, uniforms: torch.Tensor, tokens: Optional[t
     """Draft tokens (paper Sec. 3.1): tokens[b,i] ~ softmax(draft_logits[b,i] / T_b) by inverse CDF at
     uniforms[b,i] (argmax for T_b = 0); -1 beyond gamma_b.  uniforms: [B, gamma_max] fp32."""
     L = load_library()
+    nat, addr = _entry(L)
+    got = nat.sample(addr["speckv_sample_draft"], addr["speckv_sample_workspace_size"], batch, uniforms, tokens, row_status,
+                     workspace) if nat else None
+    if got is not None:
+        rc, tokens, row_status = got
+        if rc != OK:
+            raise SpeckvError(rc, "speckv_sample_draft")
+        return dict(tokens=tokens, row_status=row_status)
     c = batch._c()
     B, G, V = batch.shape()
     dev = batch.draft_logits.device
@@ -388,12 +436,18 @@ def speckv_select_gamma(feat: torch.Tensor, comp: Optional[torch.Tensor], mlp: M
     """Controller (paper Sec. 4.3, Eq. 1): scores [B, n_out], gamma_next [B]."""
     L = load_library()
     B = feat.shape[0]
-    m = mlp._c()
     dev = feat.device
     if scores is None:
         scores = torch.empty(B, mlp.n_out, dtype=torch.float32, device=dev)
     if gamma_next is None:
         gamma_next = torch.empty(B, dtype=torch.int32, device=dev)
+    nat, addr = _entry(L)
+    rc = nat.select_gamma(addr["speckv_select_gamma"], feat, comp, mlp, scores, gamma_next) if nat else None
+    if rc is not None:
+        if rc != OK:
+            raise SpeckvError(rc, "speckv_select_gamma")
+        return dict(scores=scores, gamma_next=gamma_next)
+    m = mlp._c()
     if not feat.is_cuda:
         raise ValueError("feat must be a CUDA tensor (the library has no CPU path)")
     with torch.cuda.device(dev):
@@ -409,13 +463,16 @@ def speckv_select_gamma(feat: torch.Tensor, comp: Optional[torch.Tensor], mlp: M
 def speckv_verify(batch: Batch, out: Optional[StepOutputs] = None):
     """Verification (paper Sec. 3.1 / speculative sampling): n_accepted, out_tokens, row_status."""
     L = load_library()
-    c = batch._c()
     o = out or StepOutputs.allocate(batch)
-    dev = batch.draft_logits.device
-    q = o.pointers(batch, 0)
-    with torch.cuda.device(dev):
-        rc = L.speckv_verify(C.byref(c), q["n_accepted"], q["out_tokens"], q["row_status"],
-                             q["workspace"], o.workspace.numel(), _stream(dev))
+    nat, addr = _entry(L)
+    rc = nat.verify(addr["speckv_verify"], addr["speckv_workspace_size"], batch, o) if nat else None
+    if rc is None:
+        c = batch._c()
+        dev = batch.draft_logits.device
+        q = o.pointers(batch, 0)
+        with torch.cuda.device(dev):
+            rc = L.speckv_verify(C.byref(c), q["n_accepted"], q["out_tokens"], q["row_status"],
+                                 q["workspace"], o.workspace.numel(), _stream(dev))
     if rc != OK:
         raise SpeckvError(rc, "speckv_verify")
     return dict(n_accepted=o.n_accepted, out_tokens=o.out_tokens, row_status=o.row_status)
@@ -428,9 +485,16 @@ def speckv_step(batch: Batch, comp: Optional[torch.Tensor], mlp: Mlp, out: Optio
     (created with enable_timing=True); they are recorded before and after the sweep kernel and after
     the resample kernel (the last two coincide where the sweep kernel's grid draws the tokens itself)."""
     L = load_library()
+    o = out or StepOutputs.allocate(batch, mlp.n_out)
+    if events is None:
+        nat, addr = _entry(L)
+        rc = nat.step(addr["speckv_step"], addr["speckv_workspace_size"], batch, comp, mlp, o) if nat else None
+        if rc is not None:
+            if rc != OK:
+                raise SpeckvError(rc, "speckv_step")
+            return o.as_dict()
     c = batch._c()
     m = mlp._c()
-    o = out or StepOutputs.allocate(batch, mlp.n_out)
     dev = batch.draft_logits.device
     q = o.pointers(batch, mlp.n_out)
     B = batch.shape()[0]
@@ -473,12 +537,15 @@ def speckv_shard_sweep(local: Batch, v_begin: int, shard_state: torch.Tensor, sh
                        workspace: torch.Tensor):
     """Local slice -> shard_state [B, 2G+1, 4] fp32, shard_tokl [B, G, 2] fp32 (both written)."""
     L = load_library()
-    c = local._c()
-    dev = local.draft_logits.device
-    with torch.cuda.device(dev):
-        rc = L.speckv_shard_sweep(C.byref(c), int(v_begin), _dev_ptr(shard_state, torch.float32, "shard_state"),
-                                  _dev_ptr(shard_tokl, torch.float32, "shard_tokl"), _ptr(workspace),
-                                  workspace.numel(), _stream(dev))
+    nat, addr = _entry(L)
+    rc = nat.shard_sweep(addr["speckv_shard_sweep"], local, v_begin, shard_state, shard_tokl, workspace) if nat else None
+    if rc is None:
+        c = local._c()
+        dev = local.draft_logits.device
+        with torch.cuda.device(dev):
+            rc = L.speckv_shard_sweep(C.byref(c), int(v_begin), _dev_ptr(shard_state, torch.float32, "shard_state"),
+                                      _dev_ptr(shard_tokl, torch.float32, "shard_tokl"), _ptr(workspace),
+                                      workspace.numel(), _stream(dev))
     if rc != OK:
         raise SpeckvError(rc, "speckv_shard_sweep")
 
@@ -488,17 +555,21 @@ def speckv_shard_finish(local: Batch, n_shards: int, shard_width: int, V_total: 
                         row_info: torch.Tensor):
     """Gathered states -> every step output but the sampled rows' fresh token; row_info for the draw."""
     L = load_library()
-    c = local._c()
-    m = mlp._c() if mlp is not None else None
-    dev = local.draft_logits.device
-    with torch.cuda.device(dev):
-        rc = L.speckv_shard_finish(C.byref(c), n_shards, shard_width, V_total,
-                                   _dev_ptr(all_state, torch.float32, "all_state"),
-                                   _dev_ptr(all_tokl, torch.float32, "all_tokl"),
-                                   _dev_ptr(comp, torch.float32, "comp"), C.byref(m) if m is not None else None,
-                                   _ptr(out.H), _ptr(out.C), _ptr(out.feat), _ptr(out.scores), _ptr(out.gamma_next),
-                                   _ptr(out.n_accepted), _ptr(out.out_tokens), _ptr(out.row_status),
-                                   _ptr(row_info), _stream(dev))
+    nat, addr = _entry(L)
+    rc = nat.shard_finish(addr["speckv_shard_finish"], local, n_shards, shard_width, V_total, all_state, all_tokl, comp, mlp,
+                          out, row_info) if nat else None
+    if rc is None:
+        c = local._c()
+        m = mlp._c() if mlp is not None else None
+        dev = local.draft_logits.device
+        with torch.cuda.device(dev):
+            rc = L.speckv_shard_finish(C.byref(c), n_shards, shard_width, V_total,
+                                       _dev_ptr(all_state, torch.float32, "all_state"),
+                                       _dev_ptr(all_tokl, torch.float32, "all_tokl"),
+                                       _dev_ptr(comp, torch.float32, "comp"), C.byref(m) if m is not None else None,
+                                       _ptr(out.H), _ptr(out.C), _ptr(out.feat), _ptr(out.scores), _ptr(out.gamma_next),
+                                       _ptr(out.n_accepted), _ptr(out.out_tokens), _ptr(out.row_status),
+                                       _ptr(row_info), _stream(dev))
     if rc != OK:
         raise SpeckvError(rc, "speckv_shard_finish")
 
@@ -506,11 +577,14 @@ def speckv_shard_finish(local: Batch, n_shards: int, shard_width: int, V_total: 
 def speckv_shard_draw_sums(local: Batch, row_info: torch.Tensor, shard_weight: torch.Tensor, workspace: torch.Tensor):
     """Local slice -> shard_weight [B, 2] fp64 (residual mass, target mass of the stop position)."""
     L = load_library()
-    c = local._c()
-    dev = local.draft_logits.device
-    with torch.cuda.device(dev):
-        rc = L.speckv_shard_draw_sums(C.byref(c), _ptr(row_info), _dev_ptr(shard_weight, torch.float64, "shard_weight"),
-                                      _ptr(workspace), workspace.numel(), _stream(dev))
+    nat, addr = _entry(L)
+    rc = nat.shard_draw_sums(addr["speckv_shard_draw_sums"], local, row_info, shard_weight, workspace) if nat else None
+    if rc is None:
+        c = local._c()
+        dev = local.draft_logits.device
+        with torch.cuda.device(dev):
+            rc = L.speckv_shard_draw_sums(C.byref(c), _ptr(row_info), _dev_ptr(shard_weight, torch.float64, "shard_weight"),
+                                          _ptr(workspace), workspace.numel(), _stream(dev))
     if rc != OK:
         raise SpeckvError(rc, "speckv_shard_draw_sums")
 
@@ -519,12 +593,16 @@ def speckv_shard_draw_pick(local: Batch, v_begin: int, rank: int, n_shards: int,
                            all_weight: torch.Tensor, out_tokens: torch.Tensor, workspace: torch.Tensor):
     """The shard holding the drawn token writes it into out_tokens[b, n_accepted[b]]."""
     L = load_library()
-    c = local._c()
-    dev = local.draft_logits.device
-    with torch.cuda.device(dev):
-        rc = L.speckv_shard_draw_pick(C.byref(c), int(v_begin), rank, n_shards, _ptr(row_info),
-                                      _dev_ptr(all_weight, torch.float64, "all_weight"),
-                                      _dev_ptr(out_tokens, torch.int32, "out_tokens"), _ptr(workspace),
-                                      workspace.numel(), _stream(dev))
+    nat, addr = _entry(L)
+    rc = nat.shard_draw_pick(addr["speckv_shard_draw_pick"], local, v_begin, rank, n_shards, row_info, all_weight,
+                             out_tokens, workspace) if nat else None
+    if rc is None:
+        c = local._c()
+        dev = local.draft_logits.device
+        with torch.cuda.device(dev):
+            rc = L.speckv_shard_draw_pick(C.byref(c), int(v_begin), rank, n_shards, _ptr(row_info),
+                                          _dev_ptr(all_weight, torch.float64, "all_weight"),
+                                          _dev_ptr(out_tokens, torch.int32, "out_tokens"), _ptr(workspace),
+                                          workspace.numel(), _stream(dev))
     if rc != OK:
         raise SpeckvError(rc, "speckv_shard_draw_pick")
