@@ -12,12 +12,23 @@
 
 namespace speckv {
 
+// A row's record, as the two 16-byte words it consists of
+__device__ __forceinline__ RowInfo row_info_load(const RowInfo* p) {
+    const int4 lo = __ldcg(reinterpret_cast<const int4*>(p)), hi = __ldcg(reinterpret_cast<const int4*>(p) + 1);
+    RowInfo ri;
+    ri.mode = lo.x; ri.n = lo.y; ri.u2 = __int_as_float(lo.z); ri.scale = __int_as_float(lo.w);
+    ri.lse2_p = __hiloint2double(hi.y, hi.x);
+    ri.lse2_q = __hiloint2double(hi.w, hi.z);
+    return ri;
+}
+
 struct DrawSrc {
     GranRow t, d;        // target row, draft row (residual only)
     int dg, off;         // granule g of t covers the elements of d from granule g + dg, element off, on
     int in_lo, in_hi;    // granules of t for which all granules involved are whole ones of their rows
-    float scale, lp_hi, lp_lo, lq_hi, lq_lo;  // log2(e) / T; the log2-normalisers as two floats each, so that the
-                                              // exponent keeps the bits that a single float would drop
+    float scale, lp, lq, c;  // log2(e) / T, the log2-normalisers rounded to fp32, and what the rounding took from them:
+                             // p - q = (2^(x_t * scale - lp) - c * 2^(x_d * scale - lq)) * 2^(lp - lse_p), c = 2^((lq - lse_q) - (lp - lse_p));
+                             // the last factor is common to all weights and left out
 };
 
 // The rows of a draw; the constants follow by set_norm, so that loads can go out while those are still on their way.
@@ -36,10 +47,9 @@ __device__ __forceinline__ DrawSrc make_draw(const T* trow, const T* drow, int V
 }
 __device__ __forceinline__ void set_norm(DrawSrc& s, float scale, double lse_p, double lse_q) {
     s.scale = scale;
-    s.lp_hi = static_cast<float>(lse_p);
-    s.lp_lo = static_cast<float>(lse_p - static_cast<double>(s.lp_hi));
-    s.lq_hi = static_cast<float>(lse_q);
-    s.lq_lo = static_cast<float>(lse_q - static_cast<double>(s.lq_hi));
+    s.lp = static_cast<float>(lse_p);
+    s.lq = static_cast<float>(lse_q);
+    s.c = ex2f(static_cast<float>((static_cast<double>(s.lq) - lse_q) - (static_cast<double>(s.lp) - lse_p)));
 }
 
 // ---- weights of one granule ------------------------------------------------------------------------------
@@ -52,33 +62,33 @@ __device__ __forceinline__ void gran_pairs(const uint4& g, f2 (&x)[2]) {
     x[1] = pack2(__uint_as_float(g.z), __uint_as_float(g.w));
 }
 template <typename T, bool RES>
-__device__ __forceinline__ void gran_weights(const DrawSrc& s, const uint4& t, const uint4& d, float (&w)[16 / sizeof(T)]) {
+__device__ __forceinline__ void gran_weights(float scale, float lp, float lq, float c, const uint4& t, const uint4& d,
+                                             float (&w)[16 / sizeof(T)]) {
     constexpr int NP = 8 / sizeof(T);
-    const f2 sc2 = pack2(s.scale, s.scale), ph2 = pack2(-s.lp_hi, -s.lp_hi), pl2 = pack2(s.lp_lo, s.lp_lo);
+    const f2 sc2 = pack2(scale, scale), p2 = pack2(-lp, -lp);
     f2 xt[NP];
     gran_pairs(t, xt);
     if constexpr (!RES) {
 #pragma unroll
-        for (int i = 0; i < NP; ++i) unpack2(ex2_2(sub2(fma2(xt[i], sc2, ph2), pl2)), w[2 * i], w[2 * i + 1]);
+        for (int i = 0; i < NP; ++i) unpack2(ex2_2(fma2(xt[i], sc2, p2)), w[2 * i], w[2 * i + 1]);
     } else {
-        const f2 qh2 = pack2(-s.lq_hi, -s.lq_hi), ql2 = pack2(s.lq_lo, s.lq_lo);
+        const f2 q2 = pack2(-lq, -lq), c2 = pack2(-c, -c);
         f2 xd[NP];
         gran_pairs(d, xd);
 #pragma unroll
         for (int i = 0; i < NP; ++i) {
-            const f2 p = ex2_2(sub2(fma2(xt[i], sc2, ph2), pl2));
-            const f2 q = ex2_2(sub2(fma2(xd[i], sc2, qh2), ql2));
+            const f2 p = ex2_2(fma2(xt[i], sc2, p2)), q = ex2_2(fma2(xd[i], sc2, q2));
             float lo, hi;
-            unpack2(sub2(p, q), lo, hi);
+            unpack2(fma2(q, c2, p), lo, hi);
             w[2 * i] = fmaxf(lo, 0.f);
             w[2 * i + 1] = fmaxf(hi, 0.f);
         }
     }
 }
 template <typename T, bool RES>
-__device__ __forceinline__ float gran_weight(const DrawSrc& s, const uint4& t, const uint4& d) {
+__device__ __forceinline__ float gran_weight(float scale, float lp, float lq, float c, const uint4& t, const uint4& d) {
     float w[16 / sizeof(T)];
-    gran_weights<T, RES>(s, t, d, w);
+    gran_weights<T, RES>(scale, lp, lq, c, t, d, w);
     float a = 0.f;
 #pragma unroll
     for (int j = 0; j < static_cast<int>(16 / sizeof(T)); ++j) a += w[j];
@@ -120,64 +130,92 @@ __device__ __forceinline__ uint4 draft_any(const DrawSrc& s, int g) {  // the dr
     const uint4 a = gran_any<T>(s.d, g + s.dg);
     return s.off ? gran_shift<T>(a, gran_any<T>(s.d, g + s.dg + 1), s.off) : a;
 }
+// The lane's granule g of both rows; those at or behind g1 have no weight.
+template <typename T, bool RES>
+__device__ __forceinline__ void load_weights(const DrawSrc& s, int g, int g1, float (&w)[16 / sizeof(T)]) {
+    uint4 t = gran_fill<T>(__int_as_float(0xff800000)), d = t;
+    if (g < g1) {
+        if (g >= s.in_lo && g < s.in_hi) {
+            t = ldg_stream(s.t.base + g);
+            if (RES) d = ldg_stream(s.d.base + g + s.dg);
+            if (RES && s.off) d = gran_shift<T>(d, ldg_stream(s.d.base + g + s.dg + 1), s.off);
+        } else {
+            t = gran_any<T>(s.t, g);
+            if (RES) d = draft_any<T>(s, g);
+        }
+    }
+    gran_weights<T, RES>(s.scale, s.lp, s.lq, s.c, t, d, w);
+}
 template <typename T, bool RES>
 __device__ __noinline__ double gran_weight_any(const DrawSrc s, int g) {
-    const uint4 t = gran_any<T>(s.t, g);
-    return static_cast<double>(gran_weight<T, RES>(s, t, RES ? draft_any<T>(s, g) : t));
+    float w[16 / sizeof(T)];
+    load_weights<T, RES>(s, g, 0x7fffffff, w);
+    double a = 0.0;
+#pragma unroll
+    for (int j = 0; j < static_cast<int>(16 / sizeof(T)); ++j) a += static_cast<double>(w[j]);
+    return a;
 }
 
 // ---- sums ----------------------------------------------------------------------------------------------------
-// Weight of granules [g0, g1), one warp, the same in every lane.  norm(s) sets the constants and is called once the
-// first loads are out.  Two loads per row are in flight and none is requested ahead: the other warps of the SM, not this one,
-// hide the latency, and what fits 48 registers does not spill (1,024 bf16 rows, V = 128,256: step 430 us; two requested ahead
-// 439, four in flight 435, one in flight and one ahead 436).
-template <typename T, bool RES, bool SHIFTED, class F>
-__device__ __forceinline__ double warp_weight_body(DrawSrc& s, int g0, int g1, F norm) {
+// Sum over whole granules pt[0], pt[32], ... (n left from this lane's first one on) of the weights that the row record says.
+// Two loads per row are in flight and none is requested ahead: the other warps of the SM, not this one, hide the latency, and
+// the loop, compiled by itself, keeps to the 48 registers of the sweep kernel without spilling (step of 1,024 bf16 rows,
+// V = 128,256, 430 us; two requested ahead 9 us more, four in flight 5 us more).  The record is fetched behind the first loads.
+template <typename T, bool RES, bool SHIFTED>
+__device__ __noinline__ double span_weight(const uint4* pt, const uint4* pd, int n, int off, const RowInfo* info) {
     constexpr int KU = SHIFTED ? 1 : 2;
-    const int lane = threadIdx.x & 31;
-    const int a = min(max(g0, s.in_lo), g1), e = max(min(g1, s.in_hi), a);
-    double acc = 0.0;
-    const uint4* pt = s.t.base + lane;
-    const uint4* pd = s.d.base + s.dg + lane;
     uint4 t[KU], d[KU], d1[KU];
-    auto load = [&](int g) {
+    auto load = [&]() {
 #pragma unroll
         for (int u = 0; u < KU; ++u) {
-            const int k = g + 32 * u;
             t[u] = gran_fill<T>(__int_as_float(0xff800000));
             if (RES) d[u] = t[u];
             if (RES && SHIFTED) d1[u] = t[u];
-            if (k + lane < e) {
-                t[u] = ldg_stream(pt + k);
-                if (RES) d[u] = ldg_stream(pd + k);
-                if (RES && SHIFTED) d1[u] = ldg_stream(pd + k + 1);
+            if (32 * u < n) {
+                t[u] = ldg_stream(pt + 32 * u);
+                if (RES) d[u] = ldg_stream(pd + 32 * u);
+                if (RES && SHIFTED) d1[u] = ldg_stream(pd + 32 * u + 1);
             }
         }
+        pt += 32 * KU;
+        pd += 32 * KU;
+        n -= 32 * KU;
     };
-    if (a < e) load(a);
-    norm(s);
-    // incomplete granules in front of and behind [a, e): a handful at most, one per lane
-    const int nl = a - g0, nr = g1 - e;
-    for (int k = lane; k < nl + nr; k += 32) acc += gran_weight_any<T, RES>(s, k < nl ? g0 + k : e + (k - nl));
-    for (int g = a; g < e;) {
+    load();
+    const int4 lo = __ldcg(reinterpret_cast<const int4*>(info)), hi = __ldcg(reinterpret_cast<const int4*>(info) + 1);
+    DrawSrc s;
+    set_norm(s, __int_as_float(lo.w), __hiloint2double(hi.y, hi.x), __hiloint2double(hi.w, hi.z));
+    double acc = 0.0;
+    for (;;) {
         float w = 0.f;
 #pragma unroll
-        for (int u = 0; u < KU; ++u) w += gran_weight<T, RES>(s, t[u], RES ? (SHIFTED ? gran_shift<T>(d[u], d1[u], s.off) : d[u]) : t[u]);
+        for (int u = 0; u < KU; ++u)
+            w += gran_weight<T, RES>(s.scale, s.lp, s.lq, s.c, t[u], RES ? (SHIFTED ? gran_shift<T>(d[u], d1[u], off) : d[u]) : t[u]);
         acc += static_cast<double>(w);
-        g += 32 * KU;
-        if (g < e) load(g);
+        if (n <= 0) return acc;
+        load();
+    }
+}
+// Weight of granules [g0, g1), one warp, the same in every lane.  Only the rows of s are needed; info: the row's record.
+template <typename T, bool RES>
+__device__ __forceinline__ double warp_weight(const DrawSrc& s, int g0, int g1, const RowInfo* info) {
+    const int lane = threadIdx.x & 31;
+    const int a = min(max(g0, s.in_lo), g1), e = max(min(g1, s.in_hi), a);
+    double acc = 0.0;
+    if (e - a - lane > 0) {
+        const uint4 *pt = s.t.base + a + lane, *pd = s.d.base + s.dg + a + lane;
+        acc = (RES && s.off) ? span_weight<T, RES, RES>(pt, pd, e - a - lane, s.off, info) : span_weight<T, RES, false>(pt, pd, e - a - lane, 0, info);
+    }
+    __syncwarp();
+    // incomplete granules in front of and behind [a, e): a handful at most, one per lane
+    const int nl = a - g0, nr = g1 - e;
+    if (nl + nr > 0) {
+        const RowInfo ri = row_info_load(info);
+        DrawSrc c = s;
+        set_norm(c, ri.scale, ri.lse2_p, ri.lse2_q);
+        for (int k = lane; k < nl + nr; k += 32) acc += gran_weight_any<T, RES>(c, k < nl ? g0 + k : e + (k - nl));
     }
     return warp_sum(acc);
-}
-template <typename T, bool RES, class F>
-__device__ __forceinline__ double warp_weight(DrawSrc& s, int g0, int g1, F norm) {
-    if (RES && s.off) return warp_weight_body<T, RES, RES>(s, g0, g1, norm);
-    return warp_weight_body<T, RES, false>(s, g0, g1, norm);
-}
-template <typename T, bool RES>
-__device__ __noinline__ double warp_weight_of(const DrawSrc& s, int g0, int g1) {
-    DrawSrc c = s;
-    return warp_weight<T, RES>(c, g0, g1, [](DrawSrc&) {});
 }
 
 // ---- picking -------------------------------------------------------------------------------------------------
@@ -226,22 +264,6 @@ __device__ __forceinline__ int pick_many(int n, F get, double u, double* before,
     return own * per + max(sub, 0);
 }
 
-// The lane's granule g of both rows; those at or behind g1 have no weight.
-template <typename T, bool RES>
-__device__ __forceinline__ void load_weights(const DrawSrc& s, int g, int g1, float (&w)[16 / sizeof(T)]) {
-    uint4 t = gran_fill<T>(__int_as_float(0xff800000)), d = t;
-    if (g < g1) {
-        if (g >= s.in_lo && g < s.in_hi) {
-            t = ldg_stream(s.t.base + g);
-            if (RES) d = ldg_stream(s.d.base + g + s.dg);
-            if (RES && s.off) d = gran_shift<T>(d, ldg_stream(s.d.base + g + s.dg + 1), s.off);
-        } else {
-            t = gran_any<T>(s.t, g);
-            if (RES) d = draft_any<T>(s, g);
-        }
-    }
-    gran_weights<T, RES>(s, t, d, w);
-}
 // One warp: the token among 32 consecutive granules whose weights its lanes hold (lane 0 granule g0).
 template <typename T>
 __device__ __forceinline__ int scan_weights(const DrawSrc& s, int g0, const float (&w)[16 / sizeof(T)], double tau) {
@@ -302,13 +324,19 @@ __device__ __noinline__ int find_token(const DrawSrc& s, int g0, int g1, double 
                 }
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
-                    const double a = warp_sum(static_cast<double>(gran_weight<T, false>(s, t[u], t[u])));
+                    const double a = warp_sum(static_cast<double>(gran_weight<T, false>(s.scale, s.lp, 0.f, 0.f, t[u], t[u])));
                     if (lane == 0 && k + u * nw < cnt) sh[k + u * nw] = a;
                 }
             }
         } else {
             for (int k = wi; k < cnt; k += nw) {
-                const double a = warp_weight_of<T, RES>(s, g0 + k * sub, min(g1, g0 + (k + 1) * sub));
+                double a = 0.0;
+                for (int g = g0 + k * sub; g < min(g1, g0 + (k + 1) * sub); g += 32) {
+                    load_weights<T, RES>(s, g + lane, min(g1, g0 + (k + 1) * sub), w);
+#pragma unroll
+                    for (int j = 0; j < E; ++j) a += static_cast<double>(w[j]);
+                }
+                a = warp_sum(a);
                 if (lane == 0) sh[k] = a;
             }
         }
@@ -364,15 +392,6 @@ __device__ __forceinline__ int draw_from_spans(const T* row, int V, float scale,
     return find_token<T, false>(*sh_src, g0, min(sh_src->t.ng, g0 + per_warp), tau - before, false, wi, nw, bar, sh);
 }
 
-// RowInfo as the two 16-byte words it is loaded as
-__device__ __forceinline__ RowInfo row_info_from(const int4& lo4, const int4& hi4) {
-    RowInfo ri;
-    ri.mode = lo4.x; ri.n = lo4.y; ri.u2 = __int_as_float(lo4.z); ri.scale = __int_as_float(lo4.w);
-    ri.lse2_p = __hiloint2double(hi4.y, hi4.x);
-    ri.lse2_q = __hiloint2double(hi4.w, hi4.z);
-    return ri;
-}
-
 // ----------------------------------------------------------------------------------------
 // One CTA's share of the fresh-token draw of batch row b at stop position n: share `share` of Rr, dw granules per warp.
 // The last of the row's CTAs to arrive locates the token.  A residual whose total mass is below 1e-6 cannot be told from
@@ -386,20 +405,14 @@ __device__ __forceinline__ void resample_row(const KParams& P, const int b, cons
     __shared__ double sh_sum[64];
     if (mode == RS_NONE) return;  // greedy or flagged row, or a token that the sweep's own CTA draws
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int4* ip = reinterpret_cast<const int4*>(P.info + b);
-    const int4 lo4 = __ldcg(ip), hi4 = __ldcg(ip + 1);  // on their way while the first logits are requested
     const T* trow = static_cast<const T*>(P.t) + static_cast<long long>(b) * P.tsb + static_cast<long long>(n) * P.tsp;
     const T* drow = static_cast<const T*>(P.d) + static_cast<long long>(b) * P.dsb + static_cast<long long>(n) * P.dsp;
-    DrawSrc src = make_draw<T>(trow, mode == RS_RESIDUAL ? drow : nullptr, P.V);
-    auto norm = [&](DrawSrc& s) {
-        const RowInfo ri = row_info_from(lo4, hi4);
-        set_norm(s, ri.scale, ri.lse2_p, ri.lse2_q);
-    };
+    const DrawSrc src = make_draw<T>(trow, mode == RS_RESIDUAL ? drow : nullptr, P.V);
     double* dsum = P.dsum + static_cast<long long>(b) * (kMaxShares * kWarps);
     const int span = share * kWarps + warp;
     {
         const int g0 = span * dw, g1 = min(src.t.ng, g0 + dw);
-        const double w = mode == RS_RESIDUAL ? warp_weight<T, true>(src, g0, g1, norm) : warp_weight<T, false>(src, g0, g1, norm);
+        const double w = mode == RS_RESIDUAL ? warp_weight<T, true>(src, g0, g1, P.info + b) : warp_weight<T, false>(src, g0, g1, P.info + b);
         if (lane == 0) SPECKV_ST(dsum[span], w);
     }
     __syncthreads();
@@ -408,25 +421,32 @@ __device__ __forceinline__ void resample_row(const KParams& P, const int b, cons
         const bool last = atomicAdd(P.tick2 + b, 1) == Rr - 1;
         if (last) __threadfence();
         sh_flag = last;
-        sh_src = src;
     }
     __syncthreads();
     if (!sh_flag) return;
 
     // ---- last CTA of the row: locate the threshold (every warp picks the span, redundantly) ----
-    const float u2 = __int_as_float(lo4.z);
+    const RowInfo ri = row_info_load(P.info + b);
+    if (threadIdx.x == 0) {
+        DrawSrc c = make_draw<T>(trow, mode == RS_RESIDUAL ? drow : nullptr, P.V);
+        set_norm(c, ri.scale, ri.lse2_p, ri.lse2_q);
+        sh_src = c;
+    }
+    const float u2 = ri.u2;
     double before = 0.0, total, tau;
     const int own = pick_many<true, 8>(Rr * kWarps, [&](int k) { return dbg_ok(dsum + k, 8, DBG_WS_LOAD) ? __ldcg(dsum + k) : 0.0; },
                                        static_cast<double>(u2), &before, &total, &tau);
+    __syncthreads();
+    const int ng = sh_src.t.ng;
     int tok;
-    if (mode == RS_RESIDUAL && !(total > 1e-6))
-        tok = find_token<T, false>(sh_src, 0, src.t.ng, static_cast<double>(u2), true, warp, kWarps, 1, sh_sum);
+    if (mode == RS_RESIDUAL && total > 1e-6)
+        tok = find_token<T, true>(sh_src, own * dw, min(ng, (own + 1) * dw), tau - before, false, warp, kWarps, 1, sh_sum);
+    else if (mode == RS_RESIDUAL)
+        tok = find_token<T, false>(sh_src, 0, ng, static_cast<double>(u2), true, warp, kWarps, 1, sh_sum);
     else if (own < 0)
         tok = warp == 0 ? 0 : kNotMine;  // p itself has no mass: cannot happen for a finite row
-    else if (mode == RS_RESIDUAL)
-        tok = find_token<T, true>(sh_src, own * dw, min(src.t.ng, (own + 1) * dw), tau - before, false, warp, kWarps, 1, sh_sum);
     else
-        tok = find_token<T, false>(sh_src, own * dw, min(src.t.ng, (own + 1) * dw), tau - before, false, warp, kWarps, 1, sh_sum);
+        tok = find_token<T, false>(sh_src, own * dw, min(ng, (own + 1) * dw), tau - before, false, warp, kWarps, 1, sh_sum);
     if (tok != kNotMine && lane == 0) P.out_tok[static_cast<long long>(b) * (P.G + 1) + n] = max(tok, 0);
 }
 

@@ -28,9 +28,9 @@ constexpr int kVec = 8;                 // elements per lane per step
 constexpr int kMaxShares = 32;          // CTAs that share one draw at most
 constexpr int kMaxSplit = 32;
 constexpr int kMaxGamma = 16;           // SPECKV_MAX_GAMMA
-// Measured on b256 (same box, the two builds in turn, five times): 5 CTAs x 3 loads 156.7 us, 4 x 4 161.6 us,
-// 5 x 4 163.6 us, 6 x 3 161.9 us; b256_g8 and b1024_loop the same within 0.1 %.
-constexpr int kSweepLoads = 3;  // 16-byte loads in flight per thread (bf16); fp32 uses half as many vector steps
+// Step of 256 / 1,024 bf16 rows, V = 128,256, and draft sampling of 256: 5 CTAs x 4 loads 141 / 418 / 81 us, 5 x 3 144 / 430 / 83,
+// 4 x 4 142 / 437 / 87, 6 x 3 146 / 430 / 88 (the GPU's time, one box).
+constexpr int kSweepLoads = 4;  // 16-byte loads in flight per thread (bf16); fp32 uses half as many vector steps
 constexpr int kSweepCtasPerSm = 5;  // CTAs per SM the sweep kernel is compiled for (48 registers per thread)
 constexpr float kFloor = -1.2676506002282294e30f;  // -2^100: logits below count as -inf
 constexpr uint32_t kFloorBf16x2 = 0xF180F180u;     // -2^100 as two bf16
@@ -307,16 +307,18 @@ __device__ __forceinline__ void raw_floor(Raw<float>& r) {
 //         elements of 2^((x-m)*scale), d = S = sum of 2^((x-m)*scale) * (x-m).
 //         Z = cnt + Zx; entropy (nats) = ln Z - ln2*scale*S/Z; confidence = 1/Z  (Sec. 4.2).
 //         cnt = NaN marks a NaN / +inf input.
-// TARGET  a = r (reference, log2 units = m*scale), b = Z = sum 2^(x*scale - r); c,d unused.
-//         NaN / +inf inputs surface as a non-finite Z.
+//         While it sweeps, a thread keeps its sums against r = fl(m * scale), so that an element's exponent is one
+//         fused multiply-add; partial() moves them to m itself.
+// TARGET  a = r (reference, log2 units), b = Z = sum 2^(x*scale - r); c,d unused.  Any r serves that keeps the sum in
+//         range; it is not the maximum.  NaN / +inf inputs surface as a non-finite Z.
 // ARGMAX  a = best value, b = index (bit pattern), c = bad flag (non-zero: NaN / +inf seen).
 // ----------------------------------------------------------------------------------------
 struct DraftState {
-    float m, cnt;
-    f2 za, zb, sa, sb;  // four running sums each of Zx and S, as two packed pairs
+    float m, r, cnt;
+    f2 za, zb, sa, sb;  // four running sums each of Zx and of 2^y * y, y = x * scale - r, as two packed pairs
     bool bad;
-    __device__ __forceinline__ void init(float m0) {
-        m = m0; cnt = 0.f; bad = false;
+    __device__ __forceinline__ void init(float m0, float scale) {
+        m = m0; r = __fmul_rn(m0, scale); cnt = 0.f; bad = false;
         za = zb = sa = sb = pack2(0.f, 0.f);
     }
     __device__ __forceinline__ float zsum() const { return hsum2(za) + hsum2(zb); }
@@ -335,23 +337,22 @@ struct DraftState {
         }
         float z = zsum(), sv = ssum();
         if (vmax > m) {  // everything gathered so far moves below the new maximum
-            float dm = m - vmax;
-            float f = ex2f(dm * scale);
-            float zall = cnt + z;
-            z = zall * f;
-            sv = fmaf(dm, zall, sv) * f;
+            const float rn = __fmul_rn(vmax, scale), dr = __fsub_rn(r, rn), f = ex2f(dr);
+            const float y = fmaf(m, scale, -r), zc = cnt * ex2f(y);  // the elements equal to the old maximum join the sums
+            sv = fmaf(dr, zc + z, fmaf(zc, y, sv)) * f;
+            z = (zc + z) * f;
             cnt = 0.f;
             m = vmax;
+            r = rn;
         }
 #pragma unroll
         for (int j = 0; j < kVec; ++j) {
             if (x[j] == m) {
                 cnt += 1.f;
             } else {
-                float dx = x[j] - m;
-                float e = ex2f(dx * scale);
+                const float y = fmaf(x[j], scale, -r), e = ex2f(y);
                 z += e;
-                sv = fmaf(e, dx, sv);
+                sv = fmaf(e, y, sv);
             }
         }
         za = pack2(z, 0.f); zb = pack2(0.f, 0.f);
@@ -367,17 +368,17 @@ struct DraftState {
         raw_floor(raw);
         f2 x[4];
         unpack_pairs(raw, x);
-        const f2 m2 = pack2(m, m), sc2 = pack2(scale, scale);
-        const f2 d0 = sub2(x[0], m2), d1 = sub2(x[1], m2), d2 = sub2(x[2], m2), d3 = sub2(x[3], m2);
-        const f2 e0 = ex2_2(mul2(d0, sc2)), e1 = ex2_2(mul2(d1, sc2));
-        const f2 e2 = ex2_2(mul2(d2, sc2)), e3 = ex2_2(mul2(d3, sc2));
+        const f2 sc2 = pack2(scale, scale), nr2 = pack2(-r, -r);
+        const f2 y0 = fma2(x[0], sc2, nr2), y1 = fma2(x[1], sc2, nr2), y2 = fma2(x[2], sc2, nr2), y3 = fma2(x[3], sc2, nr2);
+        const f2 e0 = ex2_2(y0), e1 = ex2_2(y1), e2 = ex2_2(y2), e3 = ex2_2(y3);
         za = add2(za, e0); zb = add2(zb, e1);
-        sa = fma2(e0, d0, sa); sb = fma2(e1, d1, sb);
+        sa = fma2(e0, y0, sa); sb = fma2(e1, y1, sb);
         za = add2(za, e2); zb = add2(zb, e3);
-        sa = fma2(e2, d2, sa); sb = fma2(e3, d3, sb);
+        sa = fma2(e2, y2, sa); sb = fma2(e3, y3, sb);
     }
-    __device__ __forceinline__ float4 partial() const {
-        return make_float4(m, bad ? __int_as_float(0x7fc00000) : cnt, zsum(), ssum());
+    __device__ __forceinline__ float4 partial(float scale) const {
+        const float d = fmaf(m, scale, -r), f = ex2f(-d), z = zsum();  // y against m itself is smaller by d, a rounding
+        return make_float4(m, bad ? __int_as_float(0x7fc00000) : cnt, z * f, fmaf(-d, z, ssum()) * f / scale);
     }
 };
 
@@ -397,36 +398,36 @@ __device__ __forceinline__ float4 merge_draft(float4 a, float4 b, float scale) {
     return r;
 }
 
+constexpr float kBigSum = 1.1529215e18f;  // 2^60
+
+// The sums of a group of steps are gathered apart and looked at once: an element far above the reference shows as a sum
+// beyond 2^60 (or an overflow, or a NaN), and only then is the group read again and the reference raised.  No element
+// is compared with anything: 24 instructions per 8 bf16 elements instead of 30 (with the draft's exponent in one
+// fused multiply-add and four loads in flight: draft sampling of 256 rows, V = 128,256, 83 -> 81 us, step 142.5 -> 141).
 struct TargetState {
-    float m, r;
-    f2 za, zb;
-    __device__ __forceinline__ void init(float m0, float scale) {
-        m = m0; r = m0 * scale;
-        za = zb = pack2(0.f, 0.f);
-    }
+    float r, z;
+    __device__ __forceinline__ void init(float m0, float scale) { r = __fmul_rn(m0, scale); z = 0.f; }
     template <typename T>
-    __device__ __forceinline__ void step(const Raw<T>& raw, float scale) {
-        if (raw_exceeds<true>(raw, m)) {  // a new maximum (or NaN): move the reference
-            float vmax = raw_max(raw);
-            if (vmax == vmax) {  // NaN needs no rescale; it poisons Z below
-                float rn = vmax * scale;
-                float f = ex2f(r - rn);
-                za = pack2((hsum2(za) + hsum2(zb)) * f, 0.f);
-                zb = pack2(0.f, 0.f);
-                r = rn; m = vmax;
-            }
-        }
+    __device__ __forceinline__ void add(const Raw<T>& raw, float scale, f2& ga, f2& gb) const {
         f2 x[4];
         unpack_pairs(raw, x);
         const f2 sc2 = pack2(scale, scale), nr2 = pack2(-r, -r);
         const f2 e0 = ex2_2(fma2(x[0], sc2, nr2)), e1 = ex2_2(fma2(x[1], sc2, nr2));
         const f2 e2 = ex2_2(fma2(x[2], sc2, nr2)), e3 = ex2_2(fma2(x[3], sc2, nr2));
-        za = add2(za, e0); zb = add2(zb, e1);
-        za = add2(za, e2); zb = add2(zb, e3);
+        ga = add2(ga, e0); gb = add2(gb, e1);
+        ga = add2(ga, e2); gb = add2(gb, e3);
     }
-    __device__ __forceinline__ float4 partial() const {
-        return make_float4(r, hsum2(za) + hsum2(zb), 0.f, 0.f);
+    // one step with its maximum taken first
+    template <typename T>
+    __device__ __forceinline__ void careful(const Raw<T>& raw, float scale) {
+        const float v = raw_max(raw), rn = __fmul_rn(v, scale);
+        if (!(v < __int_as_float(0x7f800000))) { z = __int_as_float(0x7fc00000); return; }
+        if (rn > r) { z *= ex2f(__fsub_rn(r, rn)); r = rn; }
+        f2 ga = pack2(0.f, 0.f), gb = ga;
+        add(raw, scale, ga, gb);
+        z += hsum2(add2(ga, gb));
     }
+    __device__ __forceinline__ float4 partial() const { return make_float4(r, z, 0.f, 0.f); }
 };
 
 __device__ __forceinline__ float4 merge_target(float4 a, float4 b) {
@@ -635,33 +636,62 @@ __device__ __forceinline__ float4 sweep_warp(const GranRow& row, int lo, int hi,
     }
 
     DraftState ds; TargetState ts; ArgmaxState as;
-    if constexpr (PATH == PATH_DRAFT) ds.init(m0);
+    if constexpr (PATH == PATH_DRAFT) ds.init(m0, scale);
     else if constexpr (PATH == PATH_TARGET) ts.init(m0, scale);
     else as.init(m0);
 
-    auto process = [&](const Raw<T>& v, int g) {  // g: granule of the first half
-        if constexpr (PATH == PATH_DRAFT) ds.template step<T>(v, scale);
-        else if constexpr (PATH == PATH_TARGET) ts.template step<T>(v, scale);
-        else as.template step<T>(v, g * E - row.shift(), GS == 2 ? (g + 32) * E - row.shift() : g * E - row.shift() + kVec / 2);
-    };
-    if (first_edge || last_edge) process(edge, lane == 0 ? 0 : row.ng - 1);
-
-    int i = 0;
-    for (; i + U <= n_main; i += U) {
+    if constexpr (PATH == PATH_TARGET) {
+        if (first_edge || last_edge) ts.template careful<T>(edge, scale);
+        // steps i .. i+n-1 went into ga, gb
+        auto close = [&](f2 ga, f2 gb, int i, int n) {
+            const float g = hsum2(add2(ga, gb));
+            if (g < kBigSum) {
+                ts.z += g;
+            } else {
+#pragma unroll 1
+                for (int k = i; k < i + n; ++k) ts.template careful<T>(load(k), scale);
+            }
+        };
+        int i = 0;
+        for (; i + U <= n_main; i += U) {
+            f2 ga = pack2(0.f, 0.f), gb = ga;
 #pragma unroll
-        for (int k = 0; k < U; ++k) {
-            const Raw<T> cur = buf[k];
-            const int nx = i + U + k;
-            if (nx < n_main) buf[k] = load(nx);
-            process(cur, a + lane + 32 * GS * (i + k));
+            for (int k = 0; k < U; ++k) {
+                const Raw<T> cur = buf[k];
+                const int nx = i + U + k;
+                if (nx < n_main) buf[k] = load(nx);
+                ts.template add<T>(cur, scale, ga, gb);
+            }
+            close(ga, gb, i, U);
         }
-    }
+        f2 ga = pack2(0.f, 0.f), gb = ga;
 #pragma unroll
-    for (int k = 0; k < U; ++k)
-        if (i + k < n_main) process(buf[k], a + lane + 32 * GS * (i + k));
+        for (int k = 0; k < U; ++k)
+            if (i + k < n_main) ts.template add<T>(buf[k], scale, ga, gb);
+        close(ga, gb, i, n_main - i);
+    } else {
+        auto process = [&](const Raw<T>& v, int g) {  // g: granule of the first half
+            if constexpr (PATH == PATH_DRAFT) ds.template step<T>(v, scale);
+            else as.template step<T>(v, g * E - row.shift(), GS == 2 ? (g + 32) * E - row.shift() : g * E - row.shift() + kVec / 2);
+        };
+        if (first_edge || last_edge) process(edge, lane == 0 ? 0 : row.ng - 1);
+        int i = 0;
+        for (; i + U <= n_main; i += U) {
+#pragma unroll
+            for (int k = 0; k < U; ++k) {
+                const Raw<T> cur = buf[k];
+                const int nx = i + U + k;
+                if (nx < n_main) buf[k] = load(nx);
+                process(cur, a + lane + 32 * GS * (i + k));
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < U; ++k)
+            if (i + k < n_main) process(buf[k], a + lane + 32 * GS * (i + k));
+    }
 
     float4 part;
-    if constexpr (PATH == PATH_DRAFT) part = ds.partial();
+    if constexpr (PATH == PATH_DRAFT) part = ds.partial(scale);
     else if constexpr (PATH == PATH_TARGET) part = ts.partial();
     else part = as.partial();
     return warp_merge<PATH>(part, scale);
@@ -1066,7 +1096,7 @@ __device__ __noinline__ void decide_position(const KParams& P, int b, int gam, f
 // publishes where the walk stops if it stops there, so that CTAs which have not started yet can leave
 // target rows behind that position unread.  early[b] = stop position + 1, or G + 2 when the walk passes k.
 template <typename T>
-__device__ __forceinline__ void prefix_epilogue(const KParams& P, int b, int gam, float Tf, RowDecide* pos) {
+__device__ __noinline__ void prefix_epilogue(const KParams& P, int b, int gam, float Tf, RowDecide* pos) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long row0 = static_cast<long long>(b) * P.J;
     if (warp <= P.k_early && warp <= gam)

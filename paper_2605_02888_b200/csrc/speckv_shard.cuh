@@ -90,14 +90,12 @@ __global__ void __launch_bounds__(kThreads, 4) shard_sums_kernel(const __grid_co
     const bool res = ri.mode == RS_RESIDUAL;
     const T* trow = static_cast<const T*>(P.t) + static_cast<long long>(b) * P.tsb + static_cast<long long>(ri.n) * P.tsp;
     const T* drow = static_cast<const T*>(P.d) + static_cast<long long>(b) * P.dsb + static_cast<long long>(ri.n) * P.dsp;
-    DrawSrc src = make_draw<T>(trow, res ? drow : nullptr, P.V);
-    set_norm(src, ri.scale, ri.lse2_p, ri.lse2_q);
-    auto norm = [](DrawSrc&) {};
+    const DrawSrc src = make_draw<T>(trow, res ? drow : nullptr, P.V);
     double* dr = P.dsum + static_cast<long long>(b) * (kMaxShares * kWarps);
     double* dp = P.dsum2 + static_cast<long long>(b) * (kMaxShares * kWarps);
     const int span = share * kWarps + warp, g0 = span * P.draw_pw, g1 = min(src.t.ng, g0 + P.draw_pw);
-    const double wr = res ? warp_weight<T, true>(src, g0, g1, norm) : 0.0;
-    const double wp = warp_weight<T, false>(src, g0, g1, norm);
+    const double wr = res ? warp_weight<T, true>(src, g0, g1, P.info + b) : 0.0;
+    const double wp = warp_weight<T, false>(src, g0, g1, P.info + b);
     if (lane == 0) {
         SPECKV_ST(dr[span], wr);
         SPECKV_ST(dp[span], wp);

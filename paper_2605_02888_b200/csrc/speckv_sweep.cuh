@@ -8,7 +8,7 @@ namespace speckv {
 
 // Row epilogue of the sliced sweep: a whole CTA, a warp per position.
 template <typename T>
-__device__ __forceinline__ void row_epilogue_cta(const KParams& P, int b, int gam, float Tf, RowDecide* pos, double* sh_sum,
+__device__ __noinline__ void row_epilogue_cta(const KParams& P, int b, int gam, float Tf, RowDecide* pos, double* sh_sum,
                                                  DrawSrc* sh_src) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool verify = (P.mode & MODE_VERIFY) != 0;

@@ -50,3 +50,20 @@ def test_edge_elements_count(dtype, where):
     out = _check(s, w)
     st = out["row_status"].cpu().numpy()
     assert np.array_equal(st, np.array([4, 0, 0, 4, 0, 0]))
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("jump", [30.0, 50.0, 300.0, 3.0e4])
+def test_target_elements_far_above_the_reference(dtype, jump):
+    # the sweep's reference is a maximum over its first loads; an element far above it, in one lane's later granules, makes
+    # that lane's group sum large (30: below 2^60), beyond 2^60 (50) or infinite (300), and the group is read again
+    w = synth.Workload("g", B=12, gamma_max=3, V=70001, dtype=dtype, gamma_mode="ragged", temperature=1.0, sigma_d=(0.5,), seed=5)
+    s = synth.make_step(w, 0, DEV)
+    for b in range(w.B):
+        s["target"][b, :, 20000 + 4001 * b] = jump
+        if b % 2:  # climbing: every group of the lane's raises the reference again
+            s["target"][b, :, 30000:30000 + 60 * 512:512] += torch.arange(60, device=DEV).to(s["target"].dtype) * (jump / 60)
+        if b % 3 == 0:
+            s["draft"][b] = s["target"][b, :3]
+            s["draft_tokens"][b] = 20000 + 4001 * b
+    _check(s, w)
