@@ -67,6 +67,8 @@ cudaError_t dbg_register(cudaStream_t cs, const speckv_batch* bt, bool target, c
 #endif
 }
 
+constexpr int kSlots = 740;  // CTA slots of the chip: 5 on each of 148 SMs
+
 // Vocabulary slices per logit row for a sweep over J logit rows per batch row, one CTA each, and the granules that one
 // warp takes of a slice: P.nsplit, P.per_warp.  aligned: every row starts on the 16-byte grid.
 void choose_slices(KParams& P, speckv_dtype dt, bool aligned) {
@@ -77,7 +79,6 @@ void choose_slices(KParams& P, speckv_dtype dt, bool aligned) {
     // Small batches: enough CTAs to fill the slots of the chip once (5 on each of 148 SMs).  Aiming at more starts a second
     // round of short CTAs: with 1,184 instead of 740, step of 64 bf16 rows, V = 32,000, 37.7 us instead of 33.1, of 37 rows,
     // V = 50,257, 32.6 instead of 31.1; one row the same.
-    constexpr int kSlots = 740;
     const long long rows = static_cast<long long>(P.B) * P.J;
     const long long want = (kSlots + rows - 1) / (rows > 0 ? rows : 1);
     if (want > ns) ns = static_cast<int>(want > kMaxSplit ? kMaxSplit : want);
@@ -352,8 +353,13 @@ constexpr int kPipeMinB = 384;
         // positions, and a later position's test would come too late for the CTAs behind it anyway)
         P.k_early = P.G >= 2 ? kEarlyPositions - 1 : 0;
         P.read_all = (bt->flags & SPECKV_READ_ALL_TARGET_ROWS) ? 1 : 0;
-        P.tick_early = P.rowq + 2 * P.B;
-        P.early = P.rowq + 3 * P.B;
+        // ... where the grid has that many CTAs: the third generation has to start after the first one's tests, that is
+        // one and a half rounds of CTA slots behind it (one row, V = 32,000: taking the tests for nothing cost 4 us of 20)
+        const long long ahead = static_cast<long long>(P.B) * P.nsplit * (2 * (P.k_early + 1) + P.G - P.k_early - 1);
+        if (2 * ahead >= 3 * kSlots) {
+            P.tick_early = P.rowq + 2 * P.B;
+            P.early = P.rowq + 3 * P.B;
+        }
     }
     P.rs_reverse = staged ? 1 : 0;  // the ring sweep ends all at once: no drain for the resample kernel to fill
     P.Lg = static_cast<int>(row_bytes / 16);

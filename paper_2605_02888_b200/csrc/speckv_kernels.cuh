@@ -750,74 +750,58 @@ __device__ __forceinline__ CtlRegs ctl_load(const KParams& P, int b, int lane) {
     c.compk = (P.comp && lane < P.n_comp) ? __ldg(P.comp + static_cast<long long>(b) * P.n_comp + lane) : 0.f;
     return c;
 }
-// f4 = Hbar, cbar, Hmax, cmin.  fp32 throughout: 164 multiply-adds on values of order one.
+// f4 = Hbar, cbar, Hmax, cmin.  fp32 throughout: 164 multiply-adds on values of order one.  All outputs' reductions run
+// together, output by output only the last comparison: five shuffle steps instead of five per output, and a third of the
+// code (a row epilogue is one pass over cold instructions; the controller was 2.0 to 3.6 us of it).
 __device__ __forceinline__ void ctl_eval(const KParams& P, const CtlRegs& c, const float (&f4)[4],
                                          float* scores_row, int* gamma_next) {
     const int lane = threadIdx.x & 31;
-    if (P.layout == 2) {
-        // Sec. 4.3 as printed: a_hat = f([Hbar, cbar, Hmax, cmin, comp.., gamma_j]) for every candidate
-        float x[8];
-        x[0] = f4[0]; x[1] = f4[1]; x[2] = f4[2]; x[3] = f4[3];
+    // inputs x[0..n_in) in the layout's order: four signals (layout 0: three, without Hmax), then the compression features;
+    // layout 2 has the candidate gamma as its last input
+    const int n_sig = P.layout == 0 ? 3 : 4;
+    const int n_x = P.layout == 2 ? P.n_in - 1 : P.n_in;
+    float h = c.b1, wg = 0.f, xl = 0.f;  // hidden pre-activation (without gamma); gamma's weight; x[lane]
 #pragma unroll
-        for (int k = 4; k < 8; ++k) {
-            const float cv = __shfl_sync(0xffffffffu, c.compk, k - 4);
-            x[k] = (k < P.n_in - 1) ? cv : 0.f;
-        }
-        float base = c.b1, wg = 0.f, xl = 0.f;  // hidden pre-activation without gamma; gamma's weight; x[lane]
-#pragma unroll
-        for (int f = 0; f < 8; ++f) {
-            if (f < P.n_in - 1) base = fmaf(c.w1[f], x[f], base);
-            if (f == P.n_in - 1) wg = c.w1[f];
-            if (f == lane) xl = x[f];
-        }
-        const float b2 = __shfl_sync(0xffffffffu, c.b2k, 0);
-        float best = 0.f;
-        int best_j = 0;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            if (j < P.n_out) {  // uniform across the warp
-                const float g = static_cast<float>(P.gch[j]);
-                float term;
-                if (P.n_hidden > 0) {
-                    const float h = fmaf(wg, g, base);
-                    term = (lane < P.n_hidden && h > 0.f) ? c.w2[0] * h : 0.f;
-                } else {
-                    term = lane < P.n_in - 1 ? c.w2[0] * xl : (lane == P.n_in - 1 ? c.w2[0] * g : 0.f);
-                }
-                const float a_hat = warp_sumf(term) + b2;
-                const float e = (P.transform == 0) ? fmaf(a_hat, g, 1.f) : a_hat;
-                if (scores_row && lane == 0) scores_row[j] = e;
-                if (j == 0 || e > best) { best = e; best_j = j; }
-            }
-        }
-        if (gamma_next && lane == 0) *gamma_next = P.gch[best_j];
-        return;
+    for (int f = 0; f < 8; ++f) {
+        const float cv = __shfl_sync(0xffffffffu, c.compk, (f - n_sig) & 31);
+        const float sig = f == 0 ? f4[0] : f == 1 ? f4[1] : f == 2 ? (P.layout == 0 ? f4[3] : f4[2]) : f4[3];
+        const float x = f < n_sig ? sig : cv;
+        if (f < n_x) h = fmaf(c.w1[f], x, h);
+        if (P.layout == 2 && f == n_x) wg = c.w1[f];
+        if (f == lane && f < n_x) xl = x;
     }
-    float x[8];
-    const int first_comp = (P.layout == 0) ? 3 : 4;
-    if (P.layout == 0) { x[0] = f4[0]; x[1] = f4[1]; x[2] = f4[3]; x[3] = 0.f; }
-    else { x[0] = f4[0]; x[1] = f4[1]; x[2] = f4[2]; x[3] = f4[3]; }
-#pragma unroll
-    for (int k = 3; k < 8; ++k) {
-        const float cv = __shfl_sync(0xffffffffu, c.compk, (k - first_comp) & 31);
-        if (k >= first_comp) x[k] = (k < P.n_in) ? cv : 0.f;
-    }
-    float h = c.b1;
-#pragma unroll
-    for (int f = 0; f < 8; ++f)
-        if (f < P.n_in) h = fmaf(c.w1[f], x[f], h);
-    h = (lane < P.n_hidden && h > 0.f) ? h : 0.f;
-    float best = 0.f;
-    int best_j = 0;
+    float t[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-        const float b2 = __shfl_sync(0xffffffffu, c.b2k, j);
-        if (j < P.n_out) {  // uniform across the warp
-            const float o = warp_sumf(c.w2[j] * h) + b2;
-            const float e = (P.transform == 0) ? fmaf(o, static_cast<float>(P.gch[j]), 1.f) : o;
-            if (scores_row && lane == 0) scores_row[j] = e;
-            if (j == 0 || e > best) { best = e; best_j = j; }
+        const float g = static_cast<float>(P.gch[j]);
+        if (P.layout == 2 && P.n_hidden == 0) {  // Sec. 4.3 as printed, linear
+            t[j] = lane < n_x ? c.w2[0] * xl : (lane == n_x ? c.w2[0] * g : 0.f);
+        } else {
+            const float hj = P.layout == 2 ? fmaf(wg, g, h) : h;
+            t[j] = (lane < P.n_hidden && hj > 0.f) ? (P.layout == 2 ? c.w2[0] : c.w2[j]) * hj : 0.f;
         }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) t[j] += __shfl_xor_sync(0xffffffffu, t[j], o);
+    }
+    // lane j: output j
+    float v = t[0];
+#pragma unroll
+    for (int j = 1; j < 8; ++j) v = lane == j ? t[j] : v;
+    const float b2 = P.layout == 2 ? __shfl_sync(0xffffffffu, c.b2k, 0) : c.b2k;
+    const int g = P.gch[lane & 7];
+    const float o = v + b2;
+    const float e = (P.transform == 0) ? fmaf(o, static_cast<float>(g), 1.f) : o;
+    if (scores_row && lane < P.n_out) scores_row[lane] = e;
+    // the lowest index with the largest score; a NaN never wins against what stands before it
+    float best = __shfl_sync(0xffffffffu, e, 0);
+    int best_j = 0;
+#pragma unroll
+    for (int j = 1; j < 8; ++j) {
+        const float ej = __shfl_sync(0xffffffffu, e, j);
+        if (j < P.n_out && ej > best) { best = ej; best_j = j; }
     }
     if (gamma_next && lane == 0) *gamma_next = P.gch[best_j];
 }
@@ -1123,54 +1107,50 @@ __device__ __forceinline__ int row_status0(const KParams& P, int gam, float Tf) 
     return (gam < 1 || gam > P.G ? 1 : 0) | (!(Tf >= 0.f) || Tf == __int_as_float(0x7f800000) ? 8 : 0);
 }
 
-// Second half of a row epilogue (one warp): the walk over the positions, every output of the row except a drawn token.
-// dec: what lane i has learned about position i; ctl: the controller's parameters, fetched beforehand.
-// Order: what the resample kernel needs (acceptance, stop position, normalisers), the row's
-// completion flag, then the signals and the controller.
-// own_bonus: a bonus token is drawn by the caller (from the sweep's spans), not by the CTAs that wait for the flag.
-__device__ __noinline__ void row_finish(const KParams& P, int b, int gam, float Tf, const RowDecide& dec, const CtlRegs& ctl,
-                                        bool own_bonus) {
+// The walk over the positions (one warp, lane i holding position i's decision): where it ends, and the row's status.
+//
+// The positions are walked in order; the walk ends at the first one whose target row is non-finite
+// (which flags the row), whose draft token is out of range, or whose token is rejected.  Target rows
+// behind that position are not part of the step (Sec. 3.1 discards what follows the first mismatch):
+// whatever they hold flags nothing.  A non-finite draft row flags the row wherever it is.
+__device__ __forceinline__ int row_walk(const KParams& P, int gam, float Tf, const RowDecide& dec, int* stop_at) {
+    const int lane = threadIdx.x & 31;
+    const bool verify = (P.mode & MODE_VERIFY) != 0;
+    int status = row_status0(P, gam, Tf);
+    const bool tg_on = !status && verify && lane <= gam;
+    const unsigned stop = __ballot_sync(0xffffffffu, tg_on && (dec.tbad || (lane < gam && (dec.badtok || !dec.accept))));
+    const int first = stop ? (__ffs(stop) - 1) : gam;
+    const bool tbad_first = __shfl_sync(0xffffffffu, dec.tbad ? 1 : 0, first & 31) != 0;
+    const bool any_dbad = __any_sync(0xffffffffu, dec.dbad), any_badtok = __any_sync(0xffffffffu, dec.badtok);
+    if (status == 0) status = (any_dbad || (verify && tbad_first) ? 4 : 0) | (any_badtok ? 2 : 0);
+    *stop_at = (status == 0 && verify) ? first : 0;
+    return status;
+}
+
+// What the walk decides (one warp): status, accepted count, tokens except a drawn one, the record a draw needs and the
+// row's completion flag.  own_bonus: a bonus token is drawn by the caller (from the sweep's spans), not by the CTAs
+// that wait for the flag.
+__device__ __noinline__ void finish_verify(const KParams& P, int b, int gam, float Tf, const RowDecide& dec, bool own_bonus) {
     const int lane = threadIdx.x & 31;
     const int G = P.G;
     const bool verify = (P.mode & MODE_VERIFY) != 0;
-    int status = row_status0(P, gam, Tf);
     const bool greedy = (Tf == 0.f);
-    const float scale = static_cast<float>(kLog2e / static_cast<double>(greedy ? 1.f : Tf));
-    const bool tg_on = !status && verify && lane <= gam;
-    const int x = dec.x;
-    const float u_res = dec.u_res, Hi = dec.Hi, ci = dec.ci;
-    const double lse2_q = dec.lse2_q, lse2_p = dec.lse2_p;
-    const int amax = dec.amax;
-    const bool tbad = dec.tbad, badtok = dec.badtok, accept = dec.accept;
-    const bool any_dbad = __any_sync(0xffffffffu, dec.dbad);
-
-    // The positions are walked in order; the walk ends at the first one whose target row is non-finite
-    // (which flags the row), whose draft token is out of range, or whose token is rejected.  Target rows
-    // behind that position are not part of the step (Sec. 3.1 discards what follows the first mismatch):
-    // whatever they hold flags nothing.  A non-finite draft row flags the row wherever it is.
-    const unsigned stop = __ballot_sync(0xffffffffu, tg_on && (tbad || (lane < gam && (badtok || !accept))));
-    const int first = stop ? (__ffs(stop) - 1) : gam;
-    const bool tbad_first = __shfl_sync(0xffffffffu, tbad ? 1 : 0, first & 31) != 0;
-    if (status == 0) {
-        if (any_dbad || (verify && tbad_first)) status |= 4;
-        if (__any_sync(0xffffffffu, badtok)) status |= 2;
-    }
-    const int n = (status == 0 && verify) ? first : 0;
-
+    int n;
+    const int status = row_walk(P, gam, Tf, dec, &n);
     const int rs_mode = (verify && status == 0 && !greedy) ? (n < gam ? RS_RESIDUAL : RS_BONUS) : RS_NONE;
     if (verify) {
         // fresh token: known here for greedy rows, drawn by the resample step otherwise
-        const int amax_n = __shfl_sync(0xffffffffu, amax, n);
-        const double lp_n = __shfl_sync(0xffffffffu, lse2_p, n);
-        const double lq_n = __shfl_sync(0xffffffffu, lse2_q, n < gam ? n : 0);
-        const float u2_n = __shfl_sync(0xffffffffu, u_res, n);
-        if (lane <= G) {
+        const int amax_n = __shfl_sync(0xffffffffu, dec.amax, n);
+        const double lp_n = __shfl_sync(0xffffffffu, dec.lse2_p, n);
+        const double lq_n = __shfl_sync(0xffffffffu, dec.lse2_q, n < gam ? n : 0);
+        const float u2_n = __shfl_sync(0xffffffffu, dec.u_res, n);
+        if (lane <= G && !(own_bonus && rs_mode == RS_BONUS && lane == n)) {
             int v = -1;
             if (status == 0) {
-                if (lane < n) v = x;
+                if (lane < n) v = dec.x;
                 else if (lane == n && greedy) v = amax_n;
             }
-            if (!(own_bonus && rs_mode == RS_BONUS && lane == n)) P.out_tok[static_cast<long long>(b) * (G + 1) + lane] = v;
+            P.out_tok[static_cast<long long>(b) * (G + 1) + lane] = v;
         }
         if (lane == 0) {
             P.n_acc[b] = n;
@@ -1178,7 +1158,7 @@ __device__ __noinline__ void row_finish(const KParams& P, int b, int gam, float 
             ri.mode = rs_mode;
             ri.n = n;
             ri.u2 = (status == 0 && !greedy) ? u2_n : 0.f;
-            ri.scale = scale;
+            ri.scale = static_cast<float>(kLog2e / static_cast<double>(greedy ? 1.f : Tf));
             ri.lse2_p = lp_n;
             ri.lse2_q = lq_n;
             SPECKV_ST(P.info[b], ri);
@@ -1186,29 +1166,37 @@ __device__ __noinline__ void row_finish(const KParams& P, int b, int gam, float 
     }
     if (P.status && lane == 0) P.status[b] = status;
     row_done_signal(P, b, own_bonus && rs_mode == RS_BONUS ? RS_NONE : rs_mode, n);
+}
 
-    // signals
+// The signals and the controller's outputs (one warp); ctl: the controller's parameters, fetched beforehand.
+__device__ __noinline__ void finish_signals(const KParams& P, int b, int gam, float Tf, const RowDecide& dec, const CtlRegs& ctl) {
+    const int lane = threadIdx.x & 31;
+    const int G = P.G;
+    int n;
+    const int status = row_walk(P, gam, Tf, dec, &n);
     const float in_bits = P.bits ? static_cast<float>(kLog2e) : 1.f;
-    const float Hout = (status == 0 && lane < gam) ? Hi * in_bits : 0.f;
-    const float Cout = (status == 0 && lane < gam) ? ci : 0.f;
-    float f4[4] = {0.f, 0.f, 0.f, 0.f};
-    if (status == 0) {
-        f4[0] = warp_sumf(Hout) / static_cast<float>(gam);
-        f4[1] = warp_sumf(Cout) / static_cast<float>(gam);
-        f4[2] = warp_maxf(Hout);
-        f4[3] = -warp_maxf(lane < gam ? -Cout : -2.f);
+    const float Hout = (status == 0 && lane < gam) ? dec.Hi * in_bits : 0.f;
+    const float Cout = (status == 0 && lane < gam) ? dec.ci : 0.f;
+    float f4[4] = {Hout, Cout, Hout, (status == 0 && lane < gam) ? -Cout : -2.f};
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        f4[0] += __shfl_xor_sync(0xffffffffu, f4[0], o);
+        f4[1] += __shfl_xor_sync(0xffffffffu, f4[1], o);
+        f4[2] = fmaxf(f4[2], __shfl_xor_sync(0xffffffffu, f4[2], o));
+        f4[3] = fmaxf(f4[3], __shfl_xor_sync(0xffffffffu, f4[3], o));
     }
+    f4[0] = status == 0 ? f4[0] / static_cast<float>(gam) : 0.f;
+    f4[1] = status == 0 ? f4[1] / static_cast<float>(gam) : 0.f;
+    f4[3] = status == 0 ? -f4[3] : 0.f;
     if (lane < G) {
         if (P.H) P.H[static_cast<long long>(b) * G + lane] = Hout;
         if (P.C) P.C[static_cast<long long>(b) * G + lane] = Cout;
     }
     if (P.feat && lane < 4)
         P.feat[static_cast<long long>(b) * 4 + lane] = lane == 0 ? f4[0] : lane == 1 ? f4[1] : lane == 2 ? f4[2] : f4[3];
-
     if (P.mode & MODE_MLP) {
         if (status == 0) {
-            ctl_eval(P, ctl, f4, P.scores ? P.scores + static_cast<long long>(b) * P.n_out : nullptr,
-                     P.gamma_next + b);
+            ctl_eval(P, ctl, f4, P.scores ? P.scores + static_cast<long long>(b) * P.n_out : nullptr, P.gamma_next + b);
         } else {
             if (P.scores && lane < P.n_out) P.scores[static_cast<long long>(b) * P.n_out + lane] = 0.f;
             if (lane == 0) P.gamma_next[b] = 0;
@@ -1229,7 +1217,8 @@ __device__ __noinline__ void row_epilogue(const KParams& P, int b, int gam, floa
     if ((P.mode & MODE_MLP) && !status) ctl = ctl_load(P, b, threadIdx.x & 31);
     RowDecide dec;
     row_decide<T>(P, b, gam, Tf, status, 32, pd, nd, pt, nt, dec);
-    row_finish(P, b, gam, Tf, dec, ctl, false);
+    finish_verify(P, b, gam, Tf, dec, false);
+    finish_signals(P, b, gam, Tf, dec, ctl);
 }
 
 // Epilogue of a vocabulary shard's sweep (one warp per batch row): lane i merges this shard's nd

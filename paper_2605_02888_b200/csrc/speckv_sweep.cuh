@@ -6,36 +6,36 @@
 
 namespace speckv {
 
-// Row epilogue of the sliced sweep: a whole CTA, a warp per position.
+// Row epilogue of the sliced sweep: a whole CTA.  A warp per position decides; then, side by side, warp 0 walks the positions
+// and raises the row's flag, warp 1 writes the signals and runs the controller, and warps 2.. draw a bonus token from the sums
+// that the sweep left of the target row at position gamma.  Latency-bound (cold instructions and dependent round trips): one
+// after the other in one warp this took 6.6 us behind the last partial of a lone row, this way @@EPI@@.
+constexpr int kDrawWarp0 = 2;
 template <typename T>
 __device__ __noinline__ void row_epilogue_cta(const KParams& P, int b, int gam, float Tf, RowDecide* pos, double* sh_sum,
-                                                 DrawSrc* sh_src) {
+                                              DrawSrc* sh_src) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool verify = (P.mode & MODE_VERIFY) != 0;
     const long long row0 = static_cast<long long>(b) * P.J;
     const int n_pos = row_status0(P, gam, Tf) ? 0 : verify ? gam + 1 : gam;
-    // the parameters travel while the positions are decided; warp 0 takes the last turns, so it has the fewest positions
+    // the parameters travel while the positions are decided; warps 0 and 1 take the last turns
     CtlRegs ctl;
-    if (warp == 0 && (P.mode & MODE_MLP) && n_pos) ctl = ctl_load(P, b, lane);
+    if (warp == 1 && (P.mode & MODE_MLP) && n_pos) ctl = ctl_load(P, b, lane);
     for (int i = kWarps - 1 - warp; i < n_pos; i += kWarps)
         decide_position<T>(P, b, gam, Tf, i, P.part + (row0 + (verify ? P.G + 1 + i : i)) * P.nsplit, P.part + (row0 + i) * P.nsplit,
                            P.nsplit, pos[i]);
     __syncthreads();
-    // A bonus draw: every position accepted, nothing flagged (every warp finds the same).  Warps 1.. draw the token from the
-    // sums that the sweep left of the target row at position gamma while warp 0 writes the other outputs.
-    bool bonus = false;
-    if (verify && n_pos && Tf != 0.f) {
+    if (warp >= kDrawWarp0) {
+        // a bonus draw: every position accepted, nothing flagged
+        if (!verify || !n_pos || Tf == 0.f) return;
         bool ends = false;
         if (lane < n_pos) ends = pos[lane].dbad || pos[lane].tbad || pos[lane].badtok || !pos[lane].accept;
-        bonus = !__any_sync(0xffffffffu, ends);
-    }
-    if (warp != 0) {
-        if (!bonus) return;
+        if (__any_sync(0xffffffffu, ends)) return;
         const T* row = static_cast<const T*>(P.t) + static_cast<long long>(b) * P.tsb + static_cast<long long>(gam) * P.tsp;
         const float scale = static_cast<float>(kLog2e / static_cast<double>(Tf));
         const int n = P.nsplit * kWarps;
         const int tok = draw_from_spans<T>(row, P.V, scale, P.spans + static_cast<long long>(b) * n, n, P.per_warp, pos[gam].u_res,
-                                           warp - 1, kWarps - 1, 1, sh_sum, sh_src);
+                                           warp - kDrawWarp0, kWarps - kDrawWarp0, 1, sh_sum, sh_src);
         if (tok != kNotMine && lane == 0) P.out_tok[static_cast<long long>(b) * (P.G + 1) + gam] = max(tok, 0);
         return;
     }
@@ -43,7 +43,8 @@ __device__ __noinline__ void row_epilogue_cta(const KParams& P, int b, int gam, 
     dec.x = -1; dec.u_res = 0.f; dec.Hi = dec.ci = 0.f; dec.lse2_q = dec.lse2_p = 0.0; dec.amax = -1;
     dec.dbad = dec.tbad = dec.badtok = false; dec.accept = true;
     if (lane < n_pos) dec = pos[lane];
-    row_finish(P, b, gam, Tf, dec, ctl, true);
+    if (warp == 0) finish_verify(P, b, gam, Tf, dec, true);
+    else if (P.mode & MODE_SIGNALS) finish_signals(P, b, gam, Tf, dec, ctl);
 }
 
 // ----------------------------------------------------------------------------------------
