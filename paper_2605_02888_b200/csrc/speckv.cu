@@ -29,7 +29,7 @@ inline size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 struct Plan {
     int J_full;      // logit rows per batch row with verification: 2*G + 1
-    size_t off_tick, off_info, off_part, off_tokl, off_spans, off_dsum, total;
+    size_t off_tick, off_info, off_part, off_tokl, off_spans, off_dsum, off_list, total;
     size_t total_signals;  // what the signals alone may use: the scratch array of speckv_signals_static is held against it
 };
 
@@ -127,6 +127,7 @@ Plan make_plan(const speckv_batch* bt) {
     p.total_signals = off < kAlign ? kAlign : off;
     p.off_spans = off; off = align_up(off + B * kMaxSplit * kWarps * sizeof(float2));
     p.off_dsum = off; off = align_up(off + B * kMaxShares * kWarps * sizeof(double));
+    p.off_list = off; off = align_up(off + B * p.J_full * sizeof(int2));
     p.total = off < kAlign ? kAlign : off;
     return p;
 }
@@ -225,31 +226,43 @@ cudaError_t launch_pipe(const KParams& P, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-// After the register-staged sweep the fresh tokens are drawn by extra CTAs of the same launch; the rows swept last have their fresh tokens drawn by more, shorter CTAs (see resample_body)
-constexpr int kRsTailRows = 32;  // b256, same box, builds in turn: 16 rows 158.7 us, 32 rows 156.6 us, 64 rows 156.7 us, 128 rows 157.2 us
-constexpr int kRsTailMult = 2;
+constexpr int kPrepRows = 32;  // batch rows per CTA of the preparing kernel at least; 64 CTAs at most
+
+// The sliced sweep: list and cleared counters, then the sweep with n_draw CTAs behind it.  The sweep is a programmatic
+// dependent launch: its CTAs are placed while the preparing kernel runs and wait for its end.
+template <typename T>
+cudaError_t launch_sliced(KParams P, long long n_draw, cudaStream_t st, cudaEvent_t before_sweep) {
+    constexpr int U = sizeof(T) == 2 ? kSweepLoads : (kSweepLoads + 1) / 2;
+    P.n_draw = static_cast<int>(n_draw);
+    int seg = (P.B + 63) / 64;
+    seg = seg < kPrepRows ? kPrepRows : (seg + 31) / 32 * 32;
+    prep_kernel<<<static_cast<unsigned>((P.B + seg - 1) / seg), kThreads, 0, st>>>(P, seg);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    if (before_sweep) cudaEventRecord(before_sweep, st);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(static_cast<long long>(P.B) * P.J * P.nsplit + n_draw));
+    cfg.blockDim = dim3(kThreads);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, sweep_kernel<T, U>, P);
+}
 
 template <typename T>
-cudaError_t launch_all(KParams P, cudaStream_t st, const Events& ev, bool ring) {
-    constexpr int U = sizeof(T) == 2 ? kSweepLoads : (kSweepLoads + 1) / 2;
+cudaError_t launch_all(const KParams& P, cudaStream_t st, const Events& ev, bool ring) {
     const bool verify = (P.mode & MODE_VERIFY) != 0;
-    P.rs_tail = 0; P.R2 = P.R; P.draw_pw2 = P.draw_pw;
-    bool merged = verify && !ring && P.rdone;
-    if (merged && P.B >= 4 * kRsTailRows && P.R * kRsTailMult <= kMaxShares && P.draw_pw >= 64) {
-        P.rs_tail = kRsTailRows;
-        P.R2 = P.R * kRsTailMult;
-        P.draw_pw2 = (P.draw_pw + kRsTailMult - 1) / kRsTailMult;
-    }
-    const long long n_draw = static_cast<long long>(P.B - P.rs_tail) * P.R + static_cast<long long>(P.rs_tail) * P.R2;
-    merged = merged && P.n_sweep + n_draw <= 0x7fffffffLL;
-    if (ev.before_sweep) cudaEventRecord(ev.before_sweep, st);
+    const long long n_draw = static_cast<long long>(P.B) * P.R;
+    const bool merged = verify && !ring && static_cast<long long>(P.B) * P.J * P.nsplit + n_draw <= 0x7fffffffLL;
     cudaError_t e;
     if (ring) {
+        if (ev.before_sweep) cudaEventRecord(ev.before_sweep, st);
         e = launch_pipe<T>(P, st);
     } else {
-        const long long grid = P.n_sweep + (merged ? n_draw : 0);
-        sweep_kernel<T, U><<<static_cast<unsigned>(grid), kThreads, 0, st>>>(P);
-        e = cudaGetLastError();
+        e = launch_sliced<T>(P, merged ? n_draw : 0, st, ev.before_sweep);
     }
     if (e != cudaSuccess) return e;
     if (ev.after_sweep) cudaEventRecord(ev.after_sweep, st);
@@ -320,14 +333,10 @@ speckv_status run(const speckv_batch* bt, int mode, const float* comp, const spe
     P.dsum = reinterpret_cast<double*>(w + pl.off_dsum);
 
     if (static_cast<long long>(P.B) * P.J * P.nsplit > 0x7fffffffLL) return SPECKV_ERR_UNSUPPORTED;
-    P.n_sweep = P.B * P.J * P.nsplit;
 
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     if (dbg_register(cs, bt, verify, ws, ws_bytes) != cudaSuccess) return SPECKV_ERR_CUDA;
     const long long row_bytes = static_cast<long long>(P.V) * es;
-
-    if (cudaMemsetAsync(P.tick1, 0, (6 * static_cast<size_t>(P.B) + 4) * sizeof(int), cs) != cudaSuccess)
-        return SPECKV_ERR_CUDA;
 
     // the staged sweep wants whole 16-byte granules per row and a batch its per-row tables can hold
     // Which sweep.  Measured on B200 (full-size workloads, same inputs): fp32 logits are bound by
@@ -341,6 +350,13 @@ speckv_status run(const speckv_batch* bt, int mode, const float* comp, const spe
 constexpr int kPipeMinB = 384;
     const bool staged = bt->dtype == SPECKV_F32 && aligned && row_bytes % 16 == 0 && P.B <= kPipeMaxB && P.B >= kPipeMinB &&
                         !(bt->flags & SPECKV_SCHEDULE_SLICED);
+    if (staged) {
+        if (cudaMemsetAsync(P.tick1, 0, (6 * static_cast<size_t>(P.B) + 4) * sizeof(int), cs) != cudaSuccess) return SPECKV_ERR_CUDA;
+    } else {
+        P.n_list = P.qcount; P.q_front = P.qhead; P.q_back = P.qtail;  // the ring's counters and queue are not in use
+        // signals: behind their partials, which take a third of that region; verification: a region of its own
+        P.list = reinterpret_cast<int2*>(verify ? w + pl.off_list : reinterpret_cast<char*>(P.part + static_cast<size_t>(P.B) * P.J * P.nsplit));
+    }
     // completion flags per batch row and the logits at the draft tokens: only the register-staged sweep
     // overlaps the resample work with its own tail; after the ring sweep the resample kernel starts when
     // everything is done and a flag would only cost it a round trip
@@ -361,7 +377,6 @@ constexpr int kPipeMinB = 384;
             P.early = P.rowq + 3 * P.B;
         }
     }
-    P.rs_reverse = staged ? 1 : 0;  // the ring sweep ends all at once: no drain for the resample kernel to fill
     P.Lg = static_cast<int>(row_bytes / 16);
     P.Lp = (P.Lg + kStageGran - 1) / kStageGran * kStageGran;
     cudaError_t e;
@@ -443,7 +458,7 @@ cudaError_t static_scratch_address(void** out) {
 
 // ---- vocabulary-sharded verification (speckv_shard.cuh) ----
 struct ShardPlan {
-    size_t off_tick, off_part, off_dsum, off_dsum2, total;
+    size_t off_tick, off_part, off_dsum, off_dsum2, off_list, total;
 };
 ShardPlan make_shard_plan(const speckv_batch* bt) {
     ShardPlan p;
@@ -453,6 +468,7 @@ ShardPlan make_shard_plan(const speckv_batch* bt) {
     p.off_part = off; off = align_up(off + B * J * kMaxSplit * sizeof(float4));
     p.off_dsum = off; off = align_up(off + B * kMaxShares * kWarps * sizeof(double));
     p.off_dsum2 = off; off = align_up(off + B * kMaxShares * kWarps * sizeof(double));
+    p.off_list = off; off = align_up(off + B * J * sizeof(int2));
     p.total = off < kAlign ? kAlign : off;
     return p;
 }
@@ -486,6 +502,8 @@ speckv_status shard_params(const speckv_batch* bt, void* ws, size_t ws_bytes, KP
     P.part = reinterpret_cast<float4*>(w + pl.off_part);
     P.dsum = reinterpret_cast<double*>(w + pl.off_dsum);
     P.dsum2 = reinterpret_cast<double*>(w + pl.off_dsum2);
+    P.list = reinterpret_cast<int2*>(w + pl.off_list);
+    P.n_list = P.qcount; P.q_front = P.qhead; P.q_back = P.qtail;
     return SPECKV_OK;
 }
 bool shard_aligned(const speckv_batch* bt) {
@@ -645,11 +663,12 @@ speckv_status speckv_internal_wait_probe(int32_t B, int32_t* row_status, int32_t
     // the draw kernel on its own, one CTA per batch row, with completion flags that nothing raises
     KParams P{};
     P.B = B; P.G = 1; P.V = 256; P.J = 3; P.R = 1; P.draw_pw = 8;
-    P.R2 = 1; P.draw_pw2 = 8; P.mode = MODE_VERIFY;
+    P.mode = MODE_VERIFY;
     P.wait_limit = g_wait_limit.load(std::memory_order_relaxed);
     P.status = row_status; P.out_tok = out_tokens;
     P.rdone = static_cast<int*>(workspace);
     P.tick2 = P.rdone + B;
+    P.q_front = P.q_back = P.tick2;  // the draws' tickets are not reached
     cudaStream_t cs = static_cast<cudaStream_t>(cuda_stream);
     {
         speckv_batch none{};
@@ -681,7 +700,6 @@ speckv_status speckv_shard_sweep(const speckv_batch* local, int64_t v_begin, flo
     const bool al = shard_aligned(local);
     choose_slices(P, local->dtype, al);
     if (static_cast<long long>(P.B) * P.J * P.nsplit > 0x7fffffffLL) return SPECKV_ERR_UNSUPPORTED;
-    P.n_sweep = P.B * P.J * P.nsplit;
     P.v_begin = static_cast<int>(v_begin);
     P.export_state = 1;
     P.state = reinterpret_cast<float4*>(shard_state);
@@ -692,11 +710,8 @@ speckv_status speckv_shard_sweep(const speckv_batch* local, int64_t v_begin, flo
                                 {shard_tokl, static_cast<size_t>(P.B) * P.G * sizeof(float2)}};
         if (dbg_register(cs, local, true, workspace, workspace_bytes, ex, 2) != cudaSuccess) return SPECKV_ERR_CUDA;
     }
-    if (cudaMemsetAsync(P.tick1, 0, (3 * static_cast<size_t>(P.B) + 4) * sizeof(int), cs) != cudaSuccess)
-        return SPECKV_ERR_CUDA;
     if (cudaMemsetAsync(shard_tokl, 0, static_cast<size_t>(P.B) * P.G * sizeof(float2), cs) != cudaSuccess)
         return SPECKV_ERR_CUDA;
-    const unsigned grid = static_cast<unsigned>(P.n_sweep);
     constexpr int Ub = kSweepLoads, Uf = (kSweepLoads + 1) / 2;
     // A slice row is short (V / n_shards columns).  One CTA per short row is mostly overhead and the
     // ring sweep pays per logit row as well (segment hand-over to its epilogue warp), so rows of up to
@@ -712,12 +727,8 @@ speckv_status speckv_shard_sweep(const speckv_batch* local, int64_t v_begin, flo
         }
         return cudaGetLastError() == cudaSuccess ? SPECKV_OK : SPECKV_ERR_CUDA;
     }
-    if (local->dtype == SPECKV_BF16) {
-        sweep_kernel<__nv_bfloat16, Ub><<<grid, kThreads, 0, cs>>>(P);
-    } else {
-        sweep_kernel<float, Uf><<<grid, kThreads, 0, cs>>>(P);
-    }
-    return cudaGetLastError() == cudaSuccess ? SPECKV_OK : SPECKV_ERR_CUDA;
+    const cudaError_t e = local->dtype == SPECKV_BF16 ? launch_sliced<__nv_bfloat16>(P, 0, cs, nullptr) : launch_sliced<float>(P, 0, cs, nullptr);
+    return e == cudaSuccess ? SPECKV_OK : SPECKV_ERR_CUDA;
 }
 
 speckv_status speckv_shard_finish(const speckv_batch* local, int32_t n_shards, int32_t shard_width, int32_t V_total,

@@ -453,46 +453,38 @@ __device__ __forceinline__ void resample_row(const KParams& P, const int b, cons
 template <typename T>
 __device__ __forceinline__ void resample_body(const KParams& P, const int bid) {
     __shared__ int sh_wait;
-    // one-dimensional grid, R consecutive CTAs per batch row: the CTAs of a row are neighbours in
-    // launch order, so rows finish one after the other and their searches overlap the other rows' sums
-    // the last rs_tail draws (in launch order) are cut into R2 >= R shares: their rows are the last to
-    // be swept, nothing is left to overlap their draw with, and more CTAs per row shorten it
-    const int n_head = (P.B - P.rs_tail) * P.R;
-    const bool tail = bid >= n_head;
-    const int Rr = tail ? P.R2 : P.R;
-    const int dw = tail ? P.draw_pw2 : P.draw_pw;
-    const int bq = tail ? (P.B - P.rs_tail) + (bid - n_head) / Rr : bid / Rr;
-    const int share = tail ? (bid - n_head) % Rr : bid % Rr;
-    const int b = P.rs_reverse ? P.B - 1 - bq : bq;
-    // With completion flags a CTA waits only for its own batch row (rows
-    // are taken in the order the sweep finishes them unless rs_reverse is set) and the stop positions of finished rows are
-    // summed while the sweep drains; every sweep CTA is resident or done before the first CTA that draws
-    // starts, so the wait ends, and it is bounded all the same.  Without flags (a programmatic dependent launch behind the
-    // ring sweep) the CTA waits for the whole sweep grid.
-    int mode, n;
+    // one-dimensional grid, R consecutive CTAs per draw
+    const int g = bid / P.R, share = bid - g * P.R;
+    int mode, n, b;
     if (P.rdone) {
-        if (threadIdx.x == 0) sh_wait = row_done_wait(P.rdone + b, P.wait_limit);
+        // Group g takes the row in slot g of the draw queue.  Every sweep CTA is resident or done before the first CTA that
+        // draws starts, so all slots get filled and the wait ends; it is bounded all the same.
+        if (threadIdx.x == 0) sh_wait = row_done_wait(P.rdone + g, P.wait_limit);
         __syncthreads();
         const int v = sh_wait;
         if (!v) {
-            // Gave up.  The mark goes on the row's flag: if the row epilogue has already written the
-            // status (the flag went up just after the last poll) the bit is added here, otherwise the
-            // epilogue finds the mark when it raises the flag and adds the bit itself.
+            // Gave up.  The mark goes on the slot: if the row epilogue has already written the
+            // status (the slot was filled just after the last poll) the bit is added here, otherwise the
+            // epilogue finds the mark when it takes the slot and adds the bit itself.
             if (threadIdx.x == 0 && share == 0) {
-                const int old = atomicOr(P.rdone + b, kRowDoneTimeout);
-                if ((old & 1) && P.status) atomicOr(P.status + b, 16);
+                const int old = atomicOr(P.rdone + g, kSlotTimeout);
+                if ((old & kSlotDone) && P.status) atomicOr(P.status + (old & 0xffffff), 16);
             }
             return;
         }
-        mode = (v >> 8) & 3;
-        n = (v >> 16) & 0xff;
+        b = v & 0xffffff;
+        mode = (v >> 24) & 1 ? RS_RESIDUAL : RS_NONE;
+        n = (v >> 25) & 15;
     } else {
+        // A programmatic dependent launch behind the ring sweep: waits for the whole sweep; last batch row first (those rows
+        // are the freshest in L2).
         asm volatile("griddepcontrol.wait;" ::: "memory");
+        b = P.B - 1 - g;
         const int4 lo4 = __ldcg(reinterpret_cast<const int4*>(P.info + b));
         mode = lo4.x;
         n = lo4.y;
     }
-    resample_row<T>(P, b, mode, n, share, Rr, dw);
+    resample_row<T>(P, b, mode, n, share, P.R, P.draw_pw);
 }
 
 template <typename T>

@@ -83,11 +83,13 @@ static_assert(sizeof(RowInfo) == 32, "the resample kernel reads a RowInfo as two
 struct KParams {
     int B, G, V, J, nsplit, R, mode, bits;
     int per_warp;  // sweep kernel: 16-byte granules of a logit row that one warp folds; a slice is kWarps times that
-    int n_sweep;  // sweep kernel: CTAs that sweep; the rest of the grid (if any) does the resample work
+    int2* list;     // sliced sweep: one entry per logit row to sweep, in the order of the grid (prep_kernel)
+    int* n_list;    //   and how many there are; CTAs behind the last one draw
+    int n_draw;     // sliced sweep: CTAs that may draw (R per batch row), 0 = none
     int draw_pw;  // draw: granules of the stop position that one warp sums; R CTAs of kWarps warps per batch row
-    int rs_tail, R2, draw_pw2;  // draw: the last rs_tail rows in launch order use R2 CTAs each
+    int *q_front, *q_back;  // draw queue: rows with a residual draw fill rdone from the front, the others from the back
     int wait_limit;  // polls a resample CTA spends on its row's completion flag before it gives the row up
-    // Generation order of the sweep grid (verification, early != nullptr): first the draft and target rows of
+    // Generation order of the sweep (verification, early != nullptr): first the draft and target rows of
     // positions 0..k_early of every batch row, then the remaining draft rows, last the remaining target rows,
     // which are left unread where the walk is already known to have stopped at a position <= k_early.
     int k_early, read_all;
@@ -109,7 +111,7 @@ struct KParams {
     int *tick1, *tick2;
     int *qcount, *qhead, *qtail, *rowq;  // staged sweep: next quantum to hand out; queue of completed batch rows
     float2* tokl;  // [B, G] (draft logit, target logit) at the draft token, left by the register-staged sweep; may be NULL
-    int* rdone;  // verification: rdone[b] = 1 once batch row b's epilogue has written everything the resample kernel reads
+    int* rdone;  // verification: the draw queue's slots, one per batch row (row_done_signal); draft-side sampling: row status
     RowInfo* info;
     float4* part;
     float2* spans;  // (reference, sum) of every warp's range of the row a plain draw may need: verification [B, nsplit * kWarps]
@@ -578,124 +580,139 @@ __device__ __noinline__ uint4 gran_edge(const GranRow r, int g, float pad) {
 }
 
 // ----------------------------------------------------------------------------------------
-// One WARP sweeps granules [lo, hi) of one logit row and returns the merged partial in every lane.  Lane l owns
+// One WARP sweeps granules [lo, hi) of one logit row.  Lane l owns
 // granules l, l+32, ... of the range; a step folds kVec elements per lane (bf16: one granule, fp32: two granules 32
 // apart, so that every load of the warp covers 512 contiguous bytes), U steps are in flight.  Warps of a CTA take
 // adjacent ranges and never wait for one another once the loop runs.
-// CTA_WARM: the warps of the CTA sweep ranges of the same row and share their warm starts (one
-// barrier, every warp of the CTA must call); false: the warp is on its own row.
+//   start   requests the first U steps: all it takes is the row's address
+//   warm    the reference the sums start from: the largest element of the first steps, over the warp, or over the CTA whose
+//           warps sweep ranges of the same row (one barrier, every warp must call)
+//   run     folds the range and returns the merged partial in every lane
 // ----------------------------------------------------------------------------------------
-template <typename T, int PATH, int U, bool CTA_WARM = true>
-__device__ __forceinline__ float4 sweep_warp(const GranRow& row, int lo, int hi, float scale, volatile float* sh_m0) {
-    constexpr int E = 16 / sizeof(T);
-    constexpr int GS = kVec / E;  // granules per lane and step
-    const float pad = (PATH == PATH_DRAFT) ? kFloor : __int_as_float(0xff800000);
-    const int lane = threadIdx.x & 31;
-    const int a = max(lo, row.whole_lo());
-    const int left = min(hi, row.whole_hi()) - a - lane;  // whole granules from this lane's first one on
-    const int n_main = left > 0 ? (left + 32 * GS - 1) / (32 * GS) : 0;
-    const uint4* p = row.base + a + lane;
-    auto load = [&](int k) {
+template <typename T, int U>
+struct WarpSweep {
+    static constexpr int E = 16 / sizeof(T);
+    static constexpr int GS = kVec / E;  // granules per lane and step
+    const uint4* p;
+    int a, left, n_main, meta, ng;
+    bool first_edge, last_edge;
+    Raw<T> buf[U];
+
+    __device__ __forceinline__ Raw<T> load(int k) const {
         Raw<T> r;
         r.a = ldg_stream(p + 32 * GS * k);
-        if constexpr (GS == 2) r.b = (left > 64 * k + 32) ? ldg_stream(p + 64 * k + 32) : gran_fill<T>(pad);
+        if constexpr (GS == 2) r.b = (left > 64 * k + 32) ? ldg_stream(p + 64 * k + 32) : gran_fill<T>(__int_as_float(0xff800000));
         return r;
-    };
+    }
     // incomplete granules: lane 0 the row's first, lane 1 its last
-    const bool first_edge = row.shift() != 0 && lo == 0 && hi > 0;
-    const bool last_edge = row.tail() != 0 && row.ng - 1 >= lo && row.ng - 1 < hi && !(row.shift() != 0 && row.ng == 1);
-    Raw<T> edge = raw_fill<T>(pad);
-    if (first_edge && lane == 0) edge.a = gran_edge<T>(row, 0, pad);
-    if (last_edge && lane == 1) edge.a = gran_edge<T>(row, row.ng - 1, pad);
-
-    Raw<T> buf[U];
-#pragma unroll
-    for (int k = 0; k < U; ++k) {
-        buf[k] = raw_fill<T>(pad);
-        if (k < n_main) buf[k] = load(k);
+    __device__ __forceinline__ Raw<T> edge() const {
+        const int lane = threadIdx.x & 31;
+        GranRow row;
+        row.base = p - a - lane; row.ng = ng; row.meta = meta;
+        Raw<T> e = raw_fill<T>(__int_as_float(0xff800000));
+        if (first_edge && lane == 0) e.a = gran_edge<T>(row, 0, __int_as_float(0xff800000));
+        if (last_edge && lane == 1) e.a = gran_edge<T>(row, ng - 1, __int_as_float(0xff800000));
+        return e;
     }
-
-    // warm start: the warp-wide maximum of the first U steps of every lane.  A step holding
-    // NaN / +inf / only -inf contributes the floor; its owner meets the offending element again
+    __device__ __forceinline__ void start(const GranRow& row, int lo, int hi) {
+        const int lane = threadIdx.x & 31;
+        a = max(lo, row.whole_lo());
+        left = min(hi, row.whole_hi()) - a - lane;  // whole granules from this lane's first one on
+        n_main = left > 0 ? (left + 32 * GS - 1) / (32 * GS) : 0;
+        p = row.base + a + lane;
+        meta = row.meta;
+        ng = row.ng;
+        first_edge = row.shift() != 0 && lo == 0 && hi > 0;
+        last_edge = row.tail() != 0 && row.ng - 1 >= lo && row.ng - 1 < hi && !(row.shift() != 0 && row.ng == 1);
+#pragma unroll
+        for (int k = 0; k < U; ++k) {
+            buf[k] = raw_fill<T>(__int_as_float(0xff800000));
+            if (k < n_main) buf[k] = load(k);
+        }
+    }
+    // A step holding NaN / +inf / only -inf contributes the floor; its owner meets the offending element again
     // in its own state and flags it there.
-    float m0 = kFloor;
-    auto warm = [&](const Raw<T>& r) {
-        const float v = raw_max(r);
-        if (v >= kFloor && v < __int_as_float(0x7f800000)) m0 = fmaxf(m0, v);
-    };
+    template <bool CTA>
+    __device__ __forceinline__ float warm(volatile float* sh_m0) const {
+        float m0 = kFloor;
 #pragma unroll
-    for (int k = 0; k < U; ++k) warm(buf[k]);
-    if (first_edge || last_edge) warm(edge);
-    m0 = warp_maxf(m0);
-    // share the warm start across the CTA's warps (one barrier per CTA, before the streaming loop)
-    if (CTA_WARM) {
-        if (lane == 0) sh_m0[threadIdx.x >> 5] = m0;
-        __syncthreads();
+        for (int k = 0; k < U; ++k) {
+            const float v = raw_max(buf[k]);
+            if (v >= kFloor && v < __int_as_float(0x7f800000)) m0 = fmaxf(m0, v);
+        }
+        m0 = warp_maxf(m0);
+        if (CTA) {
+            if ((threadIdx.x & 31) == 0) sh_m0[threadIdx.x >> 5] = m0;
+            __syncthreads();
 #pragma unroll
-        for (int w = 0; w < kWarps; ++w) m0 = fmaxf(m0, sh_m0[w]);
+            for (int w = 0; w < kWarps; ++w) m0 = fmaxf(m0, sh_m0[w]);
+        }
+        return m0;
     }
-
-    DraftState ds; TargetState ts; ArgmaxState as;
-    if constexpr (PATH == PATH_DRAFT) ds.init(m0, scale);
-    else if constexpr (PATH == PATH_TARGET) ts.init(m0, scale);
-    else as.init(m0);
-
-    if constexpr (PATH == PATH_TARGET) {
-        if (first_edge || last_edge) ts.template careful<T>(edge, scale);
-        // steps i .. i+n-1 went into ga, gb
-        auto close = [&](f2 ga, f2 gb, int i, int n) {
-            const float g = hsum2(add2(ga, gb));
-            if (g < kBigSum) {
-                ts.z += g;
-            } else {
+    template <int PATH>
+    __device__ __forceinline__ float4 run(float m0, float scale) {
+        const int lane = threadIdx.x & 31;
+        DraftState ds; TargetState ts; ArgmaxState as;
+        if constexpr (PATH == PATH_DRAFT) ds.init(m0, scale);
+        else if constexpr (PATH == PATH_TARGET) ts.init(m0, scale);
+        else as.init(m0);
+        if constexpr (PATH == PATH_TARGET) {
+            if (first_edge || last_edge) ts.template careful<T>(edge(), scale);
+            // steps i .. i+n-1 went into ga, gb
+            auto close = [&](f2 ga, f2 gb, int i, int n) {
+                const float g = hsum2(add2(ga, gb));
+                if (g < kBigSum) {
+                    ts.z += g;
+                } else {
 #pragma unroll 1
-                for (int k = i; k < i + n; ++k) ts.template careful<T>(load(k), scale);
+                    for (int k = i; k < i + n; ++k) ts.template careful<T>(load(k), scale);
+                }
+            };
+            int i = 0;
+            for (; i + U <= n_main; i += U) {
+                f2 ga = pack2(0.f, 0.f), gb = ga;
+#pragma unroll
+                for (int k = 0; k < U; ++k) {
+                    const Raw<T> cur = buf[k];
+                    const int nx = i + U + k;
+                    if (nx < n_main) buf[k] = load(nx);
+                    ts.template add<T>(cur, scale, ga, gb);
+                }
+                close(ga, gb, i, U);
             }
-        };
-        int i = 0;
-        for (; i + U <= n_main; i += U) {
             f2 ga = pack2(0.f, 0.f), gb = ga;
 #pragma unroll
-            for (int k = 0; k < U; ++k) {
-                const Raw<T> cur = buf[k];
-                const int nx = i + U + k;
-                if (nx < n_main) buf[k] = load(nx);
-                ts.template add<T>(cur, scale, ga, gb);
+            for (int k = 0; k < U; ++k)
+                if (i + k < n_main) ts.template add<T>(buf[k], scale, ga, gb);
+            close(ga, gb, i, n_main - i);
+        } else {
+            const int shift = meta & 15;
+            auto process = [&](const Raw<T>& v, int g) {  // g: granule of the first half
+                if constexpr (PATH == PATH_DRAFT) ds.template step<T>(v, scale);
+                else as.template step<T>(v, g * E - shift, GS == 2 ? (g + 32) * E - shift : g * E - shift + kVec / 2);
+            };
+            if (first_edge || last_edge) process(edge(), lane == 0 ? 0 : ng - 1);
+            int i = 0;
+            for (; i + U <= n_main; i += U) {
+#pragma unroll
+                for (int k = 0; k < U; ++k) {
+                    const Raw<T> cur = buf[k];
+                    const int nx = i + U + k;
+                    if (nx < n_main) buf[k] = load(nx);
+                    process(cur, a + lane + 32 * GS * (i + k));
+                }
             }
-            close(ga, gb, i, U);
+#pragma unroll
+            for (int k = 0; k < U; ++k)
+                if (i + k < n_main) process(buf[k], a + lane + 32 * GS * (i + k));
         }
-        f2 ga = pack2(0.f, 0.f), gb = ga;
-#pragma unroll
-        for (int k = 0; k < U; ++k)
-            if (i + k < n_main) ts.template add<T>(buf[k], scale, ga, gb);
-        close(ga, gb, i, n_main - i);
-    } else {
-        auto process = [&](const Raw<T>& v, int g) {  // g: granule of the first half
-            if constexpr (PATH == PATH_DRAFT) ds.template step<T>(v, scale);
-            else as.template step<T>(v, g * E - row.shift(), GS == 2 ? (g + 32) * E - row.shift() : g * E - row.shift() + kVec / 2);
-        };
-        if (first_edge || last_edge) process(edge, lane == 0 ? 0 : row.ng - 1);
-        int i = 0;
-        for (; i + U <= n_main; i += U) {
-#pragma unroll
-            for (int k = 0; k < U; ++k) {
-                const Raw<T> cur = buf[k];
-                const int nx = i + U + k;
-                if (nx < n_main) buf[k] = load(nx);
-                process(cur, a + lane + 32 * GS * (i + k));
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < U; ++k)
-            if (i + k < n_main) process(buf[k], a + lane + 32 * GS * (i + k));
+        float4 part;
+        if constexpr (PATH == PATH_DRAFT) part = ds.partial(scale);
+        else if constexpr (PATH == PATH_TARGET) part = ts.partial();
+        else part = as.partial();
+        return warp_merge<PATH>(part, scale);
     }
-
-    float4 part;
-    if constexpr (PATH == PATH_DRAFT) part = ds.partial(scale);
-    else if constexpr (PATH == PATH_TARGET) part = ts.partial();
-    else part = as.partial();
-    return warp_merge<PATH>(part, scale);
-}
+};
 
 // ----------------------------------------------------------------------------------------
 // Row epilogue helpers (one warp, double precision; a few dozen values per row)
@@ -811,30 +828,33 @@ __device__ __forceinline__ void ctl_eval(const KParams& P, const CtlRegs& c, con
 // per batch row, so the cost does not show
 __device__ __forceinline__ double log2_split(double z) { return log2(z); }
 
-// End of a row epilogue (whole warp): everything the warp wrote for batch row b becomes visible
-// before the row's completion flag does.  The resample kernel polls the flag instead of waiting for
-// the whole sweep grid, so it can work on finished rows while the sweep's last CTAs drain.
-constexpr int kRowDoneTimeout = 1 << 30;  // a resample CTA gave up waiting for this row
+// End of a row epilogue (whole warp): everything the warp wrote for batch row b becomes visible, then the row takes a slot
+// of the draw queue: rows with a residual draw from the front in the order in which they complete, all others from the
+// back, so that every slot is filled once all rows are done.  Group g of the CTAs that draw waits for slot g, not for a
+// batch row: it starts on the first finished row whatever its number, and the groups that find nothing to draw come last
+// (by batch row, 1,024 rows of which a third draw spent 9 us of all CTA slots on groups with nothing to do).
+constexpr int kSlotDone = 1 << 30, kSlotTimeout = 1 << 31;  // bits 0-23: batch row, 24: a residual draw, 25-28: stop position
 __device__ __forceinline__ void row_done_signal(const KParams& P, int b, int mode, int n) {
     if (!P.rdone) return;
+    const bool draw = mode == RS_RESIDUAL;
+    int slot = 0;
+    if ((threadIdx.x & 31) == 0) slot = draw ? atomicAdd(P.q_front, 1) : P.B - 1 - atomicAdd(P.q_back, 1);
     __threadfence();
     __syncwarp();
-    // the flag carries what a resample CTA needs to start fetching logits: draw mode and stop position
-    const int v = 1 | (mode << 8) | (n << 16);
     if ((threadIdx.x & 31) == 0) {
-        const int old = atomicOr(P.rdone + b, v);
-        // a resample CTA whose bounded wait ran out before this point left its mark here: the row's fresh
+        const int old = atomicOr(P.rdone + slot, kSlotDone | b | (draw ? 1 << 24 | n << 25 : 0));
+        // a group whose bounded wait ran out before this point left its mark here: the row's fresh
         // token will never be drawn, and the status written above must say so
-        if ((old & kRowDoneTimeout) && P.status) atomicOr(P.status + b, 16);
+        if ((old & kSlotTimeout) && P.status) atomicOr(P.status + b, 16);
     }
 }
 
-// Bounded wait for a row's completion flag (one thread polls).  The flag's value, 0 when the bound ran out.
+// Bounded wait for a slot of the draw queue (one thread polls).  The slot's value, 0 when the bound ran out.
 __device__ __forceinline__ int row_done_wait(const int* flag, int limit) {
     for (int it = 0; it < limit; ++it) {
         int v;
         asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(flag) : "memory");
-        if (v & 1) return v;
+        if (v & kSlotDone) return v;
         __nanosleep(it < 64 ? 100 : 1000);
     }
     return 0;

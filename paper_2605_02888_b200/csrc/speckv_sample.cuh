@@ -40,12 +40,15 @@ __global__ void __launch_bounds__(kThreads, kSweepCtasPerSm) sample_kernel(const
     float2* spans = P.spans + static_cast<long long>(r) * n;
     {
         const int lo = (s * kWarps + warp) * P.per_warp;
+        WarpSweep<T, U> ws;
+        ws.start(make_row(row, P.V), lo, lo + P.per_warp);
+        const float m0 = ws.template warm<true>(sh_m0);
         float2 v;
         if (greedy) {
-            const float4 p = sweep_warp<T, PATH_ARGMAX, U>(make_row(row, P.V), lo, lo + P.per_warp, scale, sh_m0);
+            const float4 p = ws.template run<PATH_ARGMAX>(m0, scale);
             v = make_float2(p.z != 0.f ? __int_as_float(0x7fc00000) : p.x, p.y);
         } else {
-            const float4 p = sweep_warp<T, PATH_TARGET, U>(make_row(row, P.V), lo, lo + P.per_warp, scale, sh_m0);
+            const float4 p = ws.template run<PATH_TARGET>(m0, scale);
             v = make_float2(p.x, p.y);
         }
         if (lane == 0) SPECKV_ST(spans[s * kWarps + warp], v);

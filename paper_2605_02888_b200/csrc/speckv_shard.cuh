@@ -35,26 +35,27 @@ __global__ void __launch_bounds__(kThreads, kSweepCtasPerSm) shard_rows_kernel(c
     const bool active = row_ok && (is_target ? pos <= gam : pos < gam);
     float4 st = make_float4(0.f, 0.f, 0.f, 0.f);
     if (active) {
-        if (is_target) {
-            const T* row = static_cast<const T*>(P.t) + static_cast<long long>(b) * P.tsb + static_cast<long long>(pos) * P.tsp;
-            if (greedy) {
-                st = sweep_warp<T, PATH_ARGMAX, U, false>(make_row(row, P.V), 0, 0x7fffffff, scale, nullptr);
-                const int idx = __float_as_int(st.y);
-                if (idx != 0x7fffffff) st.y = __int_as_float(idx + P.v_begin);
-            } else {
-                st = sweep_warp<T, PATH_TARGET, U, false>(make_row(row, P.V), 0, 0x7fffffff, scale, nullptr);
+        const T* row = is_target ? static_cast<const T*>(P.t) + static_cast<long long>(b) * P.tsb + static_cast<long long>(pos) * P.tsp
+                                 : static_cast<const T*>(P.d) + static_cast<long long>(b) * P.dsb + static_cast<long long>(pos) * P.dsp;
+        WarpSweep<T, U> ws;
+        ws.start(make_row(row, P.V), 0, 0x7fffffff);
+        if (!is_target && lane == 0 && !greedy) {
+            // both logits at the draft token, if it falls into this slice
+            const int x = __ldg(P.tok + static_cast<long long>(b) * P.G + pos) - P.v_begin;
+            if (x >= 0 && x < P.V) {
+                const T* trow = static_cast<const T*>(P.t) + static_cast<long long>(b) * P.tsb + static_cast<long long>(pos) * P.tsp;
+                SPECKV_ST(P.tokl[static_cast<long long>(b) * P.G + pos], make_float2(elem_to_float(row, x), elem_to_float(trow, x)));
             }
+        }
+        const float m0 = ws.template warm<false>(nullptr);
+        if (!is_target) {
+            st = ws.template run<PATH_DRAFT>(m0, scale);
+        } else if (greedy) {
+            st = ws.template run<PATH_ARGMAX>(m0, scale);
+            const int idx = __float_as_int(st.y);
+            if (idx != 0x7fffffff) st.y = __int_as_float(idx + P.v_begin);
         } else {
-            const T* row = static_cast<const T*>(P.d) + static_cast<long long>(b) * P.dsb + static_cast<long long>(pos) * P.dsp;
-            if (lane == 0 && !greedy) {
-                // both logits at the draft token, if it falls into this slice
-                const int x = __ldg(P.tok + static_cast<long long>(b) * P.G + pos) - P.v_begin;
-                if (x >= 0 && x < P.V) {
-                    const T* trow = static_cast<const T*>(P.t) + static_cast<long long>(b) * P.tsb + static_cast<long long>(pos) * P.tsp;
-                    SPECKV_ST(P.tokl[static_cast<long long>(b) * P.G + pos], make_float2(elem_to_float(row, x), elem_to_float(trow, x)));
-                }
-            }
-            st = sweep_warp<T, PATH_DRAFT, U, false>(make_row(row, P.V), 0, 0x7fffffff, scale, nullptr);
+            st = ws.template run<PATH_TARGET>(m0, scale);
         }
     }
     if (lane == 0) P.state[static_cast<long long>(b) * P.J + j] = st;

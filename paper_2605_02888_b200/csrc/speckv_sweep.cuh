@@ -48,19 +48,123 @@ __device__ __noinline__ void row_epilogue_cta(const KParams& P, int b, int gam, 
 }
 
 // ----------------------------------------------------------------------------------------
-// Sweep kernel.  CTAs 0 .. n_sweep-1 sweep one slice of one logit row each.  With verification the
-// grid may carry B*R more CTAs behind them that draw the fresh tokens of rejected rows in the same launch:
+// What the sweep has to know before it starts: cleared counters and the list of the logit rows to sweep in grid order.  The
+// grid has CTAs for every position up to gamma_max, and gamma lives in device memory; with the list the CTAs that have work
+// come first and the surplus goes to the draws.  (One CTA per stored position, leaving again when gamma said so, cost
+// 1.8 us of a CTA slot each: 20 us of a step of 1,024 rows that use half of their positions.)
+// Grid: a segment of batch rows per CTA; every CTA reads all rows' gamma and temperature for the prefix.
+// ----------------------------------------------------------------------------------------
+enum : int { ENTRY_FLAGGED = 256 };  // entry: (batch row, row index j | generation << 6 | ENTRY_FLAGGED | gamma << 16)
+struct PrepCounts {
+    int a0, a1, b, c;  // entries of position 0 and position 1 of the first generation, of the second and the third generation
+    __device__ __forceinline__ void add(const PrepCounts& o) { a0 += o.a0; a1 += o.a1; b += o.b; c += o.c; }
+};
+__device__ __forceinline__ PrepCounts prep_counts(const KParams& P, int gam, float Tf) {
+    const int k1 = P.early ? P.k_early + 1 : 0;
+    PrepCounts r{0, 0, 0, 0};
+    if (row_status0(P, gam, Tf)) {  // one entry, for the row epilogue
+        if (k1) r.a0 = 1; else r.b = 1;
+        return r;
+    }
+    const bool verify = (P.mode & MODE_VERIFY) != 0;
+    if (k1 >= 1) r.a0 = 2;
+    if (k1 >= 2) r.a1 = 1 + (gam >= 2 ? 1 : 0);
+    r.b = max(gam - k1, 0);
+    if (verify) r.c = max(gam + 1 - k1, 0);
+    return r;
+}
+__device__ __forceinline__ PrepCounts shfl_up(const PrepCounts& v, int o) {
+    return {__shfl_up_sync(0xffffffffu, v.a0, o), __shfl_up_sync(0xffffffffu, v.a1, o), __shfl_up_sync(0xffffffffu, v.b, o),
+            __shfl_up_sync(0xffffffffu, v.c, o)};
+}
+__global__ void __launch_bounds__(kThreads) prep_kernel(const __grid_constant__ KParams P, int seg) {
+    __shared__ PrepCounts sh[2][kWarps];
+    asm volatile("griddepcontrol.launch_dependents;");  // the sweep's CTAs may be placed; they wait for this grid's end
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int b0 = blockIdx.x * seg, b1 = min(P.B, b0 + seg);
+    for (int b = b0 + threadIdx.x; b < b1; b += kThreads) {
+        P.tick1[b] = 0;
+        if (P.rdone) { P.tick2[b] = 0; P.rdone[b] = 0; }
+        if (P.early) { P.tick_early[b] = 0; P.early[b] = 0; }
+    }
+    PrepCounts before{0, 0, 0, 0}, total{0, 0, 0, 0};
+    for (int b = threadIdx.x; b < P.B; b += kThreads) {
+        const PrepCounts c = prep_counts(P, P.gamma ? P.gamma[b] : P.G, P.temp ? P.temp[b] : P.temp_scalar);
+        total.add(c);
+        if (b < b0) before.add(c);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const PrepCounts x = {__shfl_down_sync(0xffffffffu, before.a0, o), __shfl_down_sync(0xffffffffu, before.a1, o),
+                              __shfl_down_sync(0xffffffffu, before.b, o), __shfl_down_sync(0xffffffffu, before.c, o)};
+        const PrepCounts y = {__shfl_down_sync(0xffffffffu, total.a0, o), __shfl_down_sync(0xffffffffu, total.a1, o),
+                              __shfl_down_sync(0xffffffffu, total.b, o), __shfl_down_sync(0xffffffffu, total.c, o)};
+        before.add(x);
+        total.add(y);
+    }
+    if (lane == 0) { sh[0][warp] = before; sh[1][warp] = total; }
+    __syncthreads();
+    if (warp != 0) return;
+    before = total = PrepCounts{0, 0, 0, 0};
+    for (int w = 0; w < kWarps; ++w) { before.add(sh[0][w]); total.add(sh[1][w]); }
+    const int n_list = total.a0 + total.a1 + total.b + total.c;
+    if (blockIdx.x == 0 && lane == 0) {
+        *P.n_list = n_list;
+        *P.q_front = 0;
+        *P.q_back = 0;
+    }
+    const bool verify = (P.mode & MODE_VERIFY) != 0;
+    const int k1 = P.early ? P.k_early + 1 : 0;
+    // where the segment's first row starts in each generation
+    before.a1 += total.a0;
+    before.b += total.a0 + total.a1;
+    before.c += total.a0 + total.a1 + total.b;
+    for (int r0 = b0; r0 < b1; r0 += 32) {
+        const int b = r0 + lane;
+        PrepCounts c{0, 0, 0, 0};
+        int gam = 0;
+        bool flagged = false;
+        if (b < b1) {
+            gam = P.gamma ? P.gamma[b] : P.G;
+            const float Tf = P.temp ? P.temp[b] : P.temp_scalar;
+            flagged = row_status0(P, gam, Tf) != 0;
+            c = prep_counts(P, gam, Tf);
+        }
+        PrepCounts at = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const PrepCounts v = shfl_up(at, o);
+            if (lane >= o) at.add(v);
+        }
+        const PrepCounts last = {__shfl_sync(0xffffffffu, at.a0, 31), __shfl_sync(0xffffffffu, at.a1, 31), __shfl_sync(0xffffffffu, at.b, 31),
+                                 __shfl_sync(0xffffffffu, at.c, 31)};
+        at.a0 += before.a0 - c.a0; at.a1 += before.a1 - c.a1; at.b += before.b - c.b; at.c += before.c - c.c;
+        before.add(last);
+        if (b >= b1) continue;
+        auto put = [&](int i, int j, int gen) { SPECKV_ST(P.list[i], make_int2(b, j | gen << 6 | (gam & 31) << 16)); };
+        if (flagged) {
+            SPECKV_ST(P.list[k1 ? at.a0 : at.b], make_int2(b, ENTRY_FLAGGED));
+            continue;
+        }
+        const int jd = verify ? P.G + 1 : 0;  // row index of draft position 0
+        if (k1 >= 1) { put(at.a0, 0, 0); put(at.a0 + 1, jd, 0); }
+        if (k1 >= 2) { put(at.a1, 1, 0); if (gam >= 2) put(at.a1 + 1, jd + 1, 0); }
+        for (int p = k1; p < gam; ++p) put(at.b + p - k1, jd + p, 1);
+        if (verify)
+            for (int p = k1; p <= gam; ++p) put(at.c + p - k1, p, 2);
+    }
+}
+
+// ----------------------------------------------------------------------------------------
+// Sweep kernel.  CTA i sweeps slice i % nsplit of the logit row in list entry i / nsplit.  With verification the
+// grid carries more CTAs behind them that draw the fresh tokens of rejected rows in the same launch:
 // CTAs start in index order, so these start exactly when the sweep runs out of slices, wait (with
-// a bound) for their batch row's completion flag and fill the SMs that the sweep's last CTAs
+// a bound) for a row of the draw queue and fill the SMs that the sweep's last CTAs
 // leave one by one.  A second launch, even a programmatic dependent one, starts microseconds
 // after the last sweep CTA has started and leaves most of the drain unused.
 // ----------------------------------------------------------------------------------------
 template <typename T, int U>
 __global__ void __launch_bounds__(kThreads, kSweepCtasPerSm) sweep_kernel(const __grid_constant__ KParams P) {
-    if (static_cast<int>(blockIdx.x) >= P.n_sweep) {
-        resample_body<T>(P, static_cast<int>(blockIdx.x) - P.n_sweep);
-        return;
-    }
     __shared__ float4 sh_part[kWarps];
     __shared__ RowDecide sh_pos[kMaxGamma + 1];
     __shared__ DrawSrc sh_src;
@@ -68,115 +172,93 @@ __global__ void __launch_bounds__(kThreads, kSweepCtasPerSm) sweep_kernel(const 
     __shared__ int sh_last;
     __shared__ int sh_early;
     __shared__ float sh_m0[kWarps];
-    asm volatile("griddepcontrol.launch_dependents;");  // a dependent resample kernel may be scheduled as SMs free up
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // the list and the cleared counters
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool verify = (P.mode & MODE_VERIFY) != 0;
-    int b, j, s, gen = 0;
-    if (P.early) {
-        // generation order: CTAs start in index order, so a later generation starts when the earlier ones
-        // are all under way and, for all but the smallest batches, long after the first one has finished
-        const int ns = P.nsplit, k1 = P.k_early + 1;
-        const int nA = k1 * P.B * 2 * ns, nB = (P.G - k1) * P.B * ns;
-        int i = blockIdx.x, p, is_draft;
-        if (i < nA) {
-            p = i / (2 * P.B * ns); i -= p * (2 * P.B * ns);
-            b = i / (2 * ns); i -= b * (2 * ns);
-            is_draft = i / ns; s = i - is_draft * ns;
-        } else {
-            // the later generations go batch row by batch row, so that the rows complete one after another
-            gen = (i < nA + nB) ? 1 : 2;
-            i -= (gen == 1) ? nA : nA + nB;
-            const int per_b = (gen == 1 ? P.G - k1 : P.G + 1 - k1) * ns;
-            b = i / per_b; i -= b * per_b;
-            p = i / ns; s = i - p * ns;
-            p += k1;
-            is_draft = (gen == 1);
-        }
-        j = is_draft ? P.G + 1 + p : p;
-    } else {
-        const int per_row = P.J * P.nsplit;
-        b = blockIdx.x / per_row;
-        const int r = blockIdx.x - b * per_row;
-        j = r / P.nsplit;
-        s = r - j * P.nsplit;
+    const int i = static_cast<int>(blockIdx.x) / P.nsplit, s = static_cast<int>(blockIdx.x) - i * P.nsplit;
+    int2 entry = make_int2(0, 0);
+    if (i < P.B * P.J && dbg_ok(P.list + i, 8, DBG_WS_LOAD)) entry = __ldcg(P.list + i);
+    const int n_list = __ldcg(P.n_list);
+    if (i >= n_list) {
+        const int d = static_cast<int>(blockIdx.x) - n_list * P.nsplit;
+        if (d < P.n_draw) resample_body<T>(P, d);
+        return;
     }
-    // the row's gamma and temperature travel together with the one thing a CTA of the last generation has
-    // to learn first: one memory round trip before the CTA knows whether it has work
-    int gam = P.gamma ? P.gamma[b] : P.G;
-    float Tf = P.temp ? P.temp[b] : P.temp_scalar;
-    if (threadIdx.x == 0) {
-        // one thread reads what is known of the row's stop position, so that the whole CTA takes one decision
-        int e = 0;
-        if (gen == 2 && !P.read_all)
-            asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(e) : "l"(P.early + b) : "memory");
-        sh_early = e;
-    }
-    if (threadIdx.x < kWarps) sh_m0[threadIdx.x] = kFloor;
-    __syncthreads();  // before any load is issued
-    const int rem = j * P.nsplit + s;
-
-    const bool row_ok = (gam >= 1 && gam <= P.G) && (Tf >= 0.f) && (Tf != __int_as_float(0x7f800000));
-    const bool greedy = (Tf == 0.f);
-    const float scale = static_cast<float>(kLog2e / static_cast<double>(greedy ? 1.f : Tf));
-
-    // logit row handled by this CTA: with verification, j <= G are target positions and the
-    // rest draft positions; signals alone sweep draft positions only
-    const bool is_target = verify && j <= P.G;
+    const int b = entry.x, j = entry.y & 63, gen = (entry.y >> 6) & 3;
+    const bool row_ok = !(entry.y & ENTRY_FLAGGED);
+    const bool is_target = verify && j <= P.G;  // target positions come first in a batch row's numbering
     const int pos = is_target ? j : (verify ? j - (P.G + 1) : j);
-    const bool active = row_ok && (is_target ? pos <= gam : pos < gam);
-    const long long pidx = (static_cast<long long>(b) * P.J + j) * P.nsplit + s;  // this CTA's partial
-
-    // the walk stopped at a position before this one
-    const bool skipped = active && gen == 2 && sh_early != 0 && sh_early <= P.k_early + 1;
-    if (skipped) {
-        // the row epilogue never looks behind the stop position; the partial only has to be finite
-        if (threadIdx.x == 0)
-            SPECKV_ST(P.part[pidx], greedy ? make_float4(kFloor, __int_as_float(0x7fffffff), 0.f, 0.f)
-                                           : make_float4(kFloor, 0.f, 0.f, 0.f));
-    } else if (active) {
-        // this warp's granules: the CTA's slice is cut into one contiguous range per warp
-        const int lo = (s * kWarps + warp) * P.per_warp, hi = lo + P.per_warp;
-        float4 part;
-        int path;
-        if (is_target) {
-            const T* row = static_cast<const T*>(P.t) + static_cast<long long>(b) * P.tsb +
-                           static_cast<long long>(pos) * P.tsp;
-            if (greedy) { part = sweep_warp<T, PATH_ARGMAX, U>(make_row(row, P.V), lo, hi, scale, sh_m0); path = PATH_ARGMAX; }
-            else { part = sweep_warp<T, PATH_TARGET, U>(make_row(row, P.V), lo, hi, scale, sh_m0); path = PATH_TARGET; }
-            // the position a bonus token would be drawn from: this warp's sum is a span of that draw
-            if (P.spans && pos == gam && !greedy && lane == 0)
-                SPECKV_ST(P.spans[(static_cast<long long>(b) * P.nsplit + s) * kWarps + warp], make_float2(part.x, part.y));
+    int gam = entry.y >> 16;
+    float Tf;
+    if (row_ok) {
+        // the first logits are requested before anything else about the row is known
+        const T* row = is_target ? static_cast<const T*>(P.t) + static_cast<long long>(b) * P.tsb + static_cast<long long>(pos) * P.tsp
+                                 : static_cast<const T*>(P.d) + static_cast<long long>(b) * P.dsb + static_cast<long long>(pos) * P.dsp;
+        const int lo = (s * kWarps + warp) * P.per_warp;  // this warp's granules: the CTA's slice is cut into one contiguous range per warp
+        WarpSweep<T, U> ws;
+        ws.start(make_row(row, P.V), lo, lo + P.per_warp);
+        Tf = P.temp ? __ldg(P.temp + b) : P.temp_scalar;
+        if (threadIdx.x == 0) {
+            // one thread reads what is known of the row's stop position, so that the whole CTA takes one decision
+            int e = 0;
+            if (P.early && gen == 2 && !P.read_all)
+                asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(e) : "l"(P.early + b) : "memory");
+            sh_early = e;
+        }
+        const float m0 = ws.template warm<true>(sh_m0);
+        const bool greedy = (Tf == 0.f);
+        const float scale = static_cast<float>(kLog2e / static_cast<double>(greedy ? 1.f : Tf));
+        const long long pidx = (static_cast<long long>(b) * P.J + j) * P.nsplit + s;  // this CTA's partial
+        if (gen == 2 && sh_early != 0 && sh_early <= P.k_early + 1) {
+            // The walk stopped at a position before this one: the row epilogue never looks here, the partial only has to
+            // be finite.
+            if (threadIdx.x == 0)
+                SPECKV_ST(P.part[pidx], greedy ? make_float4(kFloor, __int_as_float(0x7fffffff), 0.f, 0.f)
+                                               : make_float4(kFloor, 0.f, 0.f, 0.f));
         } else {
-            const T* row = static_cast<const T*>(P.d) + static_cast<long long>(b) * P.dsb +
-                           static_cast<long long>(pos) * P.dsp;
-            if (verify && P.tokl && s == 0 && threadIdx.x == 0 && !greedy) {
-                // the acceptance test of this position needs both logits at the draft token: fetch them
-                // now, while the sweep hides the latency, and leave them for the row epilogue
-                const int x = __ldg(P.tok + static_cast<long long>(b) * P.G + pos) - P.v_begin;  // index in this slice
-                if (x >= 0 && x < P.V) {
-                    const T* trow = static_cast<const T*>(P.t) + static_cast<long long>(b) * P.tsb +
-                                    static_cast<long long>(pos) * P.tsp;
-                    SPECKV_ST(P.tokl[static_cast<long long>(b) * P.G + pos], make_float2(elem_to_float(row, x), elem_to_float(trow, x)));
+            float4 part;
+            int path;
+            if (!is_target) {
+                if (verify && P.tokl && s == 0 && threadIdx.x == 0 && !greedy) {
+                    // the acceptance test of this position needs both logits at the draft token: fetch them
+                    // now, while the sweep hides the latency, and leave them for the row epilogue
+                    const int x = __ldg(P.tok + static_cast<long long>(b) * P.G + pos) - P.v_begin;  // index in this slice
+                    if (x >= 0 && x < P.V) {
+                        const T* trow = static_cast<const T*>(P.t) + static_cast<long long>(b) * P.tsb +
+                                        static_cast<long long>(pos) * P.tsp;
+                        SPECKV_ST(P.tokl[static_cast<long long>(b) * P.G + pos], make_float2(elem_to_float(row, x), elem_to_float(trow, x)));
+                    }
                 }
+                part = ws.template run<PATH_DRAFT>(m0, scale);
+                path = PATH_DRAFT;
+            } else if (greedy) {
+                part = ws.template run<PATH_ARGMAX>(m0, scale);
+                path = PATH_ARGMAX;
+            } else {
+                part = ws.template run<PATH_TARGET>(m0, scale);
+                path = PATH_TARGET;
+                // the position a bonus token would be drawn from: this warp's sum is a span of that draw
+                if (P.spans && pos == gam && lane == 0)
+                    SPECKV_ST(P.spans[(static_cast<long long>(b) * P.nsplit + s) * kWarps + warp], make_float2(part.x, part.y));
             }
-            part = sweep_warp<T, PATH_DRAFT, U>(make_row(row, P.V), lo, hi, scale, sh_m0);
-            path = PATH_DRAFT;
+            if (lane == 0) sh_part[warp] = part;
+            __syncthreads();
+            if (warp == 0) {
+                const float4 none = (path == PATH_ARGMAX) ? make_float4(kFloor, __int_as_float(0x7fffffff), 0.f, 0.f)
+                                  : make_float4(path == PATH_TARGET ? -3.0e38f : kFloor, 0.f, 0.f, 0.f);
+                const float4 w = lane < kWarps ? sh_part[lane] : none;
+                const float4 acc = (path == PATH_DRAFT) ? warp_merge<PATH_DRAFT>(w, scale)
+                                 : (path == PATH_TARGET) ? warp_merge<PATH_TARGET>(w, scale) : warp_merge<PATH_ARGMAX>(w, scale);
+                if (lane == 0) SPECKV_ST(P.part[pidx], acc);
+            }
         }
-        if (lane == 0) sh_part[warp] = part;
-        __syncthreads();
-        if (warp == 0) {
-            const float4 none = (path == PATH_ARGMAX) ? make_float4(kFloor, __int_as_float(0x7fffffff), 0.f, 0.f)
-                              : make_float4(path == PATH_TARGET ? -3.0e38f : kFloor, 0.f, 0.f, 0.f);
-            const float4 w = lane < kWarps ? sh_part[lane] : none;
-            const float4 acc = (path == PATH_DRAFT) ? warp_merge<PATH_DRAFT>(w, scale)
-                             : (path == PATH_TARGET) ? warp_merge<PATH_TARGET>(w, scale) : warp_merge<PATH_ARGMAX>(w, scale);
-            if (lane == 0) SPECKV_ST(P.part[pidx], acc);
-        }
-    } else if (row_ok || rem != 0) {
-        return;  // unused position: nothing to count; a flagged row keeps its first CTA for the epilogue
+    } else {
+        if (s != 0) return;  // a flagged row has one CTA, for the epilogue
+        gam = P.gamma ? P.gamma[b] : P.G;
+        Tf = P.temp ? P.temp[b] : P.temp_scalar;
     }
 
-    // tickets: the last of the row's CTAs of positions 0..k_early takes their acceptance tests, the last of all its active
+    // tickets: the last of the row's CTAs of positions 0..k_early takes their acceptance tests, the last of all its
     // CTAs runs the row epilogue; nobody waits
     if (threadIdx.x == 0) {
         const int n_rows = verify ? 2 * gam + 1 : gam;
@@ -184,7 +266,7 @@ __global__ void __launch_bounds__(kThreads, kSweepCtasPerSm) sweep_kernel(const 
         const int n_pre = (min(P.k_early, gam) + 1 + min(P.k_early + 1, gam)) * P.nsplit;
         __threadfence();
         int pre = -1;
-        if (P.early && active && gen == 0) pre = atomicAdd(P.tick_early + b, 1);
+        if (P.early && row_ok && gen == 0) pre = atomicAdd(P.tick_early + b, 1);
         const int all = atomicAdd(P.tick1 + b, 1);
         const int l = (all == n_tickets - 1 ? 2 : 0) | (pre == n_pre - 1 ? 1 : 0);
         if (l) __threadfence();
