@@ -97,19 +97,20 @@ void choose_slices(KParams& P, speckv_dtype dt, bool aligned) {
 }
 
 constexpr int kEarlyPositions = 2;   // positions whose acceptance tests the sliced sweep takes ahead of the rest of the row
-constexpr int kDrawElems = 16384;    // elements of the stop position that one CTA of a draw sums
-constexpr int kDrawSmallCtas = 1184; // CTAs of a draw wanted in flight for a small batch (two per CTA slot)
-
-// CTAs per draw and granules per warp: P.R, P.draw_pw.
+// CTAs per draw and granules per warp: P.R, P.draw_pw.  16,384 elements per CTA; a small batch spreads over the CTA slots
+// (1.6 times), and many rows (of which about a third draw) share 4,096 CTAs rather than pay a CTA's start and end for every
+// 16,384 elements.  (V = 128,256, bf16, 4 / 8 / 16 / 32 CTAs per draw: step of 1,024 rows 399 / 408 / 427 / 462 us, of 256
+// rows 141 / 138 / 138 / 141.)
+constexpr int kDrawElems = 16384, kDrawSmallCtas = 1184, kDrawMostCtas = 4096;
 void choose_draw(KParams& P, speckv_dtype dt, bool aligned) {
     const int E = 16 / esize(dt);
     const int ng = (P.V + E - 1 + (aligned ? 0 : E - 1)) / E;
     int R = (P.V + kDrawElems - 1) / kDrawElems;
-    // small batches: more, shorter shares per row, so that the draw of a handful of rows still spreads over the SMs
     const int want = (kDrawSmallCtas + P.B - 1) / P.B, cap = (ng + 32 * kWarps - 1) / (32 * kWarps);  // one granule per lane at least
+    const int most = kDrawMostCtas / P.B, least = (P.V + 4 * kDrawElems - 1) / (4 * kDrawElems);
     if (want > R) R = want < cap ? want : cap > R ? cap : R;
+    else if (R > most) R = most > least ? most : least;
     if (R > kMaxShares) R = kMaxShares;
-    if (R < 1) R = 1;
     P.draw_pw = ((ng + R * kWarps - 1) / (R * kWarps) + 7) / 8 * 8;
     P.R = (ng + P.draw_pw * kWarps - 1) / (P.draw_pw * kWarps);
 }
@@ -526,7 +527,7 @@ __global__ void wait_probe_late_epilogue(KParams P) {
     if (b >= P.B) return;
     if ((threadIdx.x & 31) == 0) P.status[b] = 0;
     __syncwarp();
-    row_done_signal(P, b, RS_BONUS, 1);
+    row_done_signal(P, b, row_done_slot(P, RS_BONUS), RS_BONUS, 1);
 }
 
 }  // namespace

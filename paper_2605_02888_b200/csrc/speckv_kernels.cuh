@@ -834,15 +834,16 @@ __device__ __forceinline__ double log2_split(double z) { return log2(z); }
 // batch row: it starts on the first finished row whatever its number, and the groups that find nothing to draw come last
 // (by batch row, 1,024 rows of which a third draw spent 9 us of all CTA slots on groups with nothing to do).
 constexpr int kSlotDone = 1 << 30, kSlotTimeout = 1 << 31;  // bits 0-23: batch row, 24: a residual draw, 25-28: stop position
-__device__ __forceinline__ void row_done_signal(const KParams& P, int b, int mode, int n) {
+__device__ __forceinline__ int row_done_slot(const KParams& P, int mode) {  // whole warp; lane 0 has the answer
+    if (!P.rdone || (threadIdx.x & 31) != 0) return 0;
+    return mode == RS_RESIDUAL ? atomicAdd(P.q_front, 1) : P.B - 1 - atomicAdd(P.q_back, 1);
+}
+__device__ __forceinline__ void row_done_signal(const KParams& P, int b, int slot, int mode, int n) {
     if (!P.rdone) return;
-    const bool draw = mode == RS_RESIDUAL;
-    int slot = 0;
-    if ((threadIdx.x & 31) == 0) slot = draw ? atomicAdd(P.q_front, 1) : P.B - 1 - atomicAdd(P.q_back, 1);
     __threadfence();
     __syncwarp();
     if ((threadIdx.x & 31) == 0) {
-        const int old = atomicOr(P.rdone + slot, kSlotDone | b | (draw ? 1 << 24 | n << 25 : 0));
+        const int old = atomicOr(P.rdone + slot, kSlotDone | b | (mode == RS_RESIDUAL ? 1 << 24 | n << 25 : 0));
         // a group whose bounded wait ran out before this point left its mark here: the row's fresh
         // token will never be drawn, and the status written above must say so
         if ((old & kSlotTimeout) && P.status) atomicOr(P.status + b, 16);
@@ -979,29 +980,35 @@ __device__ __noinline__ void row_decide(const KParams& P, int b, int gam, float 
     o.dbad = dbad; o.tbad = tbad; o.badtok = badtok; o.accept = accept;
 }
 
-// The same for one position by one warp of a CTA that has all its warps at hand (the sliced sweep): lanes 0-15 gather
-// the draft row's partials, lanes 16-31 the target row's, so that up to 32 slices cost one memory round trip and four
-// shuffle steps instead of a chain of them, and one double-precision log2 serves draft row, target row and uniform.
+// The same by the warps of a CTA (the sliced sweep): a group of 32 lanes (16 where a logit row has at most 16 partials)
+// decides one position, the lower half gathering the draft row's partials and the upper half the target row's, so that
+// they cost one memory round trip and a few shuffle steps instead of a chain of them, and one double-precision log2 serves
+// draft row, target row and uniform.
 // Latency-bound: one batch row in 15 slices (fp32, V = 32,000, gamma 4), with a lane per position the prefix and the row
 // epilogue each walked a chain of 11 dependent round trips and the step took 45.1 us; this way 23.0 us.  256 rows of
-// bf16, V = 128,256: 150.5 -> 145.6 us (the chain is also the end of a large step).  The prefix epilogue and the row epilogue call this one compiled body, so that both reach the same bits.
+// bf16, V = 128,256: 150.5 -> 145.6 us (the chain is also the end of a large step).  The prefix epilogue and the row
+// epilogue call this one compiled body, so that both reach the same bits.
+// Decides positions first, first + 1 (16 lanes each) or first alone; P.part holds n = nsplit partials per logit row.
 template <typename T>
-__device__ __noinline__ void decide_position(const KParams& P, int b, int gam, float Tf, int i, const float4* pd,
-                                             const float4* pt, int n, RowDecide& o) {
-    const int lane = threadIdx.x & 31, k = lane & 15;
-    const bool tgt_half = lane >= 16;
+__device__ __noinline__ void decide_positions(const KParams& P, int b, int gam, bool greedy, float scale, int first, int n_pos,
+                                              RowDecide* out) {
+    const int lane = threadIdx.x & 31, n = P.nsplit;
+    const int half = n <= 16 ? 8 : 16;  // lanes per logit row, at most two partials each
+    const int k = lane & (half - 1), lead = lane & ~(2 * half - 1);  // lane within the row, first lane of the group
+    const bool tgt_half = (lane & half) != 0;
     const bool verify = (P.mode & MODE_VERIFY) != 0;
-    const bool greedy = (Tf == 0.f);
-    const float scale = static_cast<float>(kLog2e / static_cast<double>(greedy ? 1.f : Tf));
-    const bool dr_on = i < gam, tok_on = verify && i < gam;
+    const int i = first + (lane >= 2 * half ? 1 : 0);
+    const bool in = i < n_pos;
+    const bool dr_on = in && i < gam, tok_on = dr_on && verify;
 
     // ---- one round trip ----
-    const bool on = tgt_half ? verify : dr_on;
-    const float4* src = tgt_half ? pt : pd;
+    const bool on = tgt_half ? in && verify : dr_on;
+    const float4* src = P.part + (static_cast<long long>(b) * P.J + (tgt_half || !verify ? i : P.G + 1 + i)) * n;
     const float4 none = tgt_half && greedy ? make_float4(kFloor, __int_as_float(0x7fffffff), 0.f, 0.f)
                                            : make_float4(tgt_half ? -3.0e38f : kFloor, 0.f, 0.f, 0.f);
-    float4 a = (on && k < n) ? ldcg4(src + k) : none;
-    const float4 a2 = (on && k + 16 < n) ? ldcg4(src + k + 16) : none;
+    float4 a = none, a2 = none;
+    if (on && k < n) a = ldcg4(src + k);
+    if (on && k + half < n) a2 = ldcg4(src + k + half);
     int x = -1;
     float u_acc = 0.f, u_res = 0.f;
     float2 tl = make_float2(0.f, 0.f);
@@ -1013,32 +1020,27 @@ __device__ __noinline__ void decide_position(const KParams& P, int b, int gam, f
             u_acc = __ldg(P.u + urow);
             if (!greedy) tl = __ldcg(P.tokl + at);  // left by the sweep CTA of the draft position
         }
-        if (verify) u_res = __ldg(P.u + urow + 1);
+        if (in && verify) u_res = __ldg(P.u + urow + 1);
     }
 
     int amax = -1;
     bool tbad = false;
-    if (greedy && verify) {  // uniform across the warp; the draft half goes along and is not looked at
+    if (greedy && verify) {  // uniform across the warp; the draft lanes go along and are not looked at
         float4 g = merge_argmax(a, a2);
-#pragma unroll
-        for (int m = 8; m > 0; m >>= 1) g = merge_argmax(g, shfl_xor4(g, m));
-        amax = __shfl_sync(0xffffffffu, __float_as_int(g.y), 16);
-        const float best = __shfl_sync(0xffffffffu, g.x, 16), bad = __shfl_sync(0xffffffffu, g.z, 16);
+        for (int m = half >> 1; m > 0; m >>= 1) g = merge_argmax(g, shfl_xor4(g, m));
+        amax = __shfl_sync(0xffffffffu, __float_as_int(g.y), lead + half);
+        const float best = __shfl_sync(0xffffffffu, g.x, lead + half), bad = __shfl_sync(0xffffffffu, g.z, lead + half);
         tbad = bad != 0.f || amax == 0x7fffffff || !(best > kFloor);
     }
     // draft partial: (m, cnt, Zx, S); target partial (r, Z): both as (reference, cnt, Z, S) with the reference in log2 units
-    // for the target half
+    // for the target lanes
     const float sc = tgt_half ? 1.f : scale;
     if (tgt_half) {
         a.z = a.y; a.y = 0.f; a.w = 0.f;
+        a2.z = a2.y; a2.y = 0.f; a2.w = 0.f;
     }
-    float4 c2 = a2;
-    if (tgt_half) {
-        c2.z = c2.y; c2.y = 0.f; c2.w = 0.f;
-    }
-    float M = fmaxf(a.x, c2.x);
-#pragma unroll
-    for (int m = 8; m > 0; m >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, m));
+    float M = fmaxf(a.x, a2.x);
+    for (int m = half >> 1; m > 0; m >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, m));
     float cnt = 0.f, Z = 0.f, S = 0.f;
     auto add = [&](const float4& v) {
         const float dm = v.x - M, f = ex2f(dm * sc), za = v.y + v.z;
@@ -1048,19 +1050,19 @@ __device__ __noinline__ void decide_position(const KParams& P, int b, int gam, f
         S += top ? v.w : fmaf(dm, za, v.w) * f;
     };
     add(a);
-    add(c2);
-#pragma unroll
-    for (int m = 8; m > 0; m >>= 1) {
+    add(a2);
+    for (int m = half >> 1; m > 0; m >>= 1) {
         cnt += __shfl_xor_sync(0xffffffffu, cnt, m);
         Z += __shfl_xor_sync(0xffffffffu, Z, m);
         S += __shfl_xor_sync(0xffffffffu, S, m);
     }
-    // lane 0: draft normaliser, lane 16: target normaliser, lane 8: accept uniform (lane 8 sees the draft sums)
-    const double arg = lane == 8 ? static_cast<double>(u_acc) : static_cast<double>(cnt) + static_cast<double>(Z);
+    // the group's first lane: draft normaliser, first target lane: target normaliser, a lane between them: accept uniform
+    const int u_lane = lead + (half >> 1);
+    const double arg = lane == u_lane ? static_cast<double>(u_acc) : static_cast<double>(cnt) + static_cast<double>(Z);
     const double l2 = log2_split(arg);
-    const double l2_p = __shfl_sync(0xffffffffu, l2, 16), l2_u = __shfl_sync(0xffffffffu, l2, 8);
-    const float Rp = __shfl_sync(0xffffffffu, M, 16), Zp = __shfl_sync(0xffffffffu, Z, 16);
-    if (lane != 0) return;
+    const double l2_p = __shfl_sync(0xffffffffu, l2, lead + half), l2_u = __shfl_sync(0xffffffffu, l2, u_lane);
+    const float Rp = __shfl_sync(0xffffffffu, M, lead + half), Zp = __shfl_sync(0xffffffffu, Z, lead + half);
+    if (lane != lead || !in) return;
 
     float Hi = 0.f, ci = 0.f;
     double lse2_q = 0.0, lse2_p = 0.0;
@@ -1091,8 +1093,16 @@ __device__ __noinline__ void decide_position(const KParams& P, int b, int gam, f
             accept = (l2_u + lq) < lp;  // u * q(x) < p(x); u = 0: log2 is -inf
         }
     }
+    RowDecide& o = out[i];
     o.x = x; o.u_res = u_res; o.Hi = Hi; o.ci = ci; o.lse2_q = lse2_q; o.lse2_p = lse2_p; o.amax = amax;
     o.dbad = dbad; o.tbad = tbad; o.badtok = badtok; o.accept = accept;
+}
+// Positions 0..n_pos-1 by all warps of the CTA; the caller synchronises.  Warp 0 has the fewest.
+template <typename T>
+__device__ __forceinline__ void decide_all(const KParams& P, int b, int gam, bool greedy, float scale, int n_pos, RowDecide* pos) {
+    const int per = P.nsplit <= 16 ? 2 : 1;
+    for (int i = (kWarps - 1 - static_cast<int>(threadIdx.x >> 5)) * per; i < n_pos; i += kWarps * per)
+        decide_positions<T>(P, b, gam, greedy, scale, i, n_pos, pos);
 }
 
 // Prefix epilogue (a whole CTA): run when the partials of a batch row's first positions 0..k are in, while
@@ -1100,12 +1110,9 @@ __device__ __noinline__ void decide_position(const KParams& P, int b, int gam, f
 // publishes where the walk stops if it stops there, so that CTAs which have not started yet can leave
 // target rows behind that position unread.  early[b] = stop position + 1, or G + 2 when the walk passes k.
 template <typename T>
-__device__ __noinline__ void prefix_epilogue(const KParams& P, int b, int gam, float Tf, RowDecide* pos) {
+__device__ __noinline__ void prefix_epilogue(const KParams& P, int b, int gam, bool greedy, float scale, RowDecide* pos) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const long long row0 = static_cast<long long>(b) * P.J;
-    if (warp <= P.k_early && warp <= gam)
-        decide_position<T>(P, b, gam, Tf, warp, P.part + (row0 + P.G + 1 + warp) * P.nsplit, P.part + (row0 + warp) * P.nsplit,
-                           P.nsplit, pos[warp]);
+    decide_all<T>(P, b, gam, greedy, scale, min(P.k_early, gam) + 1, pos);
     __syncthreads();
     if (warp == 0) {
         bool ends = false;
@@ -1122,6 +1129,10 @@ __device__ __noinline__ void prefix_epilogue(const KParams& P, int b, int gam, f
     __syncthreads();  // pos is used again when the same CTA completes the row
 }
 
+// log2(e) / T, the factor of every exponent of a row (greedy rows: T = 1).
+__device__ __forceinline__ float row_scale(float Tf) {
+    return static_cast<float>(kLog2e / static_cast<double>(Tf == 0.f ? 1.f : Tf));
+}
 // Status bits a row's gamma and temperature give by themselves.
 __device__ __forceinline__ int row_status0(const KParams& P, int gam, float Tf) {
     return (gam < 1 || gam > P.G ? 1 : 0) | (!(Tf >= 0.f) || Tf == __int_as_float(0x7f800000) ? 8 : 0);
@@ -1150,7 +1161,7 @@ __device__ __forceinline__ int row_walk(const KParams& P, int gam, float Tf, con
 // What the walk decides (one warp): status, accepted count, tokens except a drawn one, the record a draw needs and the
 // row's completion flag.  own_bonus: a bonus token is drawn by the caller (from the sweep's spans), not by the CTAs
 // that wait for the flag.
-__device__ __noinline__ void finish_verify(const KParams& P, int b, int gam, float Tf, const RowDecide& dec, bool own_bonus) {
+__device__ __noinline__ void finish_verify(const KParams& P, int b, int gam, float Tf, float scale, const RowDecide& dec, bool own_bonus) {
     const int lane = threadIdx.x & 31;
     const int G = P.G;
     const bool verify = (P.mode & MODE_VERIFY) != 0;
@@ -1158,6 +1169,7 @@ __device__ __noinline__ void finish_verify(const KParams& P, int b, int gam, flo
     int n;
     const int status = row_walk(P, gam, Tf, dec, &n);
     const int rs_mode = (verify && status == 0 && !greedy) ? (n < gam ? RS_RESIDUAL : RS_BONUS) : RS_NONE;
+    const int slot = row_done_slot(P, rs_mode);  // travels while the outputs are written
     if (verify) {
         // fresh token: known here for greedy rows, drawn by the resample step otherwise
         const int amax_n = __shfl_sync(0xffffffffu, dec.amax, n);
@@ -1178,14 +1190,14 @@ __device__ __noinline__ void finish_verify(const KParams& P, int b, int gam, flo
             ri.mode = rs_mode;
             ri.n = n;
             ri.u2 = (status == 0 && !greedy) ? u2_n : 0.f;
-            ri.scale = static_cast<float>(kLog2e / static_cast<double>(greedy ? 1.f : Tf));
+            ri.scale = scale;
             ri.lse2_p = lp_n;
             ri.lse2_q = lq_n;
             SPECKV_ST(P.info[b], ri);
         }
     }
     if (P.status && lane == 0) P.status[b] = status;
-    row_done_signal(P, b, own_bonus && rs_mode == RS_BONUS ? RS_NONE : rs_mode, n);
+    row_done_signal(P, b, slot, rs_mode, n);
 }
 
 // The signals and the controller's outputs (one warp); ctl: the controller's parameters, fetched beforehand.
@@ -1237,7 +1249,7 @@ __device__ __noinline__ void row_epilogue(const KParams& P, int b, int gam, floa
     if ((P.mode & MODE_MLP) && !status) ctl = ctl_load(P, b, threadIdx.x & 31);
     RowDecide dec;
     row_decide<T>(P, b, gam, Tf, status, 32, pd, nd, pt, nt, dec);
-    finish_verify(P, b, gam, Tf, dec, false);
+    finish_verify(P, b, gam, Tf, row_scale(Tf), dec, false);
     finish_signals(P, b, gam, Tf, dec, ctl);
 }
 

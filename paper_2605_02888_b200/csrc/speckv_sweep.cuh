@@ -12,18 +12,15 @@ namespace speckv {
 // after the other in one warp this took 6.6 us behind the last partial of a lone row, this way 4 us less.
 constexpr int kDrawWarp0 = 2;
 template <typename T>
-__device__ __noinline__ void row_epilogue_cta(const KParams& P, int b, int gam, float Tf, RowDecide* pos, double* sh_sum,
+__device__ __noinline__ void row_epilogue_cta(const KParams& P, int b, int gam, float Tf, float scale, RowDecide* pos, double* sh_sum,
                                               DrawSrc* sh_src) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool verify = (P.mode & MODE_VERIFY) != 0;
-    const long long row0 = static_cast<long long>(b) * P.J;
     const int n_pos = row_status0(P, gam, Tf) ? 0 : verify ? gam + 1 : gam;
     // the parameters travel while the positions are decided; warps 0 and 1 take the last turns
     CtlRegs ctl;
     if (warp == 1 && (P.mode & MODE_MLP) && n_pos) ctl = ctl_load(P, b, lane);
-    for (int i = kWarps - 1 - warp; i < n_pos; i += kWarps)
-        decide_position<T>(P, b, gam, Tf, i, P.part + (row0 + (verify ? P.G + 1 + i : i)) * P.nsplit, P.part + (row0 + i) * P.nsplit,
-                           P.nsplit, pos[i]);
+    decide_all<T>(P, b, gam, Tf == 0.f, scale, n_pos, pos);
     __syncthreads();
     if (warp >= kDrawWarp0) {
         // a bonus draw: every position accepted, nothing flagged
@@ -32,7 +29,6 @@ __device__ __noinline__ void row_epilogue_cta(const KParams& P, int b, int gam, 
         if (lane < n_pos) ends = pos[lane].dbad || pos[lane].tbad || pos[lane].badtok || !pos[lane].accept;
         if (__any_sync(0xffffffffu, ends)) return;
         const T* row = static_cast<const T*>(P.t) + static_cast<long long>(b) * P.tsb + static_cast<long long>(gam) * P.tsp;
-        const float scale = static_cast<float>(kLog2e / static_cast<double>(Tf));
         const int n = P.nsplit * kWarps;
         const int tok = draw_from_spans<T>(row, P.V, scale, P.spans + static_cast<long long>(b) * n, n, P.per_warp, pos[gam].u_res,
                                            warp - kDrawWarp0, kWarps - kDrawWarp0, 1, sh_sum, sh_src);
@@ -43,7 +39,7 @@ __device__ __noinline__ void row_epilogue_cta(const KParams& P, int b, int gam, 
     dec.x = -1; dec.u_res = 0.f; dec.Hi = dec.ci = 0.f; dec.lse2_q = dec.lse2_p = 0.0; dec.amax = -1;
     dec.dbad = dec.tbad = dec.badtok = false; dec.accept = true;
     if (lane < n_pos) dec = pos[lane];
-    if (warp == 0) finish_verify(P, b, gam, Tf, dec, true);
+    if (warp == 0) finish_verify(P, b, gam, Tf, scale, dec, true);
     else if (P.mode & MODE_SIGNALS) finish_signals(P, b, gam, Tf, dec, ctl);
 }
 
@@ -189,7 +185,7 @@ __global__ void __launch_bounds__(kThreads, kSweepCtasPerSm) sweep_kernel(const 
     const bool is_target = verify && j <= P.G;  // target positions come first in a batch row's numbering
     const int pos = is_target ? j : (verify ? j - (P.G + 1) : j);
     int gam = entry.y >> 16;
-    float Tf;
+    float Tf, scale = 0.f;
     if (row_ok) {
         // the first logits are requested before anything else about the row is known
         const T* row = is_target ? static_cast<const T*>(P.t) + static_cast<long long>(b) * P.tsb + static_cast<long long>(pos) * P.tsp
@@ -207,7 +203,7 @@ __global__ void __launch_bounds__(kThreads, kSweepCtasPerSm) sweep_kernel(const 
         }
         const float m0 = ws.template warm<true>(sh_m0);
         const bool greedy = (Tf == 0.f);
-        const float scale = static_cast<float>(kLog2e / static_cast<double>(greedy ? 1.f : Tf));
+        scale = row_scale(Tf);
         const long long pidx = (static_cast<long long>(b) * P.J + j) * P.nsplit + s;  // this CTA's partial
         if (gen == 2 && sh_early != 0 && sh_early <= P.k_early + 1) {
             // The walk stopped at a position before this one: the row epilogue never looks here, the partial only has to
@@ -274,7 +270,7 @@ __global__ void __launch_bounds__(kThreads, kSweepCtasPerSm) sweep_kernel(const 
     }
     __syncthreads();
     const int last = sh_last;
-    if (last & 1) prefix_epilogue<T>(P, b, gam, Tf, sh_pos);
+    if (last & 1) prefix_epilogue<T>(P, b, gam, Tf == 0.f, scale, sh_pos);
     if (!(last & 2)) return;
     if (P.export_state) {
         const long long row0 = static_cast<long long>(b) * P.J;
@@ -283,7 +279,7 @@ __global__ void __launch_bounds__(kThreads, kSweepCtasPerSm) sweep_kernel(const 
                             P.part + (row0 + lane) * P.nsplit, P.nsplit);
         return;
     }
-    row_epilogue_cta<T>(P, b, gam, Tf, sh_pos, sh_sum, &sh_src);
+    row_epilogue_cta<T>(P, b, gam, Tf, scale, sh_pos, sh_sum, &sh_src);
 }
 
 }  // namespace speckv
