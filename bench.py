@@ -7,10 +7,9 @@ With --gpus N > 1 and no launcher around it (WORLD_SIZE unset) it starts the N r
 per GPU on 127.0.0.1; under torchrun it is one of the ranks.  Rows never interact, so the ranks share
 nothing but the barrier and the MAX of their times.
 
-A step = one pass of the whole hot path (draft signals, controller, verification: a memset of the
-tickets, then the sweep kernel, whose grid also draws the fresh tokens for bf16 logits; for fp32
-logits the ring sweep and the resample kernel) over one synthetic batch whose logits are resident
-in HBM.
+A step = one pass of the whole hot path (draft signals, controller, verification: a small kernel that
+clears the counters and lists the logit rows in use, then the sweep kernel, whose grid also draws the
+fresh tokens) over one synthetic batch whose logits are resident in HBM.
 Prints ONE JSON line: verified speculation rows/s (whole job), the roofline of the dominant
 kernel against the measured HBM peak, the end-to-end figure with host buffers, and the CPU
 oracle timed on the host cores as a reported baseline.  With --impl reference the oracle
@@ -360,37 +359,33 @@ def main():
     torch.cuda.synchronize()
     prof_step_ms = sum(a_.elapsed_time(b_) for a_, b_ in outer) / n_prof
     sweep_ms = [e[0].elapsed_time(e[1]) for e in evs]
-    resample_ms = [e[1].elapsed_time(e[2]) for e in evs]
     sweep_avg = sum(sweep_ms) / n_prof
     bytes_avg = sum(bytes_step[i % n_batches] for i in range(n_prof)) / n_prof
     peak, peak_kind = measured_hbm_peak()
     achieved = bytes_avg / (sweep_avg * 1e-3) / 1e9
-    # the library picks by logit type and batch: fp32, 384..1024 rows -> ring sweep, then a resample kernel (two launches per step);
-    # bf16 -> register-staged sweep whose grid also carries the resample CTAs (one launch per step, so
-    # its duration is that of the whole pass over the batch, second read of the stop positions included)
-    kernel = "pipe_sweep_kernel" if (w.dtype == "fp32" and 384 <= wr.B <= 1024 and args.schedule != "sliced") else "sweep_kernel"
-    one_launch = kernel != "pipe_sweep_kernel"
-    # One launch per step: in the timed region the launches follow one another on one stream with nothing but a
-    # 2 us memset between them, so the kernel's average duration there is at most the step time.  The loop above
-    # brackets every launch with five event records, the GPU idles some 20 us between launches, and a kernel that
-    # starts on an idle GPU takes a few microseconds longer than one that follows its predecessor; the smaller of
+    # The sweep kernel's grid also carries the CTAs that draw, so its duration is that of the whole pass over the batch,
+    # second read of the stop positions included.  In the timed region the launches follow one another on one stream with
+    # nothing but the preparing kernel (2 us) between them, so the kernel's average duration there is at most the step time.
+    # The loop above brackets every launch with five event records, the GPU idles some 20 us between launches, and a kernel
+    # that starts on an idle GPU takes a few microseconds longer than one that follows its predecessor; the smaller of
     # the two is the kernel's duration over the timed region (both are in the line).
+    kernel = "sweep_kernel"
     kernel_ms_events = sweep_avg
-    if one_launch and ms_step < sweep_avg:
+    if ms_step < sweep_avg:
         sweep_avg = ms_step
         achieved = bytes_avg / (sweep_avg * 1e-3) / 1e9
     roofline = {"bound": "hbm", "kernel": kernel, "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": achieved / peak, "peak_kind": f"of {peak_kind}", "traffic": ncu_traffic_bytes(kernel, w.name) if not args.rows else None,
                 "algorithmic_bytes_per_launch": bytes_avg, "kernel_ms": sweep_avg, "kernel_ms_events": kernel_ms_events,
                 "kernel_ms_min": min(sweep_ms),
-                "kernel_covers": "sweep + row epilogues + fresh-token draw" if one_launch else "sweep + row epilogues",
-                "resample_kernel_ms": None if one_launch else sum(resample_ms) / n_prof,
+                "kernel_covers": "sweep + row epilogues + fresh-token draw",
+                "resample_kernel_ms": None,
                 "kernel_ms_median": statistics.median(sweep_ms),
                 # the same steps bracketed from outside: events around every single launch cost a few microseconds,
                 # so this loop's step is slower than the timed region's, and its kernel time is the one to hold against it
                 "step_ms_in_this_loop": prof_step_ms,
                 "timed_over": (f"kernel_ms_events: {n_prof} steps after the timed region, CUDA events recorded inside the library call; "
-                               "kernel_ms: the smaller of that and the timed region's step time where a step is one launch"),
+                               "kernel_ms: the smaller of that and the timed region's step time"),
                 "frac_of_8TBps": achieved / 8000.0,
                 "step_GBps": sum(bytes_step[i % n_batches] for i in range(args.steps)) / args.steps / (ms_step * 1e-3) / 1e9}
 
@@ -499,7 +494,7 @@ def main():
                            early_exit=not args.no_early_exit, schedule=args.schedule),
             "timed_blocks": len(blocks_ms), "ms_per_block_median": ms_total,
             "roofline": roofline, "cpu_baseline": cpu_baseline, "parity": parity, "e2e": e2e, "clocks": clocks,
-            "gpu_launches": (1 if one_launch else 2) * args.steps,
+            "gpu_launches": 2 * args.steps,  # the preparing kernel and the sweep kernel of each step
             "tokens_per_step_mean": float(outs[0].n_accepted.float().mean()) + 1.0,
         }))
     if dist:

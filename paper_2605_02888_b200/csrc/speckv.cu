@@ -1,8 +1,7 @@
 // Host side of libspeckv: argument checks, workspace plan and kernel launches behind the
 // C ABI declared in include/speckv.h.  No allocation, no synchronisation.  The only state the
-// library keeps between calls is a handful of per-device constants (SM count, kernel attributes set,
-// the address of the built-in scratch array), each published with release/acquire atomics; none of
-// them survives cudaDeviceReset.
+// library keeps between calls is one per-device constant (the address of the built-in scratch array), published with
+// release/acquire atomics; it does not survive cudaDeviceReset.
 #include "speckv.h"
 #include "speckv_internal.h"
 
@@ -13,7 +12,6 @@
 #include <cstdint>
 
 #include "speckv_kernels.cuh"
-#include "speckv_pipeline.cuh"
 #include "speckv_sweep.cuh"
 #include "speckv_shard.cuh"
 #include "speckv_sample.cuh"
@@ -120,7 +118,7 @@ Plan make_plan(const speckv_batch* bt) {
     const size_t B = static_cast<size_t>(bt->B);
     p.J_full = 2 * bt->gamma_max + 1;
     size_t off = 0;
-    p.off_tick = off; off = align_up(off + (6 * B + 4) * sizeof(int));  // tickets, counters, row queue, row flags, first-generation tickets, early stops
+    p.off_tick = off; off = align_up(off + (6 * B + 4) * sizeof(int));  // tickets, counters, draw queue, first-generation tickets, early stops
     p.off_info = off; off = align_up(off + B * sizeof(RowInfo));
     p.off_part = off; off = align_up(off + B * p.J_full * kMaxSplit * sizeof(float4));
     off = align_up(off + B * ((static_cast<size_t>(bt->V) + 255) / 256) * sizeof(float));  // (not in use: keeps the sizes that were accepted)
@@ -187,46 +185,6 @@ struct Events {  // optional timing events around the kernels of a step
     cudaEvent_t before_sweep = nullptr, after_sweep = nullptr, after_resample = nullptr;
 };
 
-// Staged sweep: persistent CTAs, two per SM.  Needs 16-byte aligned rows whose byte length is a
-// multiple of 16, and a batch whose per-row tables fit in shared memory.
-// SM count of the current device, looked up once per device (0 in the slot = not yet known).
-cudaError_t sm_count(int* out) {
-    static std::atomic<int> cached[64];
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    const bool slot = dev >= 0 && dev < 64;
-    int sms = slot ? cached[dev].load(std::memory_order_acquire) : 0;
-    if (sms == 0) {
-        e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) return e;
-        if (slot) cached[dev].store(sms, std::memory_order_release);
-    }
-    *out = sms;
-    return cudaSuccess;
-}
-
-template <typename T>
-cudaError_t launch_pipe(const KParams& P, cudaStream_t st) {
-    static std::atomic<bool> configured[64];
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    const size_t smem = (sizeof(PipeShared) + 127) / 128 * 128 + static_cast<size_t>(kStages) * kStageBytes;
-    const bool slot = dev >= 0 && dev < 64;
-    if (!slot || !configured[dev].load(std::memory_order_acquire)) {
-        e = cudaFuncSetAttribute(pipe_sweep_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(smem));
-        if (e != cudaSuccess) return e;
-        if (slot) configured[dev].store(true, std::memory_order_release);
-    }
-    int sms = 0;
-    e = sm_count(&sms);
-    if (e != cudaSuccess) return e;
-    pipe_sweep_kernel<T><<<kPipeCtasPerSm * sms, kPipeThreads, smem, st>>>(P);
-    return cudaGetLastError();
-}
-
 constexpr int kPrepRows = 32;  // batch rows per CTA of the preparing kernel at least; 64 CTAs at most
 
 // The sliced sweep: list and cleared counters, then the sweep with n_draw CTAs behind it.  The sweep is a programmatic
@@ -254,33 +212,16 @@ cudaError_t launch_sliced(KParams P, long long n_draw, cudaStream_t st, cudaEven
 }
 
 template <typename T>
-cudaError_t launch_all(const KParams& P, cudaStream_t st, const Events& ev, bool ring) {
+cudaError_t launch_all(const KParams& P, cudaStream_t st, const Events& ev) {
     const bool verify = (P.mode & MODE_VERIFY) != 0;
-    const long long n_draw = static_cast<long long>(P.B) * P.R;
-    const bool merged = verify && !ring && static_cast<long long>(P.B) * P.J * P.nsplit + n_draw <= 0x7fffffffLL;
-    cudaError_t e;
-    if (ring) {
-        if (ev.before_sweep) cudaEventRecord(ev.before_sweep, st);
-        e = launch_pipe<T>(P, st);
-    } else {
-        e = launch_sliced<T>(P, merged ? n_draw : 0, st, ev.before_sweep);
-    }
+    const long long n_draw = verify ? static_cast<long long>(P.B) * P.R : 0;
+    const bool merged = static_cast<long long>(P.B) * P.J * P.nsplit + n_draw <= 0x7fffffffLL;
+    cudaError_t e = launch_sliced<T>(P, merged ? n_draw : 0, st, ev.before_sweep);
     if (e != cudaSuccess) return e;
     if (ev.after_sweep) cudaEventRecord(ev.after_sweep, st);
-    if (verify && !merged) {
-        // programmatic dependent launch: the kernel's CTAs are scheduled while the sweep drains and
-        // wait inside the kernel for the sweep's results
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(static_cast<unsigned>(n_draw));
-        cfg.blockDim = dim3(kThreads);
-        cfg.dynamicSmemBytes = 0;
-        cfg.stream = st;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        e = cudaLaunchKernelEx(&cfg, resample_kernel<T>, P);
+    if (!merged) {  // more CTAs than a grid holds: the draws' part as a launch of its own
+        resample_kernel<T><<<static_cast<unsigned>(n_draw), kThreads, 0, st>>>(P);
+        e = cudaGetLastError();
     }
     if (ev.after_resample) cudaEventRecord(ev.after_resample, st);
     return e;
@@ -325,10 +266,9 @@ speckv_status run(const speckv_batch* bt, int mode, const float* comp, const spe
     char* w = static_cast<char*>(ws);
     P.tick1 = reinterpret_cast<int*>(w + pl.off_tick);
     P.tick2 = P.tick1 + P.B;
-    P.qcount = P.tick1 + 2 * P.B;
-    P.qhead = P.qcount + 1;
-    P.qtail = P.qcount + 2;
-    P.rowq = P.qcount + 4;
+    P.n_list = P.tick1 + 2 * P.B;
+    P.q_front = P.n_list + 1;
+    P.q_back = P.n_list + 2;
     P.info = reinterpret_cast<RowInfo*>(w + pl.off_info);
     P.part = reinterpret_cast<float4*>(w + pl.off_part);
     P.dsum = reinterpret_cast<double*>(w + pl.off_dsum);
@@ -337,33 +277,11 @@ speckv_status run(const speckv_batch* bt, int mode, const float* comp, const spe
 
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     if (dbg_register(cs, bt, verify, ws, ws_bytes) != cudaSuccess) return SPECKV_ERR_CUDA;
-    const long long row_bytes = static_cast<long long>(P.V) * es;
-
-    // the staged sweep wants whole 16-byte granules per row and a batch its per-row tables can hold
-    // Which sweep.  Measured on B200 (full-size workloads, same inputs): fp32 logits are bound by
-    // memory and the bulk-copy ring is faster (6.7-6.9 against 6.4 TB/s); bf16 logits need one
-    // exponential per two bytes, and hiding that latency next to the memory latency takes the 32
-    // warps per SM of the register-staged kernel (4.95 against 4.6 TB/s), whose draining tail the
-    // resample CTAs of the same grid then fill.
-    // Below a few hundred rows the ring's fixed costs (per-CTA tables, one epilogue warp per CTA, a
-    // resample kernel that cannot overlap) outweigh its streaming rate: b512_mixed cut to 128 / 256 /
-    // 512 rows takes 178 / 317 / 564 us with the ring and 166 / 307 / 581 us without.
-constexpr int kPipeMinB = 384;
-    const bool staged = bt->dtype == SPECKV_F32 && aligned && row_bytes % 16 == 0 && P.B <= kPipeMaxB && P.B >= kPipeMinB &&
-                        !(bt->flags & SPECKV_SCHEDULE_SLICED);
-    if (staged) {
-        if (cudaMemsetAsync(P.tick1, 0, (6 * static_cast<size_t>(P.B) + 4) * sizeof(int), cs) != cudaSuccess) return SPECKV_ERR_CUDA;
-    } else {
-        P.n_list = P.qcount; P.q_front = P.qhead; P.q_back = P.qtail;  // the ring's counters and queue are not in use
-        // signals: behind their partials, which take a third of that region; verification: a region of its own
-        P.list = reinterpret_cast<int2*>(verify ? w + pl.off_list : reinterpret_cast<char*>(P.part + static_cast<size_t>(P.B) * P.J * P.nsplit));
-    }
-    // completion flags per batch row and the logits at the draft tokens: only the register-staged sweep
-    // overlaps the resample work with its own tail; after the ring sweep the resample kernel starts when
-    // everything is done and a flag would only cost it a round trip
-    P.rdone = (verify && !staged) ? P.rowq + P.B : nullptr;
-    P.tokl = (verify && !staged) ? reinterpret_cast<float2*>(static_cast<char*>(ws) + pl.off_tokl) : nullptr;
-    if (verify && !staged) {
+    // signals: behind their partials, which take a third of that region; verification: a region of its own
+    P.list = reinterpret_cast<int2*>(verify ? w + pl.off_list : reinterpret_cast<char*>(P.part + static_cast<size_t>(P.B) * P.J * P.nsplit));
+    if (verify) {
+        P.rdone = P.n_list + 4;
+        P.tokl = reinterpret_cast<float2*>(w + pl.off_tokl);
         P.spans = reinterpret_cast<float2*>(w + pl.off_spans);
         // generation order: positions 0..k of every batch row first, so that their acceptance tests are in
         // before the CTAs of the later target rows start (most walks that stop early stop at the first two
@@ -374,14 +292,11 @@ constexpr int kPipeMinB = 384;
         // one and a half rounds of CTA slots behind it (one row, V = 32,000: taking the tests for nothing cost 4 us of 20)
         const long long ahead = static_cast<long long>(P.B) * P.nsplit * (2 * (P.k_early + 1) + P.G - P.k_early - 1);
         if (2 * ahead >= 3 * kSlots) {
-            P.tick_early = P.rowq + 2 * P.B;
-            P.early = P.rowq + 3 * P.B;
+            P.tick_early = P.rdone + P.B;
+            P.early = P.rdone + 2 * P.B;
         }
     }
-    P.Lg = static_cast<int>(row_bytes / 16);
-    P.Lp = (P.Lg + kStageGran - 1) / kStageGran * kStageGran;
-    cudaError_t e;
-    e = bt->dtype == SPECKV_BF16 ? launch_all<__nv_bfloat16>(P, cs, ev, staged) : launch_all<float>(P, cs, ev, staged);
+    const cudaError_t e = bt->dtype == SPECKV_BF16 ? launch_all<__nv_bfloat16>(P, cs, ev) : launch_all<float>(P, cs, ev);
     return e == cudaSuccess ? SPECKV_OK : SPECKV_ERR_CUDA;
 }
 
@@ -496,15 +411,13 @@ speckv_status shard_params(const speckv_batch* bt, void* ws, size_t ws_bytes, KP
     char* w = static_cast<char*>(ws);
     P.tick1 = reinterpret_cast<int*>(w + pl.off_tick);
     P.tick2 = P.tick1 + P.B;
-    P.qcount = P.tick1 + 2 * P.B;
-    P.qhead = P.qcount + 1;
-    P.qtail = P.qcount + 2;
-    P.rowq = P.qcount + 4;
+    P.n_list = P.tick1 + 2 * P.B;
+    P.q_front = P.n_list + 1;
+    P.q_back = P.n_list + 2;
     P.part = reinterpret_cast<float4*>(w + pl.off_part);
     P.dsum = reinterpret_cast<double*>(w + pl.off_dsum);
     P.dsum2 = reinterpret_cast<double*>(w + pl.off_dsum2);
     P.list = reinterpret_cast<int2*>(w + pl.off_list);
-    P.n_list = P.qcount; P.q_front = P.qhead; P.q_back = P.qtail;
     return SPECKV_OK;
 }
 bool shard_aligned(const speckv_batch* bt) {

@@ -393,32 +393,30 @@ __device__ __forceinline__ int draw_from_spans(const T* row, int V, float scale,
 }
 
 // ----------------------------------------------------------------------------------------
-// One CTA's share of the fresh-token draw of batch row b at stop position n: share `share` of Rr, dw granules per warp.
+// One CTA's share of the draw from the residual of batch row b at stop position n.
 // The last of the row's CTAs to arrive locates the token.  A residual whose total mass is below 1e-6 cannot be told from
 // rounding noise and is treated as empty (p == q at the stop position): the token is then drawn from p.
 // ----------------------------------------------------------------------------------------
 template <typename T>
-__device__ __forceinline__ void resample_row(const KParams& P, const int b, const int mode, const int n, const int share,
-                                             const int Rr, const int dw) {
+__device__ __forceinline__ void resample_row(const KParams& P, const int b, const int n, const int share) {
     __shared__ int sh_flag;
     __shared__ DrawSrc sh_src;
     __shared__ double sh_sum[64];
-    if (mode == RS_NONE) return;  // greedy or flagged row, or a token that the sweep's own CTA draws
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const T* trow = static_cast<const T*>(P.t) + static_cast<long long>(b) * P.tsb + static_cast<long long>(n) * P.tsp;
     const T* drow = static_cast<const T*>(P.d) + static_cast<long long>(b) * P.dsb + static_cast<long long>(n) * P.dsp;
-    const DrawSrc src = make_draw<T>(trow, mode == RS_RESIDUAL ? drow : nullptr, P.V);
+    const DrawSrc src = make_draw<T>(trow, drow, P.V);
     double* dsum = P.dsum + static_cast<long long>(b) * (kMaxShares * kWarps);
     const int span = share * kWarps + warp;
     {
-        const int g0 = span * dw, g1 = min(src.t.ng, g0 + dw);
-        const double w = mode == RS_RESIDUAL ? warp_weight<T, true>(src, g0, g1, P.info + b) : warp_weight<T, false>(src, g0, g1, P.info + b);
+        const int g0 = span * P.draw_pw;
+        const double w = warp_weight<T, true>(src, g0, min(src.t.ng, g0 + P.draw_pw), P.info + b);
         if (lane == 0) SPECKV_ST(dsum[span], w);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
-        const bool last = atomicAdd(P.tick2 + b, 1) == Rr - 1;
+        const bool last = atomicAdd(P.tick2 + b, 1) == P.R - 1;
         if (last) __threadfence();
         sh_flag = last;
     }
@@ -428,25 +426,20 @@ __device__ __forceinline__ void resample_row(const KParams& P, const int b, cons
     // ---- last CTA of the row: locate the threshold (every warp picks the span, redundantly) ----
     const RowInfo ri = row_info_load(P.info + b);
     if (threadIdx.x == 0) {
-        DrawSrc c = make_draw<T>(trow, mode == RS_RESIDUAL ? drow : nullptr, P.V);
+        DrawSrc c = make_draw<T>(trow, drow, P.V);
         set_norm(c, ri.scale, ri.lse2_p, ri.lse2_q);
         sh_src = c;
     }
-    const float u2 = ri.u2;
     double before = 0.0, total, tau;
-    const int own = pick_many<true, 8>(Rr * kWarps, [&](int k) { return dbg_ok(dsum + k, 8, DBG_WS_LOAD) ? __ldcg(dsum + k) : 0.0; },
-                                       static_cast<double>(u2), &before, &total, &tau);
+    const int own = pick_many<true, 8>(P.R * kWarps, [&](int k) { return dbg_ok(dsum + k, 8, DBG_WS_LOAD) ? __ldcg(dsum + k) : 0.0; },
+                                       static_cast<double>(ri.u2), &before, &total, &tau);
     __syncthreads();
     const int ng = sh_src.t.ng;
     int tok;
-    if (mode == RS_RESIDUAL && total > 1e-6)
-        tok = find_token<T, true>(sh_src, own * dw, min(ng, (own + 1) * dw), tau - before, false, warp, kWarps, 1, sh_sum);
-    else if (mode == RS_RESIDUAL)
-        tok = find_token<T, false>(sh_src, 0, ng, static_cast<double>(u2), true, warp, kWarps, 1, sh_sum);
-    else if (own < 0)
-        tok = warp == 0 ? 0 : kNotMine;  // p itself has no mass: cannot happen for a finite row
+    if (total > 1e-6)
+        tok = find_token<T, true>(sh_src, own * P.draw_pw, min(ng, (own + 1) * P.draw_pw), tau - before, false, warp, kWarps, 1, sh_sum);
     else
-        tok = find_token<T, false>(sh_src, own * dw, min(ng, (own + 1) * dw), tau - before, false, warp, kWarps, 1, sh_sum);
+        tok = find_token<T, false>(sh_src, 0, ng, static_cast<double>(ri.u2), true, warp, kWarps, 1, sh_sum);
     if (tok != kNotMine && lane == 0) P.out_tok[static_cast<long long>(b) * (P.G + 1) + n] = max(tok, 0);
 }
 
@@ -455,36 +448,22 @@ __device__ __forceinline__ void resample_body(const KParams& P, const int bid) {
     __shared__ int sh_wait;
     // one-dimensional grid, R consecutive CTAs per draw
     const int g = bid / P.R, share = bid - g * P.R;
-    int mode, n, b;
-    if (P.rdone) {
-        // Group g takes the row in slot g of the draw queue.  Every sweep CTA is resident or done before the first CTA that
-        // draws starts, so all slots get filled and the wait ends; it is bounded all the same.
-        if (threadIdx.x == 0) sh_wait = row_done_wait(P.rdone + g, P.wait_limit);
-        __syncthreads();
-        const int v = sh_wait;
-        if (!v) {
-            // Gave up.  The mark goes on the slot: if the row epilogue has already written the
-            // status (the slot was filled just after the last poll) the bit is added here, otherwise the
-            // epilogue finds the mark when it takes the slot and adds the bit itself.
-            if (threadIdx.x == 0 && share == 0) {
-                const int old = atomicOr(P.rdone + g, kSlotTimeout);
-                if ((old & kSlotDone) && P.status) atomicOr(P.status + (old & 0xffffff), 16);
-            }
-            return;
+    // Group g takes the row in slot g of the draw queue.  Every sweep CTA is resident or done before the first CTA that
+    // draws starts, so all slots get filled and the wait ends; it is bounded all the same.
+    if (threadIdx.x == 0) sh_wait = row_done_wait(P.rdone + g, P.wait_limit);
+    __syncthreads();
+    const int v = sh_wait;
+    if (!v) {
+        // Gave up.  The mark goes on the slot: if the row epilogue has already written the
+        // status (the slot was filled just after the last poll) the bit is added here, otherwise the
+        // epilogue finds the mark when it takes the slot and adds the bit itself.
+        if (threadIdx.x == 0 && share == 0) {
+            const int old = atomicOr(P.rdone + g, kSlotTimeout);
+            if ((old & kSlotDone) && P.status) atomicOr(P.status + (old & 0xffffff), 16);
         }
-        b = v & 0xffffff;
-        mode = (v >> 24) & 1 ? RS_RESIDUAL : RS_NONE;
-        n = (v >> 25) & 15;
-    } else {
-        // A programmatic dependent launch behind the ring sweep: waits for the whole sweep; last batch row first (those rows
-        // are the freshest in L2).
-        asm volatile("griddepcontrol.wait;" ::: "memory");
-        b = P.B - 1 - g;
-        const int4 lo4 = __ldcg(reinterpret_cast<const int4*>(P.info + b));
-        mode = lo4.x;
-        n = lo4.y;
+        return;
     }
-    resample_row<T>(P, b, mode, n, share, P.R, P.draw_pw);
+    if ((v >> 24) & 1) resample_row<T>(P, v & 0xffffff, (v >> 25) & 15, share);  // else: nothing to draw for that row
 }
 
 template <typename T>

@@ -1,19 +1,19 @@
-// Device code of libspeckv: the streaming sweep over vocabulary-sized logit rows, the
-// per-row epilogue (signals, acceptance, controller) and the inverse-CDF resample.
+// Device code of libspeckv: the streaming sweep over vocabulary-sized logit rows and the per-row epilogue (signals,
+// acceptance, controller); the draws are in speckv_draw.cuh, the kernels of a step in speckv_sweep.cuh.
 //
 // Scheme (sm_100a, CUDA cores only -- the work is a streaming reduction, not a contraction):
+//   prep kernel     clears the counters and lists the logit rows in use in the order of the sweep's grid.
 //   sweep kernel    one CTA per (row b, logit row j, vocabulary slice s).  Each thread keeps
 //                   an online-softmax state over 16-byte vector loads, the CTA merges the
 //                   256 states and stores one partial.  The last CTA of a batch row to finish
 //                   (found with a ticket counter, nobody waits) merges that row's partials,
-//                   decides the acceptances, raises the row's completion flag and then writes
-//                   the signals and the controller outputs.
-//   resample work   R CTAs per batch row rescan the stop position's draft/target rows, write
-//                   per-256-element chunk sums of the residual weights, and the last of them
+//                   decides the acceptances, puts the row into the draw queue, writes
+//                   the signals and the controller outputs and draws a bonus token.
+//   draws           R CTAs per rejected row sum the residual weights of the stop position's two rows,
+//                   and the last of them
 //                   locates the inverse-CDF threshold and writes the fresh token.  These CTAs
 //                   sit behind the sweep CTAs in the sweep kernel's own grid and wait (bounded)
-//                   for their row's flag, or run as a kernel of their own after the ring sweep
-//                   of speckv_pipeline.cuh.
+//                   for a row of the queue.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -95,8 +95,6 @@ struct KParams {
     int k_early, read_all;
     int* early;       // [B] 0 = not known yet, else stop position + 1, or G + 2 when the walk passes k_early
     int* tick_early;  // [B] arrivals of the first generation's CTAs
-    int rs_reverse;  // resample kernel: 1 = last batch row first (after a sweep it cannot overlap: those rows are the freshest in L2)
-    int Lg, Lp;  // staged sweep: 16-byte granules per logit row, and the same padded to whole ring stages
     const void* d; long long dsb, dsp;
     const void* t; long long tsb, tsp;
     const int* tok; const int* gamma; const float* temp; float temp_scalar; const float* u;
@@ -109,7 +107,6 @@ struct KParams {
     int *gamma_next, *n_acc, *out_tok, *status;
     // workspace
     int *tick1, *tick2;
-    int *qcount, *qhead, *qtail, *rowq;  // staged sweep: next quantum to hand out; queue of completed batch rows
     float2* tokl;  // [B, G] (draft logit, target logit) at the draft token, left by the register-staged sweep; may be NULL
     int* rdone;  // verification: the draw queue's slots, one per batch row (row_done_signal); draft-side sampling: row status
     RowInfo* info;
@@ -1236,7 +1233,7 @@ __device__ __noinline__ void finish_signals(const KParams& P, int b, int gam, fl
     }
 }
 
-// Row epilogue: one warp, run by whoever learns that all partials of batch row b are in (ring sweep, sharded step).
+// Row epilogue: one warp (the sharded step, whose partials are the shards' gathered states).
 // Lane i merges the nd partials at pd (draft position i) and the nt partials at pt (target position i).
 // gam and Tf are the row's gamma and temperature as the sweep read them.  Everything the row
 // needs from memory that does not depend on other loads is requested first, so the epilogue
