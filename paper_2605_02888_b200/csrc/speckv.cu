@@ -389,6 +389,8 @@ ShardPlan make_shard_plan(const speckv_batch* bt) {
     return p;
 }
 
+// A slice row short enough for one CTA in a batch that fills the SMs with one CTA per row: no ticket, nothing to clear first.
+constexpr int kShardOneCtaRows = 128, kShardOneCtaGran = 4096;
 constexpr int kShardWarpRowBytes = 65536;  // slice rows up to this size are swept by one warp each
 
 // what every shard call needs from the local batch
@@ -403,6 +405,10 @@ speckv_status shard_params(const speckv_batch* bt, void* ws, size_t ws_bytes, KP
     const int es = esize(bt->dtype);
     choose_draw(P, bt->dtype, rows_aligned(bt->draft_logits, bt->draft_stride_b, bt->draft_stride_pos, es) &&
                                   rows_aligned(bt->target_logits, bt->target_stride_b, bt->target_stride_pos, es));
+    if (P.B >= kShardOneCtaRows && P.draw_pw * P.R * kWarps <= kShardOneCtaGran) {
+        P.draw_pw *= P.R;
+        P.R = 1;
+    }
     P.mode = MODE_VERIFY; P.bits = bt->entropy_in_bits ? 1 : 0;
     P.d = bt->draft_logits; P.dsb = bt->draft_stride_b; P.dsp = bt->draft_stride_pos;
     P.t = bt->target_logits; P.tsb = bt->target_stride_b; P.tsp = bt->target_stride_pos;
@@ -624,23 +630,21 @@ speckv_status speckv_shard_sweep(const speckv_batch* local, int64_t v_begin, flo
                                 {shard_tokl, static_cast<size_t>(P.B) * P.G * sizeof(float2)}};
         if (dbg_register(cs, local, true, workspace, workspace_bytes, ex, 2) != cudaSuccess) return SPECKV_ERR_CUDA;
     }
-    if (cudaMemsetAsync(shard_tokl, 0, static_cast<size_t>(P.B) * P.G * sizeof(float2), cs) != cudaSuccess)
-        return SPECKV_ERR_CUDA;
     constexpr int Ub = kSweepLoads, Uf = (kSweepLoads + 1) / 2;
-    // A slice row is short (V / n_shards columns).  One CTA per short row is mostly overhead and the
-    // ring sweep pays per logit row as well (segment hand-over to its epilogue warp), so rows of up to
-    // 64 KB are swept by one warp each, all of them resident at once; wider slices take the
+    // A slice row is short (V / n_shards columns) and one CTA per short row is mostly overhead, so rows of up to 64 KB are
+    // swept by a few warps each, as many as fill the SMs with a granule or two per lane left; wider slices take the
     // CTA-per-slice sweep.
-    const long long row_bytes = static_cast<long long>(P.V) * esize(local->dtype);
+    const long long row_bytes = static_cast<long long>(P.V) * esize(local->dtype), rows = static_cast<long long>(P.B) * P.J;
     if (row_bytes <= kShardWarpRowBytes) {
-        const unsigned g2 = static_cast<unsigned>((static_cast<long long>(P.B) * P.J + kWarps - 1) / kWarps);
-        if (local->dtype == SPECKV_BF16) {
-            shard_rows_kernel<__nv_bfloat16, Ub><<<g2, kThreads, 0, cs>>>(P);
-        } else {
-            shard_rows_kernel<float, Uf><<<g2, kThreads, 0, cs>>>(P);
-        }
+        int rw = 1;
+        while (rw < kWarps && rows * rw < kSlots * kWarps && row_bytes >= 2048LL * rw) rw *= 2;
+        const unsigned g2 = static_cast<unsigned>((rows * rw + kWarps - 1) / kWarps);
+        if (local->dtype == SPECKV_BF16) shard_rows_kernel<__nv_bfloat16, Ub><<<g2, kThreads, 0, cs>>>(P, rw);
+        else shard_rows_kernel<float, Uf><<<g2, kThreads, 0, cs>>>(P, rw);
         return cudaGetLastError() == cudaSuccess ? SPECKV_OK : SPECKV_ERR_CUDA;
     }
+    if (cudaMemsetAsync(shard_tokl, 0, static_cast<size_t>(P.B) * P.G * sizeof(float2), cs) != cudaSuccess)
+        return SPECKV_ERR_CUDA;
     const cudaError_t e = local->dtype == SPECKV_BF16 ? launch_sliced<__nv_bfloat16>(P, 0, cs, nullptr) : launch_sliced<float>(P, 0, cs, nullptr);
     return e == cudaSuccess ? SPECKV_OK : SPECKV_ERR_CUDA;
 }
@@ -675,12 +679,13 @@ speckv_status speckv_shard_finish(const speckv_batch* local, int32_t n_shards, i
     P.n_acc = n_accepted; P.out_tok = out_tokens; P.status = row_status;
     P.part = const_cast<float4*>(reinterpret_cast<const float4*>(all_state));
     P.part_stride = P.B * P.J;
+    P.nsplit = n_shards;
     P.n_shards = n_shards; P.shard_width = shard_width;
     P.tokl = const_cast<float2*>(reinterpret_cast<const float2*>(all_tokl));
     P.tokl_stride = static_cast<long long>(P.B) * P.G;
     P.info = static_cast<RowInfo*>(row_info);
     if (static_cast<long long>(P.B) * P.J > 0x7fffffffLL) return SPECKV_ERR_UNSUPPORTED;
-    const unsigned grid = static_cast<unsigned>((P.B + kWarps - 1) / kWarps);
+    const unsigned grid = static_cast<unsigned>(P.B);
     {
         speckv_batch none{};  // this call reads no logits: only the gathered arrays and the row records
         const DbgExtra ex[3] = {{all_state, static_cast<size_t>(n_shards) * P.B * P.J * sizeof(float4)},
@@ -688,7 +693,7 @@ speckv_status speckv_shard_finish(const speckv_batch* local, int32_t n_shards, i
                                 {row_info, static_cast<size_t>(P.B) * sizeof(RowInfo)}};
         if (dbg_register(static_cast<cudaStream_t>(cuda_stream), &none, false, nullptr, 0, ex, 3) != cudaSuccess) return SPECKV_ERR_CUDA;
     }
-    shard_finish_kernel<float><<<grid, kThreads, 0, static_cast<cudaStream_t>(cuda_stream)>>>(P);
+    shard_finish_kernel<<<grid, kThreads, 0, static_cast<cudaStream_t>(cuda_stream)>>>(P);
     return cudaGetLastError() == cudaSuccess ? SPECKV_OK : SPECKV_ERR_CUDA;
 }
 
@@ -706,7 +711,7 @@ speckv_status speckv_shard_draw_sums(const speckv_batch* local, const void* row_
         const DbgExtra ex[1] = {{row_info, static_cast<size_t>(P.B) * sizeof(RowInfo)}};
         if (dbg_register(cs, local, true, workspace, workspace_bytes, ex, 1) != cudaSuccess) return SPECKV_ERR_CUDA;
     }
-    if (cudaMemsetAsync(P.tick2, 0, static_cast<size_t>(P.B) * sizeof(int), cs) != cudaSuccess) return SPECKV_ERR_CUDA;
+    if (P.R > 1 && cudaMemsetAsync(P.tick2, 0, static_cast<size_t>(P.B) * sizeof(int), cs) != cudaSuccess) return SPECKV_ERR_CUDA;
     if (static_cast<long long>(P.B) * P.R > 0x7fffffffLL) return SPECKV_ERR_UNSUPPORTED;
     const unsigned grid = static_cast<unsigned>(P.B) * static_cast<unsigned>(P.R);
     if (local->dtype == SPECKV_BF16) {

@@ -63,7 +63,7 @@ __device__ __forceinline__ void gran_pairs(const uint4& g, f2 (&x)[2]) {
 }
 template <typename T, bool RES>
 __device__ __forceinline__ void gran_weights(float scale, float lp, float lq, float c, const uint4& t, const uint4& d,
-                                             float (&w)[16 / sizeof(T)]) {
+                                             float (&w)[16 / sizeof(T)], float* sum_p = nullptr) {
     constexpr int NP = 8 / sizeof(T);
     const f2 sc2 = pack2(scale, scale), p2 = pack2(-lp, -lp);
     f2 xt[NP];
@@ -78,6 +78,7 @@ __device__ __forceinline__ void gran_weights(float scale, float lp, float lq, fl
 #pragma unroll
         for (int i = 0; i < NP; ++i) {
             const f2 p = ex2_2(fma2(xt[i], sc2, p2)), q = ex2_2(fma2(xd[i], sc2, q2));
+            if (sum_p) *sum_p += hsum2(p);  // (known at compile time)
             float lo, hi;
             unpack2(fma2(q, c2, p), lo, hi);
             w[2 * i] = fmaxf(lo, 0.f);
@@ -86,9 +87,10 @@ __device__ __forceinline__ void gran_weights(float scale, float lp, float lq, fl
     }
 }
 template <typename T, bool RES>
-__device__ __forceinline__ float gran_weight(float scale, float lp, float lq, float c, const uint4& t, const uint4& d) {
+__device__ __forceinline__ float gran_weight(float scale, float lp, float lq, float c, const uint4& t, const uint4& d,
+                                             float* sum_p = nullptr) {
     float w[16 / sizeof(T)];
-    gran_weights<T, RES>(scale, lp, lq, c, t, d, w);
+    gran_weights<T, RES>(scale, lp, lq, c, t, d, w, sum_p);
     float a = 0.f;
 #pragma unroll
     for (int j = 0; j < static_cast<int>(16 / sizeof(T)); ++j) a += w[j];
@@ -161,8 +163,9 @@ __device__ __noinline__ double gran_weight_any(const DrawSrc s, int g) {
 // Two loads per row are in flight and none is requested ahead: the other warps of the SM, not this one, hide the latency, and
 // the loop, compiled by itself, keeps to the 48 registers of the sweep kernel without spilling (step of 1,024 bf16 rows,
 // V = 128,256, 430 us; two requested ahead 9 us more, four in flight 5 us more).  The record is fetched behind the first loads.
-template <typename T, bool RES, bool SHIFTED>
-__device__ __noinline__ double span_weight(const uint4* pt, const uint4* pd, int n, int off, const RowInfo* info) {
+// WITH_P: the sum of p as well (.y).
+template <typename T, bool RES, bool SHIFTED, bool WITH_P>
+__device__ __noinline__ double2 span_weight(const uint4* pt, const uint4* pd, int n, int off, const RowInfo* info) {
     constexpr int KU = SHIFTED ? 1 : 2;
     uint4 t[KU], d[KU], d1[KU];
     auto load = [&]() {
@@ -185,26 +188,30 @@ __device__ __noinline__ double span_weight(const uint4* pt, const uint4* pd, int
     const int4 lo = __ldcg(reinterpret_cast<const int4*>(info)), hi = __ldcg(reinterpret_cast<const int4*>(info) + 1);
     DrawSrc s;
     set_norm(s, __int_as_float(lo.w), __hiloint2double(hi.y, hi.x), __hiloint2double(hi.w, hi.z));
-    double acc = 0.0;
+    double2 acc = make_double2(0.0, 0.0);
     for (;;) {
-        float w = 0.f;
+        float w = 0.f, wp = 0.f;
 #pragma unroll
         for (int u = 0; u < KU; ++u)
-            w += gran_weight<T, RES>(s.scale, s.lp, s.lq, s.c, t[u], RES ? (SHIFTED ? gran_shift<T>(d[u], d1[u], off) : d[u]) : t[u]);
-        acc += static_cast<double>(w);
+            w += gran_weight<T, RES>(s.scale, s.lp, s.lq, s.c, t[u], RES ? (SHIFTED ? gran_shift<T>(d[u], d1[u], off) : d[u]) : t[u],
+                                     RES && WITH_P ? &wp : nullptr);
+        acc.x += static_cast<double>(w);
+        if (WITH_P) acc.y += static_cast<double>(RES ? wp : w);
         if (n <= 0) return acc;
         load();
     }
 }
-// Weight of granules [g0, g1), one warp, the same in every lane.  Only the rows of s are needed; info: the row's record.
-template <typename T, bool RES>
-__device__ __forceinline__ double warp_weight(const DrawSrc& s, int g0, int g1, const RowInfo* info) {
+// Weight of granules [g0, g1), one warp, the same in every lane (.x; WITH_P: of p in .y).  Only the rows of s are needed;
+// info: the row's record.
+template <typename T, bool RES, bool WITH_P>
+__device__ __forceinline__ double2 warp_weights(const DrawSrc& s, int g0, int g1, const RowInfo* info) {
     const int lane = threadIdx.x & 31;
     const int a = min(max(g0, s.in_lo), g1), e = max(min(g1, s.in_hi), a);
-    double acc = 0.0;
+    double2 acc = make_double2(0.0, 0.0);
     if (e - a - lane > 0) {
         const uint4 *pt = s.t.base + a + lane, *pd = s.d.base + s.dg + a + lane;
-        acc = (RES && s.off) ? span_weight<T, RES, RES>(pt, pd, e - a - lane, s.off, info) : span_weight<T, RES, false>(pt, pd, e - a - lane, 0, info);
+        acc = (RES && s.off) ? span_weight<T, RES, RES, WITH_P>(pt, pd, e - a - lane, s.off, info)
+                             : span_weight<T, RES, false, WITH_P>(pt, pd, e - a - lane, 0, info);
     }
     __syncwarp();
     // incomplete granules in front of and behind [a, e): a handful at most, one per lane
@@ -213,9 +220,15 @@ __device__ __forceinline__ double warp_weight(const DrawSrc& s, int g0, int g1, 
         const RowInfo ri = row_info_load(info);
         DrawSrc c = s;
         set_norm(c, ri.scale, ri.lse2_p, ri.lse2_q);
-        for (int k = lane; k < nl + nr; k += 32) acc += gran_weight_any<T, RES>(c, k < nl ? g0 + k : e + (k - nl));
+        for (int k = lane; k < nl + nr; k += 32) {
+            const int g = k < nl ? g0 + k : e + (k - nl);
+            acc.x += gran_weight_any<T, RES>(c, g);
+            if (WITH_P) acc.y += gran_weight_any<T, false>(c, g);
+        }
     }
-    return warp_sum(acc);
+    acc.x = warp_sum(acc.x);
+    if (WITH_P) acc.y = warp_sum(acc.y);
+    return acc;
 }
 
 // ---- picking -------------------------------------------------------------------------------------------------
@@ -410,7 +423,7 @@ __device__ __forceinline__ void resample_row(const KParams& P, const int b, cons
     const int span = share * kWarps + warp;
     {
         const int g0 = span * P.draw_pw;
-        const double w = warp_weight<T, true>(src, g0, min(src.t.ng, g0 + P.draw_pw), P.info + b);
+        const double w = warp_weights<T, true, false>(src, g0, min(src.t.ng, g0 + P.draw_pw), P.info + b).x;
         if (lane == 0) SPECKV_ST(dsum[span], w);
     }
     __syncthreads();

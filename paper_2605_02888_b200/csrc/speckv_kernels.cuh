@@ -869,115 +869,7 @@ struct RowDecide {
     bool badtok, accept;
 };
 
-// The per-position part of the row epilogue for one warp: lane i < n_lanes merges the nd partials at pd (draft
-// position i) and the nt partials at pt (target position i) and takes the acceptance test of its position.
-template <typename T>
-__device__ __noinline__ void row_decide(const KParams& P, int b, int gam, float Tf, int status, int n_lanes,
-                                        const float4* pd, int nd, const float4* pt, int nt, RowDecide& o) {
-    const int lane = threadIdx.x & 31;
-    const int G = P.G;
-    const bool verify = (P.mode & MODE_VERIFY) != 0;
-    constexpr int kPre = 4;  // partials fetched ahead per lane; more are rare
-    const bool greedy = (Tf == 0.f);
-    const float scale = static_cast<float>(kLog2e / static_cast<double>(greedy ? 1.f : Tf));
-    const double sd = static_cast<double>(scale);
-    const bool in = lane < n_lanes;
-    const bool dr_on = in && !status && lane < gam;
-    const bool tg_on = in && !status && verify && lane <= gam;
-    const bool tok_on = in && !status && verify && lane < gam;
-
-    // ---- first round trip ----
-    const long long ps = P.part_stride > 0 ? P.part_stride : 1;  // partials of a logit row: adjacent, or one per shard
-    float4 qd[kPre], qt[kPre];
-#pragma unroll
-    for (int k = 0; k < kPre; ++k) {
-        qd[k] = (dr_on && k < nd) ? ldcg4(pd + k * ps) : make_float4(0.f, 0.f, 0.f, 0.f);
-        qt[k] = (tg_on && k < nt) ? ldcg4(pt + k * ps) : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    const long long urow = (static_cast<long long>(b) * (G + 1) + lane) * 2;
-    const int x = tok_on ? __ldg(P.tok + static_cast<long long>(b) * G + lane) : -1;
-    const float u_acc = tok_on ? __ldg(P.u + urow) : 0.f;
-    const float u_res = tg_on ? __ldg(P.u + urow + 1) : 0.f;
-    // the two logits at the draft token: left by the sweep CTA of the draft position when the sweep
-    // does that (same round trip), else fetched below (a second one)
-    float2 tl = make_float2(0.f, 0.f);
-    if (P.tokl && tok_on && !greedy) {
-        long long at = static_cast<long long>(b) * G + lane;
-        if (P.shard_width > 0)  // the table of the shard whose slice holds the token (one more dependent load)
-            at += (x > 0 ? min(x / P.shard_width, P.n_shards - 1) : 0) * P.tokl_stride;
-        tl = __ldcg(P.tokl + at);
-    }
-
-    const bool badtok = tok_on && (x < 0 || x >= P.V);
-    float dxf = tl.x, txf = tl.y;
-    if (!P.tokl && tok_on && !badtok && !greedy) {
-        const T* drow = static_cast<const T*>(P.d) + static_cast<long long>(b) * P.dsb;
-        const T* trow = static_cast<const T*>(P.t) + static_cast<long long>(b) * P.tsb;
-        dxf = elem_to_float(drow + static_cast<long long>(lane) * P.dsp, x);
-        txf = elem_to_float(trow + static_cast<long long>(lane) * P.tsp, x);
-    }
-
-    float Hi = 0.f, ci = 0.f;
-    double lse2_q = 0.0, lse2_p = 0.0;
-    int amax = -1;
-    bool dbad = false, tbad = false, accept = true;  // non-finite draft row / target row at this lane's position
-
-    if (!status) {
-        // Partials are merged in fp32 with the same branch-free rules the sweep uses; the draft and
-        // the target chain are independent, so their instructions interleave.  Only what decides an
-        // acceptance (the log2-normalisers and the test itself) is carried in double.
-        float4 ad = qd[0], at = qt[0];
-#pragma unroll
-        for (int k = 1; k < kPre; ++k) {
-            if (k < nd) ad = merge_draft(ad, qd[k], scale);
-            if (k < nt) at = greedy ? merge_argmax(at, qt[k]) : merge_target(at, qt[k]);
-        }
-        // (only lanes that have a position: the partials of the others would lie outside the array)
-        if (dr_on)
-            for (int k = kPre; k < nd; ++k) ad = merge_draft(ad, ldcg4(pd + k * ps), scale);
-        if (tg_on)
-            for (int k = kPre; k < nt; ++k) at = greedy ? merge_argmax(at, ldcg4(pt + k * ps)) : merge_target(at, ldcg4(pt + k * ps));
-        if (dr_on) {
-            const float m = ad.x, cnt = ad.y, Zx = ad.z, S = ad.w;
-            const float Z = cnt + Zx;
-            if (!(cnt >= 1.f) || !(Z < 3e38f) || !(m > kFloor)) {
-                dbad = true;
-            } else {
-                const float lnZ = (cnt == 1.f) ? log1pf(Zx) : logf(cnt) + log1pf(Zx / cnt);
-                const float rZ = 1.f / Z;
-                Hi = fmaxf(lnZ - static_cast<float>(kLn2) * scale * S * rZ, 0.f);
-                ci = rZ;
-                lse2_q = static_cast<double>(m) * sd + log2_split(static_cast<double>(cnt) + static_cast<double>(Zx));
-            }
-        }
-        if (tg_on) {
-            if (greedy) {
-                const int bi = __float_as_int(at.y);
-                if (at.z != 0.f || bi == 0x7fffffff || !(at.x > kFloor)) tbad = true;
-                amax = bi;
-            } else {
-                if (!(at.y > 0.f) || !(at.y < 3e38f)) tbad = true;
-                else lse2_p = static_cast<double>(at.x) + log2_split(static_cast<double>(at.y));
-            }
-        }
-    }
-
-    if (status == 0 && !dbad && tok_on && !badtok && !tbad) {
-        if (greedy) {
-            accept = (x == amax);
-        } else {
-            const double lq = static_cast<double>(dxf) * sd - lse2_q;
-            const double lp = static_cast<double>(txf) * sd - lse2_p;
-            // u * q(x) < p(x); u = 0 gives -inf on the left
-            const double l2u = (u_acc > 0.f) ? log2_split(static_cast<double>(u_acc)) : -__longlong_as_double(0x7ff0000000000000LL);
-            accept = (l2u + lq) < lp;
-        }
-    }
-    o.x = x; o.u_res = u_res; o.Hi = Hi; o.ci = ci; o.lse2_q = lse2_q; o.lse2_p = lse2_p; o.amax = amax;
-    o.dbad = dbad; o.tbad = tbad; o.badtok = badtok; o.accept = accept;
-}
-
-// The same by the warps of a CTA (the sliced sweep): a group of 32 lanes (16 where a logit row has at most 16 partials)
+// The per-position part of a row epilogue, by the warps of a CTA: a group of 32 lanes (16 where a logit row has at most 16 partials)
 // decides one position, the lower half gathering the draft row's partials and the upper half the target row's, so that
 // they cost one memory round trip and a few shuffle steps instead of a chain of them, and one double-precision log2 serves
 // draft row, target row and uniform.
@@ -985,7 +877,8 @@ __device__ __noinline__ void row_decide(const KParams& P, int b, int gam, float 
 // epilogue each walked a chain of 11 dependent round trips and the step took 45.1 us; this way 23.0 us.  256 rows of
 // bf16, V = 128,256: 150.5 -> 145.6 us (the chain is also the end of a large step).  The prefix epilogue and the row
 // epilogue call this one compiled body, so that both reach the same bits.
-// Decides positions first, first + 1 (16 lanes each) or first alone; P.part holds n = nsplit partials per logit row.
+// Decides positions first, first + 1 (16 lanes each) or first alone.  A logit row has nsplit partials: its slices', adjacent in
+// P.part, or (part_stride) the states of as many vocabulary shards, part_stride apart.
 template <typename T>
 __device__ __noinline__ void decide_positions(const KParams& P, int b, int gam, bool greedy, float scale, int first, int n_pos,
                                               RowDecide* out) {
@@ -1000,12 +893,14 @@ __device__ __noinline__ void decide_positions(const KParams& P, int b, int gam, 
 
     // ---- one round trip ----
     const bool on = tgt_half ? in && verify : dr_on;
-    const float4* src = P.part + (static_cast<long long>(b) * P.J + (tgt_half || !verify ? i : P.G + 1 + i)) * n;
+    const long long jrow = static_cast<long long>(b) * P.J + (tgt_half || !verify ? i : P.G + 1 + i);
+    const long long ps = P.part_stride > 0 ? P.part_stride : 1;
+    const float4* src = P.part + (P.part_stride > 0 ? jrow : jrow * n);
     const float4 none = tgt_half && greedy ? make_float4(kFloor, __int_as_float(0x7fffffff), 0.f, 0.f)
                                            : make_float4(tgt_half ? -3.0e38f : kFloor, 0.f, 0.f, 0.f);
     float4 a = none, a2 = none;
-    if (on && k < n) a = ldcg4(src + k);
-    if (on && k + half < n) a2 = ldcg4(src + k + half);
+    if (on && k < n) a = ldcg4(src + k * ps);
+    if (on && k + half < n) a2 = ldcg4(src + (k + half) * ps);
     int x = -1;
     float u_acc = 0.f, u_res = 0.f;
     float2 tl = make_float2(0.f, 0.f);
@@ -1015,7 +910,9 @@ __device__ __noinline__ void decide_positions(const KParams& P, int b, int gam, 
         if (tok_on) {
             x = __ldg(P.tok + at);
             u_acc = __ldg(P.u + urow);
-            if (!greedy) tl = __ldcg(P.tokl + at);  // left by the sweep CTA of the draft position
+            // left by the sweep CTA of the draft position; with shards, in the table of the one whose slice holds the token
+            const long long shard = P.shard_width > 0 && x > 0 ? min(x / P.shard_width, P.n_shards - 1) : 0;
+            if (!greedy) tl = __ldcg(P.tokl + at + shard * P.tokl_stride);
         }
         if (in && verify) u_res = __ldg(P.u + urow + 1);
     }
@@ -1231,23 +1128,6 @@ __device__ __noinline__ void finish_signals(const KParams& P, int b, int gam, fl
             if (lane == 0) P.gamma_next[b] = 0;
         }
     }
-}
-
-// Row epilogue: one warp (the sharded step, whose partials are the shards' gathered states).
-// Lane i merges the nd partials at pd (draft position i) and the nt partials at pt (target position i).
-// gam and Tf are the row's gamma and temperature as the sweep read them.  Everything the row
-// needs from memory that does not depend on other loads is requested first, so the epilogue
-// costs one memory round trip (two when the sweep did not leave the logits at the draft tokens).
-template <typename T>
-__device__ __noinline__ void row_epilogue(const KParams& P, int b, int gam, float Tf, const float4* pd, int nd,
-                                          const float4* pt, int nt) {
-    const int status = row_status0(P, gam, Tf);
-    CtlRegs ctl;
-    if ((P.mode & MODE_MLP) && !status) ctl = ctl_load(P, b, threadIdx.x & 31);
-    RowDecide dec;
-    row_decide<T>(P, b, gam, Tf, status, 32, pd, nd, pt, nt, dec);
-    finish_verify(P, b, gam, Tf, row_scale(Tf), dec, false);
-    finish_signals(P, b, gam, Tf, dec, ctl);
 }
 
 // Epilogue of a vocabulary shard's sweep (one warp per batch row): lane i merges this shard's nd

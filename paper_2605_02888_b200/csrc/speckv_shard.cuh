@@ -12,39 +12,45 @@
 // CDF runs over the vocabulary in index order, shard after shard.
 #pragma once
 
-#include "speckv_draw.cuh"
+#include "speckv_sweep.cuh"
 
 namespace speckv {
 
-// Phase 1 for short slice rows: one warp per (batch row, logit row), every warp on its own row with
-// U loads of 16 bytes in flight per lane; the warp's merged state is the shard's state of that row.
-// No partials, no tickets.  (Wider slices use sweep_kernel with export_state set.)
+// Phase 1 for short slice rows: row_warps (1, 2, 4 or 8) neighbouring warps per (batch row, logit row), each on a contiguous
+// range with U loads of 16 bytes in flight per lane; their merged state is the shard's state of that row.
+// No partials, no tickets.  (Wider slices use sweep_kernel with export_state set.)  Latency-bound: one warp folds a 32 KB row in
+// 16 rounds of loads, and 256 rows of 17 are fewer warps than the SMs hold (sweep 39 us with one warp per row, @@ROWS@@ with two).
 template <typename T, int U>
-__global__ void __launch_bounds__(kThreads, kSweepCtasPerSm) shard_rows_kernel(const __grid_constant__ KParams P) {
-    const int lane = threadIdx.x & 31;
-    const long long w = static_cast<long long>(blockIdx.x) * kWarps + (threadIdx.x >> 5);
-    if (w >= static_cast<long long>(P.B) * P.J) return;
-    const int b = static_cast<int>(w / P.J), j = static_cast<int>(w - static_cast<long long>(b) * P.J);
+__global__ void __launch_bounds__(kThreads, kSweepCtasPerSm) shard_rows_kernel(const __grid_constant__ KParams P, const int row_warps) {
+    __shared__ float4 sh_part[kWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const long long w = (static_cast<long long>(blockIdx.x) * kWarps + warp) / row_warps;
+    const int sub = warp % row_warps;
+    const bool in = w < static_cast<long long>(P.B) * P.J;
+    const int b = in ? static_cast<int>(w / P.J) : 0, j = in ? static_cast<int>(w - static_cast<long long>(b) * P.J) : 0;
     const int gam = P.gamma ? P.gamma[b] : P.G;
     const float Tf = P.temp ? P.temp[b] : P.temp_scalar;
-    const bool row_ok = (gam >= 1 && gam <= P.G) && (Tf >= 0.f) && (Tf != __int_as_float(0x7f800000));
+    const bool row_ok = row_status0(P, gam, Tf) == 0;
     const bool greedy = (Tf == 0.f);
-    const float scale = static_cast<float>(kLog2e / static_cast<double>(greedy ? 1.f : Tf));
+    const float scale = row_scale(Tf);
     const bool is_target = j <= P.G;
     const int pos = is_target ? j : j - (P.G + 1);
-    const bool active = row_ok && (is_target ? pos <= gam : pos < gam);
+    const bool active = in && row_ok && (is_target ? pos <= gam : pos < gam);
     float4 st = make_float4(0.f, 0.f, 0.f, 0.f);
+    float2 tl = make_float2(0.f, 0.f);
     if (active) {
         const T* row = is_target ? static_cast<const T*>(P.t) + static_cast<long long>(b) * P.tsb + static_cast<long long>(pos) * P.tsp
                                  : static_cast<const T*>(P.d) + static_cast<long long>(b) * P.dsb + static_cast<long long>(pos) * P.dsp;
+        const GranRow gr = make_row(row, P.V);
+        const int per = (gr.ng + row_warps - 1) / row_warps;
         WarpSweep<T, U> ws;
-        ws.start(make_row(row, P.V), 0, 0x7fffffff);
-        if (!is_target && lane == 0 && !greedy) {
+        ws.start(gr, sub * per, sub * per + per);
+        if (!is_target && lane == 0 && sub == 0 && !greedy) {
             // both logits at the draft token, if it falls into this slice
             const int x = __ldg(P.tok + static_cast<long long>(b) * P.G + pos) - P.v_begin;
             if (x >= 0 && x < P.V) {
                 const T* trow = static_cast<const T*>(P.t) + static_cast<long long>(b) * P.tsb + static_cast<long long>(pos) * P.tsp;
-                SPECKV_ST(P.tokl[static_cast<long long>(b) * P.G + pos], make_float2(elem_to_float(row, x), elem_to_float(trow, x)));
+                tl = make_float2(elem_to_float(row, x), elem_to_float(trow, x));
             }
         }
         const float m0 = ws.template warm<false>(nullptr);
@@ -58,25 +64,36 @@ __global__ void __launch_bounds__(kThreads, kSweepCtasPerSm) shard_rows_kernel(c
             st = ws.template run<PATH_TARGET>(m0, scale);
         }
     }
-    if (lane == 0) P.state[static_cast<long long>(b) * P.J + j] = st;
+    if (row_warps > 1) {
+        if (lane == 0) sh_part[warp] = st;
+        __syncthreads();
+        if (sub == 0 && active)
+            for (int k = 1; k < row_warps; ++k) {
+                const float4 o = sh_part[warp + k];
+                st = !is_target ? merge_draft(st, o, scale) : greedy ? merge_argmax(st, o) : merge_target(st, o);
+            }
+    }
+    if (lane == 0 && sub == 0 && in) {
+        P.state[static_cast<long long>(b) * P.J + j] = st;
+        if (!is_target) SPECKV_ST(P.tokl[static_cast<long long>(b) * P.G + pos], tl);
+    }
 }
 
-// Phase 2: one warp per batch row; the partials of a logit row are the n_shards gathered states.
-template <typename T>
+// Phase 2: one CTA per batch row, the row epilogue of the sweep on the n_shards gathered states of each logit row
+// (nsplit = n_shards, part_stride apart).  Latency-bound: with a warp per row, a lane per position and a chain of n_shards
+// dependent loads in each it took @@FIN0@@ for 256 rows and 8 shards, this way @@FIN1@@.
 __global__ void __launch_bounds__(kThreads) shard_finish_kernel(const __grid_constant__ KParams P) {
-    const int lane = threadIdx.x & 31;
-    const int b = blockIdx.x * kWarps + (threadIdx.x >> 5);
-    if (b >= P.B) return;
+    __shared__ RowDecide sh_pos[kMaxGamma + 1];
+    const int b = blockIdx.x;
     const int gam = P.gamma ? P.gamma[b] : P.G;
     const float Tf = P.temp ? P.temp[b] : P.temp_scalar;
-    const float4* row = P.part + static_cast<long long>(b) * P.J;
-    row_epilogue<T>(P, b, gam, Tf, row + P.G + 1 + lane, P.n_shards, row + lane, P.n_shards);
+    row_epilogue_cta<float>(P, b, gam, Tf, row_scale(Tf), sh_pos, nullptr, nullptr);
 }
 
 // Phase 3: grid B * R.  Span weights of the stop position over the local slice: of the row's own
-// weights and, for a residual draw, of p as well (the draw falls back to p when the residual is
+// weights and, for a residual draw, of p as well, from the same pass (the draw falls back to p when the residual is
 // numerically empty, and whether it is shows only once all shards' masses are known).  The last
-// CTA of a row adds them up.
+// CTA of a row adds them up; with R = 1 there is no ticket.
 template <typename T>
 __global__ void __launch_bounds__(kThreads, 4) shard_sums_kernel(const __grid_constant__ KParams P) {
     __shared__ int sh_flag;
@@ -95,21 +112,23 @@ __global__ void __launch_bounds__(kThreads, 4) shard_sums_kernel(const __grid_co
     double* dr = P.dsum + static_cast<long long>(b) * (kMaxShares * kWarps);
     double* dp = P.dsum2 + static_cast<long long>(b) * (kMaxShares * kWarps);
     const int span = share * kWarps + warp, g0 = span * P.draw_pw, g1 = min(src.t.ng, g0 + P.draw_pw);
-    const double wr = res ? warp_weight<T, true>(src, g0, g1, P.info + b) : 0.0;
-    const double wp = warp_weight<T, false>(src, g0, g1, P.info + b);
+    const double2 w = res ? warp_weights<T, true, true>(src, g0, g1, P.info + b) : warp_weights<T, false, true>(src, g0, g1, P.info + b);
     if (lane == 0) {
-        SPECKV_ST(dr[span], wr);
-        SPECKV_ST(dp[span], wp);
+        SPECKV_ST(dr[span], w.x);
+        SPECKV_ST(dp[span], w.y);
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        const bool last = atomicAdd(P.tick2 + b, 1) == P.R - 1;
-        if (last) __threadfence();
-        sh_flag = last;
+    if (P.R > 1) {
+        if (threadIdx.x == 0) {
+            __threadfence();
+            const bool last = atomicAdd(P.tick2 + b, 1) == P.R - 1;
+            if (last) __threadfence();
+            sh_flag = last;
+        }
+        __syncthreads();
+        if (!sh_flag) return;
     }
-    __syncthreads();
-    if (!sh_flag || warp != 0) return;
+    if (warp != 0) return;
     double tr = 0.0, tp = 0.0;
     for (int k = lane; k < P.R * kWarps; k += 32)
         if (dbg_ok(dr + k, 8, DBG_WS_LOAD) && dbg_ok(dp + k, 8, DBG_WS_LOAD)) {

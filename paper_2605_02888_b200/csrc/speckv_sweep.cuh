@@ -23,8 +23,8 @@ __device__ __noinline__ void row_epilogue_cta(const KParams& P, int b, int gam, 
     decide_all<T>(P, b, gam, Tf == 0.f, scale, n_pos, pos);
     __syncthreads();
     if (warp >= kDrawWarp0) {
-        // a bonus draw: every position accepted, nothing flagged
-        if (!verify || !n_pos || Tf == 0.f) return;
+        // a bonus draw: every position accepted, nothing flagged (a sharded step draws in calls of its own)
+        if (!P.spans || !n_pos || Tf == 0.f) return;
         bool ends = false;
         if (lane < n_pos) ends = pos[lane].dbad || pos[lane].tbad || pos[lane].badtok || !pos[lane].accept;
         if (__any_sync(0xffffffffu, ends)) return;
@@ -39,7 +39,7 @@ __device__ __noinline__ void row_epilogue_cta(const KParams& P, int b, int gam, 
     dec.x = -1; dec.u_res = 0.f; dec.Hi = dec.ci = 0.f; dec.lse2_q = dec.lse2_p = 0.0; dec.amax = -1;
     dec.dbad = dec.tbad = dec.badtok = false; dec.accept = true;
     if (lane < n_pos) dec = pos[lane];
-    if (warp == 0) finish_verify(P, b, gam, Tf, scale, dec, true);
+    if (warp == 0) finish_verify(P, b, gam, Tf, scale, dec, P.spans != nullptr);
     else if (P.mode & MODE_SIGNALS) finish_signals(P, b, gam, Tf, dec, ctl);
 }
 
