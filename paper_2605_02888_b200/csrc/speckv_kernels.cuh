@@ -314,14 +314,14 @@ __device__ __forceinline__ void raw_floor(Raw<float>& r) {
 // ----------------------------------------------------------------------------------------
 struct DraftState {
     float m, r, cnt;
-    f2 za, zb, sa, sb;  // four running sums each of Zx and of 2^y * y, y = x * scale - r, as two packed pairs
+    f2 za, sa;  // four running sums each of Zx and of 2^y * y, y = x * scale - r, as two packed pairs
     bool bad;
     __device__ __forceinline__ void init(float m0, float scale) {
         m = m0; r = __fmul_rn(m0, scale); cnt = 0.f; bad = false;
-        za = zb = sa = sb = pack2(0.f, 0.f);
+        za = sa = pack2(0.f, 0.f);
     }
-    __device__ __forceinline__ float zsum() const { return hsum2(za) + hsum2(zb); }
-    __device__ __forceinline__ float ssum() const { return hsum2(sa) + hsum2(sb); }
+    __device__ __forceinline__ float zsum() const { return hsum2(za); }
+    __device__ __forceinline__ float ssum() const { return hsum2(sa); }
 
     template <typename T>
     __device__ __forceinline__ void slow(const Raw<T>& raw, float scale) {
@@ -354,8 +354,8 @@ struct DraftState {
                 sv = fmaf(e, y, sv);
             }
         }
-        za = pack2(z, 0.f); zb = pack2(0.f, 0.f);
-        sa = pack2(sv, 0.f); sb = pack2(0.f, 0.f);
+        za = pack2(z, 0.f);
+        sa = pack2(sv, 0.f);
     }
 
     template <typename T>
@@ -370,10 +370,8 @@ struct DraftState {
         const f2 sc2 = pack2(scale, scale), nr2 = pack2(-r, -r);
         const f2 y0 = fma2(x[0], sc2, nr2), y1 = fma2(x[1], sc2, nr2), y2 = fma2(x[2], sc2, nr2), y3 = fma2(x[3], sc2, nr2);
         const f2 e0 = ex2_2(y0), e1 = ex2_2(y1), e2 = ex2_2(y2), e3 = ex2_2(y3);
-        za = add2(za, e0); zb = add2(zb, e1);
-        sa = fma2(e0, y0, sa); sb = fma2(e1, y1, sb);
-        za = add2(za, e2); zb = add2(zb, e3);
-        sa = fma2(e2, y2, sa); sb = fma2(e3, y3, sb);
+        za = add2(za, add2(add2(e0, e1), add2(e2, e3)));
+        sa = add2(sa, fma2(e0, y0, fma2(e1, y1, fma2(e2, y2, mul2(e3, y3)))));
     }
     __device__ __forceinline__ float4 partial(float scale) const {
         const float d = fmaf(m, scale, -r), f = ex2f(-d), z = zsum();  // y against m itself is smaller by d, a rounding
