@@ -65,7 +65,8 @@ cudaError_t dbg_register(cudaStream_t cs, const speckv_batch* bt, bool target, c
 #endif
 }
 
-constexpr int kSlots = 740;  // CTA slots of the chip: 5 on each of 148 SMs
+// CTA slots of the chip for a sweep of this type (148 SMs).
+int cta_slots(speckv_dtype dt) { return 148 * (dt == SPECKV_BF16 ? SweepShape<__nv_bfloat16>::kCtas : SweepShape<float>::kCtas); }
 
 // Vocabulary slices per logit row for a sweep over J logit rows per batch row, one CTA each, and the granules that one
 // warp takes of a slice: P.nsplit, P.per_warp.  aligned: every row starts on the 16-byte grid.
@@ -74,11 +75,12 @@ void choose_slices(KParams& P, speckv_dtype dt, bool aligned) {
     const int ng = (P.V + E - 1 + (aligned ? 0 : E - 1)) / E;  // granules a row can touch
     int ns = static_cast<int>(std::lround(16.0 * ng / static_cast<double>(kSliceBytes)));
     if (ns < 1) ns = 1;
-    // Small batches: enough CTAs to fill the slots of the chip once (5 on each of 148 SMs).  Aiming at more starts a second
-    // round of short CTAs: with 1,184 instead of 740, step of 64 bf16 rows, V = 32,000, 37.7 us instead of 33.1, of 37 rows,
+    // Small batches: enough CTAs to fill the slots of the chip once.  Aiming at more starts a second
+    // round of short CTAs: with 1,184 instead of 740 (bf16), step of 64 bf16 rows, V = 32,000, 37.7 us instead of 33.1, of 37 rows,
     // V = 50,257, 32.6 instead of 31.1; one row the same.
     const long long rows = static_cast<long long>(P.B) * P.J;
-    const long long want = (kSlots + rows - 1) / (rows > 0 ? rows : 1);
+    const int slots = cta_slots(dt);
+    const long long want = (slots + rows - 1) / (rows > 0 ? rows : 1);
     if (want > ns) ns = static_cast<int>(want > kMaxSplit ? kMaxSplit : want);
     if (ns > kMaxSplit) ns = kMaxSplit;
     // At least one granule per lane; short ranges are whole rounds of the warp (a round with idle lanes costs as much as a
@@ -87,7 +89,7 @@ void choose_slices(KParams& P, speckv_dtype dt, bool aligned) {
     int pw = (ng + ns * kWarps - 1) / (ns * kWarps);
     const int near = (pw + 16) / 32 * 32 < 32 ? 32 : (pw + 16) / 32 * 32;
     if (pw >= 256) pw = (pw + 7) / 8 * 8;
-    else if (((ng + near * kWarps - 1) / (near * kWarps)) * rows <= kSlots + rows) pw = near;
+    else if (((ng + near * kWarps - 1) / (near * kWarps)) * rows <= slots + rows) pw = near;
     else pw = (pw + 31) / 32 * 32;
     while ((ng + pw * kWarps - 1) / (pw * kWarps) > kMaxSplit) pw += 32;
     P.per_warp = pw;
@@ -191,7 +193,6 @@ constexpr int kPrepRows = 32;  // batch rows per CTA of the preparing kernel at 
 // dependent launch: its CTAs are placed while the preparing kernel runs and wait for its end.
 template <typename T>
 cudaError_t launch_sliced(KParams P, long long n_draw, cudaStream_t st, cudaEvent_t before_sweep) {
-    constexpr int U = sizeof(T) == 2 ? kSweepLoads : (kSweepLoads + 1) / 2;
     P.n_draw = static_cast<int>(n_draw);
     int seg = (P.B + 63) / 64;
     seg = seg < kPrepRows ? kPrepRows : (seg + 31) / 32 * 32;
@@ -208,7 +209,7 @@ cudaError_t launch_sliced(KParams P, long long n_draw, cudaStream_t st, cudaEven
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, sweep_kernel<T, U>, P);
+    return cudaLaunchKernelEx(&cfg, sweep_kernel<T>, P);
 }
 
 template <typename T>
@@ -291,7 +292,7 @@ speckv_status run(const speckv_batch* bt, int mode, const float* comp, const spe
         // ... where the grid has that many CTAs: the third generation has to start after the first one's tests, that is
         // one and a half rounds of CTA slots behind it (one row, V = 32,000: taking the tests for nothing cost 4 us of 20)
         const long long ahead = static_cast<long long>(P.B) * P.nsplit * (2 * (P.k_early + 1) + P.G - P.k_early - 1);
-        if (2 * ahead >= 3 * kSlots) {
+        if (2 * ahead >= 3 * cta_slots(bt->dtype)) {
             P.tick_early = P.rdone + P.B;
             P.early = P.rdone + 2 * P.B;
         }
@@ -346,8 +347,8 @@ speckv_status run_sample(const speckv_batch* bt, const float* uniforms, int32_t*
     const size_t n_tick = static_cast<size_t>(P.B) * (2 + static_cast<size_t>(P.G));
     if (cudaMemsetAsync(P.tick1, 0, n_tick * sizeof(int), cs) != cudaSuccess) return SPECKV_ERR_CUDA;
     const unsigned grid = static_cast<unsigned>(P.B) * P.G * P.nsplit;
-    if (bt->dtype == SPECKV_BF16) sample_kernel<__nv_bfloat16, kSweepLoads><<<grid, kThreads, 0, cs>>>(P);
-    else sample_kernel<float, (kSweepLoads + 1) / 2><<<grid, kThreads, 0, cs>>>(P);
+    if (bt->dtype == SPECKV_BF16) sample_kernel<__nv_bfloat16><<<grid, kThreads, 0, cs>>>(P);
+    else sample_kernel<float><<<grid, kThreads, 0, cs>>>(P);
     return cudaGetLastError() == cudaSuccess ? SPECKV_OK : SPECKV_ERR_CUDA;
 }
 
@@ -630,17 +631,16 @@ speckv_status speckv_shard_sweep(const speckv_batch* local, int64_t v_begin, flo
                                 {shard_tokl, static_cast<size_t>(P.B) * P.G * sizeof(float2)}};
         if (dbg_register(cs, local, true, workspace, workspace_bytes, ex, 2) != cudaSuccess) return SPECKV_ERR_CUDA;
     }
-    constexpr int Ub = kSweepLoads, Uf = (kSweepLoads + 1) / 2;
     // A slice row is short (V / n_shards columns) and one CTA per short row is mostly overhead, so rows of up to 64 KB are
     // swept by a few warps each, as many as fill the SMs with a granule or two per lane left; wider slices take the
     // CTA-per-slice sweep.
     const long long row_bytes = static_cast<long long>(P.V) * esize(local->dtype), rows = static_cast<long long>(P.B) * P.J;
     if (row_bytes <= kShardWarpRowBytes) {
         int rw = 1;
-        while (rw < kWarps && rows * rw < kSlots * kWarps && row_bytes >= 2048LL * rw) rw *= 2;
+        while (rw < kWarps && rows * rw < cta_slots(local->dtype) * kWarps && row_bytes >= 2048LL * rw) rw *= 2;
         const unsigned g2 = static_cast<unsigned>((rows * rw + kWarps - 1) / kWarps);
-        if (local->dtype == SPECKV_BF16) shard_rows_kernel<__nv_bfloat16, Ub><<<g2, kThreads, 0, cs>>>(P, rw);
-        else shard_rows_kernel<float, Uf><<<g2, kThreads, 0, cs>>>(P, rw);
+        if (local->dtype == SPECKV_BF16) shard_rows_kernel<__nv_bfloat16><<<g2, kThreads, 0, cs>>>(P, rw);
+        else shard_rows_kernel<float><<<g2, kThreads, 0, cs>>>(P, rw);
         return cudaGetLastError() == cudaSuccess ? SPECKV_OK : SPECKV_ERR_CUDA;
     }
     if (cudaMemsetAsync(shard_tokl, 0, static_cast<size_t>(P.B) * P.G * sizeof(float2), cs) != cudaSuccess)

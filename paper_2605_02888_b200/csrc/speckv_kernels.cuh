@@ -28,10 +28,15 @@ constexpr int kVec = 8;                 // elements per lane per step
 constexpr int kMaxShares = 32;          // CTAs that share one draw at most
 constexpr int kMaxSplit = 32;
 constexpr int kMaxGamma = 16;           // SPECKV_MAX_GAMMA
-// Step of 256 / 1,024 bf16 rows, V = 128,256, and draft sampling of 256: 5 CTAs x 4 loads 141 / 418 / 81 us, 5 x 3 144 / 430 / 83,
-// 4 x 4 142 / 437 / 87, 6 x 3 146 / 430 / 88 (the GPU's time, one box).
-constexpr int kSweepLoads = 4;  // 16-byte loads in flight per thread (bf16); fp32 uses half as many vector steps
-constexpr int kSweepCtasPerSm = 5;  // CTAs per SM the sweep kernel is compiled for (48 registers per thread)
+// Loads in flight per thread (steps of kVec elements: 16 bytes of bf16, 32 of fp32) and CTAs per SM the sweep is compiled for.
+// Step of 256 / 1,024 bf16 rows, V = 128,256, and draft sampling of 256: 5 CTAs x 4 steps 141 / 418 / 81 us, 5 x 3 144 / 430 / 83,
+// 4 x 4 142 / 437 / 87, 6 x 3 146 / 430 / 88 (the GPU's time, one box).  fp32 needs twice the bytes in flight and fewer
+// instructions for them, so fewer warps with more registers: step of 512 rows, V = 151,936, verification of 96 greedy rows,
+// and step of 256 rows, V = 128,256: 4 CTAs x 4 steps 502 / 90 / 224 us, 5 x 2 512 / 94.5 / 235, 4 x 3 508 / 91 / 227,
+// 5 x 3 (spills) 680 / 111 / 306.
+template <typename T> struct SweepShape;
+template <> struct SweepShape<__nv_bfloat16> { static constexpr int kSteps = 4, kCtas = 5; };
+template <> struct SweepShape<float> { static constexpr int kSteps = 4, kCtas = 4; };
 constexpr float kFloor = -1.2676506002282294e30f;  // -2^100: logits below count as -inf
 constexpr uint32_t kFloorBf16x2 = 0xF180F180u;     // -2^100 as two bf16
 constexpr double kLn2 = 0.6931471805599453094;

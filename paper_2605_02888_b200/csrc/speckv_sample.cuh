@@ -13,8 +13,8 @@ namespace speckv {
 // grid: B * G * nsplit CTAs, one per (batch row, position, vocabulary slice).  P.spans holds [B*G, nsplit * kWarps]
 // (reference, sum) pairs, for greedy rows (best value or NaN, index); P.tick1 one counter per position, P.tick2 one per
 // batch row, P.rdone (here: a per-row status word), all zeroed by the host.
-template <typename T, int U>
-__global__ void __launch_bounds__(kThreads, kSweepCtasPerSm) sample_kernel(const __grid_constant__ KParams P) {
+template <typename T>
+__global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sample_kernel(const __grid_constant__ KParams P) {
     __shared__ int sh_last;
     __shared__ float sh_m0[kWarps];
     __shared__ DrawSrc sh_src;
@@ -40,7 +40,7 @@ __global__ void __launch_bounds__(kThreads, kSweepCtasPerSm) sample_kernel(const
     float2* spans = P.spans + static_cast<long long>(r) * n;
     {
         const int lo = (s * kWarps + warp) * P.per_warp;
-        WarpSweep<T, U> ws;
+        WarpSweep<T, SweepShape<T>::kSteps> ws;
         ws.start(make_row(row, P.V), lo, lo + P.per_warp);
         const float m0 = ws.template warm<true>(sh_m0);
         float2 v;

@@ -164,8 +164,8 @@ __global__ void __launch_bounds__(kThreads) prep_kernel(const __grid_constant__ 
 // 6.7 TB/s but drew its tokens in a launch of its own and could leave no row unread (step of 512 fp32 rows, V = 151,936:
 // 578 us with the ring, 523 this way; 384 rows 440 / 394; 1,000 rows, V = 60,000, 535 / 418).
 // ----------------------------------------------------------------------------------------
-template <typename T, int U>
-__global__ void __launch_bounds__(kThreads, kSweepCtasPerSm) sweep_kernel(const __grid_constant__ KParams P) {
+template <typename T>
+__global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sweep_kernel(const __grid_constant__ KParams P) {
     __shared__ float4 sh_part[kWarps];
     __shared__ RowDecide sh_pos[kMaxGamma + 1];
     __shared__ DrawSrc sh_src;
@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(kThreads, kSweepCtasPerSm) sweep_kernel(const 
         const T* row = is_target ? static_cast<const T*>(P.t) + static_cast<long long>(b) * P.tsb + static_cast<long long>(pos) * P.tsp
                                  : static_cast<const T*>(P.d) + static_cast<long long>(b) * P.dsb + static_cast<long long>(pos) * P.dsp;
         const int lo = (s * kWarps + warp) * P.per_warp;  // this warp's granules: the CTA's slice is cut into one contiguous range per warp
-        WarpSweep<T, U> ws;
+        WarpSweep<T, SweepShape<T>::kSteps> ws;
         ws.start(make_row(row, P.V), lo, lo + P.per_warp);
         Tf = P.temp ? __ldg(P.temp + b) : P.temp_scalar;
         if (threadIdx.x == 0) {
