@@ -637,7 +637,7 @@ speckv_status speckv_shard_sweep(const speckv_batch* local, int64_t v_begin, flo
     const long long row_bytes = static_cast<long long>(P.V) * esize(local->dtype), rows = static_cast<long long>(P.B) * P.J;
     if (row_bytes <= kShardWarpRowBytes) {
         int rw = 1;
-        while (rw < kWarps && rows * rw < cta_slots(local->dtype) * kWarps && row_bytes >= 2048LL * rw) rw *= 2;
+        while (rw < kWarps && rows * rw < 148 * 4 * kWarps && row_bytes >= 2048LL * rw) rw *= 2;
         const unsigned g2 = static_cast<unsigned>((rows * rw + kWarps - 1) / kWarps);
         if (local->dtype == SPECKV_BF16) shard_rows_kernel<__nv_bfloat16><<<g2, kThreads, 0, cs>>>(P, rw);
         else shard_rows_kernel<float><<<g2, kThreads, 0, cs>>>(P, rw);

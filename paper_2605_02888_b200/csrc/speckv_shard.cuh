@@ -20,8 +20,9 @@ namespace speckv {
 // range with U loads of 16 bytes in flight per lane; their merged state is the shard's state of that row.
 // No partials, no tickets.  (Wider slices use sweep_kernel with export_state set.)  Latency-bound: one warp folds a 32 KB row in
 // 16 rounds of loads, and 256 rows of 17 are fewer warps than the SMs hold (64 rows of 4 shards, V = 32,000: 18.4 us, several warps per row 16.4).
+// (Steps in flight: 5 of bf16, 4 of fp32 beside 4 CTAs per SM; one rank of 8 of 256 bf16 rows 54.3 us, with the sweep's shape 57.4.)
 template <typename T>
-__global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) shard_rows_kernel(const __grid_constant__ KParams P, const int row_warps) {
+__global__ void __launch_bounds__(kThreads, 4) shard_rows_kernel(const __grid_constant__ KParams P, const int row_warps) {
     __shared__ float4 sh_part[kWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long w = (static_cast<long long>(blockIdx.x) * kWarps + warp) / row_warps;
@@ -43,7 +44,7 @@ __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) shard_rows_ker
                                  : static_cast<const T*>(P.d) + static_cast<long long>(b) * P.dsb + static_cast<long long>(pos) * P.dsp;
         const GranRow gr = make_row(row, P.V);
         const int per = (gr.ng + row_warps - 1) / row_warps;
-        WarpSweep<T, SweepShape<T>::kSteps> ws;
+        WarpSweep<T, sizeof(T) == 2 ? 5 : 4> ws;
         ws.start(gr, sub * per, sub * per + per);
         if (!is_target && lane == 0 && sub == 0 && !greedy) {
             // both logits at the draft token, if it falls into this slice
