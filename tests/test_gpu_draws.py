@@ -14,7 +14,7 @@ from parity import compare_step, gpu_batch, mlp_pair, oracle_batch
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
-SIZES = [(300, 2, 700), (300, 2, 701), (3, 3, 20001), (40, 2, 151936), (300, 1, 33000), (2, 1, 1100003)]
+SIZES = [(300, 2, 700), (300, 2, 701), (3, 3, 20001), (40, 2, 151936), (300, 1, 33000), (2, 1, 1100003), (1, 1, 5000003)]
 
 
 def _workload(B, G, V, dtype, **kw):
