@@ -37,6 +37,11 @@ constexpr int kMaxGamma = 16;           // SPECKV_MAX_GAMMA
 template <typename T> struct SweepShape;
 template <> struct SweepShape<__nv_bfloat16> { static constexpr int kSteps = 4, kCtas = 5; };
 template <> struct SweepShape<float> { static constexpr int kSteps = 4, kCtas = 4; };
+// Every kernel is launched so that its CTAs may be placed as soon as all CTAs of the kernel in front of it in the stream have
+// called dependents_may_start() or ended.  It touches memory only behind wait_for_predecessors(), that is when that kernel has
+// ended and its writes are visible, and lets its own successor in after that, so what holds for one holds for the whole chain.
+__device__ __forceinline__ void wait_for_predecessors() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void dependents_may_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 constexpr float kFloor = -1.2676506002282294e30f;  // -2^100: logits below count as -inf
 constexpr uint32_t kFloorBf16x2 = 0xF180F180u;     // -2^100 as two bf16
 constexpr double kLn2 = 0.6931471805599453094;
@@ -1171,6 +1176,8 @@ __device__ __noinline__ void export_epilogue(const KParams& P, int b, int gam, f
 // Stand-alone controller: one warp per row.
 // ----------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(kThreads) select_gamma_kernel(const __grid_constant__ KParams P, const float* feat_in) {
+    wait_for_predecessors();
+    dependents_may_start();
     const int b = blockIdx.x * kWarps + (threadIdx.x >> 5);
     if (b >= P.B) return;
     float f4[4];

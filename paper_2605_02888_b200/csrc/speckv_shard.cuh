@@ -24,6 +24,8 @@ namespace speckv {
 template <typename T>
 __global__ void __launch_bounds__(kThreads, 4) shard_rows_kernel(const __grid_constant__ KParams P, const int row_warps) {
     __shared__ float4 sh_part[kWarps];
+    wait_for_predecessors();
+    dependents_may_start();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long w = (static_cast<long long>(blockIdx.x) * kWarps + warp) / row_warps;
     const int sub = warp % row_warps;
@@ -85,6 +87,8 @@ __global__ void __launch_bounds__(kThreads, 4) shard_rows_kernel(const __grid_co
 // dependent loads in each, the four calls of 256 rows and 8 shards took 12 us more (with the changes to phases 1 and 3).
 __global__ void __launch_bounds__(kThreads) shard_finish_kernel(const __grid_constant__ KParams P) {
     __shared__ RowDecide sh_pos[kMaxGamma + 1];
+    wait_for_predecessors();
+    dependents_may_start();
     const int b = blockIdx.x;
     const int gam = P.gamma ? P.gamma[b] : P.G;
     const float Tf = P.temp ? P.temp[b] : P.temp_scalar;
@@ -98,6 +102,8 @@ __global__ void __launch_bounds__(kThreads) shard_finish_kernel(const __grid_con
 template <typename T>
 __global__ void __launch_bounds__(kThreads, 4) shard_sums_kernel(const __grid_constant__ KParams P) {
     __shared__ int sh_flag;
+    wait_for_predecessors();
+    dependents_may_start();
     const int b = blockIdx.x / P.R;
     const int share = blockIdx.x - b * P.R;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -154,6 +160,8 @@ __global__ void __launch_bounds__(kThreads) shard_pick_kernel(const __grid_const
     __shared__ int sh_go;
     __shared__ int sh_mode;
     __shared__ double sh_tau;
+    wait_for_predecessors();
+    dependents_may_start();
     const int b = blockIdx.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const RowInfo ri = P.info[b];

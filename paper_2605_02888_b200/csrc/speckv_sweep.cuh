@@ -75,7 +75,8 @@ __device__ __forceinline__ PrepCounts shfl_up(const PrepCounts& v, int o) {
 }
 __global__ void __launch_bounds__(kThreads) prep_kernel(const __grid_constant__ KParams P, int seg) {
     __shared__ PrepCounts sh[2][kWarps];
-    asm volatile("griddepcontrol.launch_dependents;");  // the sweep's CTAs may be placed; they wait for this grid's end
+    wait_for_predecessors();
+    dependents_may_start();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int b0 = blockIdx.x * seg, b1 = min(P.B, b0 + seg);
     for (int b = b0 + threadIdx.x; b < b1; b += kThreads) {
@@ -173,7 +174,8 @@ __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sweep_kernel(c
     __shared__ int sh_last;
     __shared__ int sh_early;
     __shared__ float sh_m0[kWarps];
-    asm volatile("griddepcontrol.wait;" ::: "memory");  // the list and the cleared counters
+    wait_for_predecessors();  // the list and the cleared counters
+    dependents_may_start();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool verify = (P.mode & MODE_VERIFY) != 0;
     const int i = static_cast<int>(blockIdx.x) / P.nsplit, s = static_cast<int>(blockIdx.x) - i * P.nsplit;

@@ -70,3 +70,51 @@ def test_an_empty_residual_is_drawn_from_p(dtype, V):
     for b in range(B):  # fp32 weights: the threshold is known to about 1e-6 of the mass (tests/parity.py's window)
         lo, hi = np.searchsorted(cdf[b], u[b] - 1e-6, side="right"), np.searchsorted(cdf[b], u[b] + 1e-6, side="right")
         assert lo <= tok[b] <= hi, (b, lo, tok[b], hi)
+
+
+@pytest.mark.parametrize("B,G", [(1, 1), (256, 1), (911, 16), (3000, 16)])
+def test_sampling_clears_its_counters(B, G):
+    # fewer counters than one CTA clears, about a CTA's, just above and far above one pass of the clearing grid
+    w = _workload(B, G, 40, "fp32")
+    s = synth.make_step(w, 0, DEV)
+    u = torch.rand(B, G, device=DEV)
+    batch = gpu_batch(s)
+    a = speckv.speckv_sample_draft(batch, u, workspace=torch.zeros(1 << 27, dtype=torch.uint8, device=DEV))
+    b = speckv.speckv_sample_draft(batch, u, workspace=torch.full((1 << 27,), 0xFF, dtype=torch.uint8, device=DEV))
+    assert torch.equal(a["tokens"], b["tokens"]) and torch.equal(a["row_status"], b["row_status"])
+    assert ((b["tokens"] >= 0).sum(1) == s["gamma"]).all()
+
+
+def test_calls_wait_for_their_inputs():
+    # kernels that may be placed before their predecessor ends: inputs written right in front of each call, outputs read
+    # right behind it, calls of different sizes one after the other without a synchronisation between them
+    src = []
+    for k, (B, G, V) in enumerate([(1, 4, 32000), (64, 4, 32000), (16, 8, 50257), (3, 2, 2000), (200, 4, 32001)]):
+        w = _workload(B, G, V, "bf16" if k % 2 else "fp32")
+        src.append([synth.make_step(w, i, DEV) for i in range(3)])
+    gm, _ = mlp_pair(synth.make_mlp(w, DEV))
+
+    def call(s):
+        bt = gpu_batch(s)
+        sig = speckv.speckv_signals(bt)
+        got = [sig["feat"], speckv.speckv_select_gamma(sig["feat"], s["comp"], gm)["gamma_next"]]
+        s["draft_tokens"].copy_(speckv.speckv_sample_draft(bt, s["uniforms"][:, :s["draft"].shape[1], 0].contiguous())["tokens"])
+        r = speckv.speckv_step(bt, s["comp"], gm)
+        return [x.clone() for x in got + [s["draft_tokens"], r["out_tokens"], r["n_accepted"], r["feat"], r["gamma_next"]]]
+
+    def run(sync):
+        bufs = [{k: v.clone() for k, v in x[0].items() if torch.is_tensor(v)} for x in src]
+        outs = []
+        for rep in range(12):
+            for x, buf in zip(src, bufs):
+                for k, v in buf.items():
+                    v.copy_(x[rep % 3][k])
+                if sync:
+                    torch.cuda.synchronize()
+                outs.append(call(dict(x[0], **buf)))
+        torch.cuda.synchronize()
+        return outs
+
+    for a, b in zip(run(True), run(False)):
+        for x, y in zip(a, b):
+            assert torch.equal(x.nan_to_num(), y.nan_to_num())
