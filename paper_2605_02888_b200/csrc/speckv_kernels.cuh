@@ -273,20 +273,23 @@ __device__ __forceinline__ float raw_max(const Raw<float>& r) {
     return max_nan(a, b);
 }
 
-// Does any raw element exceed `m` (or is any NaN)?  `STRICT`: exceed means >, else >=.
-// For bf16 the test runs on packed pairs; `m` must be bf16-representable.
-template <bool STRICT>
+// Is any raw element >= m (or a NaN)?  For bf16 the test runs on packed pairs; m must be bf16-representable there.
 __device__ __forceinline__ bool raw_exceeds(const Raw<__nv_bfloat16>& r, float m) {
     __nv_bfloat162 mx = __hmax2_nan(__hmax2_nan(as_bf2(r.a.x), as_bf2(r.a.y)),
                                     __hmax2_nan(as_bf2(r.a.z), as_bf2(r.a.w)));
     uint32_t mb = __float_as_uint(m) >> 16;
-    __nv_bfloat162 m2 = as_bf2(mb | (mb << 16));
-    return STRICT ? !__hble2(mx, m2) : !__hblt2(mx, m2);
+    return !__hblt2(mx, as_bf2(mb | (mb << 16)));
 }
-template <bool STRICT>
-__device__ __forceinline__ bool raw_exceeds(const Raw<float>& r, float m) {
-    float mx = raw_max(r);
-    return STRICT ? !(mx <= m) : !(mx < m);
+__device__ __forceinline__ bool raw_exceeds(const Raw<float>& r, float m) { return !(raw_max(r) < m); }
+// The same for two at once.
+__device__ __forceinline__ bool raw_exceeds2(const Raw<__nv_bfloat16>& r, const Raw<__nv_bfloat16>& s, float m) {
+    const __nv_bfloat162 a = __hmax2_nan(__hmax2_nan(as_bf2(r.a.x), as_bf2(r.a.y)), __hmax2_nan(as_bf2(r.a.z), as_bf2(r.a.w)));
+    const __nv_bfloat162 b = __hmax2_nan(__hmax2_nan(as_bf2(s.a.x), as_bf2(s.a.y)), __hmax2_nan(as_bf2(s.a.z), as_bf2(s.a.w)));
+    const uint32_t u = as_u32(__hmax2_nan(a, b));
+    return !(max_nan(bf_lo(u), bf_hi(u)) < m);
+}
+__device__ __forceinline__ bool raw_exceeds2(const Raw<float>& r, const Raw<float>& s, float m) {
+    return !(max_nan(raw_max(r), raw_max(s)) < m);
 }
 
 // Clamp the raw elements from below at kFloor (NaN becomes kFloor as well).
@@ -369,11 +372,7 @@ struct DraftState {
     }
 
     template <typename T>
-    __device__ __forceinline__ void step(Raw<T> raw, float scale) {
-        if (raw_exceeds<false>(raw, m)) {  // an element >= m, or a NaN: rare after the warm start
-            slow<T>(raw, scale);
-            return;
-        }
+    __device__ __forceinline__ void add(Raw<T> raw, float scale) {  // all elements below m
         raw_floor(raw);
         f2 x[4];
         unpack_pairs(raw, x);
@@ -382,6 +381,27 @@ struct DraftState {
         const f2 e0 = ex2_2(y0), e1 = ex2_2(y1), e2 = ex2_2(y2), e3 = ex2_2(y3);
         za = add2(za, add2(add2(e0, e1), add2(e2, e3)));
         sa = add2(sa, fma2(e0, y0, fma2(e1, y1, fma2(e2, y2, mul2(e3, y3)))));
+    }
+    template <typename T>
+    __device__ __forceinline__ void step(const Raw<T>& raw, float scale) {
+        if (raw_exceeds(raw, m)) slow<T>(raw, scale);  // an element >= m, or a NaN: rare after the warm start
+        else add<T>(raw, scale);
+    }
+    // two steps with one test for both (for four the registers run out: signals of 128 bf16 rows, V = 128,256, 53 us; 48 this
+    // way; 50 with a test for each)
+    template <typename T>
+    __device__ __forceinline__ void step2(const Raw<T>& a, const Raw<T>& b, float scale) {
+        if (raw_exceeds2(a, b, m)) {
+#pragma unroll 1
+            for (int k = 0; k < 2; ++k) {
+                Raw<T> v = a;
+                if (k) v = b;
+                slow<T>(v, scale);
+            }
+        } else {
+            add<T>(a, scale);
+            add<T>(b, scale);
+        }
     }
     __device__ __forceinline__ float4 partial(float scale) const {
         const float d = fmaf(m, scale, -r), f = ex2f(-d), z = zsum();  // y against m itself is smaller by d, a rounding
@@ -453,7 +473,7 @@ struct ArgmaxState {
     // the two halves of kVec/2 elements start at vocabulary index ea and eb
     template <typename T>
     __device__ __forceinline__ void step(const Raw<T>& raw, int ea, int eb) {
-        if (!raw_exceeds<false>(raw, best)) return;
+        if (!raw_exceeds(raw, best)) return;
         float x[kVec];
         unpack<T>(raw, x);
 #pragma unroll
@@ -698,13 +718,19 @@ struct WarpSweep {
             };
             if (first_edge || last_edge) process(edge(), lane == 0 ? 0 : ng - 1);
             int i = 0;
+            // A step's registers are loaded again when it has been folded, not before: a copy of it to fold from is four registers
+            // more, and the 48 there are spilled (b256 and b1024 as above 137 / 432 us, this way with pairs of draft steps 134 / 414).
             for (; i + U <= n_main; i += U) {
 #pragma unroll
                 for (int k = 0; k < U; ++k) {
-                    const Raw<T> cur = buf[k];
-                    const int nx = i + U + k;
-                    if (nx < n_main) buf[k] = load(nx);
-                    process(cur, a + lane + 32 * GS * (i + k));
+                    if constexpr (PATH == PATH_DRAFT && U % 2 == 0) {
+                        if (k % 2) continue;
+                        ds.template step2<T>(buf[k], buf[k + 1], scale);
+                        if (i + U + k + 1 < n_main) buf[k + 1] = load(i + U + k + 1);
+                    } else {
+                        process(buf[k], a + lane + 32 * GS * (i + k));
+                    }
+                    if (i + U + k < n_main) buf[k] = load(i + U + k);
                 }
             }
 #pragma unroll

@@ -67,3 +67,25 @@ def test_target_elements_far_above_the_reference(dtype, jump):
             s["draft"][b] = s["target"][b, :3]
             s["draft_tokens"][b] = 20000 + 4001 * b
     _check(s, w)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5, 7, 8, 9, 17])
+def test_draft_maxima_and_nans_in_every_step(dtype, n):
+    # n steps per lane (pairs of them share a test for a new maximum): a maximum, a tie with it, or a NaN in each step of a lane
+    step = 256 * 8 * n
+    w = synth.Workload("g", B=2 * n + 1, gamma_max=3, V=step, dtype=dtype, gamma_mode="fixed", gamma_fixed=3, temperature=1.0,
+                       sigma_d=(0.5,), seed=n)
+    s = synth.make_step(w, 0, DEV)
+    for b in range(2 * n):
+        k = (b // 2) * 256 + 37 + b % 2
+        s["draft"][b, 0, k] = 30.0
+        s["draft"][b, 1, k] = 30.0
+        s["draft"][b, 1, (k + 1) % step] = 30.0
+        s["draft"][b, 1, (k + 300) % step] = 30.0
+        s["draft"][b, 2, k: k + 700: 256] = 20.0 + torch.arange(s["draft"][b, 2, k: k + 700: 256].numel(), device=DEV).to(s["draft"].dtype)
+    _check(s, w)
+    s["draft"][0, 0, (n - 1) * 256 + 5] = float("nan")
+    s["draft"][1, 2, (n // 2) * 256 + 5] = float("inf")
+    st = _check(s, w)["row_status"].cpu().numpy()
+    assert (st[:2] == 4).all() and (st[2:] == 0).all()
