@@ -64,14 +64,16 @@ __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sample_kernel(
         if (lane == 0) SPECKV_ST(spans[s * kWarps + warp], v);
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        const bool last = atomicAdd(P.tick1 + r, 1) == P.nsplit - 1;
-        if (last) __threadfence();
-        sh_last = last;
+    if (P.nsplit > 1) {  // else this CTA is the row's last: no ticket (256 bf16 rows, V = 128,256: 73.4 us with it, 71.3 without)
+        if (threadIdx.x == 0) {
+            __threadfence();
+            const bool last = atomicAdd(P.tick1 + r, 1) == P.nsplit - 1;
+            if (last) __threadfence();
+            sh_last = last;
+        }
+        __syncthreads();
+        if (!sh_last) return;
     }
-    __syncthreads();
-    if (!sh_last) return;
 
     // ---- the row's last CTA ----
     int tok = -1;
