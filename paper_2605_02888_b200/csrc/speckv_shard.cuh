@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(kThreads, 4) shard_sums_kernel(const __grid_co
     tr = warp_sum(tr);
     tp = warp_sum(tp);
     if (lane == 0) {
-        P.weight[2 * static_cast<long long>(b)] = tr;
+        P.weight[2 * static_cast<long long>(b)] = res ? tr : 0.0;  // a bonus row has no residual
         P.weight[2 * static_cast<long long>(b) + 1] = tp;
     }
 }

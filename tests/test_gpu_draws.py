@@ -8,7 +8,7 @@ import torch
 
 import oracle
 import paper_2605_02888_b200 as speckv
-from paper_2605_02888_b200 import synth
+from paper_2605_02888_b200 import synth, vocab_shard
 
 from parity import compare_step, gpu_batch, mlp_pair, oracle_batch
 
@@ -118,3 +118,40 @@ def test_calls_wait_for_their_inputs():
     for a, b in zip(run(True), run(False)):
         for x, y in zip(a, b):
             assert torch.equal(x.nan_to_num(), y.nan_to_num())
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("n,V", [(1, 3000), (2, 40001), (4, 40000)])
+def test_shard_masses(dtype, n, V):
+    # a rank's two masses at the stop position: of max(0, p - q) (0 where a bonus token is drawn) and of p
+    B, G = 40, 2
+    w = _workload(B, G, V, dtype, frac_identical=0.4)
+    s = synth.make_step(w, 0, DEV)
+    s["temperature"][::7] = 0.0
+    full = gpu_batch(s)
+    gm, _ = mlp_pair(synth.make_mlp(w, DEV))
+    width, bounds = vocab_shard.shard_bounds(V, n)
+    parts = [vocab_shard.slice_batch(full, a, e) for a, e in bounds]
+    bufs = [vocab_shard.ShardBuffers.allocate(p, n, 4) for p in parts]
+    for r, (p, o) in enumerate(zip(parts, bufs)):
+        speckv.speckv_shard_sweep(p, bounds[r][0], o.state, o.tokl, o.workspace)
+        bufs[0].all_state[r].copy_(o.state)
+        bufs[0].all_tokl[r].copy_(o.tokl)
+    o = bufs[0]
+    speckv.speckv_shard_finish(parts[0], n, width, V, o.all_state, o.all_tokl, s["comp"], gm, o.out, o.row_info)
+    stop = o.out.as_dict()["n_accepted"].long().cpu().numpy()
+    for r, p in enumerate(parts):
+        a, e = bounds[r]
+        bufs[r].weight.fill_(7.0)
+        speckv.speckv_shard_draw_sums(p, o.row_info, bufs[r].weight, bufs[r].workspace)
+        got = bufs[r].weight.cpu().numpy()
+        for b in range(B):
+            T, k, g = float(s["temperature"][b]), int(stop[b]), int(s["gamma"][b])
+            want = np.zeros(2)
+            if T > 0:
+                pt = torch.softmax(s["target"][b, k].double() / T, 0)
+                want[1] = pt[a:e].sum()
+                if k < g:
+                    want[0] = (pt - torch.softmax(s["draft"][b, k].double() / T, 0)).clamp(min=0)[a:e].sum()
+            # fp32 exponentials of fp32 arguments of up to ~30: 2e-6 of the mass of p, in differences too
+            assert np.abs(got[b] - want).max() <= 5e-6 * max(want[1], 1e-3), (b, got[b], want)
