@@ -19,8 +19,8 @@
  *   - Every data pointer is DEVICE memory owned by the caller.  The struct arguments
  *     themselves (speckv_batch, speckv_mlp) are HOST structs holding device pointers.
  *   - Logit tensors are row-major with the vocabulary dimension contiguous; strides are
- *     counted in ELEMENTS.  The fast path needs 16-byte aligned base pointers and row strides
- *     that are multiples of 16 bytes; anything else takes a slower element-wise path.
+ *     counted in ELEMENTS.  Rows may start at any element: they are read in 16-byte pieces of the
+ *     address space, only a piece shared with a neighbouring row element by element.
  *   - The library allocates nothing and never synchronises; work is enqueued on the
  *     caller's stream (a cudaStream_t passed as void*).  Scratch memory comes from the
  *     caller: speckv_workspace_size() bytes,
