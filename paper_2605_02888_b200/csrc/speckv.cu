@@ -83,12 +83,15 @@ void choose_slices(KParams& P, speckv_dtype dt, bool aligned) {
     const long long want = (slots + rows - 1) / (rows > 0 ? rows : 1);
     if (want > ns) ns = static_cast<int>(want > kMaxSplit ? kMaxSplit : want);
     if (ns > kMaxSplit) ns = kMaxSplit;
-    // At least one granule per lane; short ranges are whole rounds of the warp (a round with idle lanes costs as much as a
-    // full one), long ones keep to 128-byte lines.  Rounding down makes more slices: only where they still fit the small-batch
-    // count (500 rows of V = 3,000, bf16, gamma 4: 52 us with one slice per logit row, 68 us with two).
+    // At least one granule per lane, and whole steps of the warp: one with idle lanes costs as much as a full one, and lanes
+    // that differ in their number of steps part in the last round of the loop (ranges of 128-byte lines before: step of 64 bf16
+    // rows, V = 32,000, 30.2 us, this way 29.3; of 256 fp32 rows, V = 128,256, 226.5 / 222.8; draft sampling of those 113.2 / 110.9).
+    // Rounding down makes more slices: only where they still fit the small-batch count (500 rows of V = 3,000, bf16, gamma 4:
+    // 52 us with one slice per logit row, 68 us with two).
     int pw = (ng + ns * kWarps - 1) / (ns * kWarps);
     const int near = (pw + 16) / 32 * 32 < 32 ? 32 : (pw + 16) / 32 * 32;
-    if (pw >= 256) pw = (pw + 7) / 8 * 8;
+    const int step = 32 * (kVec / E);
+    if (pw >= 256) pw = (pw + step - 1) / step * step;
     else if (((ng + near * kWarps - 1) / (near * kWarps)) * rows <= slots + rows) pw = near;
     else pw = (pw + 31) / 32 * 32;
     while ((ng + pw * kWarps - 1) / (pw * kWarps) > kMaxSplit) pw += 32;
