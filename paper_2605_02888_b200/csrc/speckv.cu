@@ -86,8 +86,8 @@ void choose_slices(KParams& P, speckv_dtype dt, bool aligned) {
     // At least one granule per lane, and whole steps of the warp: one with idle lanes costs as much as a full one, and lanes
     // that differ in their number of steps part in the last round of the loop (ranges of 128-byte lines before: step of 64 bf16
     // rows, V = 32,000, 30.2 us, this way 29.3; of 256 fp32 rows, V = 128,256, 226.5 / 222.8; draft sampling of those 113.2 / 110.9).
-    // Rounding down makes more slices: only where they still fit the small-batch count (500 rows of V = 3,000, bf16, gamma 4:
-    // 52 us with one slice per logit row, 68 us with two).
+    // Rounding down makes more slices: only where they still fit the small-batch count (500 rows of V = 3,000, bf16, gamma 4, when
+    // the sweep took them: 52 us with one slice per logit row, 68 us with two).
     int pw = (ng + ns * kWarps - 1) / (ns * kWarps);
     const int near = (pw + 16) / 32 * 32 < 32 ? 32 : (pw + 16) / 32 * 32;
     const int step = 32 * (kVec / E);
@@ -116,6 +116,25 @@ void choose_draw(KParams& P, speckv_dtype dt, bool aligned) {
     if (R > kMaxShares) R = kMaxShares;
     P.draw_pw = ((ng + R * kWarps - 1) / (R * kWarps) + 7) / 8 * 8;
     P.R = (ng + P.draw_pw * kWarps - 1) / (P.draw_pw * kWarps);
+}
+
+// Short rows: one CTA per batch row (batch_row_kernel) with P.nsplit warps per logit row, as many as leave none without work.
+// The limits lie where the CTA's time, which grows with the length of its rows, meets that of a CTA per logit row, which
+// grows with their number.  Step, gamma up to 8, bf16 / fp32, sweep -> this way: 64 rows, V = 4,000, 21.5 -> 19.7 / 22.6 -> 21.7 us
+// and V = 8,000 23.0 -> 26.8 / 25.6 -> 38.0; 256 rows, V = 8,000, 41.5 -> 36.5 / 49.4 -> 44.0 and V = 16,000 48.0 -> 55.5 / 97 -> 103
+// (of 500); 1,000 rows, V = 3,000, 112 -> 63 / 129 -> 62.
+constexpr int kShortRow = 4096, kShortRowLarge = 8192, kShortRowBatch = 256;
+bool choose_batch_rows(KParams& P, speckv_dtype dt, bool aligned) {
+    if (P.V > (P.B >= kShortRowBatch ? kShortRowLarge : kShortRow)) return false;
+    const int E = 16 / esize(dt);
+    const int ng = (P.V + E - 1 + (aligned ? 0 : E - 1)) / E;
+    P.nsplit = 1;
+    while (P.J * P.nsplit * 2 <= kWarps) P.nsplit *= 2;
+    P.n_spans = P.nsplit;
+    P.per_warp = (ng + P.nsplit - 1) / P.nsplit;
+    P.R = 1;
+    P.draw_pw = (ng + kWarps - 1) / kWarps;
+    return true;
 }
 
 Plan make_plan(const speckv_batch* bt) {
@@ -237,6 +256,16 @@ cudaError_t launch_all(const KParams& P, cudaStream_t st, const Events& ev) {
     return e;
 }
 
+// A short row's batch in one launch.
+template <typename T>
+cudaError_t launch_rows(const KParams& P, cudaStream_t st, const Events& ev) {
+    if (ev.before_sweep) cudaEventRecord(ev.before_sweep, st);
+    const cudaError_t e = launch(batch_row_kernel<T>, static_cast<unsigned>(P.B), st, P);
+    if (ev.after_sweep) cudaEventRecord(ev.after_sweep, st);
+    if (ev.after_resample) cudaEventRecord(ev.after_resample, st);
+    return e;
+}
+
 // Shared driver of signals / verify / step.
 speckv_status run(const speckv_batch* bt, int mode, const float* comp, const speckv_mlp* mlp, float* H,
                   float* C, float* feat, float* scores, int32_t* gamma_next, int32_t* n_accepted,
@@ -264,6 +293,8 @@ speckv_status run(const speckv_batch* bt, int mode, const float* comp, const spe
     if (verify) aligned = aligned && rows_aligned(bt->target_logits, bt->target_stride_b, bt->target_stride_pos, es);
     choose_slices(P, bt->dtype, aligned);
     choose_draw(P, bt->dtype, aligned);
+    P.n_spans = P.nsplit * kWarps;
+    const bool by_row = choose_batch_rows(P, bt->dtype, aligned);
     P.mode = mode; P.bits = bt->entropy_in_bits ? 1 : 0;
     P.wait_limit = g_wait_limit.load(std::memory_order_relaxed);
     P.d = bt->draft_logits; P.dsb = bt->draft_stride_b; P.dsp = bt->draft_stride_pos;
@@ -289,6 +320,12 @@ speckv_status run(const speckv_batch* bt, int mode, const float* comp, const spe
     if (dbg_register(cs, bt, verify, ws, ws_bytes) != cudaSuccess) return SPECKV_ERR_CUDA;
     // signals: behind their partials, which take a third of that region; verification: a region of its own
     P.list = reinterpret_cast<int2*>(verify ? w + pl.off_list : reinterpret_cast<char*>(P.part + static_cast<size_t>(P.B) * P.J * P.nsplit));
+    if (by_row) {
+        P.tokl = reinterpret_cast<float2*>(w + pl.off_tokl);
+        P.spans = verify ? reinterpret_cast<float2*>(w + pl.off_spans) : nullptr;
+        const cudaError_t e = bt->dtype == SPECKV_BF16 ? launch_rows<__nv_bfloat16>(P, cs, ev) : launch_rows<float>(P, cs, ev);
+        return e == cudaSuccess ? SPECKV_OK : SPECKV_ERR_CUDA;
+    }
     if (verify) {
         P.rdone = P.n_list + 4;
         P.tokl = reinterpret_cast<float2*>(w + pl.off_tokl);

@@ -510,14 +510,16 @@ __device__ __forceinline__ void resample_row(const KParams& P, const int b, cons
         if (lane == 0) SPECKV_ST(dsum[span], w);
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        const bool last = atomicAdd(P.tick2 + b, 1) == P.R - 1;
-        if (last) __threadfence();
-        sh_flag = last;
+    if (P.R > 1) {
+        if (threadIdx.x == 0) {
+            __threadfence();
+            const bool last = atomicAdd(P.tick2 + b, 1) == P.R - 1;
+            if (last) __threadfence();
+            sh_flag = last;
+        }
+        __syncthreads();
+        if (!sh_flag) return;
     }
-    __syncthreads();
-    if (!sh_flag) return;
 
     // ---- last CTA of the row: locate the threshold (every warp picks the span, redundantly) ----
     const RowInfo ri = row_info_load(P.info + b);

@@ -93,6 +93,7 @@ static_assert(sizeof(RowInfo) == 32, "the resample kernel reads a RowInfo as two
 struct KParams {
     int B, G, V, J, nsplit, R, mode, bits;
     int per_warp;  // sweep kernel: 16-byte granules of a logit row that one warp folds; a slice is kWarps times that
+    int n_spans;    // verification: spans per batch row
     int2* list;     // sliced sweep: one entry per logit row to sweep, in the order of the grid (prep_kernel)
     int* n_list;    //   and how many there are; CTAs behind the last one draw
     int n_draw;     // sliced sweep: CTAs that may draw (R per batch row), 0 = none
