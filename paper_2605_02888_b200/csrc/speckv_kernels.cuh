@@ -328,7 +328,7 @@ __device__ __forceinline__ void raw_floor(Raw<float>& r) {
 // ----------------------------------------------------------------------------------------
 struct DraftState {
     float m, r, cnt;
-    f2 za, sa;  // four running sums each of Zx and of 2^y * y, y = x * scale - r, as two packed pairs
+    f2 za, sa;  // two running sums each of Zx and of 2^y * y, y = x * scale - r
     bool bad;
     __device__ __forceinline__ void init(float m0, float scale) {
         m = m0; r = __fmul_rn(m0, scale); cnt = 0.f; bad = false;
@@ -354,6 +354,7 @@ struct DraftState {
             const float y = fmaf(m, scale, -r), zc = cnt * ex2f(y);  // the elements equal to the old maximum join the sums
             sv = fmaf(dr, zc + z, fmaf(zc, y, sv)) * f;
             z = (zc + z) * f;
+            if (f == 0.f) sv = 0.f;  // a product with dr, which behind masked elements is about 2^100 * scale, may be infinite
             cnt = 0.f;
             m = vmax;
             r = rn;

@@ -1,0 +1,77 @@
+"""Logits and temperatures at the ends of their range: long masked stretches in front of the first allowed token, temperatures
+far below one, logits in the billions.  Every row of a batch reads the same logits (row stride 0), so that the kernels see
+the shapes of a large batch (one CTA or one warp per logit row) and the oracle only a few rows."""
+import math
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2605_02888_b200 as speckv
+from paper_2605_02888_b200 import synth, vocab_shard
+
+from parity import compare_step, gpu_batch, mlp_pair, oracle_batch
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+TYPES = {"bf16": torch.bfloat16, "fp32": torch.float32}
+
+
+def _shared_rows(draft, target, B, T, seed=0):
+    """B batch rows over one [G, V] draft and one [G + 1, V] target; the drafted tokens are the draft's first maxima."""
+    G = draft.shape[0]
+    g = torch.Generator(device=DEV).manual_seed(seed)
+    tok = draft.float().argmax(-1).to(torch.int32)
+    return dict(draft=draft[None].expand(B, -1, -1), target=target[None].expand(B, -1, -1),
+                draft_tokens=tok[None].expand(B, -1).contiguous(), gamma=torch.full((B,), G, dtype=torch.int32, device=DEV),
+                temperature=torch.full((B,), T, device=DEV), uniforms=torch.rand(B, G + 1, 2, generator=g, device=DEV),
+                comp=torch.zeros(B, 2, device=DEV))
+
+
+def _oracle(s, rows, om):
+    sub = {k: v[torch.as_tensor(rows, device=DEV)] for k, v in s.items()}
+    return oracle.step(oracle_batch(sub), sub["comp"].cpu().numpy(), om)
+
+
+def _check(s, n_shards=0):
+    B, G = s["draft_tokens"].shape
+    rows = np.unique(np.linspace(0, B - 1, 12).astype(int))
+    gm, om = mlp_pair(synth.make_mlp(synth.Workload("r", B=1, gamma_max=G, V=8, seed=1), DEV))
+    ref = _oracle(s, rows, om)
+    if n_shards:
+        out = vocab_shard.step_emulated(gpu_batch(s), n_shards, s["comp"], gm)
+    else:
+        out = speckv.speckv_step(gpu_batch(s), s["comp"], gm)
+        sig = speckv.speckv_signals(gpu_batch(s))
+        assert torch.equal(sig["row_status"], out["row_status"])
+        for k in ("H", "C"):
+            np.testing.assert_allclose(sig[k][rows].cpu().numpy(), ref[k], rtol=1e-5, atol=1e-7, err_msg=k)
+    torch.cuda.synchronize()
+    compare_step(out, ref, rows=rows)
+    return out, ref
+
+
+# (rows, positions, vocabulary, shards): a lane folds up to 256 elements of a row (short rows, one warp each), 390 to 510
+# (the sweep, one CTA per row or per half of an fp32 row), 512 of a slice (one warp per sharded row, two shards)
+MASKED = [(256, 4, 8192, 0), (180, 4, 100000, 0), (180, 4, 130999, 0), (560, 4, 32768, 2)]
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("B,G,V,n_shards", MASKED)
+@pytest.mark.parametrize("T", [1e-6, 2e-6, 0.8])
+def test_masked_stretch_before_the_first_allowed_token(dtype, B, G, V, n_shards, T):
+    # constrained decoding: everything but a few tokens is -inf, and those stand at the end of the row
+    ninf = float("-inf")
+    draft = torch.full((G, V), ninf, device=DEV)
+    draft[0, -3:] = torch.tensor([5.0, 5.0, 3.0], device=DEV)      # two tied maxima: H = ln 2 for T near 0
+    draft[1, -2] = -1.0                                            # one allowed token
+    draft[2, -7:] = 2.0                                            # seven tied maxima
+    draft[3, -1] = 5.0                                             # and one in front of the masked stretch
+    draft[3, 1] = 5.0
+    target = torch.full((G + 1, V), ninf, device=DEV)
+    target[:, -7:] = torch.tensor([1.0, 4.0, 4.0, 4.0, 4.0, 4.0, 4.0], device=DEV)
+    out, ref = _check(_shared_rows(draft.to(TYPES[dtype]), target.to(TYPES[dtype]), B, T, seed=V), n_shards)
+    assert (ref["row_status"] == 0).all()
+    if T < 1e-3:
+        np.testing.assert_allclose(ref["H"][0], [math.log(2), 0.0, math.log(7), math.log(2)], atol=1e-9)
