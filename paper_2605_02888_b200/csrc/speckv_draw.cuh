@@ -29,6 +29,8 @@ struct DrawSrc {
     float scale, lp, lq, c;  // log2(e) / T, the log2-normalisers rounded to fp32, and what the rounding took from them:
                              // p - q = (2^(x_t * scale - lp) - c * 2^(x_d * scale - lq)) * 2^(lp - lse_p), c = 2^((lq - lse_q) - (lp - lse_p));
                              // the last factor is common to all weights and left out
+    bool wide;               // normalisers so large that their rounding is not small: the weights take it exactly
+    float plo, qlo;          // wide: lse_p - lp and lse_q - lq
     int r0, r1;              // draw_from_spans: the chosen span (r1 <= r0: there is none)
     double tau;
 };
@@ -51,7 +53,13 @@ __device__ __forceinline__ void set_norm(DrawSrc& s, float scale, double lse_p, 
     s.scale = scale;
     s.lp = static_cast<float>(lse_p);
     s.lq = static_cast<float>(lse_q);
+    s.plo = static_cast<float>(lse_p - static_cast<double>(s.lp));
+    s.qlo = static_cast<float>(lse_q - static_cast<double>(s.lq));
     s.c = ex2f(static_cast<float>((static_cast<double>(s.lq) - lse_q) - (static_cast<double>(s.lp) - lse_p)));
+    // Left out, the common factor is within 2^(1/64) of one (normalisers below 2^19); the two masses that are compared with a
+    // constant (1e-6) and with each other over shards need no more.  At 2^28, the logits of a few hundred at T = 1e-6 or 2e8
+    // at T = 1, it would be 2^16 and a residual of any mass could pass for empty.
+    s.wide = fmaxf(fabsf(s.plo), fabsf(s.qlo)) > 0x1p-6f;
 }
 
 // ---- weights of one granule ------------------------------------------------------------------------------
@@ -86,6 +94,24 @@ __device__ __forceinline__ void gran_weights(float scale, float lp, float lq, fl
             w[2 * i] = fmaxf(lo, 0.f);
             w[2 * i + 1] = fmaxf(hi, 0.f);
         }
+    }
+}
+// The same for normalisers of any size; rarely taken.
+template <typename T, bool RES>
+__device__ __forceinline__ void gran_weights_wide(const DrawSrc& s, const uint4& t, const uint4& d, float (&w)[16 / sizeof(T)],
+                                                  float* sum_p = nullptr) {
+    constexpr int NP = 8 / sizeof(T);
+    const f2 sc2 = pack2(s.scale, s.scale), ph = pack2(-s.lp, -s.lp), pl = pack2(s.plo, s.plo), qh = pack2(-s.lq, -s.lq), ql = pack2(s.qlo, s.qlo);
+    f2 xt[NP], xd[NP];
+    gran_pairs(t, xt);
+    if (RES) gran_pairs(d, xd);
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+        const f2 p = ex2_2(sub2(fma2(xt[i], sc2, ph), pl));
+        if (sum_p) *sum_p += hsum2(p);
+        unpack2(RES ? sub2(p, ex2_2(sub2(fma2(xd[i], sc2, qh), ql))) : p, w[2 * i], w[2 * i + 1]);
+        w[2 * i] = fmaxf(w[2 * i], 0.f);
+        w[2 * i + 1] = fmaxf(w[2 * i + 1], 0.f);
     }
 }
 template <typename T, bool RES>
@@ -134,8 +160,8 @@ __device__ __forceinline__ uint4 draft_any(const DrawSrc& s, int g) {  // the dr
     const uint4 a = gran_any<T>(s.d, g + s.dg);
     return s.off ? gran_shift<T>(a, gran_any<T>(s.d, g + s.dg + 1), s.off) : a;
 }
-// The lane's granule g of both rows; those at or behind g1 have no weight.
-template <typename T, bool RES>
+// The lane's granule g of both rows; those at or behind g1 have no weight.  WIDE: normalisers of any size (s.wide).
+template <typename T, bool RES, bool WIDE = true>
 __device__ __forceinline__ void load_weights(const DrawSrc& s, int g, int g1, float (&w)[16 / sizeof(T)]) {
     uint4 t = gran_fill<T>(__int_as_float(0xff800000)), d = t;
     if (g < g1) {
@@ -148,7 +174,8 @@ __device__ __forceinline__ void load_weights(const DrawSrc& s, int g, int g1, fl
             if (RES) d = draft_any<T>(s, g);
         }
     }
-    gran_weights<T, RES>(s.scale, s.lp, s.lq, s.c, t, d, w);
+    if (WIDE && s.wide) gran_weights_wide<T, RES>(s, t, d, w);
+    else gran_weights<T, RES>(s.scale, s.lp, s.lq, s.c, t, d, w);
 }
 template <typename T, bool RES>
 __device__ __noinline__ double gran_weight_any(const DrawSrc s, int g) {
@@ -191,6 +218,24 @@ __device__ __noinline__ double2 span_weight(const uint4* pt, const uint4* pd, in
     DrawSrc s;
     set_norm(s, __int_as_float(lo.w), __hiloint2double(hi.y, hi.x), __hiloint2double(hi.w, hi.z));
     double2 acc = make_double2(0.0, 0.0);
+    if (s.wide) {  // from the start again, a granule at a time
+        n += 32 * KU;
+        pt -= 32 * KU;
+        pd -= 32 * KU;
+        for (; n > 0; n -= 32, pt += 32, pd += 32) {
+            const uint4 a = ldg_stream(pt);
+            uint4 b = a;
+            if (RES) b = ldg_stream(pd);
+            if (RES && SHIFTED) b = gran_shift<T>(b, ldg_stream(pd + 1), off);
+            float w[16 / sizeof(T)], wp = 0.f, sum = 0.f;
+            gran_weights_wide<T, RES>(s, a, b, w, WITH_P ? &wp : nullptr);
+#pragma unroll
+            for (int j = 0; j < static_cast<int>(16 / sizeof(T)); ++j) sum += w[j];
+            acc.x += static_cast<double>(sum);
+            if (WITH_P) acc.y += static_cast<double>(wp);
+        }
+        return acc;
+    }
     for (;;) {
         float w = 0.f, wp = 0.f;
 #pragma unroll
@@ -328,7 +373,7 @@ __device__ __noinline__ int find_token(const DrawSrc& s, int g0, int g1, double 
             for (int j = 0; j < E; ++j) a += static_cast<double>(w[j]);
             a = warp_sum(a);
             if (lane == 0 && wi < cnt) sh[wi] = a;
-        } else if (!RES && sub == 32) {  // four parts at a time: one round trip for them
+        } else if (!RES && sub == 32 && !s.wide) {  // four parts at a time: one round trip for them
             for (int k = wi; k < cnt; k += 4 * nw) {
                 uint4 t[4];
 #pragma unroll
@@ -419,7 +464,7 @@ __device__ __forceinline__ int draw_from_spans(const T* row, int V, float scale,
         const bool none = __any_sync(0xffffffffu, bad) || own < 0;
         if (lane == 0) {
             DrawSrc s = make_draw<T>(row, nullptr, V);
-            set_norm(s, scale, static_cast<double>(R), 0.0);
+            set_norm(s, scale, static_cast<double>(R), 0.0);  // an fp32 value: exact whatever its size
             s.r0 = none ? 0 : own * per_warp;
             s.r1 = none ? 0 : min(s.t.ng, s.r0 + per_warp);
             s.tau = tau - before;
@@ -433,7 +478,7 @@ __device__ __forceinline__ int draw_from_spans(const T* row, int V, float scale,
     const int cnt = (g1 - g0 + 31) >> 5;  // parts of one granule per lane
     float w[16 / sizeof(T)];
     if (cnt <= nw) {  // one per warp: the warp that holds the token has its weights at hand
-        load_weights<T, false>(*sh_src, g0 + wi * 32 + lane, g1, w);
+        load_weights<T, false, false>(*sh_src, g0 + wi * 32 + lane, g1, w);
         double a = 0.0;
 #pragma unroll
         for (int j = 0; j < static_cast<int>(16 / sizeof(T)); ++j) a += static_cast<double>(w[j]);
@@ -484,7 +529,7 @@ __device__ __forceinline__ int draw_from_spans(const T* row, int V, float scale,
     double before = 0.0, total, tau;
     const int own = pick_many<false, 2>(cnt, [&](int i) { return sh[i]; }, sh_src->tau, &before, &total, &tau);
     if (own < 0) return -1;
-    load_weights<T, false>(*sh_src, g0 + own * 32 + lane, g1, w);
+    load_weights<T, false, false>(*sh_src, g0 + own * 32 + lane, g1, w);
     return scan_weights<T>(*sh_src, g0 + own * 32, w, tau - before);
 }
 

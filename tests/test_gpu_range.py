@@ -75,3 +75,23 @@ def test_masked_stretch_before_the_first_allowed_token(dtype, B, G, V, n_shards,
     assert (ref["row_status"] == 0).all()
     if T < 1e-3:
         np.testing.assert_allclose(ref["H"][0], [math.log(2), 0.0, math.log(7), math.log(2)], atol=1e-9)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("V,n_shards", [(4096, 0), (40001, 0), (33000, 3)])
+@pytest.mark.parametrize("T,level", [(0.9, 0.0), (0.9, 3.0e4), (1e-6, 100.0), (1e-6, 416.0), (1e-6, -416.0), (1e-6, 960.0)])
+def test_residual_of_two_tied_tokens(dtype, V, n_shards, T, level):
+    # p has two equal maxima and q only the first of them: the residual is the second one alone, whatever the common level
+    # of the logits, and its mass of 1/2 must not be taken for an empty one.  Half of the rows reject.  (At T = 1e-6 the
+    # normaliser of a row around 416 is 6.0e8 in log2 units and 31 above the nearest fp32 value below it; around 960 it is 63.)
+    B, a, b = 40, V // 3, V - 5
+    draft = torch.full((1, V), level - 200.0, device=DEV)
+    target = draft.expand(2, -1).clone()
+    draft[0, a] = level
+    target[0, a] = target[0, b] = level
+    s = _shared_rows(draft.to(TYPES[dtype]), target.to(TYPES[dtype]), B, T, seed=7)
+    s["uniforms"][:, 0, 0] = torch.linspace(0.02, 0.98, B, device=DEV)
+    s["uniforms"][:, 0, 1] = torch.linspace(0.03, 0.97, B, device=DEV).flip(0)
+    out, ref = _check(s, n_shards)
+    rejected = out["n_accepted"] == 0
+    assert 10 < int(rejected.sum()) < 30 and (out["out_tokens"][rejected, 0] == b).all()
