@@ -37,6 +37,9 @@
  *     (Sec. 3.1) and flag nothing.
  *   - Temperature: 0 selects the greedy rule (and T = 1 for that row's signals); otherwise
  *     finite and >= 1e-6.
+ *   - |logit| / T: any size in the draft signals.  Target rows and rows that a token is sampled from keep the sum of
+ *     their exponentials against an fp32 reference in log2 units; from about 1e9 on that reference can be so far from the
+ *     row's maximum that the sum overflows, and the row is flagged SPECKV_ROW_NONFINITE.
  */
 #ifndef SPECKV_H
 #define SPECKV_H

@@ -126,13 +126,6 @@ __device__ __forceinline__ float gran_weight(float scale, float lp, float lq, fl
 }
 
 // ---- granules that are not whole, and rows that sit differently on the 16-byte grid -------------------------
-template <typename T>
-__device__ __forceinline__ uint4 gran_any(const GranRow& r, int g) {  // outside the row: -inf, that is weight 0
-    const float ninf = __int_as_float(0xff800000);
-    if (g < 0 || g >= r.ng) return gran_fill<T>(ninf);
-    if (g < r.whole_lo() || g >= r.whole_hi()) return gran_edge<T>(r, g, ninf);
-    return ldg_stream(r.base + g);
-}
 // elements off, off + 1, ... of the 2 * E elements in a and b
 template <typename T>
 __device__ __forceinline__ uint4 gran_shift(const uint4& a, const uint4& b, int off) {

@@ -321,7 +321,9 @@ __device__ __forceinline__ void raw_floor(Raw<float>& r) {
 //         Z = cnt + Zx; entropy (nats) = ln Z - ln2*scale*S/Z; confidence = 1/Z  (Sec. 4.2).
 //         cnt = NaN marks a NaN / +inf input.
 //         While it sweeps, a thread keeps its sums against r = fl(m * scale), so that an element's exponent is one
-//         fused multiply-add; partial() moves them to m itself.
+//         fused multiply-add; partial() moves them to m itself.  That needs r close to m * scale: where it is not (far(): the
+//         rounding of |r| > 2^28 is up to 2^5 and more, or kFloor * scale overflows) the warp's range is folded again by
+//         draft_far(), from differences of logits.
 // TARGET  a = r (reference, log2 units), b = Z = sum 2^(x*scale - r); c,d unused.  Any r serves that keeps the sum in
 //         range; it is not the maximum.  NaN / +inf inputs surface as a non-finite Z.
 // ARGMAX  a = best value, b = index (bit pattern), c = bad flag (non-zero: NaN / +inf seen).
@@ -404,6 +406,10 @@ struct DraftState {
             add<T>(a, scale);
             add<T>(b, scale);
         }
+    }
+    // Sums that are not to be used: see above.  A maximum far below zero that was left behind shows in what it did to them.
+    __device__ __forceinline__ bool far(const float4& part, float scale) const {
+        return !bad && (scale > 0x1p27f || (m > kFloor && !(fabsf(r) <= 0x1p28f)) || !(fabsf(part.z) + fabsf(part.w) < __int_as_float(0x7f800000)));
     }
     __device__ __forceinline__ float4 partial(float scale) const {
         const float d = fmaf(m, scale, -r), f = ex2f(-d), z = zsum();  // y against m itself is smaller by d, a rounding
@@ -606,6 +612,48 @@ __device__ __noinline__ uint4 gran_edge(const GranRow r, int g, float pad) {
     return o;
 }
 
+// Any granule, whole or not.
+template <typename T>
+__device__ __forceinline__ uint4 gran_any(const GranRow& r, int g) {  // outside the row: -inf, that is weight 0
+    const float ninf = __int_as_float(0xff800000);
+    if (g < 0 || g >= r.ng) return gran_fill<T>(ninf);
+    if (g < r.whole_lo() || g >= r.whole_hi()) return gran_edge<T>(r, g, ninf);
+    return ldg_stream(r.base + g);
+}
+
+// One warp: the draft partial of granules [lo, hi) for logits and temperatures of any size (DraftState::far), every exponent
+// (x - m) * scale from a difference of logits.  Plain rather than fast: a row takes it from |logit| / T of 2e8 on.
+template <typename T>
+__device__ __noinline__ float4 draft_far(const T* p, int V, int lo, int hi, float scale) {
+    constexpr int E = 16 / sizeof(T);
+    const GranRow row = make_row(p, V);
+    float m = kFloor, cnt = 0.f, z = 0.f, s = 0.f;  // s: of 2^y * y
+    bool bad = false;
+    for (int g = lo + (threadIdx.x & 31); g < min(hi, row.ng); g += 32) {
+        const uint4 v = gran_any<T>(row, g);
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int j = 0; j < E; ++j) {
+            float x = sizeof(T) == 4 ? __uint_as_float(w[j % 4]) : (j & 1) ? bf_hi(w[j / 2]) : bf_lo(w[j / 2]);
+            bad |= x != x || x == __int_as_float(0x7f800000);
+            x = fmaxf(x, kFloor);
+            const float y = -fabsf(x - m) * scale, e = ex2f(y);  // y may be infinite (and at scale = inf not a number where x = m)
+            if (x > m) {
+                s = e > 0.f ? fmaf(y, cnt + z, s) * e : 0.f;
+                z = (cnt + z) * e;
+                cnt = 1.f;
+                m = x;
+            } else if (x == m) {
+                cnt += 1.f;
+            } else if (e > 0.f) {
+                z += e;
+                s = fmaf(e, y, s);
+            }
+        }
+    }
+    return warp_merge<PATH_DRAFT>(make_float4(m, bad ? __int_as_float(0x7fc00000) : cnt, z, s / scale), scale);
+}
+
 // ----------------------------------------------------------------------------------------
 // One WARP sweeps granules [lo, hi) of one logit row.  Lane l owns
 // granules l, l+32, ... of the range; a step folds kVec elements per lane (bf16: one granule, fp32: two granules 32
@@ -676,8 +724,9 @@ struct WarpSweep {
         }
         return m0;
     }
+    // PATH_DRAFT: through draft() only
     template <int PATH>
-    __device__ __forceinline__ float4 run(float m0, float scale) {
+    __device__ __forceinline__ float4 run(float m0, float scale, bool* far = nullptr) {
         const int lane = threadIdx.x & 31;
         DraftState ds; TargetState ts; ArgmaxState as;
         if constexpr (PATH == PATH_DRAFT) ds.init(m0, scale);
@@ -740,10 +789,19 @@ struct WarpSweep {
                 if (i + k < n_main) process(buf[k], a + lane + 32 * GS * (i + k));
         }
         float4 part;
-        if constexpr (PATH == PATH_DRAFT) part = ds.partial(scale);
+        if constexpr (PATH == PATH_DRAFT) {
+            part = ds.partial(scale);
+            *far = __any_sync(0xffffffffu, ds.far(part, scale));
+        }
         else if constexpr (PATH == PATH_TARGET) part = ts.partial();
         else part = as.partial();
         return warp_merge<PATH>(part, scale);
+    }
+    // a draft row's range [lo, hi)
+    __device__ __forceinline__ float4 draft(float m0, float scale, const T* row, int V, int lo, int hi) {
+        bool far;
+        const float4 part = run<PATH_DRAFT>(m0, scale, &far);
+        return far ? draft_far<T>(row, V, lo, hi, scale) : part;
     }
 };
 

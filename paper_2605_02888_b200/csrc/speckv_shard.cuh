@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(kThreads, 4) shard_rows_kernel(const __grid_co
         }
         const float m0 = ws.template warm<false>(nullptr);
         if (!is_target) {
-            st = ws.template run<PATH_DRAFT>(m0, scale);
+            st = ws.draft(m0, scale, row, P.V, sub * per, sub * per + per);
         } else if (greedy) {
             st = ws.template run<PATH_ARGMAX>(m0, scale);
             const int idx = __float_as_int(st.y);

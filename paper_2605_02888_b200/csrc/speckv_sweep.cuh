@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sweep_kernel(c
                         SPECKV_ST(P.tokl[static_cast<long long>(b) * P.G + pos], make_float2(elem_to_float(row, x), elem_to_float(trow, x)));
                     }
                 }
-                part = ws.template run<PATH_DRAFT>(m0, scale);
+                part = ws.draft(m0, scale, row, P.V, lo, lo + P.per_warp);
                 path = PATH_DRAFT;
             } else if (greedy) {
                 part = ws.template run<PATH_ARGMAX>(m0, scale);
@@ -327,7 +327,7 @@ __global__ void __launch_bounds__(kThreads, 4) batch_row_kernel(const __grid_con
             }
             const float m0 = ws.template warm<false>(nullptr);
             float4 part;
-            if (!is_target) part = ws.template run<PATH_DRAFT>(m0, scale);
+            if (!is_target) part = ws.draft(m0, scale, row, P.V, sub * P.per_warp, sub * P.per_warp + P.per_warp);
             else if (greedy) part = ws.template run<PATH_ARGMAX>(m0, scale);
             else part = ws.template run<PATH_TARGET>(m0, scale);
             if (lane == 0) {

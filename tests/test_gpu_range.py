@@ -78,6 +78,33 @@ def test_masked_stretch_before_the_first_allowed_token(dtype, B, G, V, n_shards,
 
 
 @pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("B,G,V,n_shards", [(256, 5, 4096, 0), (2, 5, 40001, 0), (180, 5, 100000, 0), (12, 5, 33000, 3)])
+@pytest.mark.parametrize("T,big", [(1.0, 5.0e9), (1.0, 1.0e10), (1.0, 1.0e34), (1e-8, 20.0), (1e-9, 20.0), (1e-9, 0.25)])
+def test_draft_logits_far_beyond_the_exponent_range(dtype, B, G, V, n_shards, T, big):
+    # logit / T of 1e9 and more: neighbouring values of the exponent's reference are then hundreds apart.  The target stays
+    # where include/speckv.h wants it, at a largest |logit| / T below 2^28.
+    g = torch.Generator(device=DEV).manual_seed(V)
+    dt = TYPES[dtype]
+    unit = min(1.0, 1.0e8 * T)
+    base = (torch.randn(G + 1, V, generator=g, device=DEV) * unit).clamp(-1.5 * unit, 1.5 * unit)
+    draft, target = base[:G].clone(), base.clone()
+    draft[0, V - 1] = big                        # met late
+    draft[0, V // 2] = big                       # a tie
+    draft[1, 3] = big                            # met at once, and a smaller one behind it
+    draft[1, V - 2] = big * 0.5
+    low = -min(big, 1.0e29)                      # (below -2^100 a logit counts as -inf)
+    draft[2] = low                               # flat: H = ln V
+    draft[3, : V - 2] = float("-inf")            # masked but for two tokens, the first of which is far below the other
+    draft[3, V - 2] = low
+    draft[4] = big + base[4]                     # the common offset takes the rest with it (absorbed in part or altogether)
+    target[0, V - 1] = 1.5 * unit
+    s = _shared_rows(draft.to(dt), target.to(dt), B, T, seed=V)
+    out, ref = _check(s, n_shards)
+    assert (ref["row_status"] == 0).all()
+    assert ref["H"][0, 0] == pytest.approx(math.log(2)) and ref["H"][0, 2] == pytest.approx(math.log(V)) and ref["H"][0, 3] == 0.0
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
 @pytest.mark.parametrize("V,n_shards", [(4096, 0), (40001, 0), (33000, 3)])
 @pytest.mark.parametrize("T,level", [(0.9, 0.0), (0.9, 3.0e4), (1e-6, 100.0), (1e-6, 416.0), (1e-6, -416.0), (1e-6, 960.0)])
 def test_residual_of_two_tied_tokens(dtype, V, n_shards, T, level):
