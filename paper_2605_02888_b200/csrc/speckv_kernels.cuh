@@ -40,6 +40,9 @@ template <> struct SweepShape<float> { static constexpr int kSteps = 4, kCtas = 
 // Every kernel is launched so that its CTAs may be placed as soon as all CTAs of the kernel in front of it in the stream have
 // called dependents_may_start() or ended.  It touches memory only behind wait_for_predecessors(), that is when that kernel has
 // ended and its writes are visible, and lets its own successor in after that, so what holds for one holds for the whole chain.
+// A kernel is therefore already running while its inputs are written (the drafted tokens, the next gamma and the logits come from
+// the call in front of it), so none of them is read through the non-coherent path (__ldg, ld.global.nc), which is for data that
+// nobody writes while the kernel runs.  Plain loads cost nothing here: all cases within 0.3 %.
 __device__ __forceinline__ void wait_for_predecessors() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void dependents_may_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 constexpr float kFloor = -1.2676506002282294e30f;  // -2^100: logits below count as -inf
@@ -196,7 +199,7 @@ __device__ __forceinline__ float max_nan(float a, float b) {  // NaN-propagating
 __device__ __forceinline__ uint4 ldg_stream(const void* p) {
     uint4 v;
     if (!dbg_ok(p, 16, DBG_LOGIT16)) return make_uint4(0xff80ff80u, 0xff80ff80u, 0xff80ff80u, 0xff80ff80u);
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
                  : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
                  : "l"(p));
     return v;
@@ -842,20 +845,20 @@ __device__ __forceinline__ CtlRegs ctl_load(const KParams& P, int b, int lane) {
     CtlRegs c;
     const bool hid = lane < P.n_hidden;
 #pragma unroll
-    for (int f = 0; f < 8; ++f) c.w1[f] = (hid && f < P.n_in) ? __ldg(P.W1 + lane * P.n_in + f) : 0.f;
+    for (int f = 0; f < 8; ++f) c.w1[f] = (hid && f < P.n_in) ? P.W1[lane * P.n_in + f] : 0.f;
     if (P.layout == 2) {
         // the paper's f(x, gamma): one output head; without hidden units W2 weighs the inputs directly
 #pragma unroll
         for (int j = 1; j < 8; ++j) c.w2[j] = 0.f;
-        c.w2[0] = (P.n_hidden > 0 ? hid : lane < P.n_in) ? __ldg(P.W2 + lane) : 0.f;
-        c.b2k = lane == 0 ? __ldg(P.b2) : 0.f;
+        c.w2[0] = (P.n_hidden > 0 ? hid : lane < P.n_in) ? P.W2[lane] : 0.f;
+        c.b2k = lane == 0 ? P.b2[0] : 0.f;
     } else {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) c.w2[j] = (hid && j < P.n_out) ? __ldg(P.W2 + j * P.n_hidden + lane) : 0.f;
-        c.b2k = lane < P.n_out ? __ldg(P.b2 + lane) : 0.f;
+        for (int j = 0; j < 8; ++j) c.w2[j] = (hid && j < P.n_out) ? P.W2[j * P.n_hidden + lane] : 0.f;
+        c.b2k = lane < P.n_out ? P.b2[lane] : 0.f;
     }
-    c.b1 = hid ? __ldg(P.b1 + lane) : 0.f;
-    c.compk = (P.comp && lane < P.n_comp) ? __ldg(P.comp + static_cast<long long>(b) * P.n_comp + lane) : 0.f;
+    c.b1 = hid ? P.b1[lane] : 0.f;
+    c.compk = (P.comp && lane < P.n_comp) ? P.comp[static_cast<long long>(b) * P.n_comp + lane] : 0.f;
     return c;
 }
 // f4 = Hbar, cbar, Hmax, cmin.  fp32 throughout: 164 multiply-adds on values of order one.  All outputs' reductions run
@@ -1002,13 +1005,13 @@ __device__ __noinline__ void decide_positions(const KParams& P, int b, int gam, 
         const long long at = static_cast<long long>(b) * P.G + i;
         const long long urow = (static_cast<long long>(b) * (P.G + 1) + i) * 2;
         if (tok_on) {
-            x = __ldg(P.tok + at);
-            u_acc = __ldg(P.u + urow);
+            x = P.tok[at];
+            u_acc = P.u[urow];
             // left by the sweep CTA of the draft position; with shards, in the table of the one whose slice holds the token
             const long long shard = P.shard_width > 0 && x > 0 ? min(x / P.shard_width, P.n_shards - 1) : 0;
             if (!greedy) tl = __ldcg(P.tokl + at + shard * P.tokl_stride);
         }
-        if (in && verify) u_res = __ldg(P.u + urow + 1);
+        if (in && verify) u_res = P.u[urow + 1];
     }
 
     int amax = -1;

@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sample_kernel(
         bad = g.z != 0.f || !(g.x > kFloor);
         tok = __float_as_int(g.y);
     } else {
-        tok = draw_from_spans<T>(row, P.V, scale, spans, n, P.per_warp, __ldg(P.u + r), warp, kWarps, 1, sh_sum, &sh_src);
+        tok = draw_from_spans<T>(row, P.V, scale, spans, n, P.per_warp, P.u[r], warp, kWarps, 1, sh_sum, &sh_src);
         if (tok == kNotMine) return;
         bad = tok < 0;
     }

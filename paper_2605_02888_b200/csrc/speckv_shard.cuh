@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(kThreads, 4) shard_rows_kernel(const __grid_co
         ws.start(gr, sub * per, sub * per + per);
         if (!is_target && lane == 0 && sub == 0 && !greedy) {
             // both logits at the draft token, if it falls into this slice
-            const int x = __ldg(P.tok + static_cast<long long>(b) * P.G + pos) - P.v_begin;
+            const int x = P.tok[static_cast<long long>(b) * P.G + pos] - P.v_begin;
             if (x >= 0 && x < P.V) {
                 const T* trow = static_cast<const T*>(P.t) + static_cast<long long>(b) * P.tsb + static_cast<long long>(pos) * P.tsp;
                 tl = make_float2(elem_to_float(row, x), elem_to_float(trow, x));

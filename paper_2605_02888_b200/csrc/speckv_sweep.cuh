@@ -200,7 +200,7 @@ __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sweep_kernel(c
         const int lo = (s * kWarps + warp) * P.per_warp;  // this warp's granules: the CTA's slice is cut into one contiguous range per warp
         WarpSweep<T, SweepShape<T>::kSteps> ws;
         ws.start(make_row(row, P.V), lo, lo + P.per_warp);
-        Tf = P.temp ? __ldg(P.temp + b) : P.temp_scalar;
+        Tf = P.temp ? P.temp[b] : P.temp_scalar;
         if (threadIdx.x == 0) {
             // one thread reads what is known of the row's stop position, so that the whole CTA takes one decision
             int e = 0;
@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sweep_kernel(c
                 if (verify && P.tokl && s == 0 && threadIdx.x == 0 && !greedy) {
                     // the acceptance test of this position needs both logits at the draft token: fetch them
                     // now, while the sweep hides the latency, and leave them for the row epilogue
-                    const int x = __ldg(P.tok + static_cast<long long>(b) * P.G + pos) - P.v_begin;  // index in this slice
+                    const int x = P.tok[static_cast<long long>(b) * P.G + pos] - P.v_begin;  // index in this slice
                     if (x >= 0 && x < P.V) {
                         const T* trow = static_cast<const T*>(P.t) + static_cast<long long>(b) * P.tsb +
                                         static_cast<long long>(pos) * P.tsp;
@@ -305,8 +305,8 @@ __global__ void __launch_bounds__(kThreads, 4) batch_row_kernel(const __grid_con
     dependents_may_start();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, b = blockIdx.x;
     const bool verify = (P.mode & MODE_VERIFY) != 0;
-    const int gam = P.gamma ? __ldg(P.gamma + b) : P.G;
-    const float Tf = P.temp ? __ldg(P.temp + b) : P.temp_scalar, scale = row_scale(Tf);
+    const int gam = P.gamma ? P.gamma[b] : P.G;
+    const float Tf = P.temp ? P.temp[b] : P.temp_scalar, scale = row_scale(Tf);
     const bool greedy = (Tf == 0.f);
     if (!row_status0(P, gam, Tf)) {
         const int n_rows = verify ? 2 * gam + 1 : gam, sub = warp % P.nsplit;
@@ -319,7 +319,7 @@ __global__ void __launch_bounds__(kThreads, 4) batch_row_kernel(const __grid_con
             ws.start(make_row(row, P.V), sub * P.per_warp, sub * P.per_warp + P.per_warp);
             if (verify && !is_target && !greedy && lane == 0 && sub == 0) {  // both logits at the draft token
                 const long long at = static_cast<long long>(b) * P.G + pos;
-                const int x = __ldg(P.tok + at);
+                const int x = P.tok[at];
                 if (x >= 0 && x < P.V) {
                     const T* trow = static_cast<const T*>(P.t) + static_cast<long long>(b) * P.tsb + static_cast<long long>(pos) * P.tsp;
                     SPECKV_ST(P.tokl[at], make_float2(elem_to_float(row, x), elem_to_float(trow, x)));

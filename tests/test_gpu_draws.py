@@ -121,6 +121,47 @@ def test_calls_wait_for_their_inputs():
 
 
 @pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("B,V", [(1, 2000), (40, 4096), (300, 8000), (24, 9001)])
+def test_calls_read_what_the_call_before_them_wrote(dtype, B, V):
+    # gamma and the drafted tokens go from call to call in the buffers that the kernels wrote them to, with nothing launched
+    # between (short vocabularies: the step is one kernel, the sampling kernel its direct predecessor; a vocabulary that is swept)
+    w = synth.Workload("d", B=B, gamma_max=8, V=V, dtype=dtype, gamma_mode="choices", temperature=0.9, sigma_t=1.0,
+                       sigma_d=(0.2, 1.0, 2.0), seed=V % 97)
+    steps = [synth.make_step(w, i, DEV) for i in range(3)]
+    gm, _ = mlp_pair(synth.make_mlp(w, DEV))
+
+    def run(sync):
+        done = torch.cuda.synchronize if sync else lambda: None
+        gamma, tok = steps[0]["gamma"].clone(), torch.zeros_like(steps[0]["draft_tokens"])
+        st = torch.empty(B, dtype=torch.int32, device=DEV)
+        bts = [gpu_batch(dict(s, gamma=gamma, draft_tokens=tok)) for s in steps]
+        us = [s["uniforms"][:, :8, 0].contiguous() for s in steps]
+        outs = [speckv.StepOutputs.allocate(b, gm.n_out) for b in bts for _ in range(8)]
+        for b, o in zip(bts * 8, outs):
+            o.gamma_next = gamma  # the controller's choice is the next step's gamma
+        toks = torch.zeros(len(outs), *tok.shape, dtype=torch.int32, device=DEV)
+        ws = torch.empty(1 << 24, dtype=torch.uint8, device=DEV)
+        done()
+        for k, o in enumerate(outs):
+            s, bt = steps[k % 3], bts[k % 3]
+            speckv.speckv_sample_draft(bt, us[k % 3], tokens=tok, row_status=st, workspace=ws)
+            done()
+            speckv.speckv_step(bt, s["comp"], gm, out=o)
+            done()
+            toks[k].copy_(tok)
+            f = speckv.speckv_signals(bt, out=o)["feat"]
+            done()
+            speckv.speckv_select_gamma(f, s["comp"], gm, scores=o.scores, gamma_next=gamma)
+            done()
+        torch.cuda.synchronize()
+        assert all(int(o.row_status.abs().sum()) == 0 for o in outs)
+        return [toks] + [t for o in outs for t in o.as_dict().values()]
+
+    for a, b in zip(run(True), run(False)):
+        assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
 @pytest.mark.parametrize("n,V", [(1, 3000), (2, 40001), (4, 40000)])
 def test_shard_masses(dtype, n, V):
     # a rank's two masses at the stop position: of max(0, p - q) (0 where a bonus token is drawn) and of p
