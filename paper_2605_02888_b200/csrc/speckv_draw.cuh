@@ -96,23 +96,26 @@ __device__ __forceinline__ void gran_weights(float scale, float lp, float lq, fl
         }
     }
 }
-// The same for normalisers of any size; rarely taken.
+// The same for normalisers of any size.  Rarely taken, and out of line so that a draw, a chain of cold code, does not fetch it.
+template <typename T> struct GranW { float w[16 / sizeof(T)], p; };  // p: sum of p
 template <typename T, bool RES>
-__device__ __forceinline__ void gran_weights_wide(const DrawSrc& s, const uint4& t, const uint4& d, float (&w)[16 / sizeof(T)],
-                                                  float* sum_p = nullptr) {
+__device__ __noinline__ GranW<T> gran_weights_wide(float scale, float lp, float plo, float lq, float qlo, uint4 t, uint4 d) {
     constexpr int NP = 8 / sizeof(T);
-    const f2 sc2 = pack2(s.scale, s.scale), ph = pack2(-s.lp, -s.lp), pl = pack2(s.plo, s.plo), qh = pack2(-s.lq, -s.lq), ql = pack2(s.qlo, s.qlo);
+    const f2 sc2 = pack2(scale, scale), ph = pack2(-lp, -lp), pl = pack2(plo, plo), qh = pack2(-lq, -lq), ql = pack2(qlo, qlo);
     f2 xt[NP], xd[NP];
     gran_pairs(t, xt);
     if (RES) gran_pairs(d, xd);
+    GranW<T> o;
+    o.p = 0.f;
 #pragma unroll
     for (int i = 0; i < NP; ++i) {
         const f2 p = ex2_2(sub2(fma2(xt[i], sc2, ph), pl));
-        if (sum_p) *sum_p += hsum2(p);
-        unpack2(RES ? sub2(p, ex2_2(sub2(fma2(xd[i], sc2, qh), ql))) : p, w[2 * i], w[2 * i + 1]);
-        w[2 * i] = fmaxf(w[2 * i], 0.f);
-        w[2 * i + 1] = fmaxf(w[2 * i + 1], 0.f);
+        o.p += hsum2(p);
+        unpack2(RES ? sub2(p, ex2_2(sub2(fma2(xd[i], sc2, qh), ql))) : p, o.w[2 * i], o.w[2 * i + 1]);
+        o.w[2 * i] = fmaxf(o.w[2 * i], 0.f);
+        o.w[2 * i + 1] = fmaxf(o.w[2 * i + 1], 0.f);
     }
+    return o;
 }
 template <typename T, bool RES>
 __device__ __forceinline__ float gran_weight(float scale, float lp, float lq, float c, const uint4& t, const uint4& d,
@@ -167,8 +170,13 @@ __device__ __forceinline__ void load_weights(const DrawSrc& s, int g, int g1, fl
             if (RES) d = draft_any<T>(s, g);
         }
     }
-    if (WIDE && s.wide) gran_weights_wide<T, RES>(s, t, d, w);
-    else gran_weights<T, RES>(s.scale, s.lp, s.lq, s.c, t, d, w);
+    if (WIDE && s.wide) {
+        const GranW<T> o = gran_weights_wide<T, RES>(s.scale, s.lp, s.plo, s.lq, s.qlo, t, d);
+#pragma unroll
+        for (int j = 0; j < static_cast<int>(16 / sizeof(T)); ++j) w[j] = o.w[j];
+    } else {
+        gran_weights<T, RES>(s.scale, s.lp, s.lq, s.c, t, d, w);
+    }
 }
 template <typename T, bool RES>
 __device__ __noinline__ double gran_weight_any(const DrawSrc s, int g) {
@@ -220,12 +228,12 @@ __device__ __noinline__ double2 span_weight(const uint4* pt, const uint4* pd, in
             uint4 b = a;
             if (RES) b = ldg_stream(pd);
             if (RES && SHIFTED) b = gran_shift<T>(b, ldg_stream(pd + 1), off);
-            float w[16 / sizeof(T)], wp = 0.f, sum = 0.f;
-            gran_weights_wide<T, RES>(s, a, b, w, WITH_P ? &wp : nullptr);
+            const GranW<T> o = gran_weights_wide<T, RES>(s.scale, s.lp, s.plo, s.lq, s.qlo, a, b);
+            float sum = 0.f;
 #pragma unroll
-            for (int j = 0; j < static_cast<int>(16 / sizeof(T)); ++j) sum += w[j];
+            for (int j = 0; j < static_cast<int>(16 / sizeof(T)); ++j) sum += o.w[j];
             acc.x += static_cast<double>(sum);
-            if (WITH_P) acc.y += static_cast<double>(wp);
+            if (WITH_P) acc.y += static_cast<double>(o.p);
         }
         return acc;
     }
