@@ -21,6 +21,12 @@ namespace {
 using namespace speckv;
 
 constexpr int kSliceBytes = 262144;  // bytes of one logit row that one sweep CTA streams
+// Draft sampling has no row epilogue and no draw behind it, so its slices are cut for balance.  fp32 rows: half as long, since the
+// last round of CTAs weighs more when fewer of them share an SM (V = 84,032, slices of 256 / 128 KB: 120 rows of 5 59.9 -> 45.1 us,
+// 500 of 3 110.6 -> 91.1, 1,000 of 4 178.5 -> 143.5; V = 151,936, 64 of 8 69.8 -> 59.3; with a persistent share of chunks per CTA,
+// the way before, 54.4 / 100.8 / 157.3 / 71.2).  Rows below 64 KB are cut only where that does not start a second round: 64 rows of
+// 8 positions, V = 3,000, fp32 13.8 -> 8.7 us, V = 6,000, bf16 13.6 -> 9.1.
+constexpr int kSampleF32SliceBytes = 131072, kSampleWholeBytes = 65536;
 constexpr size_t kAlign = 256;
 
 inline size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
@@ -69,18 +75,19 @@ cudaError_t dbg_register(cudaStream_t cs, const speckv_batch* bt, bool target, c
 int cta_slots(speckv_dtype dt) { return 148 * (dt == SPECKV_BF16 ? SweepShape<__nv_bfloat16>::kCtas : SweepShape<float>::kCtas); }
 
 // Vocabulary slices per logit row for a sweep over J logit rows per batch row, one CTA each, and the granules that one
-// warp takes of a slice: P.nsplit, P.per_warp.  aligned: every row starts on the 16-byte grid.
-void choose_slices(KParams& P, speckv_dtype dt, bool aligned) {
+// warp takes of a slice: P.nsplit, P.per_warp.  aligned: every row starts on the 16-byte grid.  sample: draft sampling.
+void choose_slices(KParams& P, speckv_dtype dt, bool aligned, bool sample = false) {
     const int E = 16 / esize(dt);
     const int ng = (P.V + E - 1 + (aligned ? 0 : E - 1)) / E;  // granules a row can touch
-    int ns = static_cast<int>(std::lround(16.0 * ng / static_cast<double>(kSliceBytes)));
+    const bool whole = sample && 16LL * ng < kSampleWholeBytes;  // not more CTAs than slots
+    int ns = static_cast<int>(std::lround(16.0 * ng / static_cast<double>(sample && dt == SPECKV_F32 ? kSampleF32SliceBytes : kSliceBytes)));
     if (ns < 1) ns = 1;
     // Small batches: enough CTAs to fill the slots of the chip once.  Aiming at more starts a second
     // round of short CTAs: with 1,184 instead of 740 (bf16), step of 64 bf16 rows, V = 32,000, 37.7 us instead of 33.1, of 37 rows,
     // V = 50,257, 32.6 instead of 31.1; one row the same.
     const long long rows = static_cast<long long>(P.B) * P.J;
     const int slots = cta_slots(dt);
-    const long long want = (slots + rows - 1) / (rows > 0 ? rows : 1);
+    const long long want = (slots + (whole ? 0 : rows - 1)) / (rows > 0 ? rows : 1);
     if (want > ns) ns = static_cast<int>(want > kMaxSplit ? kMaxSplit : want);
     if (ns > kMaxSplit) ns = kMaxSplit;
     // At least one granule per lane, and whole steps of the warp: one with idle lanes costs as much as a full one, and lanes
@@ -92,7 +99,7 @@ void choose_slices(KParams& P, speckv_dtype dt, bool aligned) {
     const int near = (pw + 16) / 32 * 32 < 32 ? 32 : (pw + 16) / 32 * 32;
     const int step = 32 * (kVec / E);
     if (pw >= 256) pw = (pw + step - 1) / step * step;
-    else if (((ng + near * kWarps - 1) / (near * kWarps)) * rows <= slots + rows) pw = near;
+    else if (((ng + near * kWarps - 1) / (near * kWarps)) * rows <= slots + (whole ? 0 : rows)) pw = near;
     else pw = (pw + 31) / 32 * 32;
     while ((ng + pw * kWarps - 1) / (pw * kWarps) > kMaxSplit) pw += 32;
     P.per_warp = pw;
@@ -376,7 +383,7 @@ speckv_status run_sample(const speckv_batch* bt, const float* uniforms, int32_t*
     P.B = bt->B; P.G = bt->gamma_max; P.V = bt->V;
     P.J = bt->gamma_max;
     const bool aligned = rows_aligned(bt->draft_logits, bt->draft_stride_b, bt->draft_stride_pos, esize(bt->dtype));
-    choose_slices(P, bt->dtype, aligned);
+    choose_slices(P, bt->dtype, aligned, true);
     P.d = bt->draft_logits; P.dsb = bt->draft_stride_b; P.dsp = bt->draft_stride_pos;
     P.gamma = bt->gamma; P.temp = bt->temperature; P.temp_scalar = bt->temperature_scalar;
     P.u = uniforms;

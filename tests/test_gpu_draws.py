@@ -50,6 +50,23 @@ def test_sampled_drafts(dtype, B, G, V):
     assert (tok[clear] == ref["tokens"][clear]).all() and clear.mean() > 0.9
 
 
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("B,G,V", [(74, 8, 3000), (93, 8, 6001), (9, 8, 16380), (9, 8, 16384), (75, 8, 32767), (120, 5, 49151),
+                                   (80, 8, 49153), (120, 5, 84032)])
+def test_sampled_drafts_over_slices(dtype, B, G, V):
+    # rows below and above 64 KB, as many as there are CTA slots and a few more; fp32 rows of one, two and three slices of 128 KB
+    w = _workload(B, G, V, dtype)
+    s = synth.make_step(w, 0, DEV)
+    s["gamma"][:] = G
+    u = torch.rand(B, G, device=DEV)
+    rows = np.arange(0, B, max(1, B // 10))
+    out = speckv.speckv_sample_draft(gpu_batch(s), u)
+    ref = oracle.sample_draft(oracle_batch(s, rows=rows), u.cpu().numpy()[rows])
+    clear = ref["near"] == 0
+    assert (out["tokens"].cpu().numpy()[rows][clear] == ref["tokens"][clear]).all() and clear.mean() > 0.8
+    assert (out["row_status"] == 0).all() and (out["tokens"] >= 0).all()
+
+
 @pytest.mark.parametrize("dtype,V", [("bf16", 5000), ("fp32", 5001), ("bf16", 300007)])
 def test_an_empty_residual_is_drawn_from_p(dtype, V):
     # draft == target and a drafted token without probability: rejected with nothing in the residual
