@@ -354,16 +354,20 @@ speckv_status run(const speckv_batch* bt, int mode, const float* comp, const spe
     return e == cudaSuccess ? SPECKV_OK : SPECKV_ERR_CUDA;
 }
 
-// Draft-side sampling: its own workspace plan (one draw per drafted position).
+// Draft-side sampling: its own workspace plan (one draw per drafted position).  A position has a span for every warp that a row of
+// this length can keep busy with a granule per lane, wherever it sits on the 16-byte grid.
 struct SamplePlan {
     size_t off_tick, off_spans, total;
+    int most_spans;
 };
 SamplePlan make_sample_plan(const speckv_batch* bt) {
     SamplePlan p;
     const size_t B = static_cast<size_t>(bt->B), G = static_cast<size_t>(bt->gamma_max);
     size_t off = 0;
     p.off_tick = off; off = align_up(off + (B * G + 2 * B) * sizeof(int));  // tickets per position and per row, row status
-    p.off_spans = off; off = align_up(off + B * G * kMaxSplit * kWarps * sizeof(float2));
+    const int E = 16 / esize(bt->dtype), ng = (bt->V + 2 * (E - 1)) / E, warps = (ng + 31) / 32;
+    p.most_spans = warps < kMaxSplit * kWarps ? warps : kMaxSplit * kWarps;
+    p.off_spans = off; off = align_up(off + B * G * p.most_spans * sizeof(float2));
     p.total = off < kAlign ? kAlign : off;
     return p;
 }
@@ -384,6 +388,8 @@ speckv_status run_sample(const speckv_batch* bt, const float* uniforms, int32_t*
     P.J = bt->gamma_max;
     const bool aligned = rows_aligned(bt->draft_logits, bt->draft_stride_b, bt->draft_stride_pos, esize(bt->dtype));
     choose_slices(P, bt->dtype, aligned, true);
+    // (per_warp is 32 at least, so a warp behind the last span has no granule)
+    P.n_spans = P.nsplit * kWarps < pl.most_spans ? P.nsplit * kWarps : pl.most_spans;
     P.d = bt->draft_logits; P.dsb = bt->draft_stride_b; P.dsp = bt->draft_stride_pos;
     P.gamma = bt->gamma; P.temp = bt->temperature; P.temp_scalar = bt->temperature_scalar;
     P.u = uniforms;

@@ -96,7 +96,7 @@ static_assert(sizeof(RowInfo) == 32, "the resample kernel reads a RowInfo as two
 struct KParams {
     int B, G, V, J, nsplit, R, mode, bits;
     int per_warp;  // sweep kernel: 16-byte granules of a logit row that one warp folds; a slice is kWarps times that
-    int n_spans;    // verification: spans per batch row
+    int n_spans;    // spans per batch row (verification) or position (draft sampling)
     int2* list;     // sliced sweep: one entry per logit row to sweep, in the order of the grid (prep_kernel)
     int* n_list;    //   and how many there are; CTAs behind the last one draw
     int n_draw;     // sliced sweep: CTAs that may draw (R per batch row), 0 = none
@@ -126,7 +126,7 @@ struct KParams {
     RowInfo* info;
     float4* part;
     float2* spans;  // (reference, sum) of every warp's range of the row a plain draw may need: verification [B, nsplit * kWarps]
-                    // (target position gamma_b), draft-side sampling [B * G, nsplit * kWarps]
+                    // (target position gamma_b), draft-side sampling [B * G, n_spans]
     double* dsum;   // draw: [B, kMaxShares * kWarps] span weights of the stop position
     double* dsum2;  // shard draw: the same of p beside the residual's
     // vocabulary-sharded verification (speckv_shard.cuh); all zero otherwise

@@ -10,8 +10,8 @@
 
 namespace speckv {
 
-// grid: B * G * nsplit CTAs, one per (batch row, position, vocabulary slice).  P.spans holds [B*G, nsplit * kWarps]
-// (reference, sum) pairs, for greedy rows (best value or NaN, index); P.tick1 one counter per position, P.tick2 one per
+// grid: B * G * nsplit CTAs, one per (batch row, position, vocabulary slice).  P.spans holds [B*G, n_spans]
+// (reference, sum) pairs, one per warp that can have granules, for greedy rows (best value or NaN, index); P.tick1 one counter per position, P.tick2 one per
 // batch row, P.rdone (here: a per-row status word), all zeroed by clear_kernel.
 // (A kernel, since nothing can be launched ahead of the end of a memset: sampling of 24 fp32 rows, V = 32,000, 14.4 us with
 // that, 10.7 this way; of one bf16 row, V = 128,256, 12.4 / 8.8.)
@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sample_kernel(
     const bool greedy = (Tf == 0.f);
     const float scale = static_cast<float>(kLog2e / static_cast<double>(greedy ? 1.f : Tf));
     const T* row = static_cast<const T*>(P.d) + static_cast<long long>(b) * P.dsb + static_cast<long long>(i) * P.dsp;
-    const int n = P.nsplit * kWarps;
+    const int n = P.n_spans;
     float2* spans = P.spans + static_cast<long long>(r) * n;
     {
         const int lo = (s * kWarps + warp) * P.per_warp;
@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sample_kernel(
             const float4 p = ws.template run<PATH_TARGET>(m0, scale);
             v = make_float2(p.x, p.y);
         }
-        if (lane == 0) SPECKV_ST(spans[s * kWarps + warp], v);
+        if (lane == 0 && s * kWarps + warp < n) SPECKV_ST(spans[s * kWarps + warp], v);
     }
     __syncthreads();
     if (P.nsplit > 1) {  // else this CTA is the row's last: no ticket (256 bf16 rows, V = 128,256: 73.4 us with it, 71.3 without)

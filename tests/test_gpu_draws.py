@@ -2,6 +2,8 @@
 per lane, one level of 8 and of up to 64 parts and two levels deep; draft and target rows that sit differently on the 16-byte
 grid; bonus draws (from the sweep's sums), residual draws, draws from p behind an empty residual, draft-side sampling.
 Against the oracle under the rules of tests/parity.py, and against a cumulative sum in float64 where the oracle flags."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -65,6 +67,28 @@ def test_sampled_drafts_over_slices(dtype, B, G, V):
     clear = ref["near"] == 0
     assert (out["tokens"].cpu().numpy()[rows][clear] == ref["tokens"][clear]).all() and clear.mean() > 0.8
     assert (out["row_status"] == 0).all() and (out["tokens"] >= 0).all()
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("B,G,V", [(1, 1, 1), (1, 1, 255), (2, 3, 257), (1, 2, 2049), (1, 1, 32001), (1, 1, 65535), (2, 1, 65537),
+                                   (1, 1, 200001), (300, 2, 1025)])
+def test_sampling_stays_within_its_workspace(dtype, B, G, V):
+    # exactly as many bytes as were asked for, what lies behind them unchanged: rows of fewer granules than a slice has lanes, the
+    # most slices, unaligned rows
+    w = _workload(B, G, V, dtype)
+    s = synth.make_step(w, 0, DEV)
+    s["temperature"][::3] = 0.0
+    u = torch.rand(B, G, device=DEV)
+    batch = gpu_batch(s)
+    n, c = ctypes.c_size_t(0), batch._c()
+    assert speckv.load_library().speckv_sample_workspace_size(ctypes.byref(c), ctypes.byref(n)) == 0
+    mem = torch.full((n.value + 8192,), 0x5A, dtype=torch.uint8, device=DEV)
+    a = speckv.speckv_sample_draft(batch, u, workspace=mem[:n.value])
+    assert (mem[n.value:] == 0x5A).all()
+    rows = np.arange(0, B, max(1, B // 20))
+    ref = oracle.sample_draft(oracle_batch(s, rows=rows), u.cpu().numpy()[rows])
+    clear = ref["near"] == 0
+    assert (a["tokens"].cpu().numpy()[rows][clear] == ref["tokens"][clear]).all()
 
 
 @pytest.mark.parametrize("dtype,V", [("bf16", 5000), ("fp32", 5001), ("bf16", 300007)])

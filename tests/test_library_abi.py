@@ -76,6 +76,21 @@ def test_workspace_size_and_argument_checks_without_a_gpu():
     assert L.speckv_select_gamma(4, 0x100, None, C.byref(m), None, 0x100, None) == binding.ERR_UNSUPPORTED
 
 
+def test_sampling_workspace_does_not_outgrow_the_buffers_in_use():
+    # a buffer of the size that was asked for when the sums were kept per 256 elements (44 bytes and 12 per chunk of each
+    # position) goes on being accepted, whatever the vocabulary; a size for more rows serves fewer
+    L = speckv.load_library()
+    n = C.c_size_t(0)
+    up = lambda x: -(-x // 256) * 256
+    for dtype in (binding.F32, binding.BF16):
+        for V in [*range(1, 600, 7), 1000, 2304, 4096, 8191, 20000, 31738, 31999, 32000, 32001, 32641, 33000, 50257, 65536, 151936, 1 << 24]:
+            for B, G in ((1, 1), (3, 4), (64, 8), (1000, 16)):
+                assert L.speckv_sample_workspace_size(C.byref(_cb(B=B, gamma_max=G, V=V, dtype=dtype)), C.byref(n)) == binding.OK
+                pos, chunks = B * G, -(-V // 256)
+                before = sum(up(x) for x in ((2 * B + pos) * 4, pos * 32, pos * 512, pos * chunks * 4, pos * chunks * 8))
+                assert n.value <= before, (dtype, V, B, G, n.value, before)
+
+
 def test_binding_refuses_cpu_tensors():
     import torch
     with pytest.raises(ValueError, match="CUDA"):
