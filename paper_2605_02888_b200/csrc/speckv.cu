@@ -75,8 +75,9 @@ cudaError_t dbg_register(cudaStream_t cs, const speckv_batch* bt, bool target, c
 int cta_slots(speckv_dtype dt) { return 148 * (dt == SPECKV_BF16 ? SweepShape<__nv_bfloat16>::kCtas : SweepShape<float>::kCtas); }
 
 // Vocabulary slices per logit row for a sweep over J logit rows per batch row, one CTA each, and the granules that one
-// warp takes of a slice: P.nsplit, P.per_warp.  aligned: every row starts on the 16-byte grid.  sample: draft sampling.
-void choose_slices(KParams& P, speckv_dtype dt, bool aligned, bool sample = false) {
+// warp takes of a slice: P.nsplit, P.per_warp.  aligned: every row starts on the 16-byte grid.  sample: draft sampling.  most: what
+// the partials of a row have room for, or its epilogue time for.
+void choose_slices(KParams& P, speckv_dtype dt, bool aligned, bool sample = false, int most = kMaxSplit) {
     const int E = 16 / esize(dt);
     const int ng = (P.V + E - 1 + (aligned ? 0 : E - 1)) / E;  // granules a row can touch
     const bool whole = sample && 16LL * ng < kSampleWholeBytes;  // not more CTAs than slots
@@ -88,8 +89,8 @@ void choose_slices(KParams& P, speckv_dtype dt, bool aligned, bool sample = fals
     const long long rows = static_cast<long long>(P.B) * P.J;
     const int slots = cta_slots(dt);
     const long long want = (slots + (whole ? 0 : rows - 1)) / (rows > 0 ? rows : 1);
-    if (want > ns) ns = static_cast<int>(want > kMaxSplit ? kMaxSplit : want);
-    if (ns > kMaxSplit) ns = kMaxSplit;
+    if (want > ns) ns = static_cast<int>(want > most ? most : want);
+    if (ns > most) ns = most;
     // At least one granule per lane, and whole steps of the warp: one with idle lanes costs as much as a full one, and lanes
     // that differ in their number of steps part in the last round of the loop (ranges of 128-byte lines before: step of 64 bf16
     // rows, V = 32,000, 30.2 us, this way 29.3; of 256 fp32 rows, V = 128,256, 226.5 / 222.8; draft sampling of those 113.2 / 110.9).
@@ -101,7 +102,7 @@ void choose_slices(KParams& P, speckv_dtype dt, bool aligned, bool sample = fals
     if (pw >= 256) pw = (pw + step - 1) / step * step;
     else if (((ng + near * kWarps - 1) / (near * kWarps)) * rows <= slots + (whole ? 0 : rows)) pw = near;
     else pw = (pw + 31) / 32 * 32;
-    while ((ng + pw * kWarps - 1) / (pw * kWarps) > kMaxSplit) pw += 32;
+    while ((ng + pw * kWarps - 1) / (pw * kWarps) > most) pw += 32;
     P.per_warp = pw;
     P.nsplit = (ng + pw * kWarps - 1) / (pw * kWarps);
 }
@@ -452,6 +453,9 @@ ShardPlan make_shard_plan(const speckv_batch* bt) {
 
 // A slice row short enough for one CTA in a batch that fills the SMs with one CTA per row: no ticket, nothing to clear first.
 constexpr int kShardOneCtaRows = 128, kShardOneCtaGran = 4096;
+// Slices of a wide slice row at most: one lane of export_epilogue merges a logit row's partials one after the other (one row,
+// gamma 2, V = 31,680, fp32: this call 20.8 us with up to 32 slices, 16.6 with 16, as many as it had before the sweep aimed at whole steps).
+constexpr int kExportSplit = 16;
 constexpr int kShardWarpRowBytes = 65536;  // slice rows up to this size are swept by one warp each
 
 // what every shard call needs from the local batch
@@ -678,7 +682,7 @@ speckv_status speckv_shard_sweep(const speckv_batch* local, int64_t v_begin, flo
     if (st != SPECKV_OK || local->B == 0) return st;
     if (!shard_state || !shard_tokl || v_begin < 0 || v_begin > (1LL << 30)) return SPECKV_ERR_INVALID_ARG;
     const bool al = shard_aligned(local);
-    choose_slices(P, local->dtype, al);
+    choose_slices(P, local->dtype, al, false, kExportSplit);
     if (static_cast<long long>(P.B) * P.J * P.nsplit > 0x7fffffffLL) return SPECKV_ERR_UNSUPPORTED;
     P.v_begin = static_cast<int>(v_begin);
     P.export_state = 1;

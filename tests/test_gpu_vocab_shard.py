@@ -74,6 +74,16 @@ def test_flagged_rows_and_token_in_every_shard():
     assert (ref["row_status"][[2, 3, 4, 5]] != 0).all() and (ref["row_status"][[0, 1]] == 0).all()
 
 
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("B,G,V,n_shards", [(1, 2, 31680, 1), (1, 8, 70001, 2), (2, 16, 151936, 1), (1, 1, 300007, 2)])
+def test_few_rows_of_wide_slices(dtype, B, G, V, n_shards):
+    # slice rows above 64 KB in as many parts as one lane merges
+    w = synth.Workload("t", B=B, gamma_max=G, V=V, dtype=dtype, gamma_mode="fixed", gamma_fixed=G, temperature=0.8, sigma_t=1.5,
+                       sigma_d=(0.3, 0.6), seed=V)
+    s, out, ref = _both(w, n_shards)
+    compare_step(out, ref)
+
+
 def test_bounds_helper():
     width, b = vocab_shard.shard_bounds(128256, 8)
     assert width == 16032 and b[0] == (0, 16032) and b[-1] == (7 * 16032, 128256)
