@@ -217,14 +217,14 @@ struct Events {  // optional timing events around the kernels of a step
     cudaEvent_t before_sweep = nullptr, after_sweep = nullptr, after_resample = nullptr;
 };
 
-// Launches kThreads-thread CTAs as a programmatic dependent of what is in front of it in the stream (wait_for_predecessors), so
+// Launches CTAs as a programmatic dependent of what is in front of it in the stream (wait_for_predecessors), so
 // that the launch itself is over when that ends.  Calls one after the other in a stream: step of 1 fp32 row, V = 32,000, 19.5 ->
 // 17.9 us, of 64 bf16 rows 34.2 -> 32.3, signals and controller of 128, V = 128,256, 52.6 -> 49.2, a rank's four calls 66.4 -> 61.2.
 template <class... Params, class... Args>
-cudaError_t launch(void (*kernel)(Params...), unsigned grid, cudaStream_t st, const Args&... args) {
+cudaError_t launch_threads(void (*kernel)(Params...), unsigned grid, unsigned threads, cudaStream_t st, const Args&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3(threads);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -232,6 +232,10 @@ cudaError_t launch(void (*kernel)(Params...), unsigned grid, cudaStream_t st, co
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+template <class... Params, class... Args>
+cudaError_t launch(void (*kernel)(Params...), unsigned grid, cudaStream_t st, const Args&... args) {
+    return launch_threads(kernel, grid, kThreads, st, args...);
 }
 
 constexpr int kPrepRows = 32;  // batch rows per CTA of the preparing kernel at least; 64 CTAs at most
@@ -456,6 +460,12 @@ constexpr int kShardOneCtaRows = 128, kShardOneCtaGran = 4096;
 // Slices of a wide slice row at most: one lane of export_epilogue merges a logit row's partials one after the other (one row,
 // gamma 2, V = 31,680, fp32: this call 20.8 us with up to 32 slices, 16.6 with 16, as many as it had before the sweep aimed at whole steps).
 constexpr int kExportSplit = 16;
+// Batches with more rows than the chip has slots for CTAs of 256 threads: two warps per row (finish of 8,000 rows, gamma 2 / 8 / 16,
+// 57.5 / 61.7 / 78.0 -> 31.3 / 46.7 / 64.6 us; of 500 rows, gamma 16, the four calls 35.9 -> 40.5, so below that eight).
+constexpr int kShardManyRows = 741;
+// Slice rows of a step or two per lane, one warp each: two steps in flight beside 5 CTAs per SM (8,000 rows, gamma 16, V = 128,
+// fp32, 188 -> 163 us; 1,024 rows, bf16, 25.9 -> 22.3).
+constexpr int kShardTinyRowBytes = 2048;
 constexpr int kShardWarpRowBytes = 65536;  // slice rows up to this size are swept by one warp each
 
 // what every shard call needs from the local batch
@@ -702,8 +712,12 @@ speckv_status speckv_shard_sweep(const speckv_batch* local, int64_t v_begin, flo
         int rw = 1;
         while (rw < kWarps && rows * rw < 148 * 4 * kWarps && row_bytes >= 2048LL * rw) rw *= 2;
         const unsigned g2 = static_cast<unsigned>((rows * rw + kWarps - 1) / kWarps);
-        const cudaError_t e = local->dtype == SPECKV_BF16 ? launch(shard_rows_kernel<__nv_bfloat16>, g2, cs, P, rw)
-                                                          : launch(shard_rows_kernel<float>, g2, cs, P, rw);
+        const bool bf16 = local->dtype == SPECKV_BF16;
+        cudaError_t e;
+        if (rw == 1 && row_bytes <= kShardTinyRowBytes)
+            e = bf16 ? launch(shard_rows_kernel<__nv_bfloat16, 2, 5>, g2, cs, P, rw) : launch(shard_rows_kernel<float, 2, 5>, g2, cs, P, rw);
+        else
+            e = bf16 ? launch(shard_rows_kernel<__nv_bfloat16, 5, 4>, g2, cs, P, rw) : launch(shard_rows_kernel<float, 4, 4>, g2, cs, P, rw);
         return e == cudaSuccess ? SPECKV_OK : SPECKV_ERR_CUDA;
     }
     if (cudaMemsetAsync(shard_tokl, 0, static_cast<size_t>(P.B) * P.G * sizeof(float2), cs) != cudaSuccess)
@@ -756,7 +770,8 @@ speckv_status speckv_shard_finish(const speckv_batch* local, int32_t n_shards, i
                                 {row_info, static_cast<size_t>(P.B) * sizeof(RowInfo)}};
         if (dbg_register(static_cast<cudaStream_t>(cuda_stream), &none, false, nullptr, 0, ex, 3) != cudaSuccess) return SPECKV_ERR_CUDA;
     }
-    return launch(shard_finish_kernel, grid, static_cast<cudaStream_t>(cuda_stream), P) == cudaSuccess ? SPECKV_OK : SPECKV_ERR_CUDA;
+    const unsigned threads = P.B >= kShardManyRows ? 64 : kThreads;
+    return launch_threads(shard_finish_kernel, grid, threads, static_cast<cudaStream_t>(cuda_stream), P) == cudaSuccess ? SPECKV_OK : SPECKV_ERR_CUDA;
 }
 
 speckv_status speckv_shard_draw_sums(const speckv_batch* local, const void* row_info, double* shard_weight,
@@ -801,8 +816,11 @@ speckv_status speckv_shard_draw_pick(const speckv_batch* local, int64_t v_begin,
         if (dbg_register(cs, local, true, workspace, workspace_bytes, ex, 1) != cudaSuccess) return SPECKV_ERR_CUDA;
     }
     const unsigned grid = static_cast<unsigned>(P.B);
-    const cudaError_t e = local->dtype == SPECKV_BF16 ? launch(shard_pick_kernel<__nv_bfloat16>, grid, cs, P)
-                                                      : launch(shard_pick_kernel<float>, grid, cs, P);
+    // as many warps as a span has parts of one granule per lane (8,000 rows, V = 128 and 2,000: 45 and 51 -> 11 and 12 us)
+    unsigned threads = 32;
+    while (threads < kThreads && threads < static_cast<unsigned>(P.draw_pw)) threads *= 2;
+    const cudaError_t e = local->dtype == SPECKV_BF16 ? launch_threads(shard_pick_kernel<__nv_bfloat16>, grid, threads, cs, P)
+                                                      : launch_threads(shard_pick_kernel<float>, grid, threads, cs, P);
     return e == cudaSuccess ? SPECKV_OK : SPECKV_ERR_CUDA;
 }
 

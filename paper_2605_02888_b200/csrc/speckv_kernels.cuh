@@ -1091,8 +1091,8 @@ __device__ __noinline__ void decide_positions(const KParams& P, int b, int gam, 
 // Positions 0..n_pos-1 by all warps of the CTA; the caller synchronises.  Warp 0 has the fewest.
 template <typename T>
 __device__ __forceinline__ void decide_all(const KParams& P, int b, int gam, bool greedy, float scale, int n_pos, RowDecide* pos) {
-    const int per = P.nsplit <= 16 ? 2 : 1;
-    for (int i = (kWarps - 1 - static_cast<int>(threadIdx.x >> 5)) * per; i < n_pos; i += kWarps * per)
+    const int per = P.nsplit <= 16 ? 2 : 1, nw = static_cast<int>(blockDim.x >> 5);
+    for (int i = (nw - 1 - static_cast<int>(threadIdx.x >> 5)) * per; i < n_pos; i += nw * per)
         decide_positions<T>(P, b, gam, greedy, scale, i, n_pos, pos);
 }
 

@@ -21,8 +21,8 @@ namespace speckv {
 // No partials, no tickets.  (Wider slices use sweep_kernel with export_state set.)  Latency-bound: one warp folds a 32 KB row in
 // 16 rounds of loads, and 256 rows of 17 are fewer warps than the SMs hold (64 rows of 4 shards, V = 32,000: 18.4 us, several warps per row 16.4).
 // (Steps in flight: 5 of bf16, 4 of fp32 beside 4 CTAs per SM; one rank of 8 of 256 bf16 rows 54.3 us, with the sweep's shape 57.4.)
-template <typename T>
-__global__ void __launch_bounds__(kThreads, 4) shard_rows_kernel(const __grid_constant__ KParams P, const int row_warps) {
+template <typename T, int U, int CTAS>
+__global__ void __launch_bounds__(kThreads, CTAS) shard_rows_kernel(const __grid_constant__ KParams P, const int row_warps) {
     __shared__ float4 sh_part[kWarps];
     wait_for_predecessors();
     dependents_may_start();
@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(kThreads, 4) shard_rows_kernel(const __grid_co
                                  : static_cast<const T*>(P.d) + static_cast<long long>(b) * P.dsb + static_cast<long long>(pos) * P.dsp;
         const GranRow gr = make_row(row, P.V);
         const int per = (gr.ng + row_warps - 1) / row_warps;
-        WarpSweep<T, sizeof(T) == 2 ? 5 : 4> ws;
+        WarpSweep<T, U> ws;
         ws.start(gr, sub * per, sub * per + per);
         if (!is_target && lane == 0 && sub == 0 && !greedy) {
             // both logits at the draft token, if it falls into this slice
@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(kThreads, 4) shard_rows_kernel(const __grid_co
     }
 }
 
-// Phase 2: one CTA per batch row, the row epilogue of the sweep on the n_shards gathered states of each logit row
+// Phase 2: one CTA (of two warps at least) per batch row, the row epilogue of the sweep on the n_shards gathered states of each logit row
 // (nsplit = n_shards, part_stride apart).  Latency-bound: with a warp per row, a lane per position and a chain of n_shards
 // dependent loads in each, the four calls of 256 rows and 8 shards took 12 us more (with the changes to phases 1 and 3).
 __global__ void __launch_bounds__(kThreads) shard_finish_kernel(const __grid_constant__ KParams P) {
@@ -218,8 +218,8 @@ __global__ void __launch_bounds__(kThreads) shard_pick_kernel(const __grid_const
     __syncthreads();
     if (own < 0) return;
     const int g0 = own * P.draw_pw, g1 = min(sh_src.t.ng, g0 + P.draw_pw);
-    const int tok = res ? find_token<T, true>(sh_src, g0, g1, tau - before, false, warp, kWarps, 1, sh_sum)
-                        : find_token<T, false>(sh_src, g0, g1, tau - before, false, warp, kWarps, 1, sh_sum);
+    const int tok = res ? find_token<T, true>(sh_src, g0, g1, tau - before, false, warp, blockDim.x >> 5, 1, sh_sum)
+                        : find_token<T, false>(sh_src, g0, g1, tau - before, false, warp, blockDim.x >> 5, 1, sh_sum);
     if (lane == 0 && tok >= 0) P.out_tok[static_cast<long long>(b) * (P.G + 1) + ri.n] = tok + P.v_begin;
 }
 

@@ -84,6 +84,16 @@ def test_few_rows_of_wide_slices(dtype, B, G, V, n_shards):
     compare_step(out, ref)
 
 
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("B,G,V,n_shards", [(740, 2, 300, 2), (741, 16, 130, 1), (900, 16, 600, 3), (1200, 1, 2500, 2), (741, 5, 4100, 1)])
+def test_many_rows_of_narrow_slices(dtype, B, G, V, n_shards):
+    # two warps per row in the second call, slice rows of one to a few steps in the first, one to four warps in the last
+    w = synth.Workload("t", B=B, gamma_max=G, V=V, dtype=dtype, gamma_mode="ragged", temperature_mode="mixed", sigma_t=1.5,
+                       sigma_d=synth.SIGMA_LEVELS, frac_identical=0.2, seed=V)
+    s, out, ref = _both(w, n_shards)
+    compare_step(out, ref)
+
+
 def test_bounds_helper():
     width, b = vocab_shard.shard_bounds(128256, 8)
     assert width == 16032 and b[0] == (0, 16032) and b[-1] == (7 * 16032, 128256)
