@@ -127,13 +127,29 @@ void choose_draw(KParams& P, speckv_dtype dt, bool aligned) {
 }
 
 // Short rows: one CTA per batch row (batch_row_kernel) with P.nsplit warps per logit row, as many as leave none without work.
-// The limits lie where the CTA's time, which grows with the length of its rows, meets that of a CTA per logit row, which
-// grows with their number.  Step, gamma up to 8, bf16 / fp32, sweep -> this way: 64 rows, V = 4,000, 21.5 -> 19.7 / 22.6 -> 21.7 us
-// and V = 8,000 23.0 -> 26.8 / 25.6 -> 38.0; 256 rows, V = 8,000, 41.5 -> 36.5 / 49.4 -> 44.0 and V = 16,000 48.0 -> 55.5 / 97 -> 103
-// (of 500); 1,000 rows, V = 3,000, 112 -> 63 / 129 -> 62.
-constexpr int kShortRow = 4096, kShortRowLarge = 8192, kShortRowBatch = 256;
+// The limits lie where the CTA's time, which grows with the length and the number of its rows, meets that of a CTA per logit
+// row, which grows with their number in the batch.  Sweep -> this way (gamma fixed at its largest):
+//   step, bf16 / fp32: 64 rows, gamma 8, V = 4,000, 24.4 -> 19.9 / 24.5 -> 21.5 us; 256 rows, gamma 8, V = 8,000, 55 -> 38 / 63 -> 48;
+//   1,000 rows, gamma 8, V = 3,000, 112 -> 63 / 129 -> 62
+//   few rows of many positions, fp32: step of 4 rows, V = 4,000, gamma 8 17.9 -> 20.5, gamma 16 19.4 -> 30.0, gamma 16, V = 2,000
+//   19.0 -> 22.9 (ragged, where half of the positions are used, 15.4 -> 12.6); signals of 16 rows, V = 4,000, gamma 12 14.0 -> 14.4,
+//   gamma 16 11.4 -> 14.8, gamma 8 10.9 -> 9.9; of 40 rows, gamma 16 (bf16) 16.4 -> 12.6
+//   1,024 rows, gamma 4, V = 14,528, step 132 -> 114 / equal;
+//   large batches, fp32: 1,100 rows, gamma 4, V = 12,000, signals 62.3 -> 48.5, step 153.5 -> 133.9; 4,000 rows, gamma 4, V = 14,528,
+//   signals 157.7 -> 132.1; 12,000 rows, gamma 2, signals V = 20,000 402 -> 328 (gamma 1, V = 14,528 215 -> 209), step V = 14,528
+//   equal, V = 20,000 8 % more.  300 rows, gamma 4, V = 12,000: step 53.7 -> 54.7.
+bool short_rows(const KParams& P) {
+    const bool verify = (P.mode & MODE_VERIFY) != 0;
+    const long long rows = static_cast<long long>(P.B) * P.J, work = static_cast<long long>(P.J) * P.V;  // work: elements of one CTA
+    if (P.B >= 2048 && !verify) return P.V <= (P.J > 1 ? 20480 : 12288);
+    if (P.B >= 1024) return P.V <= 15360;
+    if (P.B >= 256) return P.V <= 8192;
+    if (P.V > 4096) return false;
+    if (verify) return rows > 160 || work <= 98304;
+    return rows > 256 || work <= (rows > 160 ? 45056 : 36864);
+}
 bool choose_batch_rows(KParams& P, speckv_dtype dt, bool aligned) {
-    if (P.V > (P.B >= kShortRowBatch ? kShortRowLarge : kShortRow)) return false;
+    if (!short_rows(P)) return false;
     const int E = 16 / esize(dt);
     const int ng = (P.V + E - 1 + (aligned ? 0 : E - 1)) / E;
     P.nsplit = 1;
@@ -306,8 +322,9 @@ speckv_status run(const speckv_batch* bt, int mode, const float* comp, const spe
     choose_slices(P, bt->dtype, aligned);
     choose_draw(P, bt->dtype, aligned);
     P.n_spans = P.nsplit * kWarps;
+    P.mode = mode;
     const bool by_row = choose_batch_rows(P, bt->dtype, aligned);
-    P.mode = mode; P.bits = bt->entropy_in_bits ? 1 : 0;
+    P.bits = bt->entropy_in_bits ? 1 : 0;
     P.wait_limit = g_wait_limit.load(std::memory_order_relaxed);
     P.d = bt->draft_logits; P.dsb = bt->draft_stride_b; P.dsp = bt->draft_stride_pos;
     P.t = bt->target_logits; P.tsb = bt->target_stride_b; P.tsp = bt->target_stride_pos;

@@ -17,7 +17,9 @@ DEV = "cuda:0"
 
 @pytest.mark.parametrize("dtype", ["bf16", "fp32"])
 @pytest.mark.parametrize("B,G,V", [(9, 1, 4096), (9, 2, 4095), (40, 3, 4097), (5, 8, 4001), (255, 2, 8192), (256, 2, 8192),
-                                   (256, 4, 8191), (256, 1, 8193), (300, 16, 2), (33, 16, 511), (1, 4, 1)])
+                                   (256, 4, 8191), (256, 1, 8193), (300, 16, 2), (33, 16, 511), (1, 4, 1), (4, 16, 2979), (4, 16, 2978),
+                                   (5, 16, 2979), (10, 16, 2305), (10, 16, 2304), (16, 16, 2816), (16, 16, 2817), (17, 16, 4096), (1024, 1, 15360),
+                                   (1023, 1, 8193), (1024, 1, 15361), (2048, 1, 12289), (2048, 2, 15359), (2050, 2, 20480), (2050, 2, 20481)])
 def test_step_and_its_parts(dtype, B, G, V):
     w = synth.Workload("s", B=B, gamma_max=G, V=V, dtype=dtype, gamma_mode="ragged", temperature_mode="mixed", sigma_t=1.0,
                        sigma_d=(0.2, 1.0, 2.0), frac_identical=0.2, seed=B + V)
