@@ -209,6 +209,7 @@ speckv_status speckv_signals_static(const speckv_batch* batch, float* H, float* 
  *   speckv_shard_sweep      local slice -> shard_state [B, 2*gamma_max+1, 4] fp32, shard_tokl [B, gamma_max, 2] fp32
  *      -- all-gather both over the shards, in shard order: all_state [n_shards, B, 2*gamma_max+1, 4],
  *         all_tokl [n_shards, B, gamma_max, 2]
+ *         (shard_state and all_state 16-byte aligned, shard_tokl and all_tokl 8-byte)
  *   speckv_shard_finish     every output of speckv_step except the fresh token of sampled rows (its
  *                           slot holds -1), and row_info (SPECKV_ROW_INFO_BYTES per row, opaque,
  *                           16-byte aligned) for the next two calls; identical on every shard

@@ -708,6 +708,7 @@ speckv_status speckv_shard_sweep(const speckv_batch* local, int64_t v_begin, flo
     speckv_status st = shard_params(local, workspace, workspace_bytes, P, pl);
     if (st != SPECKV_OK || local->B == 0) return st;
     if (!shard_state || !shard_tokl || v_begin < 0 || v_begin > (1LL << 30)) return SPECKV_ERR_INVALID_ARG;
+    if (reinterpret_cast<uintptr_t>(shard_state) % 16 != 0 || reinterpret_cast<uintptr_t>(shard_tokl) % 8 != 0) return SPECKV_ERR_INVALID_ARG;
     const bool al = shard_aligned(local);
     choose_slices(P, local->dtype, al, false, kExportSplit);
     if (static_cast<long long>(P.B) * P.J * P.nsplit > 0x7fffffffLL) return SPECKV_ERR_UNSUPPORTED;
@@ -797,7 +798,7 @@ speckv_status speckv_shard_draw_sums(const speckv_batch* local, const void* row_
     ShardPlan pl;
     speckv_status st = shard_params(local, workspace, workspace_bytes, P, pl);
     if (st != SPECKV_OK || local->B == 0) return st;
-    if (!row_info || !shard_weight) return SPECKV_ERR_INVALID_ARG;
+    if (!row_info || !shard_weight || reinterpret_cast<uintptr_t>(row_info) % 16 != 0) return SPECKV_ERR_INVALID_ARG;
     P.info = static_cast<RowInfo*>(const_cast<void*>(row_info));
     P.weight = shard_weight;
     cudaStream_t cs = static_cast<cudaStream_t>(cuda_stream);
@@ -820,7 +821,7 @@ speckv_status speckv_shard_draw_pick(const speckv_batch* local, int64_t v_begin,
     ShardPlan pl;
     speckv_status st = shard_params(local, workspace, workspace_bytes, P, pl);
     if (st != SPECKV_OK || local->B == 0) return st;
-    if (!row_info || !all_weight || !out_tokens) return SPECKV_ERR_INVALID_ARG;
+    if (!row_info || !all_weight || !out_tokens || reinterpret_cast<uintptr_t>(row_info) % 16 != 0) return SPECKV_ERR_INVALID_ARG;
     if (n_shards < 1 || n_shards > 32 || rank < 0 || rank >= n_shards || v_begin < 0 || v_begin > (1LL << 30))
         return SPECKV_ERR_INVALID_ARG;
     P.info = static_cast<RowInfo*>(const_cast<void*>(row_info));

@@ -76,6 +76,20 @@ def test_workspace_size_and_argument_checks_without_a_gpu():
     assert L.speckv_select_gamma(4, 0x100, None, C.byref(m), None, 0x100, None) == binding.ERR_UNSUPPORTED
 
 
+def test_shard_calls_refuse_buffers_off_the_grid_of_their_records():
+    # the kernels read and write these in words of 16 bytes (states, row records) and 8 (token logits)
+    L = speckv.load_library()
+    b = _cb(V=4000, draft_stride_b=8 * 4000, draft_stride_pos=4000, target_logits=0x1000, target_stride_b=9 * 4000,
+            target_stride_pos=4000, draft_tokens=0x1000, uniforms=0x1000)
+    ok, big = 0x1000, 1 << 30
+    bad = binding.ERR_INVALID_ARG
+    for off in (4, 8):
+        assert L.speckv_shard_sweep(C.byref(b), 0, ok + off, ok, 0x100, big, None) == bad
+        assert L.speckv_shard_draw_sums(C.byref(b), ok + off, ok, 0x100, big, None) == bad
+        assert L.speckv_shard_draw_pick(C.byref(b), 0, 0, 2, ok + off, ok, ok, 0x100, big, None) == bad
+    assert L.speckv_shard_sweep(C.byref(b), 0, ok, ok + 4, 0x100, big, None) == bad
+
+
 def test_sampling_workspace_does_not_outgrow_the_buffers_in_use():
     # a buffer of the size that was asked for when the sums were kept per 256 elements (44 bytes and 12 per chunk of each
     # position) goes on being accepted, whatever the vocabulary; a size for more rows serves fewer
