@@ -52,28 +52,36 @@ def build(force: bool = False, verbose: bool = False, debug: bool = False) -> st
     return out
 
 
-TORCH_LIB_PATH = os.path.join(_CSRC, "_speckv_torch.so")
+def torch_lib_path() -> str:
+    """Where the native argument marshalling built for this Python and this torch lies.  It reads torch's C++ objects directly, so
+    one built for another torch must not be loaded, and the name says which one it is for."""
+    import sysconfig
+
+    import torch
+    tag = f"torch{torch.__version__}.{sysconfig.get_config_var('SOABI')}.abi{int(torch.compiled_with_cxx11_abi())}"
+    return os.path.join(_CSRC, "_speckv_torch." + "".join(c if c.isalnum() or c in ".-" else "_" for c in tag) + ".so")
 
 
 def build_torch(force: bool = False) -> str:
     """Compile the native argument marshalling (csrc/speckv_torch.cpp, host code only) against the installed torch if it is
     missing or older than its sources; return its path."""
     deps = [os.path.join(_CSRC, "speckv_torch.cpp"), os.path.join(_INC, "speckv.h")]
-    if not force and os.path.exists(TORCH_LIB_PATH) and all(os.path.getmtime(d) <= os.path.getmtime(TORCH_LIB_PATH) for d in deps):
-        return TORCH_LIB_PATH
+    out = torch_lib_path()
+    if not force and os.path.exists(out) and all(os.path.getmtime(d) <= os.path.getmtime(out) for d in deps):
+        return out
     import sysconfig
 
     import torch
     from torch.utils import cpp_extension
     cuda = os.path.dirname(os.path.dirname(_nvcc())) if os.path.sep in _nvcc() else "/usr/local/cuda"
     inc = [*cpp_extension.include_paths(), sysconfig.get_paths()["include"], os.path.join(cuda, "include"), _INC]
-    tmp = TORCH_LIB_PATH + f".tmp{os.getpid()}"
+    tmp = out + f".tmp{os.getpid()}"
     cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared",
            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}", *(a for d in inc for a in ("-isystem", d)),
            "-o", tmp, deps[0], *(f"-L{d}" for d in cpp_extension.library_paths()), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
     subprocess.check_call(cmd)
-    os.replace(tmp, TORCH_LIB_PATH)
-    return TORCH_LIB_PATH
+    os.replace(tmp, out)
+    return out
 
 
 if __name__ == "__main__":

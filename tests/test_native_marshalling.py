@@ -1,12 +1,13 @@
 """The native argument marshalling: it refuses (and leaves to the Python path, which raises) whatever the Python checks
 refuse, and makes the same call for everything else."""
 import dataclasses
+import os
 
 import pytest
 import torch
 
 import paper_2605_02888_b200 as speckv
-from paper_2605_02888_b200 import binding, synth
+from paper_2605_02888_b200 import binding, build, synth
 
 from parity import gpu_batch, mlp_pair
 
@@ -29,6 +30,21 @@ def test_cpu_tensors_and_odd_objects_are_left_to_the_python_path():
         nat.step(addr["speckv_step"])
     with pytest.raises(ValueError):
         speckv.speckv_sample_draft(b, torch.zeros(2, 2))
+
+
+def test_a_module_built_for_another_torch_is_not_loaded(monkeypatch):
+    here = build.torch_lib_path()
+    for name, value in (("__version__", "9.9.9+cu999"), ("compiled_with_cxx11_abi", lambda abi=torch.compiled_with_cxx11_abi(): not abi)):
+        with monkeypatch.context() as m:
+            m.setattr(torch, name, value)
+            other = build.torch_lib_path()
+            assert other != here and not os.path.exists(other)
+            # it would have to be built; where that fails the Python path does the calls
+            m.setattr(build.subprocess, "check_call", lambda *a, **k: (_ for _ in ()).throw(OSError("no compiler")))
+            m.setattr(binding, "_native", None)
+            with pytest.warns(UserWarning, match="native argument marshalling"):
+                assert binding._entry(speckv.load_library())[0] is False
+    assert build.torch_lib_path() == here
 
 
 @pytest.mark.gpu
