@@ -85,7 +85,9 @@ def load_library(path: Optional[str] = None) -> C.CDLL:
     L.speckv_verify.argtypes = [C.POINTER(_CBatch), vp, vp, vp, vp, sz, vp]
     L.speckv_step.restype = C.c_int
     L.speckv_step.argtypes = [C.POINTER(_CBatch), vp, C.POINTER(_CMlp)] + [vp] * 8 + [vp, sz, vp]
-    # include/speckv_internal.h: the benchmark's timing aid and two test hooks
+    # include/speckv_internal.h: the benchmark's timing aid and the tests' hooks
+    L.speckv_internal_plan.restype = C.c_int
+    L.speckv_internal_plan.argtypes = [C.POINTER(_CBatch), C.c_int, vp]
     L.speckv_step_profiled.restype = C.c_int
     L.speckv_step_profiled.argtypes = L.speckv_step.argtypes + [vp, vp, vp]
     L.speckv_internal_set_wait_limit.restype = C.c_int

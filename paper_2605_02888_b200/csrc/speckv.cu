@@ -294,6 +294,21 @@ cudaError_t launch_rows(const KParams& P, cudaStream_t st, const Events& ev) {
     return e;
 }
 
+// How a call of signals / verify / step is cut: sizes, slices and draws.  Returns whether it takes a CTA per batch row.
+bool plan_call(KParams& P, const speckv_batch* bt, int mode) {
+    const bool verify = (mode & MODE_VERIFY) != 0;
+    P.B = bt->B; P.G = bt->gamma_max; P.V = bt->V;
+    P.J = verify ? 2 * bt->gamma_max + 1 : bt->gamma_max;
+    P.mode = mode;
+    const int es = esize(bt->dtype);
+    bool aligned = rows_aligned(bt->draft_logits, bt->draft_stride_b, bt->draft_stride_pos, es);
+    if (verify) aligned = aligned && rows_aligned(bt->target_logits, bt->target_stride_b, bt->target_stride_pos, es);
+    choose_slices(P, bt->dtype, aligned);
+    choose_draw(P, bt->dtype, aligned);
+    P.n_spans = P.nsplit * kWarps;
+    return choose_batch_rows(P, bt->dtype, aligned);
+}
+
 // Shared driver of signals / verify / step.
 speckv_status run(const speckv_batch* bt, int mode, const float* comp, const speckv_mlp* mlp, float* H,
                   float* C, float* feat, float* scores, int32_t* gamma_next, int32_t* n_accepted,
@@ -314,16 +329,7 @@ speckv_status run(const speckv_batch* bt, int mode, const float* comp, const spe
     if (ws_bytes < (verify ? pl.total : pl.total_signals)) return SPECKV_ERR_WORKSPACE;
 
     KParams P{};
-    P.B = bt->B; P.G = bt->gamma_max; P.V = bt->V;
-    P.J = verify ? pl.J_full : bt->gamma_max;
-    const int es = esize(bt->dtype);
-    bool aligned = rows_aligned(bt->draft_logits, bt->draft_stride_b, bt->draft_stride_pos, es);
-    if (verify) aligned = aligned && rows_aligned(bt->target_logits, bt->target_stride_b, bt->target_stride_pos, es);
-    choose_slices(P, bt->dtype, aligned);
-    choose_draw(P, bt->dtype, aligned);
-    P.n_spans = P.nsplit * kWarps;
-    P.mode = mode;
-    const bool by_row = choose_batch_rows(P, bt->dtype, aligned);
+    const bool by_row = plan_call(P, bt, mode);
     P.bits = bt->entropy_in_bits ? 1 : 0;
     P.wait_limit = g_wait_limit.load(std::memory_order_relaxed);
     P.d = bt->draft_logits; P.dsb = bt->draft_stride_b; P.dsp = bt->draft_stride_pos;
@@ -394,6 +400,14 @@ SamplePlan make_sample_plan(const speckv_batch* bt) {
     return p;
 }
 
+void plan_sample(KParams& P, const speckv_batch* bt, const SamplePlan& pl) {
+    P.B = bt->B; P.G = bt->gamma_max; P.V = bt->V;
+    P.J = bt->gamma_max;
+    choose_slices(P, bt->dtype, rows_aligned(bt->draft_logits, bt->draft_stride_b, bt->draft_stride_pos, esize(bt->dtype)), true);
+    // (per_warp is 32 at least, so a warp behind the last span has no granule)
+    P.n_spans = P.nsplit * kWarps < pl.most_spans ? P.nsplit * kWarps : pl.most_spans;
+}
+
 speckv_status run_sample(const speckv_batch* bt, const float* uniforms, int32_t* tokens, int32_t* row_status,
                          void* ws, size_t ws_bytes, void* stream) {
     speckv_status st = check_batch(bt, false);
@@ -406,12 +420,7 @@ speckv_status run_sample(const speckv_batch* bt, const float* uniforms, int32_t*
     if (ws_bytes < pl.total) return SPECKV_ERR_WORKSPACE;
 
     KParams P{};
-    P.B = bt->B; P.G = bt->gamma_max; P.V = bt->V;
-    P.J = bt->gamma_max;
-    const bool aligned = rows_aligned(bt->draft_logits, bt->draft_stride_b, bt->draft_stride_pos, esize(bt->dtype));
-    choose_slices(P, bt->dtype, aligned, true);
-    // (per_warp is 32 at least, so a warp behind the last span has no granule)
-    P.n_spans = P.nsplit * kWarps < pl.most_spans ? P.nsplit * kWarps : pl.most_spans;
+    plan_sample(P, bt, pl);
     P.d = bt->draft_logits; P.dsb = bt->draft_stride_b; P.dsp = bt->draft_stride_pos;
     P.gamma = bt->gamma; P.temp = bt->temperature; P.temp_scalar = bt->temperature_scalar;
     P.u = uniforms;
@@ -664,6 +673,19 @@ speckv_status speckv_internal_debug_report(unsigned long long* out4, int reset, 
 int speckv_internal_set_wait_limit(int polls) {
     if (polls < 1) polls = 1;
     return g_wait_limit.exchange(polls);
+}
+
+speckv_status speckv_internal_plan(const speckv_batch* batch, int call, int32_t* plan) {
+    if (!plan || call < 0 || call > 2) return SPECKV_ERR_INVALID_ARG;
+    const speckv_status st = check_batch(batch, call == 1);
+    if (st != SPECKV_OK) return st;
+    if (batch->B == 0) return SPECKV_ERR_INVALID_ARG;
+    KParams P{};
+    bool by_row = false;
+    if (call == 2) plan_sample(P, batch, make_sample_plan(batch));
+    else by_row = plan_call(P, batch, call == 1 ? MODE_SIGNALS | MODE_VERIFY : MODE_SIGNALS);
+    plan[0] = by_row; plan[1] = P.nsplit; plan[2] = P.per_warp; plan[3] = P.n_spans; plan[4] = P.R; plan[5] = P.draw_pw;
+    return SPECKV_OK;
 }
 
 speckv_status speckv_internal_wait_probe(int32_t B, int32_t* row_status, int32_t* out_tokens, void* workspace,

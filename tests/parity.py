@@ -2,6 +2,8 @@
 the CPU oracle and compare element by element under the stated acceptance rules."""
 from __future__ import annotations
 
+import ctypes
+
 import numpy as np
 import torch
 
@@ -45,6 +47,14 @@ def gpu_batch(s: dict, entropy_in_bits=False, temperature_scalar=None, flags=0) 
                         temperature=s.get("temperature"),
                         temperature_scalar=1.0 if temperature_scalar is None else temperature_scalar,
                         uniforms=s.get("uniforms"), entropy_in_bits=entropy_in_bits, flags=flags)
+
+
+def plan_of(c_batch, call: str) -> dict:
+    """How a call on this batch (binding._CBatch) is cut; call: "signals", "step" or "sample".  Host arithmetic only."""
+    out = (ctypes.c_int32 * 6)()
+    rc = speckv.load_library().speckv_internal_plan(ctypes.byref(c_batch), ("signals", "step", "sample").index(call), out)
+    assert rc == 0, rc
+    return dict(zip(("by_row", "slices", "per_warp", "spans", "draw_ctas", "draw_per_warp"), out))
 
 
 def mlp_pair(w: dict, **kw):

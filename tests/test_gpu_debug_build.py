@@ -2,7 +2,7 @@
 logit load and every workspace access of every kernel is compared with the extents of the call's buffers
 and an access outside them is skipped and counted, never performed.  The shapes most likely to expose an
 index mistake go through it here - vocabularies that are not a multiple of anything, ragged gamma, padded
-and misaligned rows, broadcast rows (stride 0), the ring sweep's ragged stages, every target row read, the
+and misaligned rows, broadcast rows (stride 0), large batches with early exit, every target row read, the
 sharded step, draft sampling - and the count must stay at zero with results that match the oracle.  A
 self-test has the checker look at two addresses that no call registered (they are compared, not
 dereferenced) to show that it would have counted them."""
@@ -17,7 +17,7 @@ import oracle
 import paper_2605_02888_b200 as speckv
 from paper_2605_02888_b200 import binding, build, synth, vocab_shard
 
-from parity import compare_step, gpu_batch, mlp_pair, oracle_batch
+from parity import compare_step, gpu_batch, mlp_pair, oracle_batch, plan_of
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
@@ -59,7 +59,7 @@ def _check(w, flags=0, step=0):
 
 def test_no_access_leaves_its_buffers(debug_library):
     L = debug_library
-    # odd vocabularies, ragged gamma, both types: sliced sweep with scalar heads and tails
+    # odd vocabularies, ragged gamma, both types: rows with incomplete first and last granules
     for dtype in ("fp32", "bf16"):
         for V, B, G in ((8, 1, 1), (33, 3, 4), (257, 2, 8), (4099, 3, 5), (20000, 5, 16)):
             w = synth.Workload("d", B=B, gamma_max=G, V=V, dtype=dtype, gamma_mode="ragged", temperature_mode="mixed",
@@ -80,14 +80,16 @@ def test_no_access_leaves_its_buffers(debug_library):
         w = synth.Workload("d", B=B, gamma_max=3, V=V, dtype=dtype, gamma_mode="ragged", temperature=0.8,
                            sigma_d=(0.6,), seed=3)
         _check(w)
-        _check(w, flags=binding.SCHEDULE_SLICED | binding.READ_ALL_TARGET_ROWS)
+        _check(w, flags=binding.READ_ALL_TARGET_ROWS)
     assert _violations(L)[0] == 0, _violations(L)
-    # the ring sweep (fp32, 384 rows and more) with rows that are not whole stages
-    w = synth.Workload("d", B=400, gamma_max=2, V=4100, dtype="fp32", gamma_mode="ragged", temperature=0.9,
-                       sigma_d=(0.5,), seed=4)
-    _check(w)
+    # large fp32 batches: a CTA for each batch row, the sweep with early exit, rows off the 16-byte grid in both
+    for V, by_row in ((4100, 1), (8195, 0)):
+        w = synth.Workload("d", B=400, gamma_max=2, V=V, dtype="fp32", gamma_mode="ragged", temperature=0.9,
+                           sigma_d=(0.5,), seed=4)
+        s, _, _ = _check(w)
+        assert plan_of(gpu_batch(s)._c(), "step")["by_row"] == by_row
     assert _violations(L)[0] == 0, _violations(L)
-    # padded rows (stride > V), misaligned base (element-wise path), one target row broadcast to all (stride 0)
+    # padded rows (stride > V), misaligned base, one target row broadcast to all (stride 0)
     w = synth.Workload("d", B=7, gamma_max=4, V=1000, dtype="bf16", gamma_mode="ragged", temperature=0.9,
                        sigma_d=(0.5,), seed=5)
     s = synth.make_step(w, 0, DEV)
@@ -104,6 +106,15 @@ def test_no_access_leaves_its_buffers(debug_library):
     bro = dict(s, target=s["target"][:1].expand(w.B, -1, -1))
     out = speckv.speckv_verify(gpu_batch(bro))
     torch.cuda.synchronize()
+    assert _violations(L)[0] == 0, _violations(L)
+    # logits whose draft ranges are folded again from differences, draws with normalisers of any size
+    w = synth.Workload("d", B=5, gamma_max=3, V=20001, dtype="bf16", gamma_mode="ragged", temperature=1e-6, sigma_d=(0.5,), seed=7)
+    s = synth.make_step(w, 0, DEV)
+    gm, om = mlp_pair(synth.make_mlp(w, DEV))
+    s2 = dict(s, draft=(s["draft"].float() - 700.0).to(torch.bfloat16), target=(s["target"].float() - 700.0).to(torch.bfloat16))
+    out = speckv.speckv_step(gpu_batch(s2), s["comp"], gm)
+    torch.cuda.synchronize()
+    compare_step(out, oracle.step(oracle_batch(s2), s["comp"].cpu().numpy(), om))
     assert _violations(L)[0] == 0, _violations(L)
     # sharded step (ragged last shard) and draft sampling
     w = synth.Workload("d", B=9, gamma_max=5, V=4099, dtype="fp32", gamma_mode="ragged", temperature=0.8,

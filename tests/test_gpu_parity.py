@@ -10,7 +10,7 @@ import oracle
 import paper_2605_02888_b200 as speckv
 from paper_2605_02888_b200 import binding, synth
 
-from parity import close, compare_step, gpu_batch, mlp_pair, np_logits, oracle_batch
+from parity import close, compare_step, gpu_batch, mlp_pair, np_logits, oracle_batch, plan_of
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
@@ -120,7 +120,7 @@ def test_b256_full_batch_sampled_rows():
 
 
 def test_b512_mixed_full_batch_sampled_rows():
-    # fp32 logits at full size: the bulk-copy ring sweep in the configuration the benchmark can time
+    # fp32 logits at full size, in the configuration the benchmark can time
     w = synth.WORKLOADS["b512_mixed"]
     attrs = synth.row_attrs(w)
     greedy = np.nonzero(attrs.temperature.numpy() == 0)[0]
@@ -136,14 +136,16 @@ def test_b512_mixed_full_batch_sampled_rows():
     assert np.all(ot[np.arange(w.B), n] >= 0) and np.all(ot[np.arange(w.B), n] < w.V)
 
 
-def test_batches_beyond_the_ring_sweep_table_take_the_other_kernel():
-    # more rows than the staged sweep's per-row tables hold: same results from the register-staged kernel
-    w = synth.Workload("t", B=1100, gamma_max=2, V=512, dtype="fp32", gamma_mode="ragged", temperature=0.9,
+@pytest.mark.parametrize("V", [512, 16100])
+def test_batches_of_more_than_a_thousand_rows(V):
+    # short rows, a CTA for each batch row, and rows that the sweep takes
+    w = synth.Workload("t", B=1100, gamma_max=2, V=V, dtype="fp32", gamma_mode="ragged", temperature=0.9,
                        sigma_d=synth.SIGMA_LEVELS, seed=12)
     rows = np.array([0, 1, 511, 1023, 1024, 1099])
     s, out, ref = _run_both(w, rows=rows)
+    assert plan_of(gpu_batch(s)._c(), "step")["by_row"] == (V == 512)
     compare_step(out, ref, rows=rows)
-    w2 = synth.scaled(w, B=1024)   # the largest batch the ring sweep takes
+    w2 = synth.scaled(w, B=1024)
     s, out, ref = _run_both(w2, rows=rows[:4])
     compare_step(out, ref, rows=rows[:4])
 
@@ -241,8 +243,7 @@ def test_sample_draft_against_oracle(dtype, V):
     assert (s["temperature"] == 0).any() and (s["temperature"] > 0).any()
 
 
-def test_sample_draft_very_long_rows_take_the_two_pass_form():
-    # more chunks per row than the one-pass kernel stages: normaliser sweep, then the weights
+def test_sample_draft_of_very_long_rows():
     w = synth.Workload("t", B=3, gamma_max=2, V=600_000, dtype="fp32", gamma_mode="fixed", gamma_fixed=2,
                        temperature_mode="mixed", sigma_d=(0.5,), seed=33)
     s = synth.make_step(w, 0, DEV)
@@ -373,7 +374,7 @@ def test_gamma_max_16_and_strided_views():
     out2 = speckv.speckv_step(gpu_batch(s2), s["comp"], gm)
     for k in out:
         assert torch.equal(out[k], out2[k]), k
-    # misaligned base (element offset 1) takes the element-wise path and gives the same results
+    # misaligned base (element offset 1): other granules, the same results
     off_t = torch.zeros(w.B * (w.gamma_max + 1) * 1000 + 1, dtype=torch.bfloat16, device=DEV)
     off_t[1:] = s["target"].flatten()
     s3 = dict(s); s3["target"] = off_t[1:].view(w.B, w.gamma_max + 1, 1000)
@@ -381,35 +382,39 @@ def test_gamma_max_16_and_strided_views():
     compare_step(out3, ref)
 
 
-def test_ring_sweep_with_padded_rows_and_ragged_ends_fp32():
-    # fp32 logits in a wider buffer: rows 16-byte aligned but not adjacent, V not a multiple of a block
-    # (the ring sweep is chosen for fp32 batches of 384 to 1024 rows)
-    w = synth.Workload("e", B=390, gamma_max=6, V=5004, dtype="fp32", gamma_mode="ragged", temperature_mode="mixed",
+@pytest.mark.parametrize("V", [5004, 9004])
+def test_padded_rows_and_ragged_ends_fp32(V):
+    # fp32 logits in a wider buffer: rows 16-byte aligned but not adjacent, V not a multiple of a block; a CTA for each batch row
+    # and the sweep with early exit
+    w = synth.Workload("e", B=390, gamma_max=6, V=V, dtype="fp32", gamma_mode="ragged", temperature_mode="mixed",
                        sigma_d=(0.4,), frac_onehot=0.05, frac_identical=0.05, seed=14)
     s = synth.make_step(w, 0, DEV)
     gm, om = mlp_pair(synth.make_mlp(w, DEV))
+    assert plan_of(gpu_batch(s)._c(), "step")["by_row"] == (V == 5004)
     ref = oracle.step(oracle_batch(s), s["comp"].cpu().numpy(), om)
     out = speckv.speckv_step(gpu_batch(s), s["comp"], gm)
     compare_step(out, ref)
-    pt = torch.full((w.B, w.gamma_max + 2, 5120), 3.0, device=DEV)
-    pd = torch.full((w.B, w.gamma_max + 1, 5120), 3.0, device=DEV)
+    pt = torch.full((w.B, w.gamma_max + 2, V + 116), 3.0, device=DEV)
+    pd = torch.full((w.B, w.gamma_max + 1, V + 116), 3.0, device=DEV)
     pt[:, 1:w.gamma_max + 2, :w.V] = s["target"]; pd[:, :w.gamma_max, :w.V] = s["draft"]
     s2 = dict(s); s2["target"] = pt[:, 1:w.gamma_max + 2, :w.V]; s2["draft"] = pd[:, :w.gamma_max, :w.V]
     out2 = speckv.speckv_step(gpu_batch(s2), s["comp"], gm)
     for k in out:
         assert torch.equal(out[k], out2[k]), k
-    # an element offset of one breaks the 16-byte alignment: the register-staged kernel's element-wise path
+    # an element offset of one: rows off the 16-byte grid
     flat = torch.zeros(s["target"].numel() + 1, device=DEV)
     flat[1:] = s["target"].flatten()
     s3 = dict(s); s3["target"] = flat[1:].view_as(s["target"])
     compare_step(speckv.speckv_step(gpu_batch(s3), s["comp"], gm), ref)
-    # the same aligned batch through the sliced sweep, asked for by flag
-    compare_step(speckv.speckv_step(gpu_batch(s, flags=binding.SCHEDULE_SLICED), s["comp"], gm), ref)
+    # every target row read; the scheduling hint, which has no effect
+    for flags in (binding.READ_ALL_TARGET_ROWS, binding.SCHEDULE_SLICED):
+        _same_bits(out2, speckv.speckv_step(gpu_batch(s, flags=flags), s["comp"], gm))
 
 
-@pytest.mark.parametrize("name,B,V", [("b256", 16, 128256), ("b512_mixed", 16, 151936), ("b512_mixed", 400, 8000)])
+@pytest.mark.parametrize("name,B,V", [("b256", 16, 128256), ("b512_mixed", 16, 151936), ("b512_mixed", 400, 8000),
+                                      ("b512_mixed", 400, 9000)])
 def test_results_are_deterministic(name, B, V):
-    w = synth.scaled(synth.WORKLOADS[name], B=B, V=V)   # 400 fp32 rows: the ring sweep
+    w = synth.scaled(synth.WORKLOADS[name], B=B, V=V)   # 400 fp32 rows: a CTA for each, and the sweep with early exit
     s = synth.make_step(w, 0, DEV)
     gm, _ = mlp_pair(synth.make_mlp(w, DEV))
     a = {k: v.clone() for k, v in speckv.speckv_step(gpu_batch(s), s["comp"], gm).items()}
@@ -446,7 +451,7 @@ def _same_bits(a, b):
 
 @pytest.mark.parametrize("B,V", [(256, 128256), (300, 8200), (24, 50264)])
 def test_target_rows_behind_a_rejection_are_skipped_without_changing_anything(B, V):
-    # the sliced sweep leaves target rows unread when a rejection at position 0 or 1 is known before their CTAs
+    # the sweep leaves target rows unread when a rejection at position 0 or 1 is known before their CTAs
     # start (a matter of timing, so the full-size batch, where it does happen, a batch of short rows and a small
     # batch, where it mostly does not): with and without the skipping the outputs are the same bits; and they
     # stay the same when every target row behind a row's stop position is overwritten with NaN, read or not
@@ -471,11 +476,11 @@ def test_target_rows_behind_a_rejection_are_skipped_without_changing_anything(B,
 
 
 @pytest.mark.parametrize("name,B,V,flags", [("b256", 64, 32000, 0), ("b512_mixed", 400, 8000, 0), ("b512_mixed", 32, 8000, 0),
-                                            ("b512_mixed", 400, 8000, 4)])
+                                            ("b512_mixed", 400, 9000, 0), ("b512_mixed", 400, 9000, 1)])
 def test_step_can_be_captured_in_a_cuda_graph(name, B, V, flags):
     # the library only enqueues work on the caller's stream (no allocation, no synchronisation), so a step
-    # can be recorded once and replayed: single-launch path, ring sweep + dependent resample kernel, fp32 fallback,
-    # and the sliced sweep asked for by flag for a batch that would take the ring (flags = 4, SPECKV_SCHEDULE_SLICED)
+    # can be recorded once and replayed: the sweep behind its list, a CTA for each batch row, early exit on and off
+    # (flags = 1, SPECKV_READ_ALL_TARGET_ROWS)
     w = synth.scaled(synth.WORKLOADS[name], B=B, V=V)
     s = synth.make_step(w, 0, DEV)
     gm, _ = mlp_pair(synth.make_mlp(w, DEV))
@@ -502,7 +507,7 @@ def test_step_can_be_captured_in_a_cuda_graph(name, B, V, flags):
 
 def test_steps_overlapping_on_several_streams_match_their_serial_results():
     # each call has its own workspace and outputs; the kernels of different calls share the SMs, among them
-    # CTAs that wait for a flag of their own grid and the persistent ring sweep
+    # CTAs that wait for a slot of their own grid's queue
     cfgs = [synth.scaled(synth.WORKLOADS["b256"], B=200), synth.scaled(synth.WORKLOADS["b512_mixed"], B=64, V=32000),
             synth.scaled(synth.WORKLOADS["b1024_loop"], B=300, V=50000), synth.scaled(synth.WORKLOADS["b512_mixed"], B=400, V=16000)]
     items = []

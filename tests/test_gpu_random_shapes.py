@@ -38,10 +38,9 @@ def test_random_shapes(seed):
             out = speckv.speckv_step(gpu_batch(s), s["comp"], gm)
             torch.cuda.synchronize()
             compare_step(out, ref)
-        for flags in (binding.SCHEDULE_SLICED, binding.READ_ALL_TARGET_ROWS):   # the other kernel choice; every target row read
-            out = speckv.speckv_step(gpu_batch(s, flags=flags), s["comp"], gm)
-            torch.cuda.synchronize()
-            compare_step(out, ref)
+        out = speckv.speckv_step(gpu_batch(s, flags=binding.READ_ALL_TARGET_ROWS), s["comp"], gm)
+        torch.cuda.synchronize()
+        compare_step(out, ref)
         if V >= 64 and rnd.random() < 0.4:
             n_shards = rnd.choice([2, 3, 4])
             out = vocab_shard.step_emulated(gpu_batch(s), n_shards, s["comp"], gm)
@@ -59,7 +58,7 @@ def test_random_shapes(seed):
 def test_random_edge_inputs(seed):
     """Masked vocabularies (-inf in the same columns of draft and target), temperatures changed after the
     draft tokens were drawn (1e-6 .. 50: tokens of vanishing probability under both models), planted NaN,
-    +inf, all -inf rows and zero uniforms."""
+    +inf, all -inf rows and zero uniforms.  (Long masked stretches and the ends of the logits' range: test_gpu_range.py.)"""
     rnd = random.Random(seed)
     for it in range(40):
         B = rnd.choice([4, 20, 70, 300, 400])
@@ -99,7 +98,7 @@ def test_random_edge_inputs(seed):
         out = speckv.speckv_step(gpu_batch(s), s["comp"], gm)
         torch.cuda.synchronize()
         compare_step(out, ref)
-        out = speckv.speckv_step(gpu_batch(s, flags=binding.SCHEDULE_SLICED | binding.READ_ALL_TARGET_ROWS), s["comp"], gm)
+        out = speckv.speckv_step(gpu_batch(s, flags=binding.READ_ALL_TARGET_ROWS), s["comp"], gm)
         torch.cuda.synchronize()
         compare_step(out, ref)
         if V >= 1000:

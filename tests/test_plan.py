@@ -1,0 +1,75 @@
+"""How a call is cut into CTAs and warps, over sizes, types and alignments: every granule of a row belongs to a warp, whatever
+the rule gives, and the partials, span sums and draw sums fit the places that the workspace has for them.  Host arithmetic, no GPU."""
+import ctypes as C
+import random
+
+import pytest
+
+import paper_2605_02888_b200 as speckv
+from paper_2605_02888_b200 import binding
+
+from parity import plan_of
+
+
+def batch(B, G, V, dtype, offset=0, pad=0):
+    """offset: elements by which the logits start off a 16-byte boundary; pad: elements between rows"""
+    b = binding._CBatch()
+    es = 2 if dtype == "bf16" else 4
+    b.B, b.gamma_max, b.V, b.dtype = B, G, V, binding.BF16 if dtype == "bf16" else binding.F32
+    b.draft_logits = b.target_logits = 0x10000 + offset * es
+    b.draft_stride_pos = b.target_stride_pos = V + pad
+    b.draft_stride_b, b.target_stride_b = G * (V + pad), (G + 1) * (V + pad)
+    b.draft_tokens = b.uniforms = 0x10000
+    b.temperature_scalar = 1.0
+    return b
+
+
+def check(b, call):
+    p = plan_of(b, call)
+    E = 8 if b.dtype == binding.BF16 else 4
+    aligned = all(x % 16 == 0 for x in (b.draft_logits, b.draft_stride_pos * 16 // E, b.draft_stride_b * 16 // E)) and \
+        (call != "step" or (b.target_stride_b * 16 // E) % 16 == 0)
+    ng = -(-b.V // E) if aligned else (b.V + 2 * (E - 1)) // E   # granules a row can touch
+    warps = p["slices"] if p["by_row"] else 8 * p["slices"]
+    assert warps * p["per_warp"] >= ng, (p, ng)
+    assert 1 <= p["slices"] <= 32 and p["spans"] <= warps
+    if p["by_row"]:
+        assert call != "sample" and 8 % p["slices"] == 0 and p["spans"] == p["slices"]
+    else:
+        assert p["per_warp"] >= 32 and p["per_warp"] % 32 == 0
+        assert p["spans"] * p["per_warp"] >= ng          # a warp without a place for its sum has no granule
+    if call == "step":
+        assert 1 <= p["draw_ctas"] <= 32 and p["draw_ctas"] * 8 * p["draw_per_warp"] >= ng
+    if call == "sample":
+        n = C.c_size_t(0)
+        assert speckv.load_library().speckv_sample_workspace_size(C.byref(b), C.byref(n)) == 0
+        assert n.value >= 4 * (b.B * b.gamma_max + 2 * b.B) + 8 * b.B * b.gamma_max * p["spans"]
+    return p
+
+
+@pytest.mark.parametrize("call", ["signals", "step", "sample"])
+def test_every_granule_has_a_warp(call):
+    rnd = random.Random(5)
+    edges = [1, 7, 8, 9, 255, 256, 257, 4095, 4096, 4097, 8191, 8192, 8193, 12288, 12289, 15360, 15361, 16383, 20480, 20481, 32000, 32768,
+             50257, 128256, 151936, 1 << 20, (1 << 24) + 5]
+    seen = set()
+    for k in range(4000):
+        V = rnd.choice(edges) if k % 2 else int(2 ** rnd.uniform(0, 21))
+        B, G = int(2 ** rnd.uniform(0, 12)), rnd.randint(1, 16)
+        dtype = rnd.choice(["bf16", "fp32"])
+        p = check(batch(B, G, V, dtype, offset=rnd.choice([0, 0, 1, 3]), pad=rnd.choice([0, 0, 8, 5])), call)
+        seen.add(("row", p["slices"]) if p["by_row"] else p["slices"])
+    assert {1, 2, 15, 16, 17, 32} <= seen and {("row", n) for n in {"signals": (1, 2, 4, 8), "step": (1, 2)}.get(call, ())} <= seen, seen
+
+
+def test_which_batches_take_a_cta_per_row():
+    by_row = lambda call, B, G, V: bool(plan_of(batch(B, G, V, "fp32"), call)["by_row"])
+    # short rows in small batches; few of them with many positions go through the sweep
+    assert by_row("step", 1, 8, 4096) and not by_row("step", 1, 8, 4097)
+    assert not by_row("step", 4, 16, 4000) and by_row("step", 4, 16, 2978) and by_row("step", 5, 16, 4000)
+    assert not by_row("signals", 4, 12, 4000) and by_row("signals", 4, 8, 4000) and by_row("signals", 40, 16, 4096)
+    # longer ones with more rows
+    assert by_row("step", 256, 8, 8192) and not by_row("step", 255, 8, 8192)
+    assert by_row("step", 1024, 8, 15360) and not by_row("step", 1024, 8, 15361) and not by_row("step", 4096, 8, 15361)
+    assert by_row("signals", 2048, 2, 20480) and not by_row("signals", 2048, 1, 20480)
+    assert not any(plan_of(batch(B, 4, V, "bf16"), "sample")["by_row"] for B in (1, 64, 4096) for V in (100, 4000, 9000))
