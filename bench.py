@@ -237,7 +237,6 @@ def main():
     ap.add_argument("--no-e2e", action="store_true")
     ap.add_argument("--no-early-exit", action="store_true",
                     help="read every target row (SPECKV_READ_ALL_TARGET_ROWS): the all-positions reference for GB/s")
-    ap.add_argument("--schedule", default="auto", choices=["auto", "sliced"], help="kernel choice hint passed to the library")
     ap.add_argument("--min-seconds", type=float, default=0.5, help="the timed blocks are repeated until this much time has passed")
     ap.add_argument("--dry-run", action="store_true", help="exercise the launcher and the rank plumbing on CPU (gloo), no kernels")
     args = ap.parse_args()
@@ -275,8 +274,7 @@ def main():
         binding._lib = binding.load_library(args.lib)
 
     from paper_2605_02888_b200 import binding as _b
-    flags = (_b.READ_ALL_TARGET_ROWS if args.no_early_exit else 0) | \
-            {"auto": 0, "sliced": _b.SCHEDULE_SLICED}[args.schedule]
+    flags = _b.READ_ALL_TARGET_ROWS if args.no_early_exit else 0
 
     def gpu_batch(s):
         return speckv.Batch(draft_logits=s["draft"], target_logits=s["target"], draft_tokens=s["draft_tokens"],
@@ -491,10 +489,10 @@ def main():
             "config": dict(config_of(w), mean_gamma=float(gam.float().mean()),
                            l2=f"{n_batches} resident batches of {bytes_step[0] / 1e6:.0f} MB alternate (each larger than L2)",
                            parallelism=f"dp{world} (rows sharded, no collective)",
-                           early_exit=not args.no_early_exit, schedule=args.schedule),
+                           early_exit=not args.no_early_exit),
             "timed_blocks": len(blocks_ms), "ms_per_block_median": ms_total,
             "roofline": roofline, "cpu_baseline": cpu_baseline, "parity": parity, "e2e": e2e, "clocks": clocks,
-            "gpu_launches": 2 * args.steps,  # the preparing kernel and the sweep kernel of each step
+            "gpu_launches": 2 * args.steps,  # the preparing kernel and the sweep kernel of each step (no workload has short rows)
             "tokens_per_step_mean": float(outs[0].n_accepted.float().mean()) + 1.0,
         }))
     if dist:

@@ -181,9 +181,10 @@ speckv_status speckv_step(const speckv_batch* batch, const float* comp, const sp
  * library holds that much memory until the process exits.  The caller still owns and passes the
  * inputs and the outputs; arguments, results and row_status are exactly those of speckv_signals.
  *
- *   - A batch that needs more scratch than SPECKV_STATIC_SCRATCH_BYTES is refused with
- *     SPECKV_ERR_STATIC_LIMIT before anything is enqueued (B = 256, gamma_max = 8, V = 128256
- *     needs 2.7 MB; speckv_workspace_size() says 3.8 MB for it because it covers verification too).
+ *   - A batch is refused with SPECKV_ERR_STATIC_LIMIT before anything is enqueued when the signals'
+ *     scratch and four bytes per batch row and 256 columns exceed SPECKV_STATIC_SCRATCH_BYTES
+ *     (B = 256, gamma_max = 8, V = 128256: 2.8 MB; speckv_workspace_size() says 3.3 MB for it because
+ *     it covers verification too).
  *   - The call allocates and frees nothing.  The first call on each device looks up the
  *     array's device address (cudaGetSymbolAddress with that device current) and remembers it;
  *     make that first call outside any stream capture.

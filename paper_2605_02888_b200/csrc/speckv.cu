@@ -34,7 +34,7 @@ inline size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 struct Plan {
     int J_full;      // logit rows per batch row with verification: 2*G + 1
     size_t off_tick, off_info, off_part, off_tokl, off_spans, off_dsum, off_list, total;
-    size_t total_signals;  // what the signals alone may use: the scratch array of speckv_signals_static is held against it
+    size_t total_signals;  // what the signals alone use
 };
 
 inline int esize(speckv_dtype dt) { return dt == SPECKV_BF16 ? 2 : 4; }
@@ -134,7 +134,7 @@ void choose_draw(KParams& P, speckv_dtype dt, bool aligned) {
 //   few rows of many positions, fp32: step of 4 rows, V = 4,000, gamma 8 17.9 -> 20.5, gamma 16 19.4 -> 30.0, gamma 16, V = 2,000
 //   19.0 -> 22.9 (ragged, where half of the positions are used, 15.4 -> 12.6); signals of 16 rows, V = 4,000, gamma 12 14.0 -> 14.4,
 //   gamma 16 11.4 -> 14.8, gamma 8 10.9 -> 9.9; of 40 rows, gamma 16 (bf16) 16.4 -> 12.6
-//   1,024 rows, gamma 4, V = 14,528, step 132 -> 114 / equal;
+//   1,024 rows, gamma 4, V = 14,528: step, bf16 132 -> 114, fp32 equal
 //   large batches, fp32: 1,100 rows, gamma 4, V = 12,000, signals 62.3 -> 48.5, step 153.5 -> 133.9; 4,000 rows, gamma 4, V = 14,528,
 //   signals 157.7 -> 132.1; 12,000 rows, gamma 2, signals V = 20,000 402 -> 328 (gamma 1, V = 14,528 215 -> 209), step V = 14,528
 //   equal, V = 20,000 8 % more.  300 rows, gamma 4, V = 12,000: step 53.7 -> 54.7.
@@ -169,7 +169,6 @@ Plan make_plan(const speckv_batch* bt) {
     p.off_tick = off; off = align_up(off + (6 * B + 4) * sizeof(int));  // tickets, counters, draw queue, first-generation tickets, early stops
     p.off_info = off; off = align_up(off + B * sizeof(RowInfo));
     p.off_part = off; off = align_up(off + B * p.J_full * kMaxSplit * sizeof(float4));
-    off = align_up(off + B * ((static_cast<size_t>(bt->V) + 255) / 256) * sizeof(float));  // (not in use: keeps the sizes that were accepted)
     p.off_tokl = off; off = align_up(off + B * static_cast<size_t>(bt->gamma_max) * sizeof(float2));
     p.total_signals = off < kAlign ? kAlign : off;
     p.off_spans = off; off = align_up(off + B * kMaxSplit * kWarps * sizeof(float2));
@@ -181,6 +180,12 @@ Plan make_plan(const speckv_batch* bt) {
 
 // what the caller must provide
 size_t workspace_total(const speckv_batch* bt) { return make_plan(bt).total; }
+
+// What is held against the scratch array of speckv_signals_static: the signals' scratch and a word per 256 columns of every batch
+// row, which it once had.  More than is used, so that the batches that are refused stay the same.
+size_t static_figure(const speckv_batch* bt) {
+    return make_plan(bt).total_signals + align_up(static_cast<size_t>(bt->B) * ((static_cast<size_t>(bt->V) + 255) / 256) * sizeof(float));
+}
 
 // polls a waiting CTA spends before it gives a row up (SPECKV_ROW_TIMEOUT); lowered by tests only
 std::atomic<int> g_wait_limit{1 << 20};
@@ -575,7 +580,7 @@ speckv_status speckv_signals_static(const speckv_batch* batch, float* H, float* 
     speckv_status st = check_batch(batch, false);
     if (st != SPECKV_OK) return st;
     if (batch->B == 0) return SPECKV_OK;
-    if (make_plan(batch).total_signals > SPECKV_STATIC_SCRATCH_BYTES) return SPECKV_ERR_STATIC_LIMIT;
+    if (static_figure(batch) > SPECKV_STATIC_SCRATCH_BYTES) return SPECKV_ERR_STATIC_LIMIT;
     void* scratch = nullptr;
     if (static_scratch_address(&scratch) != cudaSuccess || !scratch) return SPECKV_ERR_CUDA;
     // run() clears the ticket counters on the caller's stream; nothing else needs a known start

@@ -14,6 +14,7 @@
 //                   locates the inverse-CDF threshold and writes the fresh token.  These CTAs
 //                   sit behind the sweep CTAs in the sweep kernel's own grid and wait (bounded)
 //                   for a row of the queue.
+//   short rows      one CTA per batch row does all of that in one launch (batch_row_kernel).
 #pragma once
 
 #include <cuda_bf16.h>
@@ -76,7 +77,7 @@ __device__ __forceinline__ bool dbg_ok(const void* p, unsigned bytes, int kind) 
 #else
 __device__ __forceinline__ bool dbg_ok(const void*, unsigned, int) { return true; }
 #endif
-enum : int { DBG_LOGIT16 = 1, DBG_LOGIT1 = 2, DBG_WS_LOAD = 3, DBG_WS_STORE = 4, DBG_COPY = 5 };
+enum : int { DBG_LOGIT16 = 1, DBG_LOGIT1 = 2, DBG_WS_LOAD = 3, DBG_WS_STORE = 4 };
 
 enum : int { MODE_SIGNALS = 1, MODE_VERIFY = 2, MODE_MLP = 4 };
 enum : int { PATH_DRAFT = 0, PATH_TARGET = 1, PATH_ARGMAX = 2 };
@@ -507,13 +508,6 @@ __device__ __forceinline__ float4 merge_argmax(float4 a, float4 b) {
     return o;
 }
 
-template <int PATH>
-__device__ __forceinline__ float4 merge_any(float4 a, float4 b, float scale) {
-    if constexpr (PATH == PATH_DRAFT) return merge_draft(a, b, scale);
-    else if constexpr (PATH == PATH_TARGET) return merge_target(a, b);
-    else return merge_argmax(a, b);
-}
-
 __device__ __forceinline__ float4 shfl_xor4(float4 v, int mask) {
     v.x = __shfl_xor_sync(0xffffffffu, v.x, mask);
     v.y = __shfl_xor_sync(0xffffffffu, v.y, mask);
@@ -823,17 +817,6 @@ __device__ __forceinline__ double warp_sum(double v) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
-__device__ __forceinline__ double warp_max(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
-}
-__device__ __forceinline__ double warp_min(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmin(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
-}
-
 // Controller (Sec. 4.3, Eq. 1) for one row, executed by a full warp.  The parameters are fetched
 // first, all at once (ctl_load), so that their memory latency overlaps whatever comes between
 // the load and the evaluation.  Lane k holds hidden unit k's weights, b2[k] and comp[k].

@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(kThreads) prep_kernel(const __grid_constant__ 
 // after the last sweep CTA has started and leaves most of the drain unused.
 // Bound by memory: a CTA streams its 256 KB in 22 us beside 4 others per SM, 6.3 TB/s over the chip while about 530 of the
 // 740 resident CTAs stream; the others are starting (2.8 us) or merging and taking tickets (3 us).  It is the one sweep for
-// all types and sizes: a persistent ring of bulk copies, which fp32 batches of 384 to 1,024 rows took before, streamed at
+// all types and all rows but short ones (batch_row_kernel): a persistent ring of bulk copies, which fp32 batches of 384 to 1,024 rows took before, streamed at
 // 6.7 TB/s but drew its tokens in a launch of its own and could leave no row unread (step of 512 fp32 rows, V = 151,936:
 // 578 us with the ring, 523 this way; 384 rows 440 / 394; 1,000 rows, V = 60,000, 535 / 418).
 // ----------------------------------------------------------------------------------------
@@ -294,7 +294,8 @@ __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sweep_kernel(c
 // fold a logit row, each a contiguous range whose partial is also a span of a bonus draw; the row epilogue and the residual
 // draw follow in the same CTA.  Latency-bound: a CTA's life is a chain of about 10 us behind its loads, so what counts is that
 // a batch row has one such chain and one CTA, not one CTA's start, merge and ticket (6 us) for every logit row (step of 500
-// rows, V = 3,000, gamma up to 8: bf16 64.8 -> 36.5 us, fp32 72.4 -> 37.0; of 8 to 16 rows about 20 -> 17).
+// rows, V = 3,000, gamma up to 8: bf16 64.8 -> 36.5 us, fp32 72.4 -> 37.0; of 8 to 16 rows about 20 -> 17).  Which batches: short_rows()
+// in speckv.cu.
 // ----------------------------------------------------------------------------------------
 template <typename T>
 __global__ void __launch_bounds__(kThreads, 4) batch_row_kernel(const __grid_constant__ KParams P) {
