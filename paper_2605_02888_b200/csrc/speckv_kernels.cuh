@@ -445,7 +445,8 @@ constexpr float kBigSum = 1.1529215e18f;  // 2^60
 // fused multiply-add and four loads in flight: draft sampling of 256 rows, V = 128,256, 83 -> 81 us, step 142.5 -> 141).
 struct TargetState {
     float r, z;
-    __device__ __forceinline__ void init(float m0, float scale) { r = __fmul_rn(m0, scale); z = 0.f; }
+    // (finite also where masked elements stand in front, m0 = kFloor, and the temperature is so low that kFloor * scale overflows)
+    __device__ __forceinline__ void init(float m0, float scale) { r = fmaxf(__fmul_rn(m0, scale), -3.0e38f); z = 0.f; }
     template <typename T>
     __device__ __forceinline__ void add(const Raw<T>& raw, float scale, f2& ga, f2& gb) const {
         f2 x[4];

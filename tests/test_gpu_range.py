@@ -105,6 +105,24 @@ def test_draft_logits_far_beyond_the_exponent_range(dtype, B, G, V, n_shards, T,
 
 
 @pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("B,V,n_shards", [(256, 4096, 0), (3, 40001, 0), (300, 60000, 0), (12, 33000, 3)])
+def test_masked_rows_at_temperatures_next_to_zero(dtype, B, V, n_shards):
+    # -2^100 / T is beyond fp32 here; draft and target allow a few tokens behind a masked stretch
+    G, T = 3, 1e-9
+    draft = torch.full((G, V), float("-inf"), device=DEV)
+    draft[:, -4:] = torch.tensor([0.25, 0.125, 0.25, -0.25], device=DEV)
+    target = torch.full((G + 1, V), float("-inf"), device=DEV)
+    target[:, -4:] = torch.tensor([0.25, 0.125, 0.25, 0.25], device=DEV)
+    s = _shared_rows(draft.to(TYPES[dtype]), target.to(TYPES[dtype]), B, T, seed=V)
+    out, ref = _check(s, n_shards)
+    assert (ref["row_status"] == 0).all() and len(set(ref["n_accepted"])) > 1
+    u = s["uniforms"][:, :G, 0].contiguous()
+    got = speckv.speckv_sample_draft(gpu_batch(s), u)
+    assert (got["row_status"] == 0).all()
+    assert (got["tokens"] == torch.where(u < 0.5, V - 4, V - 2)).float().mean() > 0.99
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
 @pytest.mark.parametrize("V,n_shards", [(4096, 0), (40001, 0), (33000, 3)])
 @pytest.mark.parametrize("T,level", [(0.9, 0.0), (0.9, 3.0e4), (1e-6, 100.0), (1e-6, 416.0), (1e-6, -416.0), (1e-6, 960.0)])
 def test_residual_of_two_tied_tokens(dtype, V, n_shards, T, level):
