@@ -60,12 +60,17 @@ def test_sampled_drafts_over_slices(dtype, B, G, V):
     w = _workload(B, G, V, dtype)
     s = synth.make_step(w, 0, DEV)
     s["gamma"][:] = G
-    u = torch.rand(B, G, device=DEV)
+    u = torch.rand(B, G, device=DEV, generator=torch.Generator(DEV).manual_seed(V))
     rows = np.arange(0, B, max(1, B // 10))
     out = speckv.speckv_sample_draft(gpu_batch(s), u)
     ref = oracle.sample_draft(oracle_batch(s, rows=rows), u.cpu().numpy()[rows])
     clear = ref["near"] == 0
-    assert (out["tokens"].cpu().numpy()[rows][clear] == ref["tokens"][clear]).all() and clear.mean() > 0.8
+    # A uniform is flagged where it lies within 1e-6 of a boundary of the CDF: with a probability of at most the sum of
+    # min(p, 2e-6) over the vocabulary, and a row with any of its G.  Rows are independent; four standard deviations and one row.
+    p = torch.softmax(s["draft"][torch.as_tensor(rows, device=DEV)].double() / 0.9, -1)
+    flagged = 1.0 - torch.prod(1.0 - p.clamp(max=2e-6).sum(-1), -1)
+    most = float(flagged.sum() + 4.0 * (flagged * (1.0 - flagged)).sum().sqrt()) + 1.0
+    assert (out["tokens"].cpu().numpy()[rows][clear] == ref["tokens"][clear]).all() and (~clear).sum() <= most
     assert (out["row_status"] == 0).all() and (out["tokens"] >= 0).all()
 
 
