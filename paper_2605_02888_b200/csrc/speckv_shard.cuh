@@ -87,12 +87,15 @@ __global__ void __launch_bounds__(kThreads, CTAS) shard_rows_kernel(const __grid
 // dependent loads in each, the four calls of 256 rows and 8 shards took 12 us more (with the changes to phases 1 and 3).
 __global__ void __launch_bounds__(kThreads) shard_finish_kernel(const __grid_constant__ KParams P) {
     __shared__ RowDecide sh_pos[kMaxGamma + 1];
+    __shared__ __align__(16) KParams sh_P;
+    params_to_shared(P, &sh_P, 0);
+    __syncthreads();
     wait_for_predecessors();
     dependents_may_start();
     const int b = blockIdx.x;
     const int gam = P.gamma ? P.gamma[b] : P.G;
     const float Tf = P.temp ? P.temp[b] : P.temp_scalar;
-    row_epilogue_cta<float>(P, b, gam, Tf, row_scale(Tf), sh_pos, nullptr, nullptr);
+    row_epilogue_cta<float>(sh_P, b, gam, Tf, row_scale(Tf), sh_pos, nullptr, nullptr);
 }
 
 // Phase 3: grid B * R.  Span weights of the stop position over the local slice: of the row's own

@@ -174,6 +174,7 @@ __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sweep_kernel(c
     __shared__ int sh_last;
     __shared__ int sh_early;
     __shared__ float sh_m0[kWarps];
+    __shared__ __align__(16) KParams sh_P;
     wait_for_predecessors();  // the list and the cleared counters
     dependents_may_start();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -275,18 +276,19 @@ __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sweep_kernel(c
         if (l) __threadfence();
         sh_last = l;
     }
+    params_to_shared(P, &sh_P, 32);  // while the tickets travel
     __syncthreads();
     const int last = sh_last;
-    if (last & 1) prefix_epilogue<T>(P, b, gam, Tf == 0.f, scale, sh_pos);
+    if (last & 1) prefix_epilogue<T>(sh_P, b, gam, Tf == 0.f, scale, sh_pos);
     if (!(last & 2)) return;
     if (P.export_state) {
         const long long row0 = static_cast<long long>(b) * P.J;
         if (warp == 0)
-            export_epilogue(P, b, gam, Tf, P.part + (row0 + P.G + 1 + lane) * P.nsplit, P.nsplit,
+            export_epilogue(sh_P, b, gam, Tf, P.part + (row0 + P.G + 1 + lane) * P.nsplit, P.nsplit,
                             P.part + (row0 + lane) * P.nsplit, P.nsplit);
         return;
     }
-    row_epilogue_cta<T>(P, b, gam, Tf, scale, sh_pos, sh_sum, &sh_src);
+    row_epilogue_cta<T>(sh_P, b, gam, Tf, scale, sh_pos, sh_sum, &sh_src);
 }
 
 // ----------------------------------------------------------------------------------------
@@ -302,6 +304,8 @@ __global__ void __launch_bounds__(kThreads, 4) batch_row_kernel(const __grid_con
     __shared__ RowDecide sh_pos[kMaxGamma + 1];
     __shared__ DrawSrc sh_src;
     __shared__ double sh_sum[64];
+    __shared__ __align__(16) KParams sh_P;
+    params_to_shared(P, &sh_P, 0);
     wait_for_predecessors();
     dependents_may_start();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, b = blockIdx.x;
@@ -337,9 +341,9 @@ __global__ void __launch_bounds__(kThreads, 4) batch_row_kernel(const __grid_con
                     SPECKV_ST(P.spans[static_cast<long long>(b) * P.nsplit + sub], make_float2(part.x, part.y));
             }
         }
-        __syncthreads();
     }
-    row_epilogue_cta<T>(P, b, gam, Tf, scale, sh_pos, sh_sum, &sh_src);
+    __syncthreads();
+    row_epilogue_cta<T>(sh_P, b, gam, Tf, scale, sh_pos, sh_sum, &sh_src);
     if (!verify) return;
     __syncthreads();
     const RowInfo ri = row_info_load(P.info + b);
