@@ -161,6 +161,23 @@ bool choose_batch_rows(KParams& P, speckv_dtype dt, bool aligned) {
     return true;
 }
 
+// A small batch whose sweep has no generations: its CTAs find their work themselves (a thread per batch row), and its draws belong
+// to batch rows.  CTAs per draw: 64 granules per warp, two loads a lane, as far as the span sums' places and the CTA slots go (1.6
+// times, as choose_draw).
+void choose_direct(KParams& P, speckv_dtype dt, bool aligned) {
+    if (P.B > kDirectMostB || P.early) return;
+    P.direct = 1;
+    if (!(P.mode & MODE_VERIFY)) return;
+    const int E = 16 / esize(dt);
+    const int ng = (P.V + E - 1 + (aligned ? 0 : E - 1)) / E;
+    int R = (ng + kWarps * 64 - 1) / (kWarps * 64);
+    const int most = kDirectSums / kWarps, fit = kDrawSmallCtas / P.B;
+    if (R > most) R = most;
+    if (R > fit) R = fit < 1 ? 1 : fit;
+    P.draw_pw = ((ng + R * kWarps - 1) / (R * kWarps) + 7) / 8 * 8;
+    P.R = (ng + P.draw_pw * kWarps - 1) / (P.draw_pw * kWarps);
+}
+
 Plan make_plan(const speckv_batch* bt) {
     Plan p;
     const size_t B = static_cast<size_t>(bt->B);
@@ -265,12 +282,20 @@ constexpr int kPrepRows = 32;  // batch rows per CTA of the preparing kernel at 
 template <typename T>
 cudaError_t launch_sliced(KParams P, long long n_draw, cudaStream_t st, cudaEvent_t before_sweep) {
     P.n_draw = static_cast<int>(n_draw);
+    const unsigned grid = static_cast<unsigned>(static_cast<long long>(P.B) * P.J * P.nsplit + n_draw);
+    if (P.direct) {
+        const int words = P.rdone ? P.B * P.R * kWarps : P.B;
+        cudaError_t e = launch(prep_direct_kernel, static_cast<unsigned>((words + kThreads - 1) / kThreads), st, P);
+        if (e != cudaSuccess) return e;
+        if (before_sweep) cudaEventRecord(before_sweep, st);
+        return launch(sweep_kernel<T>, grid, st, P);
+    }
     int seg = (P.B + 63) / 64;
     seg = seg < kPrepRows ? kPrepRows : (seg + 31) / 32 * 32;
     cudaError_t e = launch(prep_kernel, static_cast<unsigned>((P.B + seg - 1) / seg), st, P, seg);
     if (e != cudaSuccess) return e;
     if (before_sweep) cudaEventRecord(before_sweep, st);
-    return launch(sweep_kernel<T>, static_cast<unsigned>(static_cast<long long>(P.B) * P.J * P.nsplit + n_draw), st, P);
+    return launch(sweep_kernel<T>, grid, st, P);
 }
 
 template <typename T>
@@ -299,15 +324,20 @@ cudaError_t launch_rows(const KParams& P, cudaStream_t st, const Events& ev) {
     return e;
 }
 
+// Does every logit row of the call start on the 16-byte grid?
+bool call_aligned(const speckv_batch* bt, bool verify) {
+    const int es = esize(bt->dtype);
+    return rows_aligned(bt->draft_logits, bt->draft_stride_b, bt->draft_stride_pos, es) &&
+           (!verify || rows_aligned(bt->target_logits, bt->target_stride_b, bt->target_stride_pos, es));
+}
+
 // How a call of signals / verify / step is cut: sizes, slices and draws.  Returns whether it takes a CTA per batch row.
 bool plan_call(KParams& P, const speckv_batch* bt, int mode) {
     const bool verify = (mode & MODE_VERIFY) != 0;
     P.B = bt->B; P.G = bt->gamma_max; P.V = bt->V;
     P.J = verify ? 2 * bt->gamma_max + 1 : bt->gamma_max;
     P.mode = mode;
-    const int es = esize(bt->dtype);
-    bool aligned = rows_aligned(bt->draft_logits, bt->draft_stride_b, bt->draft_stride_pos, es);
-    if (verify) aligned = aligned && rows_aligned(bt->target_logits, bt->target_stride_b, bt->target_stride_pos, es);
+    const bool aligned = call_aligned(bt, verify);
     choose_slices(P, bt->dtype, aligned);
     choose_draw(P, bt->dtype, aligned);
     P.n_spans = P.nsplit * kWarps;
@@ -383,6 +413,7 @@ speckv_status run(const speckv_batch* bt, int mode, const float* comp, const spe
             P.early = P.rdone + 2 * P.B;
         }
     }
+    choose_direct(P, bt->dtype, call_aligned(bt, verify));
     const cudaError_t e = bt->dtype == SPECKV_BF16 ? launch_all<__nv_bfloat16>(P, cs, ev) : launch_all<float>(P, cs, ev);
     return e == cudaSuccess ? SPECKV_OK : SPECKV_ERR_CUDA;
 }

@@ -101,6 +101,8 @@ struct KParams {
     int2* list;     // sliced sweep: one entry per logit row to sweep, in the order of the grid (prep_kernel)
     int* n_list;    //   and how many there are; CTAs behind the last one draw
     int n_draw;     // sliced sweep: CTAs that may draw (R per batch row), 0 = none
+    int direct;  // sweep kernel: a small batch, whose CTAs find their work from gamma and the temperatures themselves, without a list,
+                 // and whose draws belong to batch rows, without a queue
     int draw_pw;  // draw: granules of the stop position that one warp sums; R CTAs of kWarps warps per batch row
     int *q_front, *q_back;  // draw queue: rows with a residual draw fill rdone from the front, the others from the back
     int wait_limit;  // polls a resample CTA spends on its row's completion flag before it gives the row up
@@ -212,6 +214,16 @@ __device__ __forceinline__ uint4 ldg_stream(const void* p) {
     asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
                  : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
                  : "l"(p));
+    return v;
+}
+// The same for a kernel that reads before its griddepcontrol.wait: straight from L2, since a line that L1 still holds of an
+// earlier kernel's read may be older than what has been written since.
+__device__ __forceinline__ uint4 ldg_early(const void* p) {
+    uint4 v;
+    if (!dbg_ok(p, 16, DBG_LOGIT16)) return make_uint4(0xff80ff80u, 0xff80ff80u, 0xff80ff80u, 0xff80ff80u);
+    asm volatile("ld.relaxed.gpu.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "l"(p) : "memory");
     return v;
 }
 __device__ __forceinline__ __nv_bfloat162 as_bf2(uint32_t u) {
@@ -680,10 +692,12 @@ struct WarpSweep {
     bool first_edge, last_edge;
     Raw<T> buf[U];
 
+    template <bool EARLY = false>
     __device__ __forceinline__ Raw<T> load(int k) const {
+        auto ld = [](const uint4* q) { return EARLY ? ldg_early(q) : ldg_stream(q); };
         Raw<T> r;
-        r.a = ldg_stream(p + 32 * GS * k);
-        if constexpr (GS == 2) r.b = (left > 64 * k + 32) ? ldg_stream(p + 64 * k + 32) : gran_fill<T>(__int_as_float(0xff800000));
+        r.a = ld(p + 32 * GS * k);
+        if constexpr (GS == 2) r.b = (left > 64 * k + 32) ? ld(p + 64 * k + 32) : gran_fill<T>(__int_as_float(0xff800000));
         return r;
     }
     // incomplete granules: lane 0 the row's first, lane 1 its last
@@ -696,6 +710,7 @@ struct WarpSweep {
         if (last_edge && lane == 1) e.a = gran_edge<T>(row, ng - 1, __int_as_float(0xff800000));
         return e;
     }
+    template <bool EARLY = false>  // in front of the kernel's griddepcontrol.wait
     __device__ __forceinline__ void start(const GranRow& row, int lo, int hi) {
         const int lane = threadIdx.x & 31;
         a = max(lo, row.whole_lo());
@@ -709,7 +724,7 @@ struct WarpSweep {
 #pragma unroll
         for (int k = 0; k < U; ++k) {
             buf[k] = raw_fill<T>(__int_as_float(0xff800000));
-            if (k < n_main) buf[k] = load(k);
+            if (k < n_main) buf[k] = load<EARLY>(k);
         }
     }
     // A step holding NaN / +inf / only -inf contributes the floor; its owner meets the offending element again
@@ -925,7 +940,7 @@ __device__ __forceinline__ int row_done_slot(const KParams& P, int mode) {  // w
     if (!P.rdone || (threadIdx.x & 31) != 0) return 0;
     return mode == RS_RESIDUAL ? atomicAdd(P.q_front, 1) : P.B - 1 - atomicAdd(P.q_back, 1);
 }
-__device__ __forceinline__ void row_done_signal(const KParams& P, int b, int slot, int mode, int n) {
+__device__ __forceinline__ void row_done_signal(const KParams& P, int b, int slot, int mode, int n) {  // (direct grid: slot b)
     if (!P.rdone) return;
     __threadfence();
     __syncwarp();
@@ -933,8 +948,54 @@ __device__ __forceinline__ void row_done_signal(const KParams& P, int b, int slo
         const int old = atomicOr(P.rdone + slot, kSlotDone | b | (mode == RS_RESIDUAL ? 1 << 24 | n << 25 : 0));
         // a group whose bounded wait ran out before this point left its mark here: the row's fresh
         // token will never be drawn, and the status written above must say so
-        if ((old & kSlotTimeout) && P.status) atomicOr(P.status + b, 16);
+        if ((old & kSlotTimeout) && (!P.direct || mode == RS_RESIDUAL)) {
+            if (P.status) atomicOr(P.status + b, 16);
+            if (P.direct) P.out_tok[static_cast<long long>(b) * (P.G + 1) + n] = -1;
+        }
     }
+}
+
+// A row's record as the drawing CTAs of a direct grid wait for it: two 16-byte words, each stored at once, each of which tells
+// whether it has been stored (prep_direct_kernel leaves all bits set; neither a mode nor a normaliser looks like that).  No
+// fence and no counter between the decision and the draw: with them (a slot of the queue taken, the record, a fence, the flag)
+// the drawing CTAs went on 2 us later.
+__device__ __forceinline__ void row_info_publish(RowInfo* p, const RowInfo& ri) {
+    if (!dbg_ok(p, sizeof(RowInfo), DBG_WS_STORE)) return;
+    asm volatile("{ .reg .b128 v; .reg .b64 lo, hi; mov.b64 lo, {%1, %2}; mov.b64 hi, {%3, %4}; mov.b128 v, {lo, hi}; st.relaxed.gpu.global.b128 [%0], v; }"
+                 :: "l"(p), "r"(ri.mode), "r"(ri.n), "r"(__float_as_int(ri.u2)), "r"(__float_as_int(ri.scale)) : "memory");
+    asm volatile("{ .reg .b128 v; mov.b128 v, {%1, %2}; st.relaxed.gpu.global.b128 [%0], v; }"
+                 :: "l"(reinterpret_cast<char*>(p) + 16), "l"(__double_as_longlong(ri.lse2_p)), "l"(__double_as_longlong(ri.lse2_q)) : "memory");
+}
+// A span's sum, as one word that tells whether it has been stored.
+__device__ __forceinline__ void span_publish(double2* p, double w) {
+    if (!dbg_ok(p, sizeof(double2), DBG_WS_STORE)) return;
+    asm volatile("{ .reg .b128 v; mov.b128 v, {%1, %2}; st.relaxed.gpu.global.b128 [%0], v; }" :: "l"(p), "l"(__double_as_longlong(w)), "l"(0ll) : "memory");
+}
+__device__ __forceinline__ bool span_read(const double2* p, double* w) {
+    long long a = 0, b = 0;
+    if (dbg_ok(p, sizeof(double2), DBG_WS_LOAD))
+        asm volatile("{ .reg .b128 v; ld.relaxed.gpu.global.b128 v, [%2]; mov.b128 {%0, %1}, v; }" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+    *w = __longlong_as_double(a);
+    return b == 0;
+}
+// One thread; false when the bound ran out.
+__device__ __forceinline__ bool row_info_wait(const RowInfo* p, int limit, RowInfo* out) {
+    for (int it = 0; it < limit; ++it) {
+        long long a, b, c, d;
+        asm volatile("{ .reg .b128 v; ld.relaxed.gpu.global.b128 v, [%2]; mov.b128 {%0, %1}, v; }" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+        asm volatile("{ .reg .b128 v; ld.relaxed.gpu.global.b128 v, [%2]; mov.b128 {%0, %1}, v; }" : "=l"(c), "=l"(d) : "l"(reinterpret_cast<const char*>(p) + 16) : "memory");
+        if (static_cast<int>(a) != -1 && c != -1) {
+            out->mode = static_cast<int>(a);
+            out->n = static_cast<int>(a >> 32);
+            out->u2 = __int_as_float(static_cast<int>(b));
+            out->scale = __int_as_float(static_cast<int>(b >> 32));
+            out->lse2_p = __longlong_as_double(c);
+            out->lse2_q = __longlong_as_double(d);
+            return true;
+        }
+        __nanosleep(it < 256 ? 100 : 1000);
+    }
+    return false;
 }
 
 // Bounded wait for a slot of the draw queue (one thread polls).  The slot's value, 0 when the bound ran out.
@@ -1157,14 +1218,24 @@ __device__ __noinline__ void finish_verify(const KParams& P, int b, int gam, flo
     int n;
     const int status = row_walk(P, gam, Tf, dec, &n);
     const int rs_mode = (verify && status == 0 && !greedy) ? (n < gam ? RS_RESIDUAL : RS_BONUS) : RS_NONE;
-    const int slot = row_done_slot(P, rs_mode);  // travels while the outputs are written
+    const bool direct = P.direct != 0;
+    const int slot = direct ? b : row_done_slot(P, rs_mode);  // travels while the outputs are written
     if (verify) {
         // fresh token: known here for greedy rows, drawn by the resample step otherwise
         const int amax_n = __shfl_sync(0xffffffffu, dec.amax, n);
         const double lp_n = __shfl_sync(0xffffffffu, dec.lse2_p, n);
         const double lq_n = __shfl_sync(0xffffffffu, dec.lse2_q, n < gam ? n : 0);
         const float u2_n = __shfl_sync(0xffffffffu, dec.u_res, n);
-        if (lane <= G && !(own_bonus && rs_mode == RS_BONUS && lane == n)) {
+        RowInfo ri;
+        ri.mode = rs_mode;
+        ri.n = n;
+        ri.u2 = (status == 0 && !greedy) ? u2_n : 0.f;
+        ri.scale = scale;
+        ri.lse2_p = lp_n;
+        ri.lse2_q = lq_n;
+        if (direct && lane == 0) row_info_publish(P.info + b, ri);
+        // (a direct grid's draw may be done before this: its place is left alone)
+        if (lane <= G && !(own_bonus && rs_mode == RS_BONUS && lane == n) && !(direct && rs_mode == RS_RESIDUAL && lane == n)) {
             int v = -1;
             if (status == 0) {
                 if (lane < n) v = dec.x;
@@ -1174,14 +1245,7 @@ __device__ __noinline__ void finish_verify(const KParams& P, int b, int gam, flo
         }
         if (lane == 0) {
             P.n_acc[b] = n;
-            RowInfo ri;
-            ri.mode = rs_mode;
-            ri.n = n;
-            ri.u2 = (status == 0 && !greedy) ? u2_n : 0.f;
-            ri.scale = scale;
-            ri.lse2_p = lp_n;
-            ri.lse2_q = lq_n;
-            SPECKV_ST(P.info[b], ri);
+            if (!direct) SPECKV_ST(P.info[b], ri);
         }
     }
     if (P.status && lane == 0) P.status[b] = status;

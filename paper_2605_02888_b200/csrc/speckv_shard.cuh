@@ -122,7 +122,8 @@ __global__ void __launch_bounds__(kThreads, 4) shard_sums_kernel(const __grid_co
     double* dr = P.dsum + static_cast<long long>(b) * (kMaxShares * kWarps);
     double* dp = P.dsum2 + static_cast<long long>(b) * (kMaxShares * kWarps);
     const int span = share * kWarps + warp, g0 = span * P.draw_pw, g1 = min(src.t.ng, g0 + P.draw_pw);
-    const double2 w = res ? warp_weights<T, true, true>(src, g0, g1, P.info + b) : warp_weights<T, false, true>(src, g0, g1, P.info + b);
+    const double2 w = res ? warp_weights<T, true, true>(src, g0, g1, NormOfRecord{P.info + b})
+                           : warp_weights<T, false, true>(src, g0, g1, NormOfRecord{P.info + b});
     if (lane == 0) {
         SPECKV_ST(dr[span], w.x);
         SPECKV_ST(dp[span], w.y);

@@ -152,8 +152,75 @@ __global__ void __launch_bounds__(kThreads) prep_kernel(const __grid_constant__ 
     }
 }
 
+// Small batches are latency-bound: 42 MB stream in 7 us, and the step around them took 33 us.  A direct grid (choose_direct() in
+// speckv.cu) takes from that chain what is not work: its CTAs ask for their first logits 2.5 us earlier, since they need no list, and
+// a row's draw starts and ends on words that it waits for (direct_draw).  Step of 16 bf16 rows, V = 128,256, 30.7 -> 25.2 us; of 64,
+// V = 32,000, 27.5 -> 24.4; of 37, V = 50,257, 27.1 -> 22.9; of one fp32 row, V = 32,000, 13.4 -> 11.1; signals of 128 bf16 rows,
+// V = 128,256, 48.7 -> 45.9.
+//
+// A direct grid needs cleared counters, empty records and empty sums, and nothing of that before its CTAs have folded their slices:
+// this kernel lets them start at once, and they wait for its end behind their first loads.
+__global__ void __launch_bounds__(kThreads) prep_direct_kernel(const __grid_constant__ KParams P) {
+    wait_for_predecessors();
+    dependents_may_start();
+    const int k = blockIdx.x * kThreads + threadIdx.x;
+    if (k < P.B) {
+        P.tick1[k] = 0;
+        if (P.rdone) {
+            P.rdone[k] = 0;
+            int4* info = reinterpret_cast<int4*>(P.info + k);
+            info[0] = info[1] = make_int4(-1, -1, -1, -1);
+        }
+    }
+    const int n = P.R * kWarps;
+    if (P.rdone && k < P.B * n)
+        SPECKV_ST(reinterpret_cast<int4*>(P.dsum)[k / n * kDirectSums + k % n], make_int4(-1, -1, -1, -1));
+}
+// What CTA `entry` of a direct grid sweeps, by the whole CTA: the batch rows' logit rows follow one another (a flagged batch row has
+// one entry), targets in front of drafts.  prep_direct_kernel has waited for everything in front of it before it let this kernel
+// start, so gamma and the temperatures are complete in L2 although this kernel has not waited yet.  Returns the number of entries.
+struct DirectEntry { int2 entry; float temp; };
+constexpr int kDirectMostB = kThreads;
+__device__ __forceinline__ int direct_entry(const KParams& P, int i, DirectEntry* sh, int* sh_scan) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, b = threadIdx.x;
+    const bool verify = (P.mode & MODE_VERIFY) != 0;
+    int cnt = 0, gam = 0;
+    float Tf = 0.f;
+    bool flagged = false;
+    if (b < P.B) {
+        gam = P.gamma ? __ldcg(P.gamma + b) : P.G;
+        Tf = P.temp ? __ldcg(P.temp + b) : P.temp_scalar;
+        flagged = row_status0(P, gam, Tf) != 0;
+        cnt = flagged ? 1 : verify ? 2 * gam + 1 : gam;
+    }
+    int incl = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+    }
+    if (lane == 31) sh_scan[warp] = incl;
+    __syncthreads();
+    int at = incl - cnt, total = 0;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) {
+        const int v = sh_scan[w];
+        at += w < warp ? v : 0;
+        total += v;
+    }
+    const int q = i - at;
+    if (q >= 0 && q < cnt) {
+        const int j = !verify || q <= gam ? q : P.G + 1 + q - (gam + 1);
+        sh->entry = make_int2(b, flagged ? ENTRY_FLAGGED : (j | 1 << 6 | (gam & 31) << 16));
+        sh->temp = Tf;
+    }
+    __syncthreads();
+    return total;
+}
+
 // ----------------------------------------------------------------------------------------
-// Sweep kernel.  CTA i sweeps slice i % nsplit of the logit row in list entry i / nsplit.  With verification the
+// Sweep kernel.  CTA i sweeps slice i % nsplit of the logit row in list entry i / nsplit (direct grid: of the i / nsplit-th logit row
+// in use).  With verification the
 // grid carries more CTAs behind them that draw the fresh tokens of rejected rows in the same launch:
 // CTAs start in index order, so these start exactly when the sweep runs out of slices, wait (with
 // a bound) for a row of the draw queue and fill the SMs that the sweep's last CTAs
@@ -175,17 +242,31 @@ __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sweep_kernel(c
     __shared__ int sh_early;
     __shared__ float sh_m0[kWarps];
     __shared__ __align__(16) KParams sh_P;
-    wait_for_predecessors();  // the list and the cleared counters
-    dependents_may_start();
+    __shared__ DirectEntry sh_entry;
+    __shared__ int sh_scan[kWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool verify = (P.mode & MODE_VERIFY) != 0;
     const int i = static_cast<int>(blockIdx.x) / P.nsplit, s = static_cast<int>(blockIdx.x) - i * P.nsplit;
     int2 entry = make_int2(0, 0);
-    if (i < P.B * P.J && dbg_ok(P.list + i, 8, DBG_WS_LOAD)) entry = __ldcg(P.list + i);
-    const int n_list = __ldcg(P.n_list);
+    int n_list;
+    if (P.direct) {
+        n_list = direct_entry(P, i, &sh_entry, sh_scan);
+        entry = sh_entry.entry;
+    } else {
+        wait_for_predecessors();  // the list and the cleared counters
+        dependents_may_start();
+        if (i < P.B * P.J && dbg_ok(P.list + i, 8, DBG_WS_LOAD)) entry = __ldcg(P.list + i);
+        n_list = __ldcg(P.n_list);
+    }
     if (i >= n_list) {
         const int d = static_cast<int>(blockIdx.x) - n_list * P.nsplit;
-        if (d < P.n_draw) resample_body<T>(P, d);
+        if (P.direct) {
+            wait_for_predecessors();
+            dependents_may_start();
+            if (d < P.n_draw) direct_draw<T>(P, d, &sh_src, sh_sum);
+        } else if (d < P.n_draw) {
+            resample_body<T>(P, d);
+        }
         return;
     }
     const int b = entry.x, j = entry.y & 63, gen = (entry.y >> 6) & 3;
@@ -200,8 +281,15 @@ __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sweep_kernel(c
                                  : static_cast<const T*>(P.d) + static_cast<long long>(b) * P.dsb + static_cast<long long>(pos) * P.dsp;
         const int lo = (s * kWarps + warp) * P.per_warp;  // this warp's granules: the CTA's slice is cut into one contiguous range per warp
         WarpSweep<T, SweepShape<T>::kSteps> ws;
-        ws.start(make_row(row, P.V), lo, lo + P.per_warp);
-        Tf = P.temp ? P.temp[b] : P.temp_scalar;
+        if (P.direct) {
+            ws.template start<true>(make_row(row, P.V), lo, lo + P.per_warp);
+            wait_for_predecessors();
+            dependents_may_start();
+            Tf = sh_entry.temp;
+        } else {
+            ws.start(make_row(row, P.V), lo, lo + P.per_warp);
+            Tf = P.temp ? P.temp[b] : P.temp_scalar;
+        }
         if (threadIdx.x == 0) {
             // one thread reads what is known of the row's stop position, so that the whole CTA takes one decision
             int e = 0;
@@ -257,6 +345,10 @@ __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sweep_kernel(c
             }
         }
     } else {
+        if (P.direct) {
+            wait_for_predecessors();
+            dependents_may_start();
+        }
         if (s != 0) return;  // a flagged row has one CTA, for the epilogue
         gam = P.gamma ? P.gamma[b] : P.G;
         Tf = P.temp ? P.temp[b] : P.temp_scalar;
