@@ -318,6 +318,25 @@ __device__ __forceinline__ bool raw_exceeds2(const Raw<float>& r, const Raw<floa
     return !(max_nan(raw_max(r), raw_max(s)) < m);
 }
 
+// How many raw elements equal m; they become -inf.
+__device__ __forceinline__ float raw_take_equal(Raw<__nv_bfloat16>& r, float m) {  // m is bf16-representable
+    float n = 0.f;
+    auto take = [&](uint32_t& w) {  // by value, so that the two zeros are equal
+        if (bf_lo(w) == m) { w = (w & 0xFFFF0000u) | 0xFF80u; n += 1.f; }
+        if (bf_hi(w) == m) { w = (w & 0x0000FFFFu) | 0xFF800000u; n += 1.f; }
+    };
+    take(r.a.x); take(r.a.y); take(r.a.z); take(r.a.w);
+    return n;
+}
+__device__ __forceinline__ float raw_take_equal(Raw<float>& r, float m) {
+    float n = 0.f;
+    auto take = [&](uint32_t& w) {
+        if (__uint_as_float(w) == m) { w = 0xFF800000u; n += 1.f; }
+    };
+    take(r.a.x); take(r.a.y); take(r.a.z); take(r.a.w);
+    take(r.b.x); take(r.b.y); take(r.b.z); take(r.b.w);
+    return n;
+}
 // Clamp the raw elements from below at kFloor (NaN becomes kFloor as well).
 __device__ __forceinline__ void raw_floor(Raw<__nv_bfloat16>& r) {
     const __nv_bfloat162 f = as_bf2(kFloorBf16x2);
@@ -335,6 +354,20 @@ __device__ __forceinline__ void raw_floor(Raw<float>& r) {
     r.b.y = __float_as_uint(fmaxf(__uint_as_float(r.b.y), kFloor));
     r.b.z = __float_as_uint(fmaxf(__uint_as_float(r.b.z), kFloor));
     r.b.w = __float_as_uint(fmaxf(__uint_as_float(r.b.w), kFloor));
+}
+
+// ----------------------------------------------------------------------------------------
+// Sums and maxima over the warp
+// ----------------------------------------------------------------------------------------
+__device__ __forceinline__ float warp_sumf(float v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+__device__ __forceinline__ float warp_maxf(float v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
 }
 
 // ----------------------------------------------------------------------------------------
@@ -364,40 +397,34 @@ struct DraftState {
     __device__ __forceinline__ float zsum() const { return hsum2(za); }
     __device__ __forceinline__ float ssum() const { return hsum2(sa); }
 
-    template <typename T>
-    __device__ __forceinline__ void slow(const Raw<T>& raw, float scale) {
-        float x[kVec];
-        unpack<T>(raw, x);
-        float vmax = kFloor;
-#pragma unroll
-        for (int j = 0; j < kVec; ++j) {
-            bad |= (x[j] != x[j]) || (x[j] == __int_as_float(0x7f800000));
-            x[j] = fmaxf(x[j], kFloor);
-            vmax = fmaxf(vmax, x[j]);
-        }
-        float z = zsum(), sv = ssum();
-        if (vmax > m) {  // everything gathered so far moves below the new maximum
-            const float rn = __fmul_rn(vmax, scale), dr = __fsub_rn(r, rn), f = ex2f(dr);
-            const float y = fmaf(m, scale, -r), zc = cnt * ex2f(y);  // the elements equal to the old maximum join the sums
-            sv = fmaf(dr, zc + z, fmaf(zc, y, sv)) * f;
-            z = (zc + z) * f;
-            if (f == 0.f) sv = 0.f;  // a product with dr, which behind masked elements is about 2^100 * scale, may be infinite
-            cnt = 0.f;
-            m = vmax;
-            r = rn;
-        }
-#pragma unroll
-        for (int j = 0; j < kVec; ++j) {
-            if (x[j] == m) {
-                cnt += 1.f;
-            } else {
-                const float y = fmaf(x[j], scale, -r), e = ex2f(y);
-                z += e;
-                sv = fmaf(e, y, sv);
-            }
-        }
-        za = pack2(z, 0.f);
+    // The warp's maximum m is the same in all lanes, and a step in which any lane holds an element >= m (or a NaN) is taken by all
+    // of them here: the new maximum is the warp's, so that from then on only a still larger element comes this way.
+    // (A maximum per lane left each of the elements above the first reference to come here by itself, about as many as the range is
+    // longer than what the reference was taken from, at 200 instructions each; the range takes 45 a step.)
+    __device__ __forceinline__ void raise(float v, float scale) {  // everything gathered so far moves below the new maximum v > m
+        const float rn = __fmul_rn(v, scale), dr = __fsub_rn(r, rn), f = ex2f(dr);
+        const float y = fmaf(m, scale, -r), zc = cnt * ex2f(y);  // the elements equal to the old maximum join the sums
+        const float z = zsum();
+        float sv = fmaf(dr, zc + z, fmaf(zc, y, ssum())) * f;
+        if (f == 0.f) sv = 0.f;  // a product with dr, which behind masked elements is about 2^100 * scale, may be infinite
+        za = pack2((zc + z) * f, 0.f);
         sa = pack2(sv, 0.f);
+        cnt = 0.f;
+        m = v;
+        r = rn;
+    }
+    // the lane's largest finite element; notes a NaN / +inf
+    template <typename T>
+    __device__ __forceinline__ float finite_max(const Raw<T>& raw) {
+        const float v = raw_max(raw);
+        if (v < __int_as_float(0x7f800000)) return v;
+        bad = true;
+        return kFloor;
+    }
+    // counts the elements equal to m and takes them out of the step
+    template <typename T>
+    __device__ __forceinline__ void take_top(Raw<T>& raw) {
+        cnt += raw_take_equal(raw, m);
     }
 
     template <typename T>
@@ -413,24 +440,26 @@ struct DraftState {
     }
     template <typename T>
     __device__ __forceinline__ void step(const Raw<T>& raw, float scale) {
-        if (raw_exceeds(raw, m)) slow<T>(raw, scale);  // an element >= m, or a NaN: rare after the warm start
-        else add<T>(raw, scale);
+        Raw<T> v = raw;
+        if (__any_sync(0xffffffffu, raw_exceeds(raw, m))) {  // rare after the warm start
+            const float top = warp_maxf(finite_max<T>(v));
+            if (top > m) raise(top, scale);
+            take_top<T>(v);
+        }
+        add<T>(v, scale);
     }
     // two steps with one test for both (for four the registers run out: signals of 128 bf16 rows, V = 128,256, 53 us; 48 this
     // way; 50 with a test for each)
     template <typename T>
-    __device__ __forceinline__ void step2(const Raw<T>& a, const Raw<T>& b, float scale) {
-        if (raw_exceeds2(a, b, m)) {
-#pragma unroll 1
-            for (int k = 0; k < 2; ++k) {
-                Raw<T> v = a;
-                if (k) v = b;
-                slow<T>(v, scale);
-            }
-        } else {
-            add<T>(a, scale);
-            add<T>(b, scale);
+    __device__ __forceinline__ void step2(Raw<T>& a, Raw<T>& b, float scale) {
+        if (__any_sync(0xffffffffu, raw_exceeds2(a, b, m))) {
+            const float top = warp_maxf(fmaxf(finite_max<T>(a), finite_max<T>(b)));
+            if (top > m) raise(top, scale);
+            take_top<T>(a);
+            take_top<T>(b);
         }
+        add<T>(a, scale);
+        add<T>(b, scale);
     }
     // Sums that are not to be used: see above.  A maximum far below zero that was left behind shows in what it did to them.
     __device__ __forceinline__ bool far(const float4& part, float scale) const {
@@ -542,17 +571,6 @@ __device__ __forceinline__ float4 shfl_xor4(float4 v, int mask) {
 // Warp-level merge of the 32 per-thread partials (result valid in every lane).
 // DRAFT / TARGET: bring every lane to the warp-wide reference, then plain sums.
 // ----------------------------------------------------------------------------------------
-__device__ __forceinline__ float warp_sumf(float v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-__device__ __forceinline__ float warp_maxf(float v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
-}
-
 template <int PATH>
 __device__ __forceinline__ float4 warp_merge(float4 p, float scale) {
     if constexpr (PATH == PATH_DRAFT) {
@@ -790,10 +808,13 @@ struct WarpSweep {
                 else as.template step<T>(v, g * E - shift, GS == 2 ? (g + 32) * E - shift : g * E - shift + kVec / 2);
             };
             if (first_edge || last_edge) process(edge(), lane == 0 ? 0 : ng - 1);
+            // The lanes' votes on a draft step need all of them: the loop ends with the last step that all lanes have, and one without the
+            // last step folds nothing.
+            const int n_all = PATH == PATH_DRAFT ? __shfl_sync(0xffffffffu, n_main, 31) : n_main;
             int i = 0;
             // A step's registers are loaded again when it has been folded, not before: a copy of it to fold from is four registers
             // more, and the 48 there are spilled (b256 and b1024 as above 137 / 432 us, this way with pairs of draft steps 134 / 414).
-            for (; i + U <= n_main; i += U) {
+            for (; i + U <= n_all; i += U) {
 #pragma unroll
                 for (int k = 0; k < U; ++k) {
                     if constexpr (PATH == PATH_DRAFT && U % 2 == 0) {
@@ -806,9 +827,13 @@ struct WarpSweep {
                     if (i + U + k < n_main) buf[k] = load(i + U + k);
                 }
             }
+            const int n_any = PATH == PATH_DRAFT ? __shfl_sync(0xffffffffu, n_main, 0) : n_main;
 #pragma unroll
-            for (int k = 0; k < U; ++k)
-                if (i + k < n_main) process(buf[k], a + lane + 32 * GS * (i + k));
+            for (int k = 0; k < U; ++k) {
+                if (i + k >= n_any) continue;
+                if (PATH == PATH_DRAFT && i + k >= n_main) buf[k] = raw_fill<T>(__int_as_float(0xff800000));
+                process(buf[k], a + lane + 32 * GS * (i + k));
+            }
         }
         float4 part;
         if constexpr (PATH == PATH_DRAFT) {
