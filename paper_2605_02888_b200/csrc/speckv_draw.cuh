@@ -446,12 +446,12 @@ __device__ __forceinline__ double warp_sum8(double (&v)[8]) {
 }
 
 // A plain draw from the sums that the sweep's warps have left of a row (spans: reference in log2 units and sum, one per
-// warp range): nw warps of a CTA, one of which gets the token (find_token).  -1: the row holds a NaN / +inf or has no weight.
+// warp range, or of F pieces of it that are `piece` granules long): nw warps of a CTA, one of which gets the token (find_token).  -1: the row holds a NaN / +inf or has no weight.
 // The first warp picks the span and, once all have summed its parts, the part and the token: picking in all warps was 40 % of
 // the instructions of draft sampling, where every row is drawn from (256 bf16 rows, V = 128,256: 81 us, this way 73).
 template <typename T>
 __device__ __forceinline__ int draw_from_spans(const T* row, int V, float scale, const float2* spans, int n, int per_warp, float u,
-                                               int wi, int nw, int bar, double* sh, DrawSrc* sh_src) {
+                                               int wi, int nw, int bar, double* sh, DrawSrc* sh_src, int F = 1, int piece = 0) {
     const int lane = threadIdx.x & 31;
     if (wi == 0) {
         const int per = (n + 31) >> 5;
@@ -479,8 +479,9 @@ __device__ __forceinline__ int draw_from_spans(const T* row, int V, float scale,
         if (lane == 0) {
             DrawSrc s = make_draw<T>(row, nullptr, V);
             set_norm(s, scale, static_cast<double>(R), 0.0);  // an fp32 value: exact whatever its size
-            s.r0 = none ? 0 : own * per_warp;
-            s.r1 = none ? 0 : min(s.t.ng, s.r0 + per_warp);
+            const int w = own / F, k = own - w * F, lo = w * per_warp, a = max(lo, s.t.whole_lo());
+            s.r0 = none ? 0 : k > 0 ? a + k * piece : lo;
+            s.r1 = none ? 0 : min(s.t.ng, k < F - 1 ? min(a + (k + 1) * piece, lo + per_warp) : lo + per_warp);
             s.tau = tau - before;
             *sh_src = s;
         }

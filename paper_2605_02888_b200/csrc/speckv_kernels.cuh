@@ -98,6 +98,7 @@ struct KParams {
     int B, G, V, J, nsplit, R, mode, bits;
     int per_warp;  // sweep kernel: 16-byte granules of a logit row that one warp folds; a slice is kWarps times that
     int n_spans;    // spans per batch row (verification) or position (draft sampling)
+    int fine, fine_groups;  // draft sampling: spans per warp range, and groups of steps in each (the last one has what is left)
     int2* list;     // sliced sweep: one entry per logit row to sweep, in the order of the grid (prep_kernel)
     int* n_list;    //   and how many there are; CTAs behind the last one draw
     int n_draw;     // sliced sweep: CTAs that may draw (R per batch row), 0 = none
@@ -507,15 +508,17 @@ struct TargetState {
         ga = add2(ga, e0); gb = add2(gb, e1);
         ga = add2(ga, e2); gb = add2(gb, e3);
     }
-    // one step with its maximum taken first
+    // one step with its maximum taken first; returns what the sum gathered so far was multiplied by
     template <typename T>
-    __device__ __forceinline__ void careful(const Raw<T>& raw, float scale) {
+    __device__ __forceinline__ float careful(const Raw<T>& raw, float scale) {
         const float v = raw_max(raw), rn = __fmul_rn(v, scale);
-        if (!(v < __int_as_float(0x7f800000))) { z = __int_as_float(0x7fc00000); return; }
-        if (rn > r) { z *= ex2f(__fsub_rn(r, rn)); r = rn; }
+        if (!(v < __int_as_float(0x7f800000))) { z = __int_as_float(0x7fc00000); return 1.f; }
+        float f = 1.f;
+        if (rn > r) { f = ex2f(__fsub_rn(r, rn)); z *= f; r = rn; }
         f2 ga = pack2(0.f, 0.f), gb = ga;
         add(raw, scale, ga, gb);
         z += hsum2(add2(ga, gb));
+        return f;
     }
     __device__ __forceinline__ float4 partial() const { return make_float4(r, z, 0.f, 0.f); }
 };
@@ -691,6 +694,8 @@ __device__ __noinline__ float4 draft_far(const T* p, int V, int lo, int hi, floa
     return warp_merge<PATH_DRAFT>(make_float4(m, bad ? __int_as_float(0x7fc00000) : cnt, z, s / scale), scale);
 }
 
+constexpr int kFineStride = kThreads + 4;  // floats between the sums of a lane's pieces, so that 4 lanes each can read one piece
+constexpr int kMostFine = 8;
 // ----------------------------------------------------------------------------------------
 // One WARP sweeps granules [lo, hi) of one logit row.  Lane l owns
 // granules l, l+32, ... of the range; a step folds kVec elements per lane (bf16: one granule, fp32: two granules 32
@@ -764,9 +769,15 @@ struct WarpSweep {
         }
         return m0;
     }
-    // PATH_DRAFT: through draft() only
-    template <int PATH>
-    __device__ __forceinline__ float4 run(float m0, float scale, bool* far = nullptr) {
+    // The spans that a warp leaves of a row which is to be drawn from: its range in n pieces of `groups` times U steps each, piece k's
+    // sum in the lane's sh[k * kFineStride].
+    struct Fine {
+        float* sh;
+        int n, groups;
+    };
+    // PATH_DRAFT: through draft() only.  FINE: the pieces' sums are in shared memory, relative to the warp's reference.
+    template <int PATH, bool FINE = false>
+    __device__ __forceinline__ float4 run(float m0, float scale, bool* far = nullptr, const Fine fine = Fine()) {
         const int lane = threadIdx.x & 31;
         DraftState ds; TargetState ts; ArgmaxState as;
         if constexpr (PATH == PATH_DRAFT) ds.init(m0, scale);
@@ -774,6 +785,10 @@ struct WarpSweep {
         else as.init(m0);
         if constexpr (PATH == PATH_TARGET) {
             if (first_edge || last_edge) ts.template careful<T>(edge(), scale);
+            // FINE: ts.z is the present piece's sum, `behind` what lane 1 has of the row's last granule
+            float behind = 0.f;
+            int piece = 0, left_groups = fine.groups;
+            if (FINE && lane == 1) { behind = ts.z; ts.z = 0.f; }
             // steps i .. i+n-1 went into ga, gb
             auto close = [&](f2 ga, f2 gb, int i, int n) {
                 const float g = hsum2(add2(ga, gb));
@@ -781,7 +796,13 @@ struct WarpSweep {
                     ts.z += g;
                 } else {
 #pragma unroll 1
-                    for (int k = i; k < i + n; ++k) ts.template careful<T>(load(k), scale);
+                    for (int k = i; k < i + n; ++k) {
+                        const float f = ts.template careful<T>(load(k), scale);
+                        if (FINE && f != 1.f) {
+                            behind *= f;
+                            for (int q = 0; q < piece; ++q) fine.sh[q * kFineStride] *= f;
+                        }
+                    }
                 }
             };
             int i = 0;
@@ -795,12 +816,28 @@ struct WarpSweep {
                     ts.template add<T>(cur, scale, ga, gb);
                 }
                 close(ga, gb, i, U);
+                if (FINE && --left_groups == 0) {  // (a lane has fine.n * fine.groups whole groups at most)
+                    fine.sh[piece * kFineStride] = ts.z;
+                    ts.z = 0.f;
+                    ++piece;
+                    left_groups = fine.groups;
+                }
             }
             f2 ga = pack2(0.f, 0.f), gb = ga;
 #pragma unroll
             for (int k = 0; k < U; ++k)
                 if (i + k < n_main) ts.template add<T>(buf[k], scale, ga, gb);
             close(ga, gb, i, n_main - i);
+            if (FINE) {
+                const float R = warp_maxf(ts.r), f = ex2f(ts.r - R);
+                if (piece < fine.n) fine.sh[piece++ * kFineStride] = ts.z;
+                else fine.sh[(fine.n - 1) * kFineStride] += ts.z;
+                for (; piece < fine.n; ++piece) fine.sh[piece * kFineStride] = 0.f;
+                if (last_edge && lane == 1) fine.sh[min((ng - 1 - a) / (fine.groups * U * 32 * GS), fine.n - 1) * kFineStride] += behind;
+                if (f != 1.f)
+                    for (int q = 0; q < fine.n; ++q) fine.sh[q * kFineStride] *= f;
+                return make_float4(R, 0.f, 0.f, 0.f);
+            }
         } else {
             const int shift = meta & 15;
             auto process = [&](const Raw<T>& v, int g) {  // g: granule of the first half

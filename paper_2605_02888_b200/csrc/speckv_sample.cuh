@@ -3,7 +3,9 @@
 //
 // A drafted position is one logit row, swept like a target row: each warp leaves the sum of its contiguous range, and
 // these sums are the spans of a plain draw (speckv_draw.cuh), so the CTA that completes the row reads one warp range again
-// and nothing else.
+// and nothing else.  Of a long range it leaves the sums of up to eight pieces, so that what is read again is a granule per thread, one
+// round trip: every row is drawn from, and the ranges read again were an eighth of the traffic (256 bf16 rows of 8, V = 128,256, 70.8 ->
+// 65 us; 287 fp32 rows of 6, V = 29,184, 31.3 -> 27.9).
 #pragma once
 
 #include "speckv_draw.cuh"
@@ -27,16 +29,19 @@ __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sample_kernel(
     __shared__ float sh_m0[kWarps];
     __shared__ DrawSrc sh_src;
     __shared__ double sh_sum[64];
-    wait_for_predecessors();
-    dependents_may_start();
+    __shared__ float sh_fine[kMostFine * kFineStride];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int r = blockIdx.x / P.nsplit;  // draw: batch row b, drafted position i
     const int s = blockIdx.x - r * P.nsplit;
     const int b = r / P.G, i = r - b * P.G;
-    const int gam = P.gamma ? P.gamma[b] : P.G;
-    const float Tf = P.temp ? P.temp[b] : P.temp_scalar;
+    // clear_kernel has waited for everything in front of it before it let this kernel start: what this one reads is complete in L2
+    // although it has not waited yet, and it writes nothing before it has.
+    const int gam = P.gamma ? __ldcg(P.gamma + b) : P.G;
+    const float Tf = P.temp ? __ldcg(P.temp + b) : P.temp_scalar;
     const int bits = row_status0(P, gam, Tf);
     if (bits || i >= gam) {  // nothing to draw at this position
+        wait_for_predecessors();
+        dependents_may_start();
         if (s == 0 && threadIdx.x == 0) {
             P.out_tok[r] = -1;
             if (i == 0 && bits && P.status) P.status[b] = bits;
@@ -51,17 +56,32 @@ __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sample_kernel(
     {
         const int lo = (s * kWarps + warp) * P.per_warp;
         WarpSweep<T, SweepShape<T>::kSteps> ws;
-        ws.start(make_row(row, P.V), lo, lo + P.per_warp);
+        ws.template start<true>(make_row(row, P.V), lo, lo + P.per_warp);
+        wait_for_predecessors();
+        dependents_may_start();
         const float m0 = ws.template warm<true>(sh_m0);
-        float2 v;
+        const int at = s * kWarps + warp;
         if (greedy) {
             const float4 p = ws.template run<PATH_ARGMAX>(m0, scale);
-            v = make_float2(p.z != 0.f ? __int_as_float(0x7fc00000) : p.x, p.y);
-        } else {
+            if (lane == 0 && at * P.fine < n) SPECKV_ST(spans[at * P.fine], make_float2(p.z != 0.f ? __int_as_float(0x7fc00000) : p.x, p.y));
+        } else if (P.fine == 1) {
             const float4 p = ws.template run<PATH_TARGET>(m0, scale);
-            v = make_float2(p.x, p.y);
+            if (lane == 0 && at < n) SPECKV_ST(spans[at], make_float2(p.x, p.y));
+        } else {
+            const float4 p = ws.template run<PATH_TARGET, true>(m0, scale, nullptr, {sh_fine + threadIdx.x, P.fine, P.fine_groups});
+            __syncwarp();
+            // four lanes add up a piece
+            const int k = lane >> 2;
+            double sum = 0.0;
+            if (k < P.fine) {
+                const float* x = sh_fine + k * kFineStride + warp * 32 + (lane & 3) * 8;
+#pragma unroll
+                for (int q = 0; q < 8; ++q) sum += static_cast<double>(x[q]);
+            }
+            sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+            sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+            if (k < P.fine && (lane & 3) == 0 && at * P.fine + k < n) SPECKV_ST(spans[at * P.fine + k], make_float2(p.x, static_cast<float>(sum)));
         }
-        if (lane == 0 && s * kWarps + warp < n) SPECKV_ST(spans[s * kWarps + warp], v);
     }
     __syncthreads();
     if (P.nsplit > 1) {  // else this CTA is the row's last: no ticket (256 bf16 rows, V = 128,256: 73.4 us with it, 71.3 without)
@@ -80,7 +100,7 @@ __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sample_kernel(
     bool bad = false;
     if (greedy) {
         float4 g = make_float4(kFloor, __int_as_float(0x7fffffff), 0.f, 0.f);
-        for (int k = lane; k < n; k += 32) {
+        for (int k = lane * P.fine; k < n; k += 32 * P.fine) {
             const float2 v = dbg_ok(spans + k, 8, DBG_WS_LOAD) ? __ldcg(spans + k) : make_float2(kFloor, 0.f);
             g = merge_argmax(g, make_float4(v.x, v.y, v.x != v.x ? 1.f : 0.f, 0.f));
         }
@@ -88,7 +108,8 @@ __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sample_kernel(
         bad = g.z != 0.f || !(g.x > kFloor);
         tok = __float_as_int(g.y);
     } else {
-        tok = draw_from_spans<T>(row, P.V, scale, spans, n, P.per_warp, P.u[r], warp, kWarps, 1, sh_sum, &sh_src);
+        tok = draw_from_spans<T>(row, P.V, scale, spans, n, P.per_warp, P.u[r], warp, kWarps, 1, sh_sum, &sh_src, P.fine,
+                                 P.fine_groups * SweepShape<T>::kSteps * 32 * (kVec * static_cast<int>(sizeof(T)) / 16));
         if (tok == kNotMine) return;
         bad = tok < 0;
     }
