@@ -473,7 +473,10 @@ __device__ __forceinline__ int draw_from_spans(const T* row, int V, float scale,
             float2 x = v[0];
 #pragma unroll
             for (int q = 1; q < 8; ++q) if (i == q) x = v[q];
-            return static_cast<double>(x.y) * static_cast<double>(ex2f(x.x - R));
+            // Of a total of one or more, a span of less than 2^-100 counts as empty: its elements, below 2^-126 each, read as 0, so that
+            // a threshold of 0 would find nothing in it.
+            const double weight = static_cast<double>(x.y) * static_cast<double>(ex2f(x.x - R));
+            return weight < 0x1p-100 ? 0.0 : weight;
         }, static_cast<double>(u), &before, &total, &tau);
         const bool none = __any_sync(0xffffffffu, bad) || own < 0;
         if (lane == 0) {

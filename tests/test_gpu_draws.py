@@ -242,3 +242,36 @@ def test_shard_masses(dtype, n, V):
                     want[0] = (pt - torch.softmax(s["draft"][b, k].double() / T, 0)).clamp(min=0)[a:e].sum()
             # fp32 exponentials of fp32 arguments of up to ~30: 2e-6 of the mass of p, in differences too
             assert np.abs(got[b] - want).max() <= 5e-6 * max(want[1], 1e-3), (b, got[b], want)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("B,G,V", [(100, 8, 16384), (100, 8, 16389), (100, 8, 33003), (100, 8, 65537), (95, 8, 70007), (40, 4, 151936)])
+def test_sampled_drafts_from_pieces(dtype, B, G, V):
+    # a warp's range in one, two and up to eight pieces; rows whose front is masked, and rows with elements at their end that lie more
+    # than 2^60 above what the sums began with: the pieces summed before are brought to the new reference
+    w = _workload(B, G, V, dtype)
+    s = synth.make_step(w, 0, DEV)
+    s["gamma"][:] = G
+    s["draft"][::3, :, : V * 7 // 10] = float("-inf")
+    s["draft"][1::3, :, V - 40:] += 60.0
+    s["draft"][1::3, :, V * 9 // 16] += 59.0
+    s["draft"][2::6, :, V - 1] += 100.0
+    s["temperature"][5::7] = 0.0
+    u = torch.rand(B, G, device=DEV, generator=torch.Generator(DEV).manual_seed(V))
+    u[:, 0], u[:, 1] = 0.0, 1.0 - 2.0 ** -24
+    rows = np.arange(0, B, 11)
+    out = speckv.speckv_sample_draft(gpu_batch(s), u)
+    ref = oracle.sample_draft(oracle_batch(s, rows=rows), u.cpu().numpy()[rows])
+    tok, want = out["tokens"].cpu().numpy()[rows], ref["tokens"]
+    # The oracle flags a row where any of its uniforms is near a boundary, as the two imposed ones are; here each position by itself,
+    # from a cumulative sum in 64 bits.  A uniform is near one with a probability of at most sum(min(p, 2e-6)).
+    at = torch.as_tensor(rows, device=DEV)
+    p = torch.softmax(s["draft"][at].double() / 0.9, -1)
+    cdf = p.cumsum(-1)
+    x = u[at].double().unsqueeze(-1) * cdf[..., -1:]
+    greedy = (s["temperature"].cpu().numpy()[rows] == 0.0)[:, None]
+    clear = ((cdf - x).abs().amin(-1) > 1e-6).cpu().numpy() | greedy
+    assert (tok[clear] == want[clear]).all()
+    near = p.clamp(max=2e-6).sum(-1)[:, 2:]
+    assert (~clear[:, 2:]).sum() <= float(near.sum() + 4.0 * near.sum().sqrt()) + 1.0
+    assert (out["row_status"] == 0).all() and (out["tokens"] >= 0).all()
