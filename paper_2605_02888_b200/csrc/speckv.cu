@@ -33,7 +33,7 @@ inline size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 struct Plan {
     int J_full;      // logit rows per batch row with verification: 2*G + 1
-    size_t off_tick, off_info, off_part, off_tokl, off_spans, off_dsum, off_list, total;
+    size_t off_pos, off_tick, off_info, off_part, off_tokl, off_spans, off_dsum, off_list, total;
     size_t total_signals;  // what the signals alone use
 };
 
@@ -107,11 +107,11 @@ void choose_slices(KParams& P, speckv_dtype dt, bool aligned, bool sample = fals
     P.nsplit = (ng + pw * kWarps - 1) / (pw * kWarps);
 }
 
-constexpr int kEarlyPositions = 2;   // positions whose acceptance tests the sliced sweep takes ahead of the rest of the row
 // CTAs per draw and granules per warp: P.R, P.draw_pw.  16,384 elements per CTA; a small batch spreads over the CTA slots
 // (1.6 times), and many rows (of which about a third draw) share 4,096 CTAs rather than pay a CTA's start and end for every
 // 16,384 elements.  (V = 128,256, bf16, 4 / 8 / 16 / 32 CTAs per draw: step of 1,024 rows 399 / 408 / 427 / 462 us, of 256
 // rows 141 / 138 / 138 / 141.)
+constexpr int kBriefSlice = 131072;  // bytes of a slice from which on the test of a position beyond the second pays
 constexpr int kDrawElems = 16384, kDrawSmallCtas = 1184, kDrawMostCtas = 4096;
 void choose_draw(KParams& P, speckv_dtype dt, bool aligned) {
     const int E = 16 / esize(dt);
@@ -183,7 +183,8 @@ Plan make_plan(const speckv_batch* bt) {
     const size_t B = static_cast<size_t>(bt->B);
     p.J_full = 2 * bt->gamma_max + 1;
     size_t off = 0;
-    p.off_tick = off; off = align_up(off + (6 * B + 4) * sizeof(int));  // tickets, counters, draw queue, first-generation tickets, early stops
+    p.off_pos = off; off += 2 * B * sizeof(int);  // positions' tickets
+    p.off_tick = off; off = align_up(off + (4 * B + 4) * sizeof(int));  // tickets, counters, draw queue, early stops
     p.off_info = off; off = align_up(off + B * sizeof(RowInfo));
     p.off_part = off; off = align_up(off + B * p.J_full * kMaxSplit * sizeof(float4));
     p.off_tokl = off; off = align_up(off + B * static_cast<size_t>(bt->gamma_max) * sizeof(float2));
@@ -400,17 +401,24 @@ speckv_status run(const speckv_batch* bt, int mode, const float* comp, const spe
         P.rdone = P.n_list + 4;
         P.tokl = reinterpret_cast<float2*>(w + pl.off_tokl);
         P.spans = reinterpret_cast<float2*>(w + pl.off_spans);
-        // generation order: positions 0..k of every batch row first, so that their acceptance tests are in
-        // before the CTAs of the later target rows start (most walks that stop early stop at the first two
-        // positions, and a later position's test would come too late for the CTAs behind it anyway)
-        P.k_early = P.G >= 2 ? kEarlyPositions - 1 : 0;
+        // position 0 of every batch row first and the later target rows position by position, so that a position's acceptance test is in
+        // before the CTAs of the later target rows start
         P.read_all = (bt->flags & SPECKV_READ_ALL_TARGET_ROWS) ? 1 : 0;
         // ... where the grid has that many CTAs: the third generation has to start after the first one's tests, that is
         // one and a half rounds of CTA slots behind it (one row, V = 32,000: taking the tests for nothing cost 4 us of 20)
-        const long long ahead = static_cast<long long>(P.B) * P.nsplit * (2 * (P.k_early + 1) + P.G - P.k_early - 1);
+        const long long ahead = static_cast<long long>(P.B) * P.nsplit * (P.G + 1);
         if (2 * ahead >= 3 * cta_slots(bt->dtype)) {
-            P.tick_early = P.rdone + P.B;
-            P.early = P.rdone + 2 * P.B;
+            P.early = P.rdone + P.B;
+            P.tick_pos = reinterpret_cast<unsigned long long*>(w + pl.off_pos);
+            P.pos_bits = P.nsplit <= 7 ? 4 : 8;  // twice nsplit arrivals at most
+            // Position by position the tests of one are in before the next one's CTAs start, where a position has a round of CTAs or its
+            // CTAs are short; else batch rows that complete one after the other are worth more (position by position: 256 bf16 rows,
+            // V = 128,256, 131.9 -> 133.3 us, 96 greedy fp32 rows 85.1 -> 86.3; 512 fp32 rows, V = 151,936, 495 -> 475).  A test keeps a CTA
+            // slot for 2.5 us: of short slices only the first two positions (all of them: 1,000 fp32 rows, V = 20,000, 173 -> 184 us,
+            // 600 bf16 rows of 4, V = 14,000, 69.7 -> 76.4), and no more where the rows go one by one.
+            const bool brief = P.per_warp * kWarps * 16 < kBriefSlice;
+            P.rows_major = !brief && static_cast<long long>(P.B) * P.nsplit < cta_slots(bt->dtype);
+            P.n_tests = brief || P.rows_major ? 2 : 64 / P.pos_bits;
         }
     }
     choose_direct(P, bt->dtype, call_aligned(bt, verify));

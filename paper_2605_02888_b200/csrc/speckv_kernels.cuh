@@ -107,12 +107,14 @@ struct KParams {
     int draw_pw;  // draw: granules of the stop position that one warp sums; R CTAs of kWarps warps per batch row
     int *q_front, *q_back;  // draw queue: rows with a residual draw fill rdone from the front, the others from the back
     int wait_limit;  // polls a resample CTA spends on its row's completion flag before it gives the row up
-    // Generation order of the sweep (verification, early != nullptr): first the draft and target rows of
-    // positions 0..k_early of every batch row, then the remaining draft rows, last the remaining target rows,
-    // which are left unread where the walk is already known to have stopped at a position <= k_early.
-    int k_early, read_all;
-    int* early;       // [B] 0 = not known yet, else stop position + 1, or G + 2 when the walk passes k_early
-    int* tick_early;  // [B] arrivals of the first generation's CTAs
+    // Order of the sweep (verification): first the draft and target row of position 0 of every batch row, then the other draft rows,
+    // last the other target rows, position by position (rows_major: batch row by batch row), which are left unread where the walk is already known to have stopped in
+    // front of them (early != nullptr).
+    int read_all;
+    int* early;       // [B] the lowest position + 1 at which a test has ended the walk so far
+    unsigned long long* tick_pos;  // [B] arrivals of each position's draft and target slices, pos_bits bits each
+    int pos_bits, n_tests;  // positions from n_tests on are not tested
+    int rows_major;
     const void* d; long long dsb, dsp;
     const void* t; long long tsb, tsp;
     const int* tok; const int* gamma; const float* temp; float temp_scalar; const float* u;
@@ -1088,7 +1090,7 @@ struct RowDecide {
 // draft row, target row and uniform.
 // Latency-bound: one batch row in 15 slices (fp32, V = 32,000, gamma 4), with a lane per position the prefix and the row
 // epilogue each walked a chain of 11 dependent round trips and the step took 45.1 us; this way 23.0 us.  256 rows of
-// bf16, V = 128,256: 150.5 -> 145.6 us (the chain is also the end of a large step).  The prefix epilogue and the row
+// bf16, V = 128,256: 150.5 -> 145.6 us (the chain is also the end of a large step).  The test of a position and the row
 // epilogue call this one compiled body, so that both reach the same bits.
 // Decides positions first, first + 1 (16 lanes each) or first alone.  A logit row has nsplit partials: its slices', adjacent in
 // P.part, or (part_stride) the states of as many vocabulary shards, part_stride apart.
@@ -1216,28 +1218,15 @@ __device__ __forceinline__ void decide_all(const KParams& P, int b, int gam, boo
         decide_positions<T>(P, b, gam, greedy, scale, i, n_pos, pos);
 }
 
-// Prefix epilogue (a whole CTA): run when the partials of a batch row's first positions 0..k are in, while
-// the rest of the row is still being swept.  It takes the acceptance tests of those positions and
-// publishes where the walk stops if it stops there, so that CTAs which have not started yet can leave
-// target rows behind that position unread.  early[b] = stop position + 1, or G + 2 when the walk passes k.
+// The acceptance test of one position (one warp), run when the partials of its draft and target row are in, while the rest of the
+// batch row is still being swept.  A position that ends the walk is noted, so that CTAs which have not started yet can leave
+// the target rows behind it unread.
 template <typename T>
-__device__ __noinline__ void prefix_epilogue(const KParams& P, int b, int gam, bool greedy, float scale, RowDecide* pos) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    decide_all<T>(P, b, gam, greedy, scale, min(P.k_early, gam) + 1, pos);
-    __syncthreads();
-    if (warp == 0) {
-        bool ends = false;
-        if (lane <= P.k_early && lane <= gam) {
-            const RowDecide& d = pos[lane];
-            ends = d.tbad || d.dbad || (lane < gam && (d.badtok || !d.accept));
-        }
-        const unsigned stop = __ballot_sync(0xffffffffu, ends);
-        if (lane == 0) {
-            const int e = stop ? __ffs(stop) : P.G + 2;
-            asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(P.early + b), "r"(e) : "memory");
-        }
-    }
-    __syncthreads();  // pos is used again when the same CTA completes the row
+__device__ __noinline__ void test_position(const KParams& P, int b, int gam, bool greedy, float scale, int i, RowDecide* pos) {
+    decide_positions<T>(P, b, gam, greedy, scale, i, i + 1, pos);
+    __syncwarp();
+    const RowDecide& d = pos[i];
+    if ((threadIdx.x & 31) == 0 && (d.tbad || d.dbad || d.badtok || !d.accept)) atomicMin(P.early + b, i + 1);
 }
 
 // log2(e) / T, the factor of every exponent of a row (greedy rows: T = 1).

@@ -51,30 +51,12 @@ __device__ __noinline__ void row_epilogue_cta(const KParams& P, int b, int gam, 
 // Grid: a segment of batch rows per CTA; every CTA reads all rows' gamma and temperature for the prefix.
 // ----------------------------------------------------------------------------------------
 enum : int { ENTRY_FLAGGED = 256 };  // entry: (batch row, row index j | generation << 6 | ENTRY_FLAGGED | gamma << 16)
-struct PrepCounts {
-    int a0, a1, b, c;  // entries of position 0 and position 1 of the first generation, of the second and the third generation
-    __device__ __forceinline__ void add(const PrepCounts& o) { a0 += o.a0; a1 += o.a1; b += o.b; c += o.c; }
-};
-__device__ __forceinline__ PrepCounts prep_counts(const KParams& P, int gam, float Tf) {
-    const int k1 = P.early ? P.k_early + 1 : 0;
-    PrepCounts r{0, 0, 0, 0};
-    if (row_status0(P, gam, Tf)) {  // one entry, for the row epilogue
-        if (k1) r.a0 = 1; else r.b = 1;
-        return r;
-    }
-    const bool verify = (P.mode & MODE_VERIFY) != 0;
-    if (k1 >= 1) r.a0 = 2;
-    if (k1 >= 2) r.a1 = 1 + (gam >= 2 ? 1 : 0);
-    r.b = max(gam - k1, 0);
-    if (verify) r.c = max(gam + 1 - k1, 0);
-    return r;
-}
-__device__ __forceinline__ PrepCounts shfl_up(const PrepCounts& v, int o) {
-    return {__shfl_up_sync(0xffffffffu, v.a0, o), __shfl_up_sync(0xffffffffu, v.a1, o), __shfl_up_sync(0xffffffffu, v.b, o),
-            __shfl_up_sync(0xffffffffu, v.c, o)};
-}
 __global__ void __launch_bounds__(kThreads) prep_kernel(const __grid_constant__ KParams P, int seg) {
-    __shared__ PrepCounts sh[2][kWarps];
+    // rows of each gamma (and, last, flagged ones) in front of this CTA's segment and in all
+    constexpr int kFlagged = kMaxGamma + 1, kBins = kMaxGamma + 2;
+    __shared__ int sh[2][kBins];
+    if (threadIdx.x < 2 * kBins) sh[threadIdx.x / kBins][threadIdx.x % kBins] = 0;
+    __syncthreads();
     wait_for_predecessors();
     dependents_may_start();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -82,73 +64,96 @@ __global__ void __launch_bounds__(kThreads) prep_kernel(const __grid_constant__ 
     for (int b = b0 + threadIdx.x; b < b1; b += kThreads) {
         P.tick1[b] = 0;
         if (P.rdone) { P.tick2[b] = 0; P.rdone[b] = 0; }
-        if (P.early) { P.tick_early[b] = 0; P.early[b] = 0; }
+        if (P.early) { P.tick_pos[b] = 0; P.early[b] = 0x7fffffff; }
     }
-    PrepCounts before{0, 0, 0, 0}, total{0, 0, 0, 0};
     for (int b = threadIdx.x; b < P.B; b += kThreads) {
-        const PrepCounts c = prep_counts(P, P.gamma ? P.gamma[b] : P.G, P.temp ? P.temp[b] : P.temp_scalar);
-        total.add(c);
-        if (b < b0) before.add(c);
+        const int gam = P.gamma ? P.gamma[b] : P.G;
+        const int bin = row_status0(P, gam, P.temp ? P.temp[b] : P.temp_scalar) ? kFlagged : gam;
+        atomicAdd(&sh[1][bin], 1);
+        if (b < b0) atomicAdd(&sh[0][bin], 1);
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const PrepCounts x = {__shfl_down_sync(0xffffffffu, before.a0, o), __shfl_down_sync(0xffffffffu, before.a1, o),
-                              __shfl_down_sync(0xffffffffu, before.b, o), __shfl_down_sync(0xffffffffu, before.c, o)};
-        const PrepCounts y = {__shfl_down_sync(0xffffffffu, total.a0, o), __shfl_down_sync(0xffffffffu, total.a1, o),
-                              __shfl_down_sync(0xffffffffu, total.b, o), __shfl_down_sync(0xffffffffu, total.c, o)};
-        before.add(x);
-        total.add(y);
-    }
-    if (lane == 0) { sh[0][warp] = before; sh[1][warp] = total; }
     __syncthreads();
     if (warp != 0) return;
-    before = total = PrepCounts{0, 0, 0, 0};
-    for (int w = 0; w < kWarps; ++w) { before.add(sh[0][w]); total.add(sh[1][w]); }
-    const int n_list = total.a0 + total.a1 + total.b + total.c;
+    // lane p: rows that have a draft row at position p - 1, that is a target row at position p (gamma >= p)
+    int before = lane >= 1 && lane <= kMaxGamma ? sh[0][lane] : 0, total = lane >= 1 && lane <= kMaxGamma ? sh[1][lane] : 0;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_down_sync(0xffffffffu, before, o), y = __shfl_down_sync(0xffffffffu, total, o);
+        if (lane + o < 32) { before += x; total += y; }
+    }
+    const bool verify = (P.mode & MODE_VERIFY) != 0;
+    // First generation: position 0 of every row (one entry for a flagged one); second: the other draft rows, batch row by batch row;
+    // third: the other target rows, position by position or batch row by batch row.
+    const int ok_before = __shfl_sync(0xffffffffu, before, 1), ok_total = __shfl_sync(0xffffffffu, total, 1);
+    const int per0 = verify ? 2 : 1;
+    int at_a = per0 * ok_before + sh[0][kFlagged];
+    const int n_a = per0 * ok_total + sh[1][kFlagged];
+    int at_b = n_a, n_b = 0, at_r = ok_before;
+    for (int p = 2; p <= P.G; ++p) {
+        at_b += __shfl_sync(0xffffffffu, before, p);
+        at_r += __shfl_sync(0xffffffffu, before, p);
+        n_b += __shfl_sync(0xffffffffu, total, p);
+    }
+    int scan = lane >= 1 ? total : 0;  // rows of the third generation in front of position `lane`
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, scan, o);
+        if (lane >= o) scan += x;
+    }
+    int at_c = n_a + n_b + scan - total + before;  // lane p: where the segment's next row of position p goes
+    at_r += n_a + n_b;  // rows_major: where the segment's next row's entries of the third generation go
+    const int n_c = verify ? __shfl_sync(0xffffffffu, scan, 31) : 0;
     if (blockIdx.x == 0 && lane == 0) {
-        *P.n_list = n_list;
+        *P.n_list = n_a + n_b + n_c;
         *P.q_front = 0;
         *P.q_back = 0;
     }
-    const bool verify = (P.mode & MODE_VERIFY) != 0;
-    const int k1 = P.early ? P.k_early + 1 : 0;
-    // where the segment's first row starts in each generation
-    before.a1 += total.a0;
-    before.b += total.a0 + total.a1;
-    before.c += total.a0 + total.a1 + total.b;
+    const unsigned below = (1u << lane) - 1;
+    const int jd = verify ? P.G + 1 : 0;  // row index of draft position 0
     for (int r0 = b0; r0 < b1; r0 += 32) {
         const int b = r0 + lane;
-        PrepCounts c{0, 0, 0, 0};
         int gam = 0;
         bool flagged = false;
         if (b < b1) {
             gam = P.gamma ? P.gamma[b] : P.G;
-            const float Tf = P.temp ? P.temp[b] : P.temp_scalar;
-            flagged = row_status0(P, gam, Tf) != 0;
-            c = prep_counts(P, gam, Tf);
+            flagged = row_status0(P, gam, P.temp ? P.temp[b] : P.temp_scalar) != 0;
+            if (flagged) gam = 0;
         }
-        PrepCounts at = c;
+        auto put = [&](int i, int j, int gen) { SPECKV_ST(P.list[i], make_int2(b, j | gen << 6 | (gam & 31) << 16)); };
+        const unsigned ok = __ballot_sync(0xffffffffu, gam > 0), bad = __ballot_sync(0xffffffffu, flagged);
+        const int a = at_a + per0 * __popc(ok & below) + __popc(bad & below);
+        if (flagged) SPECKV_ST(P.list[a], make_int2(b, ENTRY_FLAGGED));
+        if (gam > 0) {
+            put(a, jd, 0);
+            if (verify) put(a + 1, 0, 0);
+        }
+        at_a += per0 * __popc(ok) + __popc(bad);
+        int more = max(gam - 1, 0), incl = more;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            const PrepCounts v = shfl_up(at, o);
-            if (lane >= o) at.add(v);
+            const int x = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += x;
         }
-        const PrepCounts last = {__shfl_sync(0xffffffffu, at.a0, 31), __shfl_sync(0xffffffffu, at.a1, 31), __shfl_sync(0xffffffffu, at.b, 31),
-                                 __shfl_sync(0xffffffffu, at.c, 31)};
-        at.a0 += before.a0 - c.a0; at.a1 += before.a1 - c.a1; at.b += before.b - c.b; at.c += before.c - c.c;
-        before.add(last);
-        if (b >= b1) continue;
-        auto put = [&](int i, int j, int gen) { SPECKV_ST(P.list[i], make_int2(b, j | gen << 6 | (gam & 31) << 16)); };
-        if (flagged) {
-            SPECKV_ST(P.list[k1 ? at.a0 : at.b], make_int2(b, ENTRY_FLAGGED));
+        for (int p = 1; p < gam; ++p) put(at_b + incl - more + p - 1, jd + p, 1);
+        at_b += __shfl_sync(0xffffffffu, incl, 31);
+        if (!verify) continue;
+        if (P.rows_major) {
+            int all = gam;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int x = __shfl_up_sync(0xffffffffu, all, o);
+                if (lane >= o) all += x;
+            }
+            for (int p = 1; p <= gam; ++p) put(at_r + all - gam + p - 1, p, 2);
+            at_r += __shfl_sync(0xffffffffu, all, 31);
             continue;
         }
-        const int jd = verify ? P.G + 1 : 0;  // row index of draft position 0
-        if (k1 >= 1) { put(at.a0, 0, 0); put(at.a0 + 1, jd, 0); }
-        if (k1 >= 2) { put(at.a1, 1, 0); if (gam >= 2) put(at.a1 + 1, jd + 1, 0); }
-        for (int p = k1; p < gam; ++p) put(at.b + p - k1, jd + p, 1);
-        if (verify)
-            for (int p = k1; p <= gam; ++p) put(at.c + p - k1, p, 2);
+        for (int p = 1; p <= P.G; ++p) {
+            const unsigned has = __ballot_sync(0xffffffffu, gam >= p);
+            const int c = __shfl_sync(0xffffffffu, at_c, p);
+            if (gam >= p) put(c + __popc(has & below), p, 2);
+            if (lane == p) at_c += __popc(has);
+        }
     }
 }
 
@@ -292,7 +297,7 @@ __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sweep_kernel(c
         }
         if (threadIdx.x == 0) {
             // one thread reads what is known of the row's stop position, so that the whole CTA takes one decision
-            int e = 0;
+            int e = 0x7fffffff;
             if (P.early && gen == 2 && !P.read_all)
                 asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(e) : "l"(P.early + b) : "memory");
             sh_early = e;
@@ -301,7 +306,7 @@ __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sweep_kernel(c
         const bool greedy = (Tf == 0.f);
         scale = row_scale(Tf);
         const long long pidx = (static_cast<long long>(b) * P.J + j) * P.nsplit + s;  // this CTA's partial
-        if (gen == 2 && sh_early != 0 && sh_early <= P.k_early + 1) {
+        if (gen == 2 && sh_early <= pos) {
             // The walk stopped at a position before this one: the row epilogue never looks here, the partial only has to
             // be finite.
             if (threadIdx.x == 0)
@@ -354,24 +359,29 @@ __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sweep_kernel(c
         Tf = P.temp ? P.temp[b] : P.temp_scalar;
     }
 
-    // tickets: the last of the row's CTAs of positions 0..k_early takes their acceptance tests, the last of all its
-    // CTAs runs the row epilogue; nobody waits
+    // tickets: the last of a position's CTAs takes its acceptance test, the last of all of the row's CTAs runs the row epilogue;
+    // nobody waits
     if (threadIdx.x == 0) {
         const int n_rows = verify ? 2 * gam + 1 : gam;
         const int n_tickets = row_ok ? n_rows * P.nsplit : 1;
-        const int n_pre = (min(P.k_early, gam) + 1 + min(P.k_early + 1, gam)) * P.nsplit;
         __threadfence();
-        int pre = -1;
-        if (P.early && row_ok && gen == 0) pre = atomicAdd(P.tick_early + b, 1);
-        const int all = atomicAdd(P.tick1 + b, 1);
-        const int l = (all == n_tickets - 1 ? 2 : 0) | (pre == n_pre - 1 ? 1 : 0);
+        int l = 0;
+        if (P.early && row_ok && pos < gam && pos < P.n_tests) {
+            const int sh = pos * P.pos_bits;
+            const unsigned long long old = atomicAdd(P.tick_pos + b, 1ull << sh);
+            l = static_cast<int>(old >> sh & ((1ull << P.pos_bits) - 1)) == 2 * P.nsplit - 1 ? 1 : 0;
+        }
+        if (atomicAdd(P.tick1 + b, 1) == n_tickets - 1) l = 2;  // (the whole row's epilogue: no test before it)
         if (l) __threadfence();
         sh_last = l;
     }
     params_to_shared(P, &sh_P, 32);  // while the tickets travel
     __syncthreads();
     const int last = sh_last;
-    if (last & 1) prefix_epilogue<T>(sh_P, b, gam, Tf == 0.f, scale, sh_pos);
+    if (last & 1) {
+        if (warp == 0) test_position<T>(sh_P, b, gam, Tf == 0.f, scale, pos, sh_pos);
+        return;
+    }
     if (!(last & 2)) return;
     if (P.export_state) {
         const long long row0 = static_cast<long long>(b) * P.J;
