@@ -111,7 +111,6 @@ void choose_slices(KParams& P, speckv_dtype dt, bool aligned, bool sample = fals
 // (1.6 times), and many rows (of which about a third draw) share 4,096 CTAs rather than pay a CTA's start and end for every
 // 16,384 elements.  (V = 128,256, bf16, 4 / 8 / 16 / 32 CTAs per draw: step of 1,024 rows 399 / 408 / 427 / 462 us, of 256
 // rows 141 / 138 / 138 / 141.)
-constexpr int kBriefSlice = 131072;  // bytes of a slice from which on the test of a position beyond the second pays
 constexpr int kDrawElems = 16384, kDrawSmallCtas = 1184, kDrawMostCtas = 4096;
 void choose_draw(KParams& P, speckv_dtype dt, bool aligned) {
     const int E = 16 / esize(dt);
@@ -161,11 +160,27 @@ bool choose_batch_rows(KParams& P, speckv_dtype dt, bool aligned) {
     return true;
 }
 
+// Does the call write one of its outputs over its gamma or its temperatures?
+bool overwrites_rows(const KParams& P) {
+    auto in = [&](const void* out, size_t words, const void* rows) {
+        const uintptr_t o = reinterpret_cast<uintptr_t>(out), r = reinterpret_cast<uintptr_t>(rows);
+        return out && rows && o < r + 4 * static_cast<size_t>(P.B) && r < o + 4 * words;
+    };
+    const size_t B = static_cast<size_t>(P.B), G = static_cast<size_t>(P.G);
+    const struct { const void* p; size_t words; } outs[] = {{P.gamma_next, B}, {P.n_acc, B}, {P.status, B}, {P.out_tok, B * (G + 1)},
+        {P.H, B * G}, {P.C, B * G}, {P.feat, 4 * B}, {P.scores, B * static_cast<size_t>(P.n_out)}};
+    for (const auto& o : outs)
+        if (in(o.p, o.words, P.gamma) || in(o.p, o.words, P.temp)) return true;
+    return false;
+}
+
 // A small batch whose sweep has no generations: its CTAs find their work themselves (a thread per batch row), and its draws belong
-// to batch rows.  CTAs per draw: 64 granules per warp, two loads a lane, as far as the span sums' places and the CTA slots go (1.6
+// to batch rows.  Not where the call writes over gamma or the temperatures (the next gamma in the place of this step's): every CTA reads
+// those of all rows, the later ones while the epilogues of the first rows write; a list is complete before the sweep starts.
+// CTAs per draw: 64 granules per warp, two loads a lane, as far as the span sums' places and the CTA slots go (1.6
 // times, as choose_draw).
 void choose_direct(KParams& P, speckv_dtype dt, bool aligned) {
-    if (P.B > kDirectMostB || P.early) return;
+    if (P.B > kDirectMostB || P.n_tests || overwrites_rows(P)) return;
     P.direct = 1;
     if (!(P.mode & MODE_VERIFY)) return;
     const int E = 16 / esize(dt);
@@ -176,6 +191,25 @@ void choose_direct(KParams& P, speckv_dtype dt, bool aligned) {
     if (R > fit) R = fit < 1 ? 1 : fit;
     P.draw_pw = ((ng + R * kWarps - 1) / (R * kWarps) + 7) / 8 * 8;
     P.R = (ng + P.draw_pw * kWarps - 1) / (P.draw_pw * kWarps);
+}
+
+// Order of the sweep and its early tests (verification, large batches): position 0 of every batch row first and the later target rows
+// position by position, so that a position's acceptance test is in before the CTAs of the later target rows start
+constexpr int kBriefSlice = 131072;  // bytes of a slice from which on the test of a position beyond the second pays
+void choose_tests(KParams& P, speckv_dtype dt) {
+    // ... where the grid has that many CTAs: the third generation has to start after the first one's tests, that is
+    // one and a half rounds of CTA slots behind it (one row, V = 32,000: taking the tests for nothing cost 4 us of 20)
+    const long long ahead = static_cast<long long>(P.B) * P.nsplit * (P.G + 1);
+    if (2 * ahead < 3 * cta_slots(dt)) return;
+    P.pos_bits = P.nsplit <= 7 ? 4 : 8;  // twice nsplit arrivals at most
+    // Position by position the tests of one are in before the next one's CTAs start, where a position has a round of CTAs or its
+    // CTAs are short; else batch rows that complete one after the other are worth more (position by position: 256 bf16 rows,
+    // V = 128,256, 131.9 -> 133.3 us, 96 greedy fp32 rows 85.1 -> 86.3; 512 fp32 rows, V = 151,936, 495 -> 475).  A test keeps a CTA
+    // slot for 2.5 us: of short slices only the first two positions (all of them: 1,000 fp32 rows, V = 20,000, 173 -> 184 us,
+    // 600 bf16 rows of 4, V = 14,000, 69.7 -> 76.4), and no more where the rows go one by one.
+    const bool brief = P.per_warp * kWarps * 16 < kBriefSlice;
+    P.rows_major = !brief && static_cast<long long>(P.B) * P.nsplit < cta_slots(dt);
+    P.n_tests = brief || P.rows_major ? 2 : 64 / P.pos_bits;
 }
 
 Plan make_plan(const speckv_batch* bt) {
@@ -332,7 +366,8 @@ bool call_aligned(const speckv_batch* bt, bool verify) {
            (!verify || rows_aligned(bt->target_logits, bt->target_stride_b, bt->target_stride_pos, es));
 }
 
-// How a call of signals / verify / step is cut: sizes, slices and draws.  Returns whether it takes a CTA per batch row.
+// How a call of signals / verify / step is cut: sizes, slices, order and draws.  Returns whether it takes a CTA per batch row.  The
+// outputs and the rows' parameters are in P already.
 bool plan_call(KParams& P, const speckv_batch* bt, int mode) {
     const bool verify = (mode & MODE_VERIFY) != 0;
     P.B = bt->B; P.G = bt->gamma_max; P.V = bt->V;
@@ -342,7 +377,10 @@ bool plan_call(KParams& P, const speckv_batch* bt, int mode) {
     choose_slices(P, bt->dtype, aligned);
     choose_draw(P, bt->dtype, aligned);
     P.n_spans = P.nsplit * kWarps;
-    return choose_batch_rows(P, bt->dtype, aligned);
+    if (choose_batch_rows(P, bt->dtype, aligned)) return true;
+    if (verify) choose_tests(P, bt->dtype);
+    choose_direct(P, bt->dtype, aligned);
+    return false;
 }
 
 // Shared driver of signals / verify / step.
@@ -365,7 +403,6 @@ speckv_status run(const speckv_batch* bt, int mode, const float* comp, const spe
     if (ws_bytes < (verify ? pl.total : pl.total_signals)) return SPECKV_ERR_WORKSPACE;
 
     KParams P{};
-    const bool by_row = plan_call(P, bt, mode);
     P.bits = bt->entropy_in_bits ? 1 : 0;
     P.wait_limit = g_wait_limit.load(std::memory_order_relaxed);
     P.d = bt->draft_logits; P.dsb = bt->draft_stride_b; P.dsp = bt->draft_stride_pos;
@@ -375,6 +412,7 @@ speckv_status run(const speckv_batch* bt, int mode, const float* comp, const spe
     if (mode & MODE_MLP) fill_mlp(P, mlp, comp);
     P.H = H; P.C = C; P.feat = feat; P.scores = scores; P.gamma_next = gamma_next;
     P.n_acc = n_accepted; P.out_tok = out_tokens; P.status = row_status;
+    const bool by_row = plan_call(P, bt, mode);
     char* w = static_cast<char*>(ws);
     P.tick1 = reinterpret_cast<int*>(w + pl.off_tick);
     P.tick2 = P.tick1 + P.B;
@@ -401,27 +439,12 @@ speckv_status run(const speckv_batch* bt, int mode, const float* comp, const spe
         P.rdone = P.n_list + 4;
         P.tokl = reinterpret_cast<float2*>(w + pl.off_tokl);
         P.spans = reinterpret_cast<float2*>(w + pl.off_spans);
-        // position 0 of every batch row first and the later target rows position by position, so that a position's acceptance test is in
-        // before the CTAs of the later target rows start
         P.read_all = (bt->flags & SPECKV_READ_ALL_TARGET_ROWS) ? 1 : 0;
-        // ... where the grid has that many CTAs: the third generation has to start after the first one's tests, that is
-        // one and a half rounds of CTA slots behind it (one row, V = 32,000: taking the tests for nothing cost 4 us of 20)
-        const long long ahead = static_cast<long long>(P.B) * P.nsplit * (P.G + 1);
-        if (2 * ahead >= 3 * cta_slots(bt->dtype)) {
+        if (P.n_tests) {
             P.early = P.rdone + P.B;
             P.tick_pos = reinterpret_cast<unsigned long long*>(w + pl.off_pos);
-            P.pos_bits = P.nsplit <= 7 ? 4 : 8;  // twice nsplit arrivals at most
-            // Position by position the tests of one are in before the next one's CTAs start, where a position has a round of CTAs or its
-            // CTAs are short; else batch rows that complete one after the other are worth more (position by position: 256 bf16 rows,
-            // V = 128,256, 131.9 -> 133.3 us, 96 greedy fp32 rows 85.1 -> 86.3; 512 fp32 rows, V = 151,936, 495 -> 475).  A test keeps a CTA
-            // slot for 2.5 us: of short slices only the first two positions (all of them: 1,000 fp32 rows, V = 20,000, 173 -> 184 us,
-            // 600 bf16 rows of 4, V = 14,000, 69.7 -> 76.4), and no more where the rows go one by one.
-            const bool brief = P.per_warp * kWarps * 16 < kBriefSlice;
-            P.rows_major = !brief && static_cast<long long>(P.B) * P.nsplit < cta_slots(bt->dtype);
-            P.n_tests = brief || P.rows_major ? 2 : 64 / P.pos_bits;
         }
     }
-    choose_direct(P, bt->dtype, call_aligned(bt, verify));
     const cudaError_t e = bt->dtype == SPECKV_BF16 ? launch_all<__nv_bfloat16>(P, cs, ev) : launch_all<float>(P, cs, ev);
     return e == cudaSuccess ? SPECKV_OK : SPECKV_ERR_CUDA;
 }
@@ -731,16 +754,20 @@ int speckv_internal_set_wait_limit(int polls) {
 }
 
 speckv_status speckv_internal_plan(const speckv_batch* batch, int call, int32_t* plan) {
-    if (!plan || call < 0 || call > 2) return SPECKV_ERR_INVALID_ARG;
-    const speckv_status st = check_batch(batch, call == 1);
+    if (!plan || call < 0 || call > 3) return SPECKV_ERR_INVALID_ARG;
+    const bool verify = call == 1 || call == 3;
+    const speckv_status st = check_batch(batch, verify);
     if (st != SPECKV_OK) return st;
     if (batch->B == 0) return SPECKV_ERR_INVALID_ARG;
     KParams P{};
+    P.gamma = batch->gamma; P.temp = batch->temperature;
+    if (call == 3) P.gamma_next = const_cast<int32_t*>(batch->gamma);
     bool by_row = false;
     if (call == 2) plan_sample(P, batch, make_sample_plan(batch));
-    else by_row = plan_call(P, batch, call == 1 ? MODE_SIGNALS | MODE_VERIFY : MODE_SIGNALS);
+    else by_row = plan_call(P, batch, verify ? MODE_SIGNALS | MODE_VERIFY : MODE_SIGNALS);
     const int fine = P.fine > 0 ? P.fine : 1;
     plan[0] = by_row; plan[1] = P.nsplit; plan[2] = P.per_warp; plan[3] = (P.n_spans + fine - 1) / fine; plan[4] = P.R; plan[5] = P.draw_pw;
+    plan[6] = P.direct;
     return SPECKV_OK;
 }
 

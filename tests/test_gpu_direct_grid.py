@@ -9,7 +9,7 @@ import oracle
 import paper_2605_02888_b200 as speckv
 from paper_2605_02888_b200 import binding, synth
 
-from parity import compare_step, gpu_batch, mlp_pair, oracle_batch
+from parity import compare_step, gpu_batch, mlp_pair, oracle_batch, plan_of
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
@@ -65,3 +65,23 @@ def test_waits_that_run_out(B):
     assert (tok == want).all()
     again = speckv.speckv_verify(gpu_batch(s))    # nothing of it stays
     assert all((again[k] == ref[k]).all() for k in ref)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("B,G,V", [(24, 8, 9001), (98, 8, 20000), (256, 2, 8193), (256, 1, 20000), (40, 8, 65541)])
+def test_next_gamma_over_this_steps_gamma(dtype, B, G, V):
+    # grids of one to three rounds of CTAs: the later ones start when the first rows have already written their next gamma
+    w, s = _step(B, G, V, dtype)
+    gm, _ = mlp_pair(synth.make_mlp(w, DEV))
+    bt = gpu_batch(s)
+    assert plan_of(bt._c(), "step")["direct"] and not plan_of(bt._c(), "step_in_place")["direct"]
+    apart = {k: v.clone() for k, v in speckv.speckv_step(bt, s["comp"], gm).items()}
+    gamma = s["gamma"].clone()
+    bt = gpu_batch(dict(s, gamma=gamma))
+    out = speckv.StepOutputs.allocate(bt, gm.n_out)
+    out.gamma_next = gamma
+    for _ in range(4):
+        gamma.copy_(s["gamma"])
+        again = speckv.speckv_step(bt, s["comp"], gm, out=out)
+        for k, v in apart.items():
+            assert torch.equal(v.view(torch.int32), again[k].view(torch.int32)), k

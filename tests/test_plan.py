@@ -73,3 +73,16 @@ def test_which_batches_take_a_cta_per_row():
     assert by_row("step", 1024, 8, 15360) and not by_row("step", 1024, 8, 15361) and not by_row("step", 4096, 8, 15361)
     assert by_row("signals", 2048, 2, 20480) and not by_row("signals", 2048, 1, 20480)
     assert not any(plan_of(batch(B, 4, V, "bf16"), "sample")["by_row"] for B in (1, 64, 4096) for V in (100, 4000, 9000))
+
+
+def test_a_step_that_writes_over_its_gamma_takes_a_list():
+    # CTAs that find their work from the gamma of all rows would see what the first rows' epilogues have written
+    for B, G, V, dtype in [(1, 4, 32000, "fp32"), (100, 8, 20000, "bf16"), (98, 8, 20000, "fp32"), (256, 1, 8193, "bf16"), (37, 8, 50257, "bf16")]:
+        b = batch(B, G, V, dtype)
+        b.gamma = 0x20000
+        b.temperature = 0x30000
+        assert plan_of(b, "step")["direct"] and plan_of(b, "signals")["direct"]
+        in_place = plan_of(b, "step_in_place")
+        assert not in_place["direct"] and not in_place["by_row"]
+        assert {k: in_place[k] for k in ("slices", "per_warp", "spans")} == {k: plan_of(b, "step")[k] for k in ("slices", "per_warp", "spans")}
+    assert plan_of(batch(100, 8, 20000, "bf16"), "step_in_place")["direct"]   # gamma_max for all rows: nothing to write over
