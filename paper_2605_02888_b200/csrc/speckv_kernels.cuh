@@ -383,8 +383,8 @@ __device__ __forceinline__ float warp_maxf(float v) {
 //         cnt = NaN marks a NaN / +inf input.
 //         While it sweeps, a thread keeps its sums against r = fl(m * scale), so that an element's exponent is one
 //         fused multiply-add; partial() moves them to m itself.  That needs r close to m * scale: where it is not (far(): the
-//         rounding of |r| > 2^28 is up to 2^5 and more, or kFloor * scale overflows) the warp's range is folded again by
-//         draft_far(), from differences of logits.
+//         rounding of |r| > 2^28 is up to 2^5 and more, or kFloor * scale overflows or is next to 0) the warp's range is folded
+//         again by draft_far(), from differences of logits.
 // TARGET  a = r (reference, log2 units), b = Z = sum 2^(x*scale - r); c,d unused.  Any r serves that keeps the sum in
 //         range; it is not the maximum.  NaN / +inf inputs surface as a non-finite Z.
 // ARGMAX  a = best value, b = index (bit pattern), c = bad flag (non-zero: NaN / +inf seen).
@@ -464,9 +464,10 @@ struct DraftState {
         add<T>(a, scale);
         add<T>(b, scale);
     }
-    // Sums that are not to be used: see above.  A maximum far below zero that was left behind shows in what it did to them.
+    // Sums that are not to be used: see above.  A maximum far below zero that was left behind shows in what it did to them.  (Below
+    // 2^-93 the exponent of kFloor is above -128, and an element that only stands for none has weight.)
     __device__ __forceinline__ bool far(const float4& part, float scale) const {
-        return !bad && (scale > 0x1p27f || (m > kFloor && !(fabsf(r) <= 0x1p28f)) || !(fabsf(part.z) + fabsf(part.w) < __int_as_float(0x7f800000)));
+        return !bad && (scale > 0x1p27f || scale < 0x1p-93f || (m > kFloor && !(fabsf(r) <= 0x1p28f)) || !(fabsf(part.z) + fabsf(part.w) < __int_as_float(0x7f800000)));
     }
     __device__ __forceinline__ float4 partial(float scale) const {
         const float d = fmaf(m, scale, -r), f = ex2f(-d), z = zsum();  // y against m itself is smaller by d, a rounding
@@ -664,7 +665,7 @@ __device__ __forceinline__ uint4 gran_any(const GranRow& r, int g) {  // outside
 }
 
 // One warp: the draft partial of granules [lo, hi) for logits and temperatures of any size (DraftState::far), every exponent
-// (x - m) * scale from a difference of logits.  Plain rather than fast: a row takes it from |logit| / T of 2e8 on.
+// (x - m) * scale from a difference of logits.  Plain rather than fast: a row takes it from |logit| / T of 2e8 on, or from T of 1.4e28.
 template <typename T>
 __device__ __noinline__ float4 draft_far(const T* p, int V, int lo, int hi, float scale) {
     constexpr int E = 16 / sizeof(T);
@@ -678,7 +679,7 @@ __device__ __noinline__ float4 draft_far(const T* p, int V, int lo, int hi, floa
         for (int j = 0; j < E; ++j) {
             float x = sizeof(T) == 4 ? __uint_as_float(w[j % 4]) : (j & 1) ? bf_hi(w[j / 2]) : bf_lo(w[j / 2]);
             bad |= x != x || x == __int_as_float(0x7f800000);
-            x = fmaxf(x, kFloor);
+            if (!(x > kFloor)) continue;  // no weight at any temperature
             const float y = -fabsf(x - m) * scale, e = ex2f(y);  // y may be infinite (and at scale = inf not a number where x = m)
             if (x > m) {
                 s = e > 0.f ? fmaf(y, cnt + z, s) * e : 0.f;

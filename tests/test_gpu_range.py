@@ -140,3 +140,20 @@ def test_residual_of_two_tied_tokens(dtype, V, n_shards, T, level):
     out, ref = _check(s, n_shards)
     rejected = out["n_accepted"] == 0
     assert 10 < int(rejected.sum()) < 30 and (out["out_tokens"][rejected, 0] == b).all()
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("B,V,n_shards", [(256, 4096, 0), (3, 40001, 0), (180, 100000, 0), (12, 33000, 3)])
+@pytest.mark.parametrize("T", [1e28, 1e29, 1e30, 1e33])
+def test_temperatures_that_flatten_everything(dtype, B, V, n_shards, T):
+    # -2^100 / T is small here: what a masked element counts as must still have no weight, and neither may what stands in for a
+    # tied maximum that is counted apart or for the elements behind a row's end
+    g = torch.Generator(device=DEV).manual_seed(V)
+    draft = torch.randn(3, V, generator=g, device=DEV)
+    draft[1] = 2.0                                  # every element is the maximum
+    draft[2, : V // 2] = float("-inf")
+    target = torch.randn(4, V, generator=g, device=DEV)
+    s = _shared_rows(draft.to(TYPES[dtype]), target.to(TYPES[dtype]), B, T, seed=V)
+    out, ref = _check(s, n_shards)
+    assert (ref["row_status"] == 0).all()
+    np.testing.assert_allclose(ref["H"][0], [math.log(V), math.log(V), math.log(V - V // 2)], rtol=1e-6)
