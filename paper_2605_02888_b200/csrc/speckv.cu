@@ -323,14 +323,14 @@ cudaError_t launch_sliced(KParams P, long long n_draw, cudaStream_t st, cudaEven
         cudaError_t e = launch(prep_direct_kernel, static_cast<unsigned>((words + kThreads - 1) / kThreads), st, P);
         if (e != cudaSuccess) return e;
         if (before_sweep) cudaEventRecord(before_sweep, st);
-        return launch(sweep_kernel<T>, grid, st, P);
+        return launch(sweep_kernel<T, true>, grid, st, P);
     }
     int seg = (P.B + 63) / 64;
     seg = seg < kPrepRows ? kPrepRows : (seg + 31) / 32 * 32;
     cudaError_t e = launch(prep_kernel, static_cast<unsigned>((P.B + seg - 1) / seg), st, P, seg);
     if (e != cudaSuccess) return e;
     if (before_sweep) cudaEventRecord(before_sweep, st);
-    return launch(sweep_kernel<T>, grid, st, P);
+    return launch(sweep_kernel<T, false>, grid, st, P);
 }
 
 template <typename T>

@@ -236,8 +236,14 @@ __device__ __forceinline__ int direct_entry(const KParams& P, int i, DirectEntry
 // all types and all rows but short ones (batch_row_kernel): a persistent ring of bulk copies, which fp32 batches of 384 to 1,024 rows took before, streamed at
 // 6.7 TB/s but drew its tokens in a launch of its own and could leave no row unread (step of 512 fp32 rows, V = 151,936:
 // 578 us with the ring, 523 this way; 384 rows 440 / 394; 1,000 rows, V = 60,000, 535 / 418).
+// A direct grid is a kernel of its own: one body with both ways of finding the work and both ways of drawing spilled 216 / 324
+// bytes (stores / loads) of bf16 and 52 / 44 of fp32 in all batches.  Apart, 32 / 32 and 20 / 16 with the list, 180 / 284 and 20 / 16
+// direct: step of 1,000 bf16 rows of 6, V = 20,000, 128.6 -> 126.3 us, of 1,024, V = 128,256, 388.5 -> 386.1, of 16 23.9 -> 23.4, of 37,
+// V = 50,257, 22.4 -> 21.9, of one fp32 row, V = 32,000, 11.3 -> 10.9, signals of 700 fp32 rows of 4, V = 30,001, 59.0 -> 57.9.  (The
+// direct grid's spills are its draw's, behind a wait: out of line, 20 / 20 bytes, signals of 128 bf16 rows, V = 128,256, take 43.1 us,
+// this way 42.5.)
 // ----------------------------------------------------------------------------------------
-template <typename T>
+template <typename T, bool DIRECT>
 __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sweep_kernel(const __grid_constant__ KParams P) {
     __shared__ float4 sh_part[kWarps];
     __shared__ RowDecide sh_pos[kMaxGamma + 1];
@@ -247,14 +253,14 @@ __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sweep_kernel(c
     __shared__ int sh_early;
     __shared__ float sh_m0[kWarps];
     __shared__ __align__(16) KParams sh_P;
-    __shared__ DirectEntry sh_entry;
+    __shared__ DirectEntry sh_entry;  // DIRECT only, as the next one
     __shared__ int sh_scan[kWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool verify = (P.mode & MODE_VERIFY) != 0;
     const int i = static_cast<int>(blockIdx.x) / P.nsplit, s = static_cast<int>(blockIdx.x) - i * P.nsplit;
     int2 entry = make_int2(0, 0);
     int n_list;
-    if (P.direct) {
+    if constexpr (DIRECT) {
         n_list = direct_entry(P, i, &sh_entry, sh_scan);
         entry = sh_entry.entry;
     } else {
@@ -265,7 +271,7 @@ __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sweep_kernel(c
     }
     if (i >= n_list) {
         const int d = static_cast<int>(blockIdx.x) - n_list * P.nsplit;
-        if (P.direct) {
+        if constexpr (DIRECT) {
             wait_for_predecessors();
             dependents_may_start();
             if (d < P.n_draw) direct_draw<T>(P, d, &sh_src, sh_sum);
@@ -286,7 +292,7 @@ __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sweep_kernel(c
                                  : static_cast<const T*>(P.d) + static_cast<long long>(b) * P.dsb + static_cast<long long>(pos) * P.dsp;
         const int lo = (s * kWarps + warp) * P.per_warp;  // this warp's granules: the CTA's slice is cut into one contiguous range per warp
         WarpSweep<T, SweepShape<T>::kSteps> ws;
-        if (P.direct) {
+        if constexpr (DIRECT) {
             ws.template start<true>(make_row(row, P.V), lo, lo + P.per_warp);
             wait_for_predecessors();
             dependents_may_start();
@@ -295,7 +301,7 @@ __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sweep_kernel(c
             ws.start(make_row(row, P.V), lo, lo + P.per_warp);
             Tf = P.temp ? P.temp[b] : P.temp_scalar;
         }
-        if (threadIdx.x == 0) {
+        if (!DIRECT && threadIdx.x == 0) {
             // one thread reads what is known of the row's stop position, so that the whole CTA takes one decision
             int e = 0x7fffffff;
             if (P.early && gen == 2 && !P.read_all)
@@ -306,7 +312,7 @@ __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sweep_kernel(c
         const bool greedy = (Tf == 0.f);
         scale = row_scale(Tf);
         const long long pidx = (static_cast<long long>(b) * P.J + j) * P.nsplit + s;  // this CTA's partial
-        if (gen == 2 && sh_early <= pos) {
+        if (!DIRECT && gen == 2 && sh_early <= pos) {
             // The walk stopped at a position before this one: the row epilogue never looks here, the partial only has to
             // be finite.
             if (threadIdx.x == 0)
@@ -350,7 +356,7 @@ __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sweep_kernel(c
             }
         }
     } else {
-        if (P.direct) {
+        if constexpr (DIRECT) {
             wait_for_predecessors();
             dependents_may_start();
         }
@@ -366,7 +372,7 @@ __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sweep_kernel(c
         const int n_tickets = row_ok ? n_rows * P.nsplit : 1;
         __threadfence();
         int l = 0;
-        if (P.early && row_ok && pos < gam && pos < P.n_tests) {
+        if (!DIRECT && P.early && row_ok && pos < gam && pos < P.n_tests) {
             const int sh = pos * P.pos_bits;
             const unsigned long long old = atomicAdd(P.tick_pos + b, 1ull << sh);
             l = static_cast<int>(old >> sh & ((1ull << P.pos_bits) - 1)) == 2 * P.nsplit - 1 ? 1 : 0;
@@ -378,12 +384,12 @@ __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sweep_kernel(c
     params_to_shared(P, &sh_P, 32);  // while the tickets travel
     __syncthreads();
     const int last = sh_last;
-    if (last & 1) {
+    if (!DIRECT && (last & 1)) {
         if (warp == 0) test_position<T>(sh_P, b, gam, Tf == 0.f, scale, pos, sh_pos);
         return;
     }
     if (!(last & 2)) return;
-    if (P.export_state) {
+    if (!DIRECT && P.export_state) {
         const long long row0 = static_cast<long long>(b) * P.J;
         if (warp == 0)
             export_epilogue(sh_P, b, gam, Tf, P.part + (row0 + P.G + 1 + lane) * P.nsplit, P.nsplit,
