@@ -517,7 +517,8 @@ speckv_status run_sample(const speckv_batch* bt, const float* uniforms, int32_t*
     cudaError_t e = launch(clear_kernel, n_clear, cs, P.tick1, n_tick);
     if (e != cudaSuccess) return SPECKV_ERR_CUDA;
     const unsigned grid = static_cast<unsigned>(P.B) * P.G * P.nsplit;
-    e = bt->dtype == SPECKV_BF16 ? launch(sample_kernel<__nv_bfloat16>, grid, cs, P) : launch(sample_kernel<float>, grid, cs, P);
+    if (P.fine > 1) e = bt->dtype == SPECKV_BF16 ? launch(sample_kernel<__nv_bfloat16, true>, grid, cs, P) : launch(sample_kernel<float, true>, grid, cs, P);
+    else e = bt->dtype == SPECKV_BF16 ? launch(sample_kernel<__nv_bfloat16, false>, grid, cs, P) : launch(sample_kernel<float, false>, grid, cs, P);
     return e == cudaSuccess ? SPECKV_OK : SPECKV_ERR_CUDA;
 }
 

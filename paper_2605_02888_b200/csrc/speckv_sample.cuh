@@ -23,13 +23,15 @@ __global__ void __launch_bounds__(kThreads) clear_kernel(int* p, int n) {
     for (int i = blockIdx.x * kThreads + threadIdx.x; i < n; i += gridDim.x * kThreads) SPECKV_ST(p[i], 0);
 }
 
-template <typename T>
+// FINE: ranges in pieces (P.fine > 1).  A kernel of its own: in one with the other the short ranges paid 12 / 4 bytes of spills (fp32; bf16
+// 60 / 44) and 8 KB of shared memory, apart neither spills (293 bf16 rows of 8, V = 1,553, 24.7 -> 23.9 us; 256 rows, V = 128,256, 65.8 ->
+// 64.9).
+template <typename T, bool FINE>
 __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sample_kernel(const __grid_constant__ KParams P) {
     __shared__ int sh_last;
     __shared__ float sh_m0[kWarps];
     __shared__ DrawSrc sh_src;
     __shared__ double sh_sum[64];
-    __shared__ float sh_fine[kMostFine * kFineStride];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int r = blockIdx.x / P.nsplit;  // draw: batch row b, drafted position i
     const int s = blockIdx.x - r * P.nsplit;
@@ -51,7 +53,7 @@ __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sample_kernel(
     const bool greedy = (Tf == 0.f);
     const float scale = static_cast<float>(kLog2e / static_cast<double>(greedy ? 1.f : Tf));
     const T* row = static_cast<const T*>(P.d) + static_cast<long long>(b) * P.dsb + static_cast<long long>(i) * P.dsp;
-    const int n = P.n_spans;
+    const int n = P.n_spans, fine = FINE ? P.fine : 1;
     float2* spans = P.spans + static_cast<long long>(r) * n;
     {
         const int lo = (s * kWarps + warp) * P.per_warp;
@@ -63,24 +65,25 @@ __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sample_kernel(
         const int at = s * kWarps + warp;
         if (greedy) {
             const float4 p = ws.template run<PATH_ARGMAX>(m0, scale);
-            if (lane == 0 && at * P.fine < n) SPECKV_ST(spans[at * P.fine], make_float2(p.z != 0.f ? __int_as_float(0x7fc00000) : p.x, p.y));
-        } else if (P.fine == 1) {
+            if (lane == 0 && at * fine < n) SPECKV_ST(spans[at * fine], make_float2(p.z != 0.f ? __int_as_float(0x7fc00000) : p.x, p.y));
+        } else if constexpr (!FINE) {
             const float4 p = ws.template run<PATH_TARGET>(m0, scale);
             if (lane == 0 && at < n) SPECKV_ST(spans[at], make_float2(p.x, p.y));
         } else {
-            const float4 p = ws.template run<PATH_TARGET, true>(m0, scale, nullptr, {sh_fine + threadIdx.x, P.fine, P.fine_groups});
+            __shared__ float sh_fine[kMostFine * kFineStride];
+            const float4 p = ws.template run<PATH_TARGET, true>(m0, scale, nullptr, {sh_fine + threadIdx.x, fine, P.fine_groups});
             __syncwarp();
             // four lanes add up a piece
             const int k = lane >> 2;
             double sum = 0.0;
-            if (k < P.fine) {
+            if (k < fine) {
                 const float* x = sh_fine + k * kFineStride + warp * 32 + (lane & 3) * 8;
 #pragma unroll
                 for (int q = 0; q < 8; ++q) sum += static_cast<double>(x[q]);
             }
             sum += __shfl_xor_sync(0xffffffffu, sum, 1);
             sum += __shfl_xor_sync(0xffffffffu, sum, 2);
-            if (k < P.fine && (lane & 3) == 0 && at * P.fine + k < n) SPECKV_ST(spans[at * P.fine + k], make_float2(p.x, static_cast<float>(sum)));
+            if (k < fine && (lane & 3) == 0 && at * fine + k < n) SPECKV_ST(spans[at * fine + k], make_float2(p.x, static_cast<float>(sum)));
         }
     }
     __syncthreads();
@@ -100,7 +103,7 @@ __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sample_kernel(
     bool bad = false;
     if (greedy) {
         float4 g = make_float4(kFloor, __int_as_float(0x7fffffff), 0.f, 0.f);
-        for (int k = lane * P.fine; k < n; k += 32 * P.fine) {
+        for (int k = lane * fine; k < n; k += 32 * fine) {
             const float2 v = dbg_ok(spans + k, 8, DBG_WS_LOAD) ? __ldcg(spans + k) : make_float2(kFloor, 0.f);
             g = merge_argmax(g, make_float4(v.x, v.y, v.x != v.x ? 1.f : 0.f, 0.f));
         }
@@ -108,8 +111,8 @@ __global__ void __launch_bounds__(kThreads, SweepShape<T>::kCtas) sample_kernel(
         bad = g.z != 0.f || !(g.x > kFloor);
         tok = __float_as_int(g.y);
     } else {
-        tok = draw_from_spans<T>(row, P.V, scale, spans, n, P.per_warp, P.u[r], warp, kWarps, 1, sh_sum, &sh_src, P.fine,
-                                 P.fine_groups * SweepShape<T>::kSteps * 32 * (kVec * static_cast<int>(sizeof(T)) / 16));
+        tok = draw_from_spans<T>(row, P.V, scale, spans, n, P.per_warp, P.u[r], warp, kWarps, 1, sh_sum, &sh_src, fine,
+                                 FINE ? P.fine_groups * SweepShape<T>::kSteps * 32 * (kVec * static_cast<int>(sizeof(T)) / 16) : 0);
         if (tok == kNotMine) return;
         bad = tok < 0;
     }
