@@ -473,10 +473,11 @@ __device__ __forceinline__ int draw_from_spans(const T* row, int V, float scale,
             float2 x = v[0];
 #pragma unroll
             for (int q = 1; q < 8; ++q) if (i == q) x = v[q];
-            // Of a total of one or more, a span of less than 2^-100 counts as empty: its elements, below 2^-126 each, read as 0, so that
-            // a threshold of 0 would find nothing in it.
-            const double weight = static_cast<double>(x.y) * static_cast<double>(ex2f(x.x - R));
-            return weight < 0x1p-100 ? 0.0 : weight;
+            // The reference is the row's largest exponent but for its rounding, 2^6 at most below 2^31.  A span of less than 2^-100 then
+            // has less than 2^-36 of the total and counts as empty: its elements, below 2^-126 each, may read as 0, so that a threshold
+            // of 0 would find nothing in it.  From 2^31 on the reference may lie so far above the row that this is all the row has.
+            const float f = ex2f(x.x - R), y = fabsf(x.x) < 0x1p31f && x.y * f < 0x1p-100f ? 0.f : x.y;
+            return static_cast<double>(y) * static_cast<double>(f);
         }, static_cast<double>(u), &before, &total, &tau);
         const bool none = __any_sync(0xffffffffu, bad) || own < 0;
         if (lane == 0) {

@@ -157,3 +157,25 @@ def test_temperatures_that_flatten_everything(dtype, B, V, n_shards, T):
     out, ref = _check(s, n_shards)
     assert (ref["row_status"] == 0).all()
     np.testing.assert_allclose(ref["H"][0], [math.log(V), math.log(V), math.log(V - V // 2)], rtol=1e-6)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("B,V", [(256, 4096), (40, 40001), (300, 60000), (40, 128256)])
+@pytest.mark.parametrize("level", [2348810240.0, 2969567232.0, -2164260864.0])
+def test_draws_from_rows_far_below_their_reference(dtype, B, V, level):
+    # beyond 2^31 in log2 units the fp32 reference of these levels lies 106 to 120 above the row's exponents, and the whole row weighs
+    # less than 2^-100: it is drawn from all the same, as a sampled draft and for a bonus token
+    scale = np.float32(math.log2(math.e))
+    assert 105 < float(np.float32(level) * scale) - float(np.float32(level)) * float(scale) < 121
+    G, a, b = 2, V // 3, V - 5
+    draft = torch.full((G, V), float("-inf"), device=DEV)
+    draft[:, a] = draft[:, b] = level
+    s = _shared_rows(draft.to(TYPES[dtype]), draft[:1].expand(G + 1, -1).to(TYPES[dtype]), B, 1.0, seed=3)
+    u = torch.linspace(0.02, 0.98, B * G, device=DEV).reshape(G, B).t().contiguous()
+    got = speckv.speckv_sample_draft(gpu_batch(s), u)
+    assert (got["row_status"] == 0).all() and torch.equal(got["tokens"], torch.where(u < 0.5, a, b).to(torch.int32))
+    s["uniforms"][:, :, 0] *= 0.9
+    s["uniforms"][:, G, 1] = u[:, 0]
+    out = speckv.speckv_verify(gpu_batch(s))
+    assert (out["row_status"] == 0).all() and (out["n_accepted"] == G).all()
+    assert torch.equal(out["out_tokens"][:, G], torch.where(u[:, 0] < 0.5, a, b).to(torch.int32))
