@@ -38,9 +38,12 @@ speckv_status speckv_internal_wait_probe(int32_t B, int32_t* row_status, int32_t
                                          size_t workspace_bytes, void* cuda_stream);
 
 /* How a call on this batch is cut (host arithmetic only; the pointers count for their alignment).  call: 0 signals, 1 verify or
- * step, 2 draft sampling, 3 a step that writes the next gamma over this one's.  plan: whether it takes a CTA per batch row; slices per logit row (there: warps per logit row);
- * 16-byte granules per warp; warp ranges with a place for their sums per batch row (sampling: per position); CTAs per residual
- * draw; granules per warp of it; whether the CTAs find their work without a list (direct grid).                                */
+ * step, 2 draft sampling, 3 a step that writes the next gamma over this one's.  plan, 12 words:
+ * whether it takes a CTA per batch row; slices per logit row (there: warps per logit row); 16-byte granules per warp; sums with a
+ * place of their own per batch row (sampling: per position); CTAs per residual draw; granules per warp of it; whether the CTAs
+ * find their work without a list (direct grid); sums per warp range (sampling: its pieces); granules per piece; positions whose
+ * acceptance test is taken ahead of the rest of the row (0: none), bits of each one's arrival counter, and whether the target rows behind
+ * the first position follow one another batch row by batch row.                                                                */
 speckv_status speckv_internal_plan(const speckv_batch* batch, int call, int32_t* plan);
 
 /* Bounds-checked build only (the library built with -DSPECKV_DEBUG, `python -m paper_2605_02888_b200.build

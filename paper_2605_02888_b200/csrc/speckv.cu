@@ -766,9 +766,12 @@ speckv_status speckv_internal_plan(const speckv_batch* batch, int call, int32_t*
     bool by_row = false;
     if (call == 2) plan_sample(P, batch, make_sample_plan(batch));
     else by_row = plan_call(P, batch, verify ? MODE_SIGNALS | MODE_VERIFY : MODE_SIGNALS);
-    const int fine = P.fine > 0 ? P.fine : 1;
-    plan[0] = by_row; plan[1] = P.nsplit; plan[2] = P.per_warp; plan[3] = (P.n_spans + fine - 1) / fine; plan[4] = P.R; plan[5] = P.draw_pw;
+    const int steps = batch->dtype == SPECKV_BF16 ? SweepShape<__nv_bfloat16>::kSteps : SweepShape<float>::kSteps;
+    plan[0] = by_row; plan[1] = P.nsplit; plan[2] = P.per_warp; plan[3] = P.n_spans; plan[4] = P.R; plan[5] = P.draw_pw;
     plan[6] = P.direct;
+    plan[7] = call == 2 ? P.fine : 1;
+    plan[8] = call == 2 ? P.fine_groups * steps * 32 * (kVec * esize(batch->dtype) / 16) : P.per_warp;
+    plan[9] = P.n_tests; plan[10] = P.pos_bits; plan[11] = P.rows_major;
     return SPECKV_OK;
 }
 

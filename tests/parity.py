@@ -52,10 +52,11 @@ def gpu_batch(s: dict, entropy_in_bits=False, temperature_scalar=None, flags=0) 
 def plan_of(c_batch, call: str) -> dict:
     """How a call on this batch (binding._CBatch) is cut; call: "signals", "step", "sample" or "step_in_place" (the next gamma over this
     step's).  Host arithmetic only."""
-    out = (ctypes.c_int32 * 7)()
+    out = (ctypes.c_int32 * 12)()
     rc = speckv.load_library().speckv_internal_plan(ctypes.byref(c_batch), ("signals", "step", "sample", "step_in_place").index(call), out)
     assert rc == 0, rc
-    return dict(zip(("by_row", "slices", "per_warp", "spans", "draw_ctas", "draw_per_warp", "direct"), out))
+    return dict(zip(("by_row", "slices", "per_warp", "spans", "draw_ctas", "draw_per_warp", "direct", "pieces", "piece", "tests", "pos_bits",
+                     "rows_major"), out))
 
 
 def mlp_pair(w: dict, **kw):

@@ -31,6 +31,10 @@ def _step(B, G, V, dtype):
                                    (256, 1, 8193), (257, 1, 8193), (3, 8, 128256)])
 def test_direct_grids(dtype, B, G, V):
     w, s = _step(B, G, V, dtype)
+    plan = plan_of(gpu_batch(s)._c(), "step")
+    assert not plan["by_row"] and plan["direct"] == (B <= 256) and plan_of(gpu_batch(s)._c(), "signals")["direct"] == (B <= 256)
+    assert plan["draw_ctas"] == {(1, "bf16"): 2, (2, "bf16"): 1, (33, "bf16"): 15, (33, "fp32"): 16, (3, "bf16"): 16, (148, "fp32"): 6}.get(
+        (B, dtype), plan["draw_ctas"])
     gm, om = mlp_pair(synth.make_mlp(w, DEV))
     rows = np.arange(B) if B * G * V < 1 << 22 else np.unique(np.r_[0:min(B, 6), np.arange(0, B, max(1, B // 16)), B - 1])
     for _ in range(2):

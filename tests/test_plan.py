@@ -32,15 +32,23 @@ def check(b, call):
     ng = -(-b.V // E) if aligned else (b.V + 2 * (E - 1)) // E   # granules a row can touch
     warps = p["slices"] if p["by_row"] else 8 * p["slices"]
     assert warps * p["per_warp"] >= ng, (p, ng)
-    assert 1 <= p["slices"] <= 32 and p["spans"] <= warps
+    assert 1 <= p["slices"] <= 32 and p["spans"] <= warps * p["pieces"]
+    assert p["pieces"] * p["piece"] >= p["per_warp"]     # every granule of a range is in one of its pieces
     if p["by_row"]:
         assert call != "sample" and 8 % p["slices"] == 0 and p["spans"] == p["slices"]
     else:
         assert p["per_warp"] >= 32 and p["per_warp"] % 32 == 0
-        assert p["spans"] * p["per_warp"] >= ng          # a warp without a place for its sum has no granule
+        assert p["spans"] // p["pieces"] * p["per_warp"] >= ng   # a warp without a place for its sum has no granule
     if call == "step":
-        assert 1 <= p["draw_ctas"] <= 32 and p["draw_ctas"] * 8 * p["draw_per_warp"] >= ng
+        # 16 bytes for each of a direct grid's sums, 8 for another's, in 32 * 8 places of 8
+        assert 1 <= p["draw_ctas"] <= (16 if p["direct"] else 32) and p["draw_ctas"] * 8 * p["draw_per_warp"] >= ng
+        # arrivals of a position: the slices of two rows; places for all tests in a word of 64 bits
+        assert p["tests"] == 0 or (2 * p["slices"] < 1 << p["pos_bits"] and p["tests"] * p["pos_bits"] <= 64)
+        assert not (p["direct"] and (p["by_row"] or p["tests"] or b.B > 256))
+    else:
+        assert p["tests"] == 0 and p["pieces"] <= (8 if call == "sample" else 1)
     if call == "sample":
+        assert p["spans"] <= 256 and not p["direct"] and (p["pieces"] == 1 or p["spans"] % p["pieces"] == 0)
         n = C.c_size_t(0)
         assert speckv.load_library().speckv_sample_workspace_size(C.byref(b), C.byref(n)) == 0
         assert n.value >= 4 * (b.B * b.gamma_max + 2 * b.B) + 8 * b.B * b.gamma_max * p["spans"]
@@ -52,14 +60,19 @@ def test_every_granule_has_a_warp(call):
     rnd = random.Random(5)
     edges = [1, 7, 8, 9, 255, 256, 257, 4095, 4096, 4097, 8191, 8192, 8193, 12288, 12289, 15360, 15361, 16383, 20480, 20481, 32000, 32768,
              50257, 128256, 151936, 1 << 20, (1 << 24) + 5]
-    seen = set()
+    seen, how = set(), set()
     for k in range(4000):
         V = rnd.choice(edges) if k % 2 else int(2 ** rnd.uniform(0, 21))
         B, G = int(2 ** rnd.uniform(0, 12)), rnd.randint(1, 16)
         dtype = rnd.choice(["bf16", "fp32"])
         p = check(batch(B, G, V, dtype, offset=rnd.choice([0, 0, 1, 3]), pad=rnd.choice([0, 0, 8, 5])), call)
         seen.add(("row", p["slices"]) if p["by_row"] else p["slices"])
+        how.add((p["direct"], p["tests"], p["pos_bits"], p["rows_major"]) if call == "step" and not p["by_row"] else p["pieces"])
     assert {1, 2, 15, 16, 17, 32} <= seen and {("row", n) for n in {"signals": (1, 2, 4, 8), "step": (1, 2)}.get(call, ())} <= seen, seen
+    if call == "step":   # direct; a list without tests; of two positions by row and by position; of all, with counters of 4 and 8 bits
+        assert {(1, 0, 0, 0), (0, 0, 0, 0), (0, 2, 4, 1), (0, 2, 4, 0), (0, 16, 4, 0), (0, 8, 8, 0)} <= how, how
+    if call == "sample":
+        assert {1, 2, 3, 5, 8} <= how, how
 
 
 def test_which_batches_take_a_cta_per_row():
