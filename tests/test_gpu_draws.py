@@ -12,7 +12,7 @@ import oracle
 import paper_2605_02888_b200 as speckv
 from paper_2605_02888_b200 import synth, vocab_shard
 
-from parity import compare_step, gpu_batch, mlp_pair, oracle_batch
+from parity import compare_step, gpu_batch, mlp_pair, oracle_batch, plan_of
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
@@ -76,16 +76,17 @@ def test_sampled_drafts_over_slices(dtype, B, G, V):
 
 @pytest.mark.parametrize("dtype", ["bf16", "fp32"])
 @pytest.mark.parametrize("B,G,V", [(1, 1, 1), (1, 1, 255), (2, 3, 257), (1, 2, 2049), (1, 1, 32001), (1, 1, 65535), (2, 1, 65537),
-                                   (1, 1, 200001), (300, 2, 1025)])
+                                   (1, 1, 200001), (300, 2, 1025), (100, 8, 33003), (40, 4, 151936), (200, 1, 300007)])
 def test_sampling_stays_within_its_workspace(dtype, B, G, V):
     # exactly as many bytes as were asked for, what lies behind them unchanged: rows of fewer granules than a slice has lanes, the
-    # most slices, unaligned rows
+    # most slices, unaligned rows, ranges in two to six pieces
     w = _workload(B, G, V, dtype)
     s = synth.make_step(w, 0, DEV)
     s["temperature"][::3] = 0.0
     u = torch.rand(B, G, device=DEV)
     batch = gpu_batch(s)
     n, c = ctypes.c_size_t(0), batch._c()
+    assert (plan_of(c, "sample")["pieces"] > 1) == (B * V > 1000000)
     assert speckv.load_library().speckv_sample_workspace_size(ctypes.byref(c), ctypes.byref(n)) == 0
     mem = torch.full((n.value + 8192,), 0x5A, dtype=torch.uint8, device=DEV)
     a = speckv.speckv_sample_draft(batch, u, workspace=mem[:n.value])
@@ -272,6 +273,11 @@ def test_sampled_drafts_from_pieces(dtype, B, G, V):
     greedy = (s["temperature"].cpu().numpy()[rows] == 0.0)[:, None]
     clear = ((cdf - x).abs().amin(-1) > 1e-6).cpu().numpy() | greedy
     assert (tok[clear] == want[clear]).all()
+    # the two imposed uniforms: a token that may be drawn, with nothing to speak of in front of it and behind it respectively
+    got = torch.as_tensor(tok, device=DEV)[:, :2].long().unsqueeze(-1)
+    share, upto = p[:, :2].gather(-1, got).squeeze(-1), (cdf[:, :2] / cdf[:, :2, -1:]).gather(-1, got).squeeze(-1)
+    sampled = torch.as_tensor(~greedy[:, 0], device=DEV)
+    assert (share[sampled] > 0).all() and (upto - share)[sampled, 0].max() <= 1e-6 and (1.0 - upto)[sampled, 1].max() <= 1e-6
     near = p.clamp(max=2e-6).sum(-1)[:, 2:]
     assert (~clear[:, 2:]).sum() <= float(near.sum() + 4.0 * near.sum().sqrt()) + 1.0
     assert (out["row_status"] == 0).all() and (out["tokens"] >= 0).all()
