@@ -451,8 +451,8 @@ def _same_bits(a, b):
 
 @pytest.mark.parametrize("B,V", [(256, 128256), (300, 8200), (24, 50264)])
 def test_target_rows_behind_a_rejection_are_skipped_without_changing_anything(B, V):
-    # the sweep leaves target rows unread when a rejection at position 0 or 1 is known before their CTAs
-    # start (a matter of timing, so the full-size batch, where it does happen, a batch of short rows and a small
+    # the sweep leaves target rows unread when a rejection at a position in front of them is known before their CTAs
+    # start (here of position 0 or 1; a matter of timing, so the full-size batch, where it does happen, a batch of short rows and a small
     # batch, where it mostly does not): with and without the skipping the outputs are the same bits; and they
     # stay the same when every target row behind a row's stop position is overwritten with NaN, read or not
     w = synth.scaled(synth.WORKLOADS["b256"], B=B, V=V)
@@ -470,6 +470,37 @@ def test_target_rows_behind_a_rejection_are_skipped_without_changing_anything(B,
     behind = (pos > n[:, None]) & (pos <= g[:, None])
     assert int(behind.sum()) > 0
     s["target"][behind] = float("nan")
+    for flags in (0, binding.READ_ALL_TARGET_ROWS):
+        for _ in range(3):
+            _same_bits(skip, speckv.speckv_step(gpu_batch(s, flags=flags), s["comp"], gm))
+
+
+@pytest.mark.parametrize("dtype,B,G,V,mode", [
+    # (tests, bits of a position's counter, rows of a batch row together): the first two positions alone, of long slices and of short
+    # ones; all positions, with counters of 4 bits, and of 8 (eight slices and more), where positions from the ninth on have none
+    ("bf16", 300, 6, 70001, (2, 4, 1)), ("fp32", 300, 6, 20000, (2, 4, 0)), ("fp32", 640, 6, 40001, (16, 4, 0)), ("bf16", 760, 4, 66000, (16, 4, 0)),
+    ("fp32", 80, 4, 530001, (8, 8, 0)), ("fp32", 80, 12, 530000, (8, 8, 0)), ("bf16", 60, 3, 1050000, (2, 8, 1))])
+def test_early_tests_at_every_position_change_nothing(dtype, B, G, V, mode):
+    # walks that end at each position in turn; the same bits with and without skipping, also with NaN in every target row behind
+    w = synth.Workload("early", B=B, gamma_max=G, V=V, dtype=dtype, gamma_mode="fixed", gamma_fixed=G, temperature=0.9, sigma_t=1.0,
+                       sigma_d=(0.3, 1.0, 2.0), seed=V % 89)
+    s = synth.make_step(w, 0, DEV)
+    s["gamma"][1::5] -= 1
+    s["temperature"][3::11] = 0.0
+    stop = torch.arange(B, device=DEV) % (G + 1)
+    pos = torch.arange(G + 1, device=DEV)[None, :]
+    s["uniforms"][:, :, 0] = torch.where(pos == stop[:, None], 1.0 - 2.0 ** -24, 0.0)   # u = 0 accepts whatever p allows
+    plan = plan_of(gpu_batch(s)._c(), "step")
+    assert (plan["tests"], plan["pos_bits"], plan["rows_major"]) == mode, plan
+    gm, om = mlp_pair(synth.make_mlp(w, DEV))
+    skip = {k: v.clone() for k, v in speckv.speckv_step(gpu_batch(s), s["comp"], gm).items()}
+    _same_bits(skip, speckv.speckv_step(gpu_batch(s, flags=binding.READ_ALL_TARGET_ROWS), s["comp"], gm))
+    n, g = skip["n_accepted"].long(), s["gamma"].long()
+    assert int(skip["row_status"].abs().sum()) == 0 and set(range(G)) <= set(n.tolist())
+    rows = np.arange(0, B, max(1, B // 4 if B * G * V > 1 << 27 else B // 16))
+    ref = oracle.step(oracle_batch(s, rows=rows), s["comp"].cpu().numpy()[rows], om)
+    compare_step(skip, ref, rows=rows)
+    s["target"][(pos > n[:, None]) & (pos <= g[:, None])] = float("nan")
     for flags in (0, binding.READ_ALL_TARGET_ROWS):
         for _ in range(3):
             _same_bits(skip, speckv.speckv_step(gpu_batch(s, flags=flags), s["comp"], gm))
