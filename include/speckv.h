@@ -39,7 +39,7 @@
  *     finite and >= 1e-6.
  *   - |logit| / T: any size in the draft signals.  Target rows and rows that a token is sampled from keep the sum of
  *     their exponentials against an fp32 reference in log2 units; from about 1e9 on that reference can be so far from the
- *     row's maximum that the sum overflows, and the row is flagged SPECKV_ROW_NONFINITE.
+ *     row's maximum that the sum overflows, or is lost below 2^-126, and the row is flagged SPECKV_ROW_NONFINITE.
  */
 #ifndef SPECKV_H
 #define SPECKV_H
@@ -163,7 +163,8 @@ speckv_status speckv_sample_draft(const speckv_batch* batch, const float* unifor
  * (plus a second look at the stop position's two rows for a residual draw, and at one short range
  * of the bonus position's row for a bonus draw).
  * gamma_next[b] is the controller's choice for the NEXT step of row b; this step verifies
- * with the gamma given in the batch.  H, C, scores may be NULL.                            */
+ * with the gamma given in the batch, which gamma_next may overwrite (at up to 256 rows such a call
+ * is a few microseconds slower).  H, C, scores may be NULL.                                 */
 speckv_status speckv_step(const speckv_batch* batch, const float* comp, const speckv_mlp* mlp,
                           float* H, float* C, float* feat, float* scores, int32_t* gamma_next,
                           int32_t* n_accepted, int32_t* out_tokens, int32_t* row_status,

@@ -191,7 +191,7 @@ __device__ __noinline__ double gran_weight_any(const DrawSrc s, int g) {
 // ---- sums ----------------------------------------------------------------------------------------------------
 // Sum over whole granules pt[0], pt[32], ... (n left from this lane's first one on) of the weights that the row record says.
 // Two loads per row are in flight (four where the record is known) and none is requested ahead: the other warps of the SM, not this one, hide the latency, and
-// the loop, compiled by itself, keeps to the 48 registers of the sweep kernel without spilling (step of 1,024 bf16 rows,
+// the loop, compiled by itself, does without the spills that the kernel around it has at 48 registers (step of 1,024 bf16 rows,
 // V = 128,256, 430 us; two requested ahead 9 us more, four in flight 5 us more).  The record is fetched behind the first loads.
 // WITH_P: the sum of p as well (.y).
 struct NormOfRecord {  // the row's record in global memory

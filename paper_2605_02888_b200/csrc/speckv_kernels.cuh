@@ -14,6 +14,9 @@
 //                   locates the inverse-CDF threshold and writes the fresh token.  These CTAs
 //                   sit behind the sweep CTAs in the sweep kernel's own grid and wait (bounded)
 //                   for a row of the queue.
+//   direct grid     small batches: prep_direct_kernel clears counters, records and sums; the sweep's CTAs find their logit row from
+//                   gamma and the temperatures themselves (direct_entry), and each batch row has drawing CTAs of its own, which wait
+//                   (bounded) for the row's record and for one another's sums; the last of them in the grid picks (direct_draw).
 //   short rows      one CTA per batch row does all of that in one launch (batch_row_kernel).
 #pragma once
 
@@ -39,8 +42,12 @@ template <typename T> struct SweepShape;
 template <> struct SweepShape<__nv_bfloat16> { static constexpr int kSteps = 4, kCtas = 5; };
 template <> struct SweepShape<float> { static constexpr int kSteps = 4, kCtas = 4; };
 // Every kernel is launched so that its CTAs may be placed as soon as all CTAs of the kernel in front of it in the stream have
-// called dependents_may_start() or ended.  It touches memory only behind wait_for_predecessors(), that is when that kernel has
+// called dependents_may_start() or ended.  It writes memory only behind wait_for_predecessors(), that is when that kernel has
 // ended and its writes are visible, and lets its own successor in after that, so what holds for one holds for the whole chain.
+// It reads behind it too, but for a direct grid's sweep and draft sampling: the kernel in front of them (prep_direct_kernel,
+// clear_kernel) writes nothing but the workspace and has waited for everything in front of it before it let them start, so gamma, the
+// temperatures and the logits are complete in L2 and are read from there, past L1 (ldg_early, __ldcg).  That holds for what no CTA of
+// the same grid writes: a step that writes the next gamma over this one's takes no direct grid (overwrites_rows() in speckv.cu).
 // A kernel is therefore already running while its inputs are written (the drafted tokens, the next gamma and the logits come from
 // the call in front of it), so none of them is read through the non-coherent path (__ldg, ld.global.nc), which is for data that
 // nobody writes while the kernel runs.  Plain loads cost nothing here: all cases within 0.3 %.
@@ -108,8 +115,8 @@ struct KParams {
     int *q_front, *q_back;  // draw queue: rows with a residual draw fill rdone from the front, the others from the back
     int wait_limit;  // polls a resample CTA spends on its row's completion flag before it gives the row up
     // Order of the sweep (verification): first the draft and target row of position 0 of every batch row, then the other draft rows,
-    // last the other target rows, position by position (rows_major: batch row by batch row), which are left unread where the walk is already known to have stopped in
-    // front of them (early != nullptr).
+    // last the other target rows, position by position (rows_major: batch row by batch row), which are left unread where the walk is
+    // already known to have stopped in front of them (early != nullptr).
     int read_all;
     int* early;       // [B] the lowest position + 1 at which a test has ended the walk so far
     unsigned long long* tick_pos;  // [B] arrivals of each position's draft and target slices, pos_bits bits each
@@ -154,7 +161,7 @@ struct KParams {
 // A kernel's parameters for the functions that are not inlined: handed a reference to the parameter itself they fetch every field
 // as global memory, a miss each the first time, and a row epilogue is a chain of cold fields.  With these copied while the tickets
 // travel and one scan less per pick (speckv_draw.cuh): step of 16 bf16 rows, V = 128,256, 33.4 -> 30.7 us, of 64, V = 32,000,
-// 30.8 -> 27.5, of 4, V = 70,528, 16.5 -> 13.7, verification of 96 greedy fp32 rows 89.7 -> 86.7.  Thread first + k copies word k; the
+// 30.8 -> 27.5, of 4, V = 70,528, 16.5 -> 13.7.  Thread first + k copies word k; the
 // caller has a barrier before the first use.
 __device__ __forceinline__ void params_to_shared(const KParams& P, KParams* sh, int first) {
     for (int k = static_cast<int>(threadIdx.x) - first; k >= 0 && k < static_cast<int>(sizeof(KParams) / 4); k += static_cast<int>(blockDim.x) - first)
